@@ -255,7 +255,7 @@ void fp_free(fp_ctx *ctx);                 /* NULL-safe; synchronises the device
    stages together, and a pass never writes the stage state that it reads, so the linked
    reads need no synchronisation beyond the launch order.
    A batch advances many independent blocks (same precision, scheme, metric order)
-   together: one persistent launch per direction pass covers the work of every
+   together: one launch per direction pass covers the work of every
    block, the three RK stages are captured once into a CUDA graph, and each call
    replays it.  Unlinked batches with local Lax-Friedrichs speeds are captured as up to
    four independent chains of the graph, each advancing a group of the blocks of about equal

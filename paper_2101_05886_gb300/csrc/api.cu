@@ -39,9 +39,8 @@ struct fp_ctx {
   BlockDev hblk;
   BlockDev *dblk = nullptr;
   BlockDev uploaded;                  // last BlockDev copied to dblk
-  std::vector<int2> hitems[3];
-  int2 *items[3] = {nullptr, nullptr, nullptr};
-  int nitems[3] = {0, 0, 0};
+  fpk::SweepItem *items[3] = {nullptr, nullptr, nullptr};
+  int ncta[3] = {0, 0, 0};            // CTAs of each direction's launch
   int nsm = 152;
   // CTA shapes of the context's sweep: [0] the primary one, [1] the alternative (nshape == 2,
   // the folded FP32 sweeps): threads (faces per chunk x lines per tile), xi rings padded (every
@@ -57,8 +56,8 @@ struct fp_batch {
   std::vector<fp_ctx *> ctx;
   std::vector<BlockDev> hblk;
   BlockDev *dblk = nullptr;
-  int2 *items[3] = {nullptr, nullptr, nullptr};
-  int nitems[3] = {0, 0, 0};
+  fpk::SweepItem *items[3] = {nullptr, nullptr, nullptr};
+  int ncta[3] = {0, 0, 0};
   double *dt_dev = nullptr;
   double *dt_host = nullptr;   // page-locked, so the per-step upload is asynchronous
   cudaEvent_t dt_ready = nullptr;  // the last upload of dt_host has been consumed
@@ -71,8 +70,8 @@ struct fp_batch {
   // are linked (a block reads its neighbours' stage states) or the LF speeds are global.
   static constexpr int kMaxBranch = 4;
   int nbranch = 1;
-  int2 *bitems[kMaxBranch][3] = {};
-  int bnitems[kMaxBranch][3] = {};
+  fpk::SweepItem *bitems[kMaxBranch][3] = {};
+  int bncta[kMaxBranch][3] = {};
   int nsm = 152;
   int nshape = 1, nt[2] = {128, 128}, pad[2] = {1, 1}, per_sm[2] = {1, 1};   // as fp_ctx (shared by all blocks)
   int shape = 0;                     // the one CTA shape the batch runs (sweep_batch_shape)
@@ -262,33 +261,34 @@ void default_tile(int dir, int nt, int *S, int *TT) {
 void fill_dirs(fp_ctx *c) {
   const int ni = c->desc.n[0], nj = c->desc.n[1], nk = c->desc.n[2], G = c->G;
   const int dims = c->desc.dims;
-  const long long qs1 = ni, qs2 = (long long)ni * nj;
-  const long long ei = ni + 2 * G, ej = nj + 2 * G;
-  const long long ms1 = ei, ms2 = ei * ej;
+  // (strides of the second transverse index do not fit 32 bits only in 2-D, where it is 0)
+  const int qs1 = ni, qs2 = (int)((long long)ni * nj);
+  const int ei = ni + 2 * G, ej = nj + 2 * G;
+  const int ms1 = ei, ms2 = (int)((long long)ei * ej);
   BlockDev &B = c->hblk;
   // direction 0: lines along i, transverse (j, k)
   {
     DirDev &D = B.dir[0];
-    D.nd = ni; D.nt1 = nj; D.nlines = (long long)nj * nk;
+    D.nd = ni; D.nt1 = nj; D.nt2 = nk;
     D.qT1 = qs1; D.qT2 = qs2; D.qsd = 1;
     D.mT1 = ms1; D.mT2 = ms2; D.msd = 1;
-    D.fT1 = ni + 1; D.fT2 = (long long)(ni + 1) * nj; D.fsd = 1;
+    D.fT1 = ni + 1; D.fT2 = (int)((ni + 1LL) * nj); D.fsd = 1;
   }
   // direction 1: lines along j, transverse (i, k)
   {
     DirDev &D = B.dir[1];
-    D.nd = nj; D.nt1 = ni; D.nlines = (long long)ni * nk;
+    D.nd = nj; D.nt1 = ni; D.nt2 = nk;
     D.qT1 = 1; D.qT2 = qs2; D.qsd = qs1;
     D.mT1 = 1; D.mT2 = ms2; D.msd = ms1;
-    D.fT1 = 1; D.fT2 = (long long)ni * (nj + 1); D.fsd = ni;
+    D.fT1 = 1; D.fT2 = (int)(ni * (nj + 1LL)); D.fsd = ni;
   }
   // direction 2: lines along k, transverse (i, j)
   {
     DirDev &D = B.dir[2];
-    D.nd = nk; D.nt1 = ni; D.nlines = (long long)ni * nj;
+    D.nd = nk; D.nt1 = ni; D.nt2 = nj;
     D.qT1 = 1; D.qT2 = qs1; D.qsd = qs2;
     D.mT1 = 1; D.mT2 = ms1; D.msd = ms2;
-    D.fT1 = 1; D.fT2 = ni; D.fsd = (long long)ni * nj;
+    D.fT1 = 1; D.fT2 = ni; D.fsd = qs2;
   }
   for (int d = 0; d < 3; ++d) {
     DirDev &D = B.dir[d];
@@ -302,8 +302,8 @@ void fill_dirs(fp_ctx *c) {
     {
       long long e[3] = {ni, nj, nk};
       e[d] = G;
-      const long long s1 = e[0], s2 = e[0] * e[1];
-      const long long st[3] = {1, s1, s2};
+      const int s1 = (int)e[0], s2 = (int)(e[0] * e[1]);
+      const int st[3] = {1, s1, s2};
       const int ta = d == 0 ? 1 : 0, tb = d == 2 ? 1 : 2;   // the line's t1 and t2 directions
       D.hsd = st[d];
       D.hT1 = st[ta];
@@ -311,13 +311,13 @@ void fill_dirs(fp_ctx *c) {
       D.hc = e[0] * e[1] * e[2];
     }
     default_tile(d, c->nt[0], &D.S, &D.TT);
-    if (d >= dims) D.nlines = 0;
+    if (d >= dims) D.nt2 = 0;
   }
   B.dims = dims;
   B.G = G;
   B.qc = (long long)ni * nj * nk;
   B.mc = c->nmet;
-  B.moff = G + G * ms1 + (dims == 3 ? G * ms2 : 0);
+  B.moff = G + (long long)G * ms1 + (dims == 3 ? (long long)G * ms2 : 0);
   B.met = c->met;
   B.q[0] = nullptr; B.q[1] = c->q1; B.q[2] = c->q2;
   B.racc = c->racc;
@@ -331,23 +331,124 @@ void fill_dirs(fp_ctx *c) {
   for (int d = 0; d < 3; ++d) B.nbr[d][0] = B.nbr[d][1] = -1;
 }
 
-void make_items(const BlockDev &B, int bidx, int d, std::vector<int2> &out) {
+// The work of one block in one direction: `tiles` tiles of TT lines, each tile row a line after
+// the other in a stream of period P = nd + 2 G (see the sweep).
+struct Stream {
+  int block;
+  long long tiles;
+  int P, S, G;
+  long long positions(long long n) const { return n * P - 2 * G; }   // first to last cell of n tiles
+};
+
+Stream stream_of(const BlockDev &B, int block, int d) {
   const DirDev &D = B.dir[d];
-  for (long long L0 = 0; L0 < D.nlines; L0 += D.TT) out.push_back(make_int2(bidx, (int)L0));
+  return {block, ((long long)D.nt1 * D.nt2 + D.TT - 1) / D.TT, D.nd + 2 * B.G, D.S, B.G};
+}
+
+// Cuts the tiles first .. tiles-1 of a stream into pieces of at most `k` chunks, the next piece
+// starting at the position where one ends (an item of n chunks finishes n S - 1 cells: its
+// first face is also its predecessor's last).  Returns their number.
+long long cut_stream(const Stream &s, long long first, long long k, std::vector<fpk::SweepItem> *out) {
+  long long tile = first, u = s.G, n = 0;
+  while (tile < s.tiles) {
+    const long long left = (s.tiles - 1 - tile) * s.P + (s.P - s.G - u);
+    const long long len = std::min(k * s.S - 1, left);
+    if (out) out->push_back({s.block, (int)tile, 1, (int)u, (int)len, -1, {0, 0}});
+    ++n;
+    u += len;
+    tile += u / s.P;
+    u %= s.P;
+    if (u >= s.P - s.G) { ++tile; u = s.G; }      // in the ghosts between two lines: on to the next line
+    if (u < s.G) u = s.G;
+  }
+  return n;
+}
+
+// the pieces of a stream's tiles from `first` on, cut as small as `most` pieces allow
+void spread_stream(const Stream &s, long long first, long long most, std::vector<fpk::SweepItem> &out) {
+  long long lo = 1, hi = (s.positions(s.tiles - first) + s.S) / s.S + 1;
+  while (lo < hi) {
+    const long long mid = (lo + hi) / 2;
+    if (cut_stream(s, first, mid, nullptr) <= most) hi = mid; else lo = mid + 1;
+  }
+  cut_stream(s, first, lo, &out);
+}
+
+// The items of one launch over direction `d`, for a device that holds `slots` CTAs at once;
+// returns the number of CTAs.  Every block gets a share g of the CTAs in proportion to its
+// positions.
+//  - xi: the share's CTAs take equal pieces of the block's stream.  Lines follow each other in
+//    memory, so neighbouring pieces share nothing.
+//  - eta, zeta: a tile is TT adjacent points wide and shares memory sectors with the next, so
+//    CTAs that run at the same time take adjacent tiles: whole rounds go in turn, CTA c the
+//    tiles c, c + g, ... (equal pieces of the stream instead read 3 times the bytes and cost 6 %
+//    on a 256^3 block), and what is left after the rounds is spread in equal pieces.
+//  - One block by itself: two rounds per CTA, so there are more CTAs than slots and those that
+//    run on faster SMs take more of them (256^3 WENO5 step: 8.93 ms, 9.75 ms with all rounds in one
+//    item, 9.97 ms with a CTA per tile in a fixed order and lines padded to chunks).  The blocks of a
+//    batch keep one item for all rounds: its graph's other branches fill the SMs that end
+//    early (64-block WENO5 step: 18.04 ms, 18.25 ms with two rounds per item).
+int make_items(const std::vector<Stream> &streams, int d, int slots, std::vector<fpk::SweepItem> &items) {
+  std::vector<std::vector<fpk::SweepItem>> cta(slots);
+  long long total = 0, done = 0;
+  for (const Stream &s : streams) total += s.tiles * s.P;
+  for (const Stream &s : streams) {
+    // the CTAs c0 .. c0 + g - 1: the block's part of the line [0, total) mapped to the slots, at
+    // least one (which it then shares with a neighbour)
+    const long long c0 = done * slots / total;
+    done += s.tiles * s.P;
+    const long long g = std::max(1LL, done * slots / total - c0);
+    const long long r = d == 0 ? 0 : s.tiles / g;
+    std::vector<fpk::SweepItem> piece;
+    if (r * g < s.tiles) spread_stream(s, r * g, g, piece);
+    const bool alone = streams.size() == 1;
+    const long long per = alone ? 2 : r;          // rounds per item
+    for (long long r0 = 0; r0 < r; r0 += per) {
+      const long long n = std::min(per, r - r0);
+      for (long long c = 0; c < g; ++c) {
+        const fpk::SweepItem it = {s.block, (int)(r0 * g + c), (int)g, s.G, (int)s.positions(n), -1, {0, 0}};
+        if (alone && r > per) cta.push_back({it}); else cta[c0 + c].push_back(it);
+      }
+    }
+    for (size_t c = 0; c < piece.size(); ++c)
+      if (alone && r > per) cta.push_back({piece[c]}); else cta[c0 + c].push_back(piece[c]);
+  }
+  // CTA c's first item at index c, the others behind
+  items.clear();
+  for (const auto &c : cta)
+    if (!c.empty()) items.push_back(c[0]);
+  int n = 0;
+  for (const auto &c : cta) {
+    if (c.empty()) continue;
+    int prev = n++;
+    for (size_t i = 1; i < c.size(); ++i) {
+      items[prev].next = (int)items.size();
+      prev = items[prev].next;
+      items.push_back(c[i]);
+    }
+  }
+  return n;
+}
+
+// the launch's items on the device (replaces *dst)
+cudaError_t put_items(const std::vector<fpk::SweepItem> &items, fpk::SweepItem **dst) {
+  cudaFree(*dst);
+  *dst = nullptr;
+  if (items.empty()) return cudaSuccess;
+  cudaError_t e = fpk::dev_alloc(dst, items.size() * sizeof(fpk::SweepItem));
+  if (e == cudaSuccess)
+    e = cudaMemcpy(*dst, items.data(), items.size() * sizeof(fpk::SweepItem), cudaMemcpyHostToDevice);
+  return e;
 }
 
 int upload_items(fp_ctx *c) {
-  for (int d = 0; d < 3; ++d) {
-    if (c->items[d]) { cudaFree(c->items[d]); c->items[d] = nullptr; }
-    c->hitems[d].clear();
-    if (d < c->desc.dims) make_items(c->hblk, 0, d, c->hitems[d]);
-    c->nitems[d] = (int)c->hitems[d].size();
-    if (c->nitems[d] == 0) continue;
-    cudaError_t e = fpk::dev_alloc(&c->items[d], c->hitems[d].size() * sizeof(int2));
-    if (e != cudaSuccess) return cuda_fail(c, e, "cudaMalloc(items)");
-    e = cudaMemcpy(c->items[d], c->hitems[d].data(), c->hitems[d].size() * sizeof(int2),
-                   cudaMemcpyHostToDevice);
-    if (e != cudaSuccess) return cuda_fail(c, e, "cudaMemcpy(items)");
+  std::vector<fpk::SweepItem> items;
+  for (int d = 0; d < c->desc.dims; ++d) {
+    const DirDev &D = c->hblk.dir[d];
+    const int a = c->nshape == 2 && D.S * D.TT == c->nt[1] ? 1 : 0;
+    c->ncta[d] = make_items({stream_of(c->hblk, 0, d)}, d, c->per_sm[a] * c->nsm, items);
+    cudaError_t e = put_items(items, &c->items[d]);
+    if (e != cudaSuccess) return cuda_fail(c, e, "sweep items");
   }
   return FP_OK;
 }
@@ -358,12 +459,6 @@ int sync_block(fp_ctx *c, cudaStream_t s) {
   if (e != cudaSuccess) return cuda_fail(c, e, "upload block descriptor");
   c->uploaded = c->hblk;
   return FP_OK;
-}
-
-int grid_for(int per_sm, int nsm, int nitems) {
-  long long g = (long long)per_sm * nsm;
-  if (g > nitems) g = nitems;
-  return g < 1 ? 1 : (int)g;
 }
 
 int validate(const fp_grid_desc *d, int ghost_nodes, std::string &why) {
@@ -548,7 +643,7 @@ int fp_init_grid(const fp_grid_desc *desc, const double *xyz, int ghost_nodes, v
   // each a quarter as long (batches pick their tiles by timing them instead)
   for (int d = 1; d < c->desc.dims; ++d) {
     DirDev &D = c->hblk.dir[d];
-    if ((D.nlines + D.TT - 1) / D.TT < (long long)c->per_sm[0] * c->nsm) { D.S = 32; D.TT = c->nt[0] / 32; }
+    if (((long long)D.nt1 * D.nt2 + D.TT - 1) / D.TT < (long long)c->per_sm[0] * c->nsm) { D.S = 32; D.TT = c->nt[0] / 32; }
   }
   int st = upload_items(c);
   if (st != FP_OK) { fp_free(c); return st; }
@@ -570,13 +665,12 @@ static int run_stage(fp_ctx *c, int stage, int rk, cudaStream_t s) {
     fpk::SweepLaunch L;
     L.blocks = c->dblk;
     L.items = c->items[d];
-    L.nitems = c->nitems[d];
+    L.grid = c->ncta[d];
     L.dir = d;
     L.mode = d == 0 ? fpk::MODE_WRITE : (d == dims - 1 ? (rk ? fpk::MODE_RK : fpk::MODE_RHS) : fpk::MODE_ADD);
     L.stage = stage;
     L.dt = c->dt_dev;
     L.alt = shape_of(c, c->hblk.dir[d]);
-    L.grid = grid_for(c->per_sm[L.alt], c->nsm, L.nitems);
     L.bnd = has_bnd(c->desc, d);
     L.glf = c->desc.global_lf;
     cudaError_t e = launch(c->is_f32, L, M, c->desc.scheme, c->desc.characteristic,
@@ -814,40 +908,24 @@ int fp_batch_launches_per_step(const fp_batch *b) {
   return b ? b->nbranch * 3 * (b->dims + (b->global_lf ? 2 : 0)) : 0;
 }
 
-static int batch_items_into(fp_batch *b, int d, const std::vector<int> *only_blocks, int2 **dst, int *ndst);
-
-static int batch_items(fp_batch *b, int d, const std::vector<int> *only_blocks) {
-  return batch_items_into(b, d, only_blocks, &b->items[d], &b->nitems[d]);
-}
-
-static int batch_items_into(fp_batch *b, int d, const std::vector<int> *only_blocks, int2 **dst, int *ndst) {
-  std::vector<std::pair<long long, int2>> work;
-  for (size_t k = 0; k < b->hblk.size(); ++k) {
-    if (only_blocks && std::find(only_blocks->begin(), only_blocks->end(), (int)k) == only_blocks->end())
-      continue;
-    const DirDev &D = b->hblk[k].dir[d];
-    for (long long L0 = 0; L0 < D.nlines; L0 += D.TT) {
-      long long lines = std::min<long long>(D.TT, D.nlines - L0);
-      work.push_back({(long long)D.nd * lines, make_int2((int)k, (int)L0)});
-    }
-  }
-  // largest items first: the persistent grid takes them in order
-  std::stable_sort(work.begin(), work.end(),
-                   [](const std::pair<long long, int2> &x, const std::pair<long long, int2> &y) {
-                     return x.first > y.first;
-                   });
-  std::vector<int2> it(work.size());
-  for (size_t k = 0; k < work.size(); ++k) it[k] = work[k].second;
-  cudaFree(*dst);
-  *dst = nullptr;
-  *ndst = (int)it.size();
-  if (it.empty()) return FP_OK;
-  cudaError_t e = fpk::dev_alloc(dst, it.size() * sizeof(int2));
-  if (e == cudaSuccess) e = cudaMemcpy(*dst, it.data(), it.size() * sizeof(int2), cudaMemcpyHostToDevice);
+// the items of direction d for all blocks or some of them (blocks in index order)
+static int batch_items_into(fp_batch *b, int d, const std::vector<int> *only_blocks, fpk::SweepItem **dst,
+                            int *ncta) {
+  std::vector<Stream> streams;
+  for (size_t k = 0; k < b->hblk.size(); ++k)
+    if (!only_blocks || std::find(only_blocks->begin(), only_blocks->end(), (int)k) != only_blocks->end())
+      streams.push_back(stream_of(b->hblk[k], (int)k, d));
+  std::vector<fpk::SweepItem> items;
+  *ncta = make_items(streams, d, b->per_sm[shape_of(b, b->hblk[0].dir[d])] * b->nsm, items);
+  cudaError_t e = put_items(items, dst);
   if (e != cudaSuccess)
     return bfail(b, e == cudaErrorMemoryAllocation ? FP_ERR_OOM : FP_ERR_CUDA,
                  std::string("batch items: ") + cudaGetErrorString(e));
   return FP_OK;
+}
+
+static int batch_items(fp_batch *b, int d, const std::vector<int> *only_blocks) {
+  return batch_items_into(b, d, only_blocks, &b->items[d], &b->ncta[d]);
 }
 
 static int batch_upload(fp_batch *b, cudaStream_t s) {
@@ -858,18 +936,17 @@ static int batch_upload(fp_batch *b, cudaStream_t s) {
   return FP_OK;
 }
 
-static int batch_pass_items(fp_batch *b, int d, int mode, int stage, cudaStream_t s, const int2 *items,
-                            int nitems) {
+static int batch_pass_items(fp_batch *b, int d, int mode, int stage, cudaStream_t s,
+                            const fpk::SweepItem *items, int ncta) {
   fpk::SweepLaunch L;
   L.blocks = b->dblk;
   L.items = items;
-  L.nitems = nitems;
+  L.grid = ncta;
   L.dir = d;
   L.mode = mode;
   L.stage = stage;
   L.dt = b->dt_dev;
   L.alt = shape_of(b, b->hblk[0].dir[d]);   // every block of a batch pass has the same shape
-  L.grid = grid_for(b->per_sm[L.alt], b->nsm, L.nitems);
   L.bnd = b->bnd[d];
   L.glf = b->global_lf;
   cudaError_t e = launch(b->is_f32, L, b->M, b->scheme, b->charwise, b->fp, s);
@@ -878,7 +955,7 @@ static int batch_pass_items(fp_batch *b, int d, int mode, int stage, cudaStream_
 }
 
 static int batch_pass(fp_batch *b, int d, int mode, int stage, cudaStream_t s) {
-  return batch_pass_items(b, d, mode, stage, s, b->items[d], b->nitems[d]);
+  return batch_pass_items(b, d, mode, stage, s, b->items[d], b->ncta[d]);
 }
 
 // Autotuner: for the batch's CTA shape, each direction and each line-length class, time every
@@ -1042,7 +1119,7 @@ int fp_batch_create_linked(fp_ctx *const *blocks, int nblocks, void *const *q_de
     std::vector<std::vector<int>> grp(b->nbranch);
     for (int k = 0; k < nblocks; ++k) grp[group_of[k]].push_back(k);
     for (int g = 0; g < b->nbranch && !st; ++g)
-      for (int d = 0; d < b->dims && !st; ++d) st = batch_items_into(b, d, &grp[g], &b->bitems[g][d], &b->bnitems[g][d]);
+      for (int d = 0; d < b->dims && !st; ++d) st = batch_items_into(b, d, &grp[g], &b->bitems[g][d], &b->bncta[g][d]);
     if (st) { fp_batch_free(b); return st; }
   }
   // capture the three RK stages x directions into one graph (one chain per branch)
@@ -1066,7 +1143,7 @@ int fp_batch_create_linked(fp_ctx *const *blocks, int nblocks, void *const *q_de
       for (int stage = 0; stage < 3 && !st && e == cudaSuccess; ++stage)
         for (int d = 0; d < b->dims && !st; ++d) {
           int mode = d == 0 ? fpk::MODE_WRITE : (d == b->dims - 1 ? fpk::MODE_RK : fpk::MODE_ADD);
-          st = batch_pass_items(b, d, mode, stage, bs[g], b->bitems[g][d], b->bnitems[g][d]);
+          st = batch_pass_items(b, d, mode, stage, bs[g], b->bitems[g][d], b->bncta[g][d]);
         }
       if (e == cudaSuccess) e = cudaEventRecord(join[g], bs[g]);
       if (e == cudaSuccess) e = cudaStreamWaitEvent(cs, join[g], 0);
@@ -1188,13 +1265,12 @@ extern "C" int fp_rhs_noalloc(fp_ctx *c, const void *q, void *dqdt, void *stream
     fpk::SweepLaunch L;
     L.blocks = S.blk;
     L.items = c->items[d];
-    L.nitems = c->nitems[d];
+    L.grid = c->ncta[d];
     L.dir = d;
     L.mode = d == 0 ? fpk::MODE_WRITE : (d == dims - 1 ? fpk::MODE_RHS : fpk::MODE_ADD);
     L.stage = 0;
     L.dt = c->dt_dev;
     L.alt = shape_of(c, c->hblk.dir[d]);
-    L.grid = grid_for(c->per_sm[L.alt], c->nsm, L.nitems);
     L.bnd = has_bnd(c->desc, d);
     L.glf = c->desc.global_lf;
     e = launch(c->is_f32, L, M, c->desc.scheme, c->desc.characteristic, c->desc.free_stream_preserving, s);

@@ -26,7 +26,7 @@ __global__ void k_cfl(const BlockDev *blk, long long ncells, int ni, int nj, int
     const int j = (int)(r % nj);
     const int k = (int)(r / nj);
     // lines of the xi direction run along i; their transverse strides are those of j and k
-    const long long mo = blk->moff + i + j * blk->dir[0].mT1 + (dims == 3 ? k * blk->dir[0].mT2 : 0);
+    const long long mo = blk->moff + i + (long long)j * blk->dir[0].mT1 + (dims == 3 ? (long long)k * blk->dir[0].mT2 : 0);
     const double rho = (double)q[idx];
     const double u = (double)q[qc + idx] / rho, v = (double)q[2 * qc + idx] / rho,
                  w = (double)q[3 * qc + idx] / rho;
@@ -87,7 +87,7 @@ __global__ void k_lam_max(const BlockDev *blocks, const int2 *items, int nitems,
       const long long r = idx / ni;
       const int j = (int)(r % nj);
       const int k = (int)(r / nj);
-      const long long mo = B->moff + i + j * B->dir[0].mT1 + (dims == 3 ? k * B->dir[0].mT2 : 0);
+      const long long mo = B->moff + i + (long long)j * B->dir[0].mT1 + (dims == 3 ? (long long)k * B->dir[0].mT2 : 0);
       const T rho = q[idx], rinv = T(1) / rho;
       const T u = q[qc + idx] * rinv, v = q[2 * qc + idx] * rinv, w = q[3 * qc + idx] * rinv;
       const T p = (g - T(1)) * (q[4 * qc + idx] - T(0.5) * rho * (u * u + v * v + w * w));

@@ -89,15 +89,16 @@ __device__ __forceinline__ P fpk_in(P p, P base, long long n, int *status) {
 #define FPK_IN(p, base, n, status) (p)
 #endif
 
-// One swept direction of one block.  A "line" runs along the swept direction; the
-// lines of a block are numbered by a flattened transverse index L = t1 + nt1 * t2.
+// One swept direction of one block.  A "line" runs along the swept direction.  Strides of one
+// grid index are 32-bit (extents are at most 2^20 and a block holds fewer than 2^31 points),
+// products with an index 64-bit.
 struct DirDev {
   int nd;              // points along the line
-  int nt1;             // extent of the first transverse coordinate
-  long long nlines;    // number of lines
-  long long qT1, qT2, qsd;  // state offsets: t1, t2 and along-line strides
-  long long mT1, mT2, msd;  // metric offsets (ghosted arrays)
-  long long fT1, fT2, fsd;  // face-metric offsets, face f+1/2 at (f+1)*fsd
+  int nt1;             // extent of the first transverse coordinate (lines are numbered t1 + nt1 t2)
+  int nt2;             // extent of the second one (0 for a direction the block does not sweep)
+  int qT1, qT2, qsd;   // state offsets: t1, t2 and along-line strides
+  int mT1, mT2, msd;   // metric offsets (ghosted arrays)
+  int fT1, fT2, fsd;   // face-metric offsets, face f+1/2 at (f+1)*fsd
   long long fc;        // face-metric component stride
   int bclo, bchi;      // boundary codes at the two line ends
   int S, TT;           // faces per chunk, lines per tile (S * TT == the variant's sweep_threads)
@@ -106,7 +107,8 @@ struct DirDev {
   // FP_BC_HALO sides: the caller's buffers of the G cells beyond each side, laid out like the
   // state with this direction's extent replaced by G (strides: t1, t2, along the line, component)
   const void *halo[2];
-  long long hT1, hT2, hsd, hc;
+  int hT1, hT2, hsd;
+  long long hc;
 };
 
 // 16-byte aligned and padded so that the sweep can copy a descriptor into shared memory in
@@ -131,15 +133,24 @@ struct alignas(16) BlockDev {
   int nbr[3][2];       // FP_BC_BLOCK sides: index of the linked block in the launch's block table
 };
 
+// A work item of the sweep: `len` consecutive positions (cells and the ghost positions between two
+// lines) of one block's stream, the first one position u0 (0 .. nd + 2 G - 1) of tile `tile`;
+// after the end of a tile's line the stream goes on with the tile `stride` further.  Item c is
+// the first of CTA c, `next` the index of the CTA's next item (-1: none).  16-byte aligned:
+// copied into shared memory in 16-byte pieces.
+struct alignas(16) SweepItem {
+  int block, tile, stride, u0;
+  int len, next, pad[2];
+};
+
 struct SweepLaunch {
   const BlockDev *blocks;
-  const int2 *items;   // (block index, first line) per work item
-  int nitems;
+  const SweepItem *items;
   int dir;
   int mode;
   int stage;           // RK stage 0,1,2 (input q[stage], output q[(stage+1)%3])
   const double *dt;    // device scalar
-  int grid;            // CTAs of the persistent launch
+  int grid;            // CTAs of the launch
   int bnd = 0;         // some block of the launch has a slip-wall or cut side in `dir`
   int glf = 0;         // the blocks of the launch use global Lax-Friedrichs speeds
   int alt = 0;         // the blocks' tiles in `dir` are of the alternative CTA shape

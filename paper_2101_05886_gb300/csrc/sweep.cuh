@@ -3,14 +3,15 @@
 // arithmetic type.
 //
 // One CTA owns a tile of TT lines along the swept direction and marches along
-// them in chunks of S faces (S * TT = 256 threads, one face per thread).  Cells
+// them in chunks of S faces (S * TT = the CTA's threads, one face per thread), from
+// the end of one line straight on to the next line of its work item.  Cells
 // enter a shared-memory ring (2S slots per line) once and are reused by every
 // face whose stencil covers them; per-cell primitives and spectral radii are
 // formed once per cell.  Face fluxes go to a second ring, and each cell's
 // residual contribution F'_{i+1/2} - F'_{i-1/2} (Eq. aderivative) is applied in
 // the epilogue: written, accumulated, scaled into dQ/dt, or fused into the
-// Runge-Kutta stage update.  Work items (block, line tile) are taken by a
-// persistent grid, so one launch covers every block of a batch.
+// Runge-Kutta stage update.  The work items of a launch are laid out on the host
+// (make_items in api.cu), so one launch covers every block of a batch.
 //
 // Face flux in difference form (Eq. my_point1 with the split of Eq.
 // flux_split_detail): with Q* = Q~_{i+1/2}/(1/J)_{i+1/2} (Eq. Q_star, order-M
@@ -349,8 +350,8 @@ __device__ __forceinline__ void dflux_pair(T g1, typename PairOf<T>::type rinvB,
 // FIX = 2 is the same sweep with the alternative CTA shape of sweep_threads (fp_internal.h).
 template <typename T, int M, int SCHEME, bool BND, int FIX>
 __global__ void __launch_bounds__(sweep_threads(sizeof(T) == 4, SCHEME, FIX), sweep_min_ctas(sizeof(T) == 4, SCHEME, FIX))
-fp_sweep(const BlockDev *__restrict__ blocks, const int2 *__restrict__ items, int nitems, int dir,
-         int mode, int stage, const double *__restrict__ dtp, int charwise_arg, int fpform_arg) {
+fp_sweep(const BlockDev *__restrict__ blocks, const SweepItem *__restrict__ items, int dir, int mode,
+         int stage, const double *__restrict__ dtp, int charwise_arg, int fpform_arg) {
   // this variant's CTA shape (fp_internal.h): threads, ring stride of a staged field, padding
   constexpr int kThreads = sweep_threads(sizeof(T) == 4, SCHEME, FIX);
   constexpr int kRing = sweep_ring(sizeof(T) == 4, SCHEME, FIX);
@@ -367,37 +368,35 @@ fp_sweep(const BlockDev *__restrict__ blocks, const int2 *__restrict__ items, in
   T *const epb = nsb + kNextFields * kThreads;              // epilogue operands, per thread
   const int tid = threadIdx.x;
   // Work-item descriptors in shared memory, double-buffered: during an item's first chunk
-  // the next item's (block, first line) and its whole block descriptor are copied in with
-  // cp.async, so an item starts without a chain of dependent global loads, and the chunk
-  // loop reads buffer pointers from here rather than through an L1 that the streamed cells
-  // keep evicting.
+  // the next item of this CTA and its whole block descriptor are copied in with cp.async, so an
+  // item starts without a chain of dependent global loads, and the chunk loop reads buffer
+  // pointers from here rather than through an L1 that the streamed cells keep evicting.
   static_assert(sizeof(BlockDev) % 16 == 0, "descriptor copied in 16-byte pieces");
   constexpr int kDescPieces = (int)(sizeof(BlockDev) / 16);
   __shared__ __align__(16) unsigned char s_desc[2][sizeof(BlockDev)];
-  __shared__ __align__(16) int2 s_item[2];
+  __shared__ __align__(16) SweepItem s_item[2];
   __shared__ T s_dt;
   __shared__ T s_lam[3];                // global Lax-Friedrichs speeds of this item's direction
   auto fetch_desc = [&](int buf, int blk) {
     for (int p = tid; p < kDescPieces; p += kThreads)
       cp_async16(s_desc[buf] + 16 * p, reinterpret_cast<const unsigned char *>(blocks + blk) + 16 * p);
   };
-  if (blockIdx.x < nitems) {            // the first item's descriptor, loaded before the loop
-    if (tid == 0) s_item[0] = items[blockIdx.x];
-    __syncthreads();
-    fetch_desc(0, s_item[0].x);
-    cp_async_commit();
-    cp_async_wait_all();
-    __syncthreads();
-  }
+  // this CTA's first item and its descriptor, loaded before the loop
+  fetch_desc(0, items[blockIdx.x].block);
+  if (tid == 0) s_item[0] = items[blockIdx.x];
+  cp_async_commit();
+  cp_async_wait_all();
+  __syncthreads();
 
   int cur = 0;
-  for (int it = blockIdx.x; it < nitems; it += gridDim.x, cur ^= 1) {
-    const int2 item = s_item[cur];
+  for (int it = blockIdx.x; it >= 0; cur ^= 1) {
+    const SweepItem &item = s_item[cur];
     const BlockDev *B = reinterpret_cast<const BlockDev *>(s_desc[cur]);
     const DirDev *D = &B->dir[dir];
-    const int nit = it + gridDim.x;
-    // the next item's (block, first line): lands by this item's prologue barrier
-    if (tid == 0 && nit < nitems) cp_async8(&s_item[cur ^ 1], items + nit);
+    const int nit = item.next;
+    // the next item: lands by this item's prologue barrier
+    if (tid < 2 && nit >= 0) cp_async16(reinterpret_cast<unsigned char *>(&s_item[cur ^ 1]) + 16 * tid,
+                                        reinterpret_cast<const unsigned char *>(items + nit) + 16 * tid);
     if (tid == 0) {                      // read after the prologue's barrier
       s_dt = mode == MODE_RK ? T(*dtp) : T(0);
       if (!FIX && B->global_lf)
@@ -417,18 +416,39 @@ fp_sweep(const BlockDev *__restrict__ blocks, const int2 *__restrict__ items, in
     const int SS = slotFast ? 1 : TT;
     const int lbase = tl * LS;
     const int wm = W - 1;
-    const int nd = D->nd;
-    const long long L = (long long)item.y + tl;
-    const bool lineOK = L < D->nlines;
-    const int t1 = lineOK ? (int)(L % D->nt1) : 0;
-    const int t2 = lineOK ? (int)(L / D->nt1) : 0;
-    const long long qbase = t1 * D->qT1 + t2 * D->qT2, qsd = D->qsd;
-    const long long mbase = B->moff + t1 * D->mT1 + t2 * D->mT2, msd = D->msd;
-    const long long fbase = t1 * D->fT1 + t2 * D->fT2, fsd = D->fsd, fcs = D->fc;
+    const int nd = D->nd, nt1 = D->nt1, nt2 = D->nt2;
+    const int qsd = D->qsd, msd = D->msd, fsd = D->fsd;
+    const long long fcs = D->fc;
     const long long qc = B->qc, mc = B->mc;
     const int G = B->G, bclo = D->bclo, bchi = D->bchi;
-    const T *__restrict__ met = static_cast<const T *>(B->met) + mbase;
-    const T *__restrict__ fmet = static_cast<const T *>(D->fmet) + fbase;
+    // The lines of a tile row are marched as one stream of positions: line after line, each with
+    // its G ghost cells at both ends (period P).  `u` is a position within its line (cell
+    // x = u - G) and (t1, t2) that line's transverse coordinates.  A chunk may cover the end of
+    // one line and the start of the next: 2 G - 1 idle faces between two lines, where whole chunks
+    // per line (32 faces along xi) left 15 idle on average, 25 % of the pass for 96 points; and
+    // the next line's loads are in flight like any others (xi pass of eight batch blocks, 1.9M
+    // points: 124.8 -> 102.4 us, 86.9M -> 73.6M warp instructions).
+    const int P = nd + 2 * G;
+    // the position w steps after the start of the item's first tile
+    auto locate = [&](int w, int &u, int &t1, int &t2) {
+      int line = item.tile * TT + tl;
+      while (w >= P) { w -= P; line += TT * item.stride; }
+      u = w;
+      t2 = line / nt1;
+      t1 = line - t2 * nt1;
+    };
+    const int step2 = TT * item.stride / nt1, step1 = TT * item.stride - step2 * nt1;
+    auto wrap = [&](int &u, int &t1, int &t2) {
+#pragma unroll 1
+      while (u >= P) {
+        u -= P;
+        t1 += step1;
+        t2 += step2;
+        if (t1 >= nt1) { t1 -= nt1; ++t2; }
+      }
+    };
+    const T *__restrict__ met = static_cast<const T *>(B->met) + B->moff;
+    const T *__restrict__ fmet = static_cast<const T *>(D->fmet);
     const T *__restrict__ qin = static_cast<const T *>(B->q[stage]);
     const T g1 = T(B->gamma - 1.0), gam = T(B->gamma);
     const int glf = FIX ? 0 : B->global_lf;
@@ -446,20 +466,22 @@ fp_sweep(const BlockDev *__restrict__ blocks, const int2 *__restrict__ items, in
       FPK_CHK_ONLY(if (o < 0 || o >= kRing) { atomicOr(B->status, ST_BOUNDS); return 0; })
       return o;
     };
-    FPK_CHK_ONLY(const T *const metb = static_cast<const T *>(B->met);
-                 const T *const fmetb = static_cast<const T *>(D->fmet);)
+    // offsets of line (t1, t2) in the state, the ghosted metrics and the face metrics
+    auto qline = [&](int t1, int t2) { return (long long)t1 * D->qT1 + (long long)t2 * D->qT2; };
+    auto mline = [&](int t1, int t2) { return (long long)t1 * D->mT1 + (long long)t2 * D->mT2; };
+    auto fline = [&](int t1, int t2) { return (long long)t1 * D->fT1 + (long long)t2 * D->fT2; };
 
-    // boundary rule of a cell index x of this line: the source cell (its first component
+    // boundary rule of cell index x of line (t1, t2): the source cell (its first component
     // at src, component stride cs), or the far-field state (far); `wall` asks for the
     // momentum to be reflected about the boundary face's normal.  Codes: 0 periodic, 1 far
     // field, 2 zero gradient, 3 slip wall (mirror cell), 4 C-grid cut (mirror cell on the line
     // with t1 reversed, wall outside the cut width), 5 another block of the batch (its cells
     // next to its opposite side, same transverse indices, same RK stage), 6 the caller's halo
     // buffer of that side (the cells another process holds, refreshed for every RK stage).
-    auto bc_source = [&](int x, const T *&src, long long &cs, bool &far,
+    auto bc_source = [&](int x, int t1, int t2, const T *&src, long long &cs, bool &far,
                          bool &wall FPK_CHK_ONLY(, const T *&sb, long long &sn)) {
       int xx = x;
-      long long qsrc = qbase;
+      int s1 = t1;
       cs = qc; far = false; wall = false;
       FPK_CHK_ONLY(sb = qin; sn = 5 * qc;)
       if (x < 0 || x >= nd) {
@@ -468,36 +490,35 @@ fp_sweep(const BlockDev *__restrict__ blocks, const int2 *__restrict__ items, in
         else if (bc == 1) far = true;
         else if (bc == 2 || !BND) xx = x < 0 ? 0 : nd - 1;
         else if (bc == 6) {   // halo buffer: index x + G below the line, x - nd above it
-          const long long hx = x < 0 ? (long long)(x + G) : (long long)(x - nd);
-          src = static_cast<const T *>(D->halo[x < 0 ? 0 : 1]) + t1 * D->hT1 + t2 * D->hT2 + hx * D->hsd;
+          const long long hx = x < 0 ? x + G : x - nd;
+          src = static_cast<const T *>(D->halo[x < 0 ? 0 : 1]) + (long long)t1 * D->hT1 + (long long)t2 * D->hT2 +
+                hx * D->hsd;
           cs = D->hc;
           FPK_CHK_ONLY(sb = static_cast<const T *>(D->halo[x < 0 ? 0 : 1]); sn = 5 * D->hc;)
           return;
-        } else if (bc == 5) {   // rare path: the line's (t1, t2) are recovered from its offset
+        } else if (bc == 5) {
           const BlockDev *NB = blocks + B->nbr[dir][x < 0 ? 0 : 1];
           const DirDev *ND = &NB->dir[dir];
-          const long long s2 = qbase / D->qT2, s1 = (qbase - s2 * D->qT2) / D->qT1;
-          src = static_cast<const T *>(NB->q[stage]) + s1 * ND->qT1 + s2 * ND->qT2 +
+          src = static_cast<const T *>(NB->q[stage]) + (long long)t1 * ND->qT1 + (long long)t2 * ND->qT2 +
                 (long long)(x < 0 ? ND->nd + x : x - nd) * ND->qsd;
           cs = NB->qc;
           FPK_CHK_ONLY(sb = static_cast<const T *>(NB->q[stage]); sn = 5 * NB->qc;)
           return;
         } else {
           xx = x < 0 ? -1 - x : 2 * nd - 1 - x;
-          const long long T1 = D->qT1;
-          const int n1 = D->nt1, cw = B->cut;
-          const int s1 = (int)((qbase / T1) % n1);
-          if (bc == 4 && (s1 < cw || s1 >= n1 - cw)) qsrc = qbase + (long long)(n1 - 1 - 2 * s1) * T1;
+          const int cw = B->cut;
+          if (bc == 4 && (t1 < cw || t1 >= nt1 - cw)) s1 = nt1 - 1 - t1;
           else wall = true;
         }
       }
-      src = qin + qsrc + (long long)xx * qsd;
+      src = qin + qline(s1, t2) + (long long)xx * qsd;
     };
 
     // global loads of one cell (Q, metric vector, 1/J) with the boundary rule applied
-    auto fetch = [&](int x, T Q[5], T k[3], T &invJ) {
+    auto fetch = [&](int x, int t1, int t2, T Q[5], T k[3], T &invJ) {
       if (x >= -G && x < nd + G) {
-        const long long mo = (long long)x * msd;
+        const long long mo = mline(t1, t2) + (long long)x * msd;
+        FPK_CHK_ONLY(const T *const metb = static_cast<const T *>(B->met);)
 #pragma unroll
         for (int a = 0; a < 3; ++a) k[a] = *FPK_IN(met + ((3LL * dir + a) * mc + mo), metb, 10 * mc, B->status);
         invJ = *FPK_IN(met + (9LL * mc + mo), metb, 10 * mc, B->status);
@@ -505,7 +526,7 @@ fp_sweep(const BlockDev *__restrict__ blocks, const int2 *__restrict__ items, in
         long long cs;
         bool far, wall;
         FPK_CHK_ONLY(const T *sb; long long sn;)
-        bc_source(x, qp, cs, far, wall FPK_CHK_ONLY(, sb, sn));
+        bc_source(x, t1, t2, qp, cs, far, wall FPK_CHK_ONLY(, sb, sn));
         if (far) {
 #pragma unroll
           for (int v = 0; v < 5; ++v) Q[v] = qb[v];
@@ -514,9 +535,9 @@ fp_sweep(const BlockDev *__restrict__ blocks, const int2 *__restrict__ items, in
           for (int v = 0; v < 5; ++v) Q[v] = __ldg(FPK_IN(qp + v * cs, sb, sn, B->status));
           // slip wall: reflect about the boundary face of this line (face -1/2 or nd-1/2)
           if (BND && wall)
-            wall_reflect<T>(Q, FPK_IN(fmet + (x < 0 ? 0LL : (long long)nd * fsd), fmetb, fcs, B->status), fcs);
+            wall_reflect<T>(Q, FPK_IN(fmet + (fline(t1, t2) + (x < 0 ? 0LL : (long long)nd * fsd)), fmet, fcs, B->status), fcs);
         }
-      } else {   // beyond every stencil that a face of this line uses
+      } else {   // before the first line of the item: no face of a line uses it
 #pragma unroll
         for (int v = 0; v < 5; ++v) Q[v] = qb[v];
         k[0] = T(1); k[1] = T(0); k[2] = T(0);
@@ -548,49 +569,41 @@ fp_sweep(const BlockDev *__restrict__ blocks, const int2 *__restrict__ items, in
       cp[CF_AC * kRing] = c * Num<T>::sqrt_(gx * gx + gy * gy + gz * gz);
     };
 
-    // asynchronous copy of one cell's loads into this thread's staging slots
-    // asynchronous copy of the face metric of face ff into staging slot `slot` (0/1,
-    // alternating between chunks)
-    auto prefetch_face = [&](int ff, int slot) {
+    // asynchronous copy of the face metric of face x + 1/2 of line (t1, t2) into staging slot
+    // `slot` (0/1, alternating between chunks)
+    auto prefetch_face = [&](int x, int t1, int t2, int slot) {
       T *dst = nsb + tid + (9 + 3 * slot) * kThreads;
+      const long long fo = fline(t1, t2) + (long long)(x + 1) * fsd;
 #pragma unroll
       for (int c = 0; c < 3; ++c)
-        cp_async_el(dst + c * kThreads, FPK_IN(fmet + c * fcs + (long long)(ff + 1) * fsd, fmetb, 3 * fcs, B->status));
+        cp_async_el(dst + c * kThreads, FPK_IN(fmet + (c * fcs + fo), fmet, 3 * fcs, B->status));
     };
-    auto prefetch_cell = [&](int x) {
+    // asynchronous copy of one cell's loads (-G <= x < nd + G) into this thread's staging slots
+    auto prefetch_cell = [&](int x, int t1, int t2) {
       T *dst = nsb + tid;
-      if (x >= -G && x < nd + G) {
-        const long long mo = (long long)x * msd;
+      const long long mo = mline(t1, t2) + (long long)x * msd;
+      FPK_CHK_ONLY(const T *const metb = static_cast<const T *>(B->met);)
 #pragma unroll
-        for (int a = 0; a < 3; ++a)
-          cp_async_el(dst + (5 + a) * kThreads, FPK_IN(met + (3LL * dir + a) * mc + mo, metb, 10 * mc, B->status));
-        cp_async_el(dst + 8 * kThreads, FPK_IN(met + 9LL * mc + mo, metb, 10 * mc, B->status));
-        const T *qp;
-        long long cs;
-        bool far, wall;
-        FPK_CHK_ONLY(const T *sb; long long sn;)
-        bc_source(x, qp, cs, far, wall FPK_CHK_ONLY(, sb, sn));
-        if (far) {
-#pragma unroll
-          for (int v = 0; v < 5; ++v) dst[v * kThreads] = qb[v];
-        } else {   // a wall ghost copies its mirror cell; the reflection is applied when staged
-#pragma unroll
-          for (int v = 0; v < 5; ++v) cp_async_el(dst + v * kThreads, FPK_IN(qp + v * cs, sb, sn, B->status));
-        }
-      } else {
+      for (int a = 0; a < 3; ++a)
+        cp_async_el(dst + (5 + a) * kThreads, FPK_IN(met + ((3LL * dir + a) * mc + mo), metb, 10 * mc, B->status));
+      cp_async_el(dst + 8 * kThreads, FPK_IN(met + (9LL * mc + mo), metb, 10 * mc, B->status));
+      const T *qp;
+      long long cs;
+      bool far, wall;
+      FPK_CHK_ONLY(const T *sb; long long sn;)
+      bc_source(x, t1, t2, qp, cs, far, wall FPK_CHK_ONLY(, sb, sn));
+      if (far) {
 #pragma unroll
         for (int v = 0; v < 5; ++v) dst[v * kThreads] = qb[v];
-        dst[5 * kThreads] = T(1);
-        dst[6 * kThreads] = T(0);
-        dst[7 * kThreads] = T(0);
-        dst[8 * kThreads] = T(1);
+      } else {   // a wall ghost copies its mirror cell; the reflection is applied when staged
+#pragma unroll
+        for (int v = 0; v < 5; ++v) cp_async_el(dst + v * kThreads, FPK_IN(qp + v * cs, sb, sn, B->status));
       }
     };
-    // asynchronous copy of the epilogue operands of cell x (residual accumulator,
-    // Q^n, metric differences, face metric of x+1/2) into this thread's slots
-    auto prefetch_epilogue = [&](int x) {
+    // asynchronous copy of the epilogue operands of a cell (state offset qo: residual
+    // accumulator, Q^n, metric differences) into this thread's slots
+    auto prefetch_epilogue = [&](long long qo) {
       T *dst = epb + tid;
-      const long long qo = qbase + (long long)x * qsd;
       if (mode != MODE_WRITE) {
         const T *ra = static_cast<const T *>(B->racc) + qo;
 #pragma unroll
@@ -611,18 +624,26 @@ fp_sweep(const BlockDev *__restrict__ blocks, const int2 *__restrict__ items, in
       }
     };
 
-    const int nch = (nd + 1 + S - 1) / S;
-    // prologue: the first chunk's window [a0-4, a0+S+4), a0 = -1, and its faces' metrics
-    if (lineOK) {
-      if (tf - 1 < nd) prefetch_face(tf - 1, 0);
+    // Within an item, faces and cells are numbered from its first cell (0, at position item.u0):
+    // ring slots go by that number.  Chunk ch computes faces a .. a+S-1, a = ch S - 1, and then
+    // finishes cells max(a, 0) .. a+S-1.
+    const int len = item.len, nch = (len + S) / S;   // faces -1 .. len - 1
+    int u, t1, t2;                       // position of this thread's face of the current chunk
+    locate(item.u0 - 1 + tf, u, t1, t2);
+    // prologue: the first chunk's window, cells [a-4, a+S+4), a = -1, and its faces' metrics
+    {
+      if (t2 < nt2 && u >= G - 1 && u < nd + G) prefetch_face(u - G, t1, t2, 0);
       cp_async_commit();
       // S >= 8, so the window's S + 8 cells are one per thread plus a second one for the
       // threads tf < 8: both loads are issued before either cell is staged
-      const bool two = tf < 8;
+      int ua, a1, a2, ub2, b1, b2;
+      locate(item.u0 - 5 + tf, ua, a1, a2);
+      locate(item.u0 - 5 + tf + S, ub2, b1, b2);
+      const bool one = a2 < nt2, two = tf < 8 && b2 < nt2;
       T Qa[5], ka[3], ija, Qb[5], kb[3], ijb;
-      fetch(-5 + tf, Qa, ka, ija);
-      if (two) fetch(-5 + tf + S, Qb, kb, ijb);
-      stage_cell(-5 + tf, Qa, ka, ija);
+      if (one) fetch(ua - G, a1, a2, Qa, ka, ija);
+      if (two) fetch(ub2 - G, b1, b2, Qb, kb, ijb);
+      if (one) stage_cell(-5 + tf, Qa, ka, ija);
       if (two) stage_cell(-5 + tf + S, Qb, kb, ijb);
     }
     cp_async_wait_all();
@@ -630,16 +651,25 @@ fp_sweep(const BlockDev *__restrict__ blocks, const int2 *__restrict__ items, in
 
     for (int ch = 0; ch < nch; ++ch) {
       const int a = ch * S - 1;                      // first face of the chunk
+      const bool more = ch + 1 < nch;
+      // this thread's face u - G + 1/2 and cell u - G of line (t1, t2)
+      const bool faceOK = t2 < nt2 && u >= G - 1 && u < nd + G && a + tf < len;
+      const bool cellOK = faceOK && u >= G && (ch > 0 || tf > 0);
       // ---- start the loads this chunk's epilogue and the next chunk need
-      const bool nextOK = lineOK && ch + 1 < nch;
-      if (lineOK && a + tf >= 0 && a + tf < nd) prefetch_epilogue(a + tf);
-      if (nextOK) prefetch_cell(a + S + 4 + tf);
-      if (nextOK && a + S + tf < nd) prefetch_face(a + S + tf, (ch + 1) & 1);
-      if (ch == 0 && nit < nitems) fetch_desc(cur ^ 1, s_item[cur ^ 1].x);   // next item's descriptor
+      if (cellOK) prefetch_epilogue(qline(t1, t2) + (long long)(u - G) * qsd);
+      if (more) {
+        int un = u + S, n1 = t1, n2 = t2;            // this thread's face of the next chunk
+        wrap(un, n1, n2);
+        if (n2 < nt2 && un >= G - 1 && un < nd + G) prefetch_face(un - G, n1, n2, (ch + 1) & 1);
+        un += 4;                                     // the cell it stages for the next chunk
+        wrap(un, n1, n2);
+        if (n2 < nt2 && a + S + tf < len) prefetch_cell(un - G, n1, n2);
+      }
+      if (ch == 0 && nit >= 0) fetch_desc(cur ^ 1, s_item[cur ^ 1].block);   // next item's descriptor
       cp_async_commit();
       // ---- one face per thread: face ff + 1/2 between cells ff and ff+1
       const int ff = a + tf;
-      if (lineOK && ff < nd) {
+      if (faceOK) {
         const int i0 = ff;
         int o[8];
 #pragma unroll
@@ -988,8 +1018,8 @@ fp_sweep(const BlockDev *__restrict__ blocks, const int2 *__restrict__ items, in
       __syncthreads();
       // ---- residual of cell x = a + tf from its two faces, then the epilogue
       const int x = a + tf;
-      if (lineOK && x >= 0 && x < nd) {
-        const long long qo = qbase + (long long)x * qsd;
+      if (cellOK) {
+        const long long qo = qline(t1, t2) + (long long)(u - G) * qsd;
         const int ox = off(x), oxm = off(x - 1);
         T R[5];
 #pragma unroll
@@ -1064,23 +1094,31 @@ fp_sweep(const BlockDev *__restrict__ blocks, const int2 *__restrict__ items, in
       }
       __syncthreads();
       // ---- stage the next chunk's new cell from this thread's staging slots
-      if (nextOK) {
-        const int xs = a + S + 4 + tf;
+      u += S;
+      wrap(u, t1, t2);
+      int uc = u + 4, c1 = t1, c2 = t2;
+      wrap(uc, c1, c2);
+      if (more && c2 < nt2 && a + S + tf < len) {
         const T *src = nsb + tid;
         T Q[5] = {src[0], src[kThreads], src[2 * kThreads], src[3 * kThreads], src[4 * kThreads]};
         const T k[3] = {src[5 * kThreads], src[6 * kThreads], src[7 * kThreads]};
-        if (BND && xs >= nd && xs < nd + G && bchi >= 3) {   // past the high end: slip-wall ghost?
-          const T *qp;
-          long long cs;
-          bool far, wall;
-          FPK_CHK_ONLY(const T *sb; long long sn;)
-          bc_source(xs, qp, cs, far, wall FPK_CHK_ONLY(, sb, sn));
-          if (wall) wall_reflect<T>(Q, FPK_IN(fmet + (long long)nd * fsd, fmetb, fcs, B->status), fcs);
+        if (BND) {                                   // a slip-wall ghost?
+          const int xs = uc - G;
+          if (xs < 0 ? bclo >= 3 : xs >= nd && bchi >= 3) {
+            const T *qp;
+            long long cs;
+            bool far, wall;
+            FPK_CHK_ONLY(const T *sb; long long sn;)
+            bc_source(xs, c1, c2, qp, cs, far, wall FPK_CHK_ONLY(, sb, sn));
+            if (wall)
+              wall_reflect<T>(Q, FPK_IN(fmet + (fline(c1, c2) + (xs < 0 ? 0LL : (long long)nd * fsd)), fmet, fcs, B->status), fcs);
+          }
         }
-        stage_cell(xs, Q, k, src[8 * kThreads]);
+        stage_cell(a + S + 4 + tf, Q, k, src[8 * kThreads]);
       }
       __syncthreads();
     }
+    it = nit;
   }
 }
 
@@ -1095,9 +1133,9 @@ template <typename T, int M, int SCHEME, bool BND, int FIX>
 cudaError_t launch_one(const SweepLaunch &L, int charwise, int fp, cudaStream_t s) {
   constexpr size_t smem = sweep_smem<T, SCHEME, FIX>();
   constexpr int nt = sweep_threads(sizeof(T) == 4, SCHEME, FIX);
-  if (L.nitems <= 0) return cudaSuccess;
-  fp_sweep<T, M, SCHEME, BND, FIX><<<L.grid, nt, smem, s>>>(L.blocks, L.items, L.nitems, L.dir, L.mode,
-                                                            L.stage, L.dt, charwise, fp);
+  if (L.grid <= 0) return cudaSuccess;
+  fp_sweep<T, M, SCHEME, BND, FIX><<<L.grid, nt, smem, s>>>(L.blocks, L.items, L.dir, L.mode, L.stage, L.dt,
+                                                            charwise, fp);
   return cudaGetLastError();
 }
 

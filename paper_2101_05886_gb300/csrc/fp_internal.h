@@ -206,8 +206,8 @@ cudaError_t build_metrics(const MetricJob &J, cudaStream_t s);
 cudaError_t convert_f64_to_f32(const double *src, float *dst, long long n, cudaStream_t s);
 
 // Global Lax-Friedrichs speeds (cfl.cu): zero, then max over (block, first point) items of
-// kLamChunk points each.
-constexpr int kLamChunk = 8192;
+// kLamChunk points each (the kernel's threads).
+constexpr int kLamChunk = 256;
 cudaError_t launch_lambda(const BlockDev *blocks, int nblocks, const int2 *items, int nitems,
                           int is_f32, int charwise, int stage, cudaStream_t s);
 

@@ -446,7 +446,26 @@ int upload_items(fp_ctx *c) {
   for (int d = 0; d < c->desc.dims; ++d) {
     const DirDev &D = c->hblk.dir[d];
     const int a = c->nshape == 2 && D.S * D.TT == c->nt[1] ? 1 : 0;
-    c->ncta[d] = make_items({stream_of(c->hblk, 0, d)}, d, c->per_sm[a] * c->nsm, items);
+    // FP64: one CTA's warps keep the SM's FP64 pipe busy (two lanes per clock and SM), so what counts is
+    // the chunks of the SM with the most: fewer CTAs than fit, if their equal shares then
+    // leave no SM with one CTA more than others (37 x 40 x 26 points, 9 passes: 1.79 ms with a share per
+    // slot).  FP32 needs the resident warps to hide latency: a share per slot.
+    int per_sm = c->per_sm[a];
+    if (!c->is_f32) {
+      long long least = -1;
+      for (int m = c->per_sm[a]; m >= 1; --m) {
+        const int n = make_items({stream_of(c->hblk, 0, d)}, d, m * c->nsm, items);
+        long long most = 0;                       // chunks of one CTA
+        for (int k = 0; k < n; ++k) {
+          long long ch = 0;
+          for (int i = k; i >= 0; i = items[i].next) ch += (items[i].len + D.S) / D.S;
+          most = std::max(most, ch);
+        }
+        const long long cost = (n + c->nsm - 1) / c->nsm * most;
+        if (least < 0 || 20 * cost < 19 * least) { least = cost; per_sm = m; }
+      }
+    }
+    c->ncta[d] = make_items({stream_of(c->hblk, 0, d)}, d, per_sm * c->nsm, items);
     cudaError_t e = put_items(items, &c->items[d]);
     if (e != cudaSuccess) return cuda_fail(c, e, "sweep items");
   }

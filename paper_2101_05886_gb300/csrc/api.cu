@@ -196,19 +196,17 @@ int has_halo(const fp_grid_desc &d) {
 int ghost_of(int M, int scheme) { return std::max(scheme == FP_WENO7_JS ? 4 : 3, M / 2); }
 
 // resident CTAs per SM of the sweep variants a context runs (folded switches or not; the fewer
-// of the plain and the boundary-rule instantiation), after opting every variant in to its
-// dynamic shared memory
+// of the plain and the boundary-rule instantiation), after opting both in to their dynamic
+// shared memory
 int prepare(int is_f32, int M, int scheme, int fix) {
   using P = int (*)(int, int);
-  const P f32[6] = {fpk::prepare_sweep_f32, fpk::prepare_sweep_f32_fix, fpk::prepare_sweep_f32_fix2,
-                    fpk::prepare_sweep_f32_bnd, fpk::prepare_sweep_f32_bnd_fix, fpk::prepare_sweep_f32_bnd_fix2};
-  const P f64[6] = {fpk::prepare_sweep_f64, fpk::prepare_sweep_f64_fix, nullptr,
-                    fpk::prepare_sweep_f64_bnd, fpk::prepare_sweep_f64_bnd_fix, nullptr};
+  const P f32[8] = {fpk::prepare_sweep_f32,     fpk::prepare_sweep_f32_fix,     fpk::prepare_sweep_f32_fix2,
+                    fpk::prepare_sweep_f32_comp, fpk::prepare_sweep_f32_bnd,    fpk::prepare_sweep_f32_bnd_fix,
+                    fpk::prepare_sweep_f32_bnd_fix2, fpk::prepare_sweep_f32_bnd_comp};
+  const P f64[8] = {fpk::prepare_sweep_f64,     fpk::prepare_sweep_f64_fix, nullptr, fpk::prepare_sweep_f64_comp,
+                    fpk::prepare_sweep_f64_bnd, fpk::prepare_sweep_f64_bnd_fix, nullptr, fpk::prepare_sweep_f64_bnd_comp};
   const P *p = is_f32 ? f32 : f64;
-  int nb[6] = {1 << 20, 1 << 20, 1 << 20, 1 << 20, 1 << 20, 1 << 20};
-  for (int v = 0; v < 6; ++v)
-    if (p[v]) nb[v] = p[v](M, scheme);
-  return std::min(nb[fix], nb[3 + fix]);
+  return std::min(p[fix](M, scheme), p[4 + fix](M, scheme));
 }
 
 // the CTA shapes of a sweep (fp_internal.h sweep_threads) and their resident CTAs per SM
@@ -230,25 +228,25 @@ int shape_of(const C *c, const fpk::DirDev &D) {
   return c->nshape == 2 && D.S * D.TT == c->nt[1] ? 1 : 0;
 }
 
-// the switches are folded for characteristic FP sweeps with local speeds (not for WENOCU6,
-// whose sweep measured 1 % slower with them folded)
+// the sweep's variant: 3 component-wise; 1 switches folded, for characteristic FP sweeps with
+// local speeds (not for WENOCU6, whose sweep measured 1 % slower with them folded); 0 the rest
 int fix_of(int scheme, int charwise, int fp, int global_lf) {
-  return charwise && fp && !global_lf && scheme != FP_WENOCU6 ? 1 : 0;
+  return !charwise ? 3 : (fp && !global_lf && scheme != FP_WENOCU6 ? 1 : 0);
 }
 
 // the variant of the launch: boundary rules compiled in when some block of the launch has such a
 // side in its direction, the switches folded as fix_of says
 cudaError_t launch(int is_f32, const fpk::SweepLaunch &L, int M, int scheme, int charwise, int fp,
                    cudaStream_t s) {
-  using F = cudaError_t (*)(const fpk::SweepLaunch &, int, int, int, int, cudaStream_t);
-  const F f32[4] = {fpk::launch_sweep_f32, fpk::launch_sweep_f32_fix, fpk::launch_sweep_f32_bnd,
-                    fpk::launch_sweep_f32_bnd_fix};
-  const F f64[4] = {fpk::launch_sweep_f64, fpk::launch_sweep_f64_fix, fpk::launch_sweep_f64_bnd,
-                    fpk::launch_sweep_f64_bnd_fix};
-  const int fix = fix_of(scheme, charwise, fp, L.glf);
-  if (is_f32 && fix && L.alt)
-    return (L.bnd ? fpk::launch_sweep_f32_bnd_fix2 : fpk::launch_sweep_f32_fix2)(L, M, scheme, charwise, fp, s);
-  return (is_f32 ? f32 : f64)[(L.bnd ? 2 : 0) + fix](L, M, scheme, charwise, fp, s);
+  using F = cudaError_t (*)(const fpk::SweepLaunch &, int, int, int, cudaStream_t);
+  const F f32[8] = {fpk::launch_sweep_f32,     fpk::launch_sweep_f32_fix,     fpk::launch_sweep_f32_fix2,
+                    fpk::launch_sweep_f32_comp, fpk::launch_sweep_f32_bnd,    fpk::launch_sweep_f32_bnd_fix,
+                    fpk::launch_sweep_f32_bnd_fix2, fpk::launch_sweep_f32_bnd_comp};
+  const F f64[8] = {fpk::launch_sweep_f64,     fpk::launch_sweep_f64_fix, nullptr, fpk::launch_sweep_f64_comp,
+                    fpk::launch_sweep_f64_bnd, fpk::launch_sweep_f64_bnd_fix, nullptr, fpk::launch_sweep_f64_bnd_comp};
+  int v = fix_of(scheme, charwise, fp, L.glf);
+  if (v == 1 && is_f32 && L.alt) v = 2;
+  return (is_f32 ? f32 : f64)[(L.bnd ? 4 : 0) + v](L, M, scheme, fp, s);
 }
 
 // default tile of a direction for a CTA of nt threads: 32 faces along xi, 8 across lines
@@ -366,7 +364,10 @@ long long cut_stream(const Stream &s, long long first, long long k, std::vector<
 
 // the pieces of a stream's tiles from `first` on, cut as small as `most` pieces allow
 void spread_stream(const Stream &s, long long first, long long most, std::vector<fpk::SweepItem> &out) {
-  long long lo = 1, hi = (s.positions(s.tiles - first) + s.S) / s.S + 1;
+  // a piece of k chunks finishes k S - 1 positions, and pieces may leave out those between lines
+  const long long n = s.tiles - first;
+  long long lo = std::max(1LL, n * (s.P - 2 * s.G) / (most * s.S));
+  long long hi = (s.positions(n) + most) / (most * s.S) + 1;
   while (lo < hi) {
     const long long mid = (lo + hi) / 2;
     if (cut_stream(s, first, mid, nullptr) <= most) hi = mid; else lo = mid + 1;

@@ -7,13 +7,13 @@
 
 namespace fpk {
 
-constexpr int kCellFields = 17;      // per-cell values staged in shared memory
+constexpr int kCellFields = 14;      // per-cell values staged in shared memory
 constexpr int kFaceFields = 10;      // per-face values staged in shared memory (W, delta)
 constexpr int kNextFields = 15;      // staged per thread: next chunk's cell (Q, k, 1/J), face metrics x2
 constexpr int kEpiFields = 13;       // epilogue operands staged per thread (accumulator, Q^n, dk)
 
 // CTA shape of a sweep variant (precision, scheme, fix: 0 switches read at run time, 1 folded,
-// 2 folded with the alternative shape): its threads, which equal faces per chunk x lines per
+// 2 folded with the alternative shape, 3 component-wise): its threads, which equal faces per chunk x lines per
 // tile, whether the rings of the xi pass (lines of 2S slots, one after the other) are padded to
 // 3S slots per line so that every tile shape is free of bank conflicts (unpadded, the xi pass
 // takes S = 32 only), and the CTAs one SM holds.
@@ -32,7 +32,7 @@ constexpr int kEpiFields = 13;       // epilogue operands staged per thread (acc
 // kernels of two shapes there would not share SMs, so a batch runs one shape throughout):
 // linear upwind the alternative (64 threads: +12 %), the others the primary.
 __host__ __device__ constexpr bool sweep_has_alt(bool f32, int scheme, int fix) {
-  return f32 && fix != 0 && scheme >= 0 && scheme <= 2;
+  return f32 && (fix == 1 || fix == 2) && scheme >= 0 && scheme <= 2;
 }
 __host__ __device__ constexpr int sweep_batch_shape(bool f32, int scheme, int fix) {
   return sweep_has_alt(f32, scheme, fix) && scheme == 1 ? 1 : 0;
@@ -57,11 +57,10 @@ enum : int {
   CF_K = 5,      // 5..7 metric vector of the swept direction (d_x, d_y, d_z)/J
   CF_INVJ = 8,   // 1/J
   CF_RINV = 9,   // 1/rho
-  CF_U = 10,     // 10..12 velocity
-  CF_H = 13,     // total enthalpy
-  CF_SQR = 14,   // sqrt(rho)
-  CF_UC = 15,    // contravariant velocity u . grad(d), grad(d) = J k
-  CF_AC = 16     // c |grad(d)|
+  CF_H = 10,     // total enthalpy
+  CF_SQR = 11,   // sqrt(rho)
+  CF_UC = 12,    // contravariant velocity u . grad(d), grad(d) = J k
+  CF_AC = 13     // c |grad(d)|
 };
 
 enum : int { MODE_WRITE = 0, MODE_ADD = 1, MODE_RHS = 2, MODE_RK = 3 };
@@ -159,29 +158,37 @@ struct SweepLaunch {
 // Launchers of the sweep, one per translation unit (sweep_<NAME>.cu): precision f32 / f64,
 // `_bnd` with the slip-wall, cut, link and halo rules compiled in, `_fix` with the
 // characteristic decomposition and the FP form fixed on, `_fix2` the same in the alternative
-// CTA shape (FP32 only).  Each returns the cudaError_t of the
+// CTA shape (FP32 only), `_comp` component-wise.  Each returns the cudaError_t of the
 // launch; prepare_sweep_<NAME> opts in to the dynamic shared memory of its 16 (M, scheme)
 // variants and returns the resident CTAs per SM of the given one.
-cudaError_t launch_sweep_f32(const SweepLaunch &L, int M, int scheme, int charwise, int fp, cudaStream_t s);
-cudaError_t launch_sweep_f32_fix(const SweepLaunch &L, int M, int scheme, int charwise, int fp, cudaStream_t s);
-cudaError_t launch_sweep_f32_bnd(const SweepLaunch &L, int M, int scheme, int charwise, int fp, cudaStream_t s);
-cudaError_t launch_sweep_f32_bnd_fix(const SweepLaunch &L, int M, int scheme, int charwise, int fp, cudaStream_t s);
-cudaError_t launch_sweep_f32_fix2(const SweepLaunch &L, int M, int scheme, int charwise, int fp, cudaStream_t s);
-cudaError_t launch_sweep_f32_bnd_fix2(const SweepLaunch &L, int M, int scheme, int charwise, int fp, cudaStream_t s);
-cudaError_t launch_sweep_f64(const SweepLaunch &L, int M, int scheme, int charwise, int fp, cudaStream_t s);
-cudaError_t launch_sweep_f64_fix(const SweepLaunch &L, int M, int scheme, int charwise, int fp, cudaStream_t s);
-cudaError_t launch_sweep_f64_bnd(const SweepLaunch &L, int M, int scheme, int charwise, int fp, cudaStream_t s);
-cudaError_t launch_sweep_f64_bnd_fix(const SweepLaunch &L, int M, int scheme, int charwise, int fp, cudaStream_t s);
+cudaError_t launch_sweep_f32(const SweepLaunch &L, int M, int scheme, int fp, cudaStream_t s);
+cudaError_t launch_sweep_f32_fix(const SweepLaunch &L, int M, int scheme, int fp, cudaStream_t s);
+cudaError_t launch_sweep_f32_fix2(const SweepLaunch &L, int M, int scheme, int fp, cudaStream_t s);
+cudaError_t launch_sweep_f32_comp(const SweepLaunch &L, int M, int scheme, int fp, cudaStream_t s);
+cudaError_t launch_sweep_f32_bnd(const SweepLaunch &L, int M, int scheme, int fp, cudaStream_t s);
+cudaError_t launch_sweep_f32_bnd_fix(const SweepLaunch &L, int M, int scheme, int fp, cudaStream_t s);
+cudaError_t launch_sweep_f32_bnd_fix2(const SweepLaunch &L, int M, int scheme, int fp, cudaStream_t s);
+cudaError_t launch_sweep_f32_bnd_comp(const SweepLaunch &L, int M, int scheme, int fp, cudaStream_t s);
+cudaError_t launch_sweep_f64(const SweepLaunch &L, int M, int scheme, int fp, cudaStream_t s);
+cudaError_t launch_sweep_f64_fix(const SweepLaunch &L, int M, int scheme, int fp, cudaStream_t s);
+cudaError_t launch_sweep_f64_comp(const SweepLaunch &L, int M, int scheme, int fp, cudaStream_t s);
+cudaError_t launch_sweep_f64_bnd(const SweepLaunch &L, int M, int scheme, int fp, cudaStream_t s);
+cudaError_t launch_sweep_f64_bnd_fix(const SweepLaunch &L, int M, int scheme, int fp, cudaStream_t s);
+cudaError_t launch_sweep_f64_bnd_comp(const SweepLaunch &L, int M, int scheme, int fp, cudaStream_t s);
 int prepare_sweep_f32(int M, int scheme);
 int prepare_sweep_f32_fix(int M, int scheme);
+int prepare_sweep_f32_fix2(int M, int scheme);
+int prepare_sweep_f32_comp(int M, int scheme);
 int prepare_sweep_f32_bnd(int M, int scheme);
 int prepare_sweep_f32_bnd_fix(int M, int scheme);
-int prepare_sweep_f32_fix2(int M, int scheme);
 int prepare_sweep_f32_bnd_fix2(int M, int scheme);
+int prepare_sweep_f32_bnd_comp(int M, int scheme);
 int prepare_sweep_f64(int M, int scheme);
 int prepare_sweep_f64_fix(int M, int scheme);
+int prepare_sweep_f64_comp(int M, int scheme);
 int prepare_sweep_f64_bnd(int M, int scheme);
 int prepare_sweep_f64_bnd_fix(int M, int scheme);
+int prepare_sweep_f64_bnd_comp(int M, int scheme);
 
 // Every device and page-locked allocation of the library goes through these two, so the
 // host-side hook fp_debug_fail_allocation can make a chosen one fail as if the device (or

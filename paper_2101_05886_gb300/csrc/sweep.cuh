@@ -41,15 +41,21 @@ namespace fpk {
 
 template <typename T> struct Num;
 template <> struct Num<double> {
-  // reciprocal of a finite nonzero x: the PTX approximation (relative error about 2^-20)
-  // refined by two Newton-Raphson steps y <- y + y (1 - x y), which square the error twice
+  // reciprocal of a finite nonzero x: the PTX approximation (relative error about 2^-20) and one
+  // step of Householder's third-order iteration, y <- y + y (e + e^2) with e = 1 - x y, which
+  // cubes the error (three operations; two Newton-Raphson steps take four)
   static __device__ __forceinline__ double rcp(double x) {
     double y;
     asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-    y = fma(y, fma(-x, y, 1.0), y);
-    return fma(y, fma(-x, y, 1.0), y);
+    const double e = fma(-x, y, 1.0);
+    return fma(y, fma(e, e, e), y);
   }
-  static __device__ __forceinline__ double div(double a, double b) { return a / b; }
+  // max(m, |x|), m >= 0: doubles without sign are ordered like their bits, and integer compares
+  // leave the FP64 pipe alone
+  static __device__ __forceinline__ double amax(double m, double x) {
+    const long long a = __double_as_longlong(m), b = __double_as_longlong(fabs(x));
+    return __longlong_as_double(a > b ? a : b);
+  }
   static __device__ __forceinline__ double sqrt_(double x) { return sqrt(x); }
   static __device__ __forceinline__ double rsqrt_(double x) { return rsqrt(x); }
   static __device__ __forceinline__ double ld(const void *p, long long i) {
@@ -64,7 +70,7 @@ template <> struct Num<float> {
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
     return r;
   }
-  static __device__ __forceinline__ float div(float a, float b) { return a * rcp(b); }
+  static __device__ __forceinline__ float amax(float m, float x) { return fmaxf(m, fabsf(x)); }
   static __device__ __forceinline__ float sqrt_(float x) {
     float r;
     asm("sqrt.approx.f32 %0, %1;" : "=f"(r) : "f"(x));
@@ -94,36 +100,47 @@ __device__ __forceinline__ dpair pmul(dpair a, dpair b) { return dpair{a.x * b.x
 template <typename P> __device__ __forceinline__ P psub(P a, P b) { return pfma(b, pmk(decltype(a.x)(-1), decltype(a.x)(-1)), a); }
 template <typename P> __device__ __forceinline__ P pc(decltype(P::x) v) { return pmk(v, v); }
 
-// Fifth-order reconstruction of a pair of five-point stencils (the + side and the
-// mirrored - side of one characteristic field) in first-difference form; returns
-// the two reconstructed values.
-template <typename T, int SCHEME>
+// WENO5-JS reconstruction of a pair of five-point stencils (the + side and the mirrored - side of
+// one characteristic field) in first-difference form; returns the two reconstructed values.
+// The stencil values come at half the size of the split values f+-, and 4 times the smoothness
+// indicators of that half-size stencil are formed, (second difference)^2 13/3 + (first)^2, one
+// operation per square: the same numbers as the indicators of f+-, with the same epsilon.
+// FP64: the weights 1/10, 6/10, 3/10 over beta^2 are brought to the common denominator
+// beta0^2 beta1^2 beta2^2, one reciprocal instead of four (a reciprocal takes three operations
+// of the FP64 pipe, which bounds that sweep; the products stay in range up to indicators of
+// 1e77).  FP32 takes the reciprocals, which run on their own unit: the products would leave
+// the FP32 range at indicators of 4e9.
+template <typename T>
 __device__ __forceinline__ typename PairOf<T>::type recon5_pair(
     typename PairOf<T>::type v0, typename PairOf<T>::type v1, typename PairOf<T>::type v2,
     typename PairOf<T>::type v3, typename PairOf<T>::type v4) {
   using P = typename PairOf<T>::type;
-  const P a = psub(v1, v0), b = psub(v2, v1), c = psub(v3, v2), d = psub(v4, v3);
-  const P r0 = pfma(pc<P>(T(5)), b, pmul(pc<P>(T(-2)), a));      // 6 (q0 - v2)
-  const P r1 = pfma(pc<P>(T(2)), c, b);                          // 6 (q1 - v2)
-  const P r2 = pfma(pc<P>(T(4)), c, pmul(pc<P>(T(-1)), d));      // 6 (q2 - v2)
-  if (SCHEME == 1) {
-    const P s = pfma(pc<P>(T(0.3)), r2, pfma(pc<P>(T(0.6)), r1, pmul(pc<P>(T(0.1)), r0)));
-    return pfma(pc<P>(T(1.0 / 6.0)), s, v2);
-  }
-  const P d0 = psub(b, a), e0 = pfma(pc<P>(T(3)), b, pmul(pc<P>(T(-1)), a));
-  const P d1 = psub(c, b), e1 = padd(b, c);
-  const P d2 = psub(d, c), e2 = pfma(pc<P>(T(-3)), c, d);
-  const P c13 = pc<P>(T(13.0 / 12.0)), q4 = pc<P>(T(0.25)), eps = pc<P>(T(1.0e-6));
-  const P b0 = pfma(c13, pmul(d0, d0), pfma(q4, pmul(e0, e0), eps));
-  const P b1 = pfma(c13, pmul(d1, d1), pfma(q4, pmul(e1, e1), eps));
-  const P b2 = pfma(c13, pmul(d2, d2), pfma(q4, pmul(e2, e2), eps));
+  // first differences a, b, c, d, two of them negated so that no combination needs a negation
+  const P a = psub(v1, v0), nb = psub(v1, v2), c = psub(v3, v2), nd = psub(v3, v4);
+  const P d0 = padd(nb, a), d1 = padd(c, nb), d2 = padd(c, nd);  // second differences (signs free)
+  const P e0 = pfma(pc<P>(T(3)), nb, a), e1 = psub(c, nb), e2 = pfma(pc<P>(T(3)), c, nd);
+  const P r0 = pfma(pc<P>(T(-2)), e0, nb);                       // 6 (q0 - v2) = 5 b - 2 a
+  const P r1 = padd(e1, c);                                      // 6 (q1 - v2) = b + 2 c
+  const P r2 = padd(e2, c);                                      // 6 (q2 - v2) = 4 c - d
+  const P c133 = pc<P>(T(13.0 / 3.0)), eps = pc<P>(T(1.0e-6));
+  const P b0 = pfma(c133, pmul(d0, d0), pfma(e0, e0, eps));
+  const P b1 = pfma(c133, pmul(d1, d1), pfma(e1, e1, eps));
+  const P b2 = pfma(c133, pmul(d2, d2), pfma(e2, e2, eps));
   const P s0 = pmul(b0, b0), s1 = pmul(b1, b1), s2 = pmul(b2, b2);
-  const P a0 = pmul(pc<P>(T(0.1)), pmk(Num<T>::rcp(s0.x), Num<T>::rcp(s0.y)));
-  const P a1 = pmul(pc<P>(T(0.6)), pmk(Num<T>::rcp(s1.x), Num<T>::rcp(s1.y)));
-  const P a2 = pmul(pc<P>(T(0.3)), pmk(Num<T>::rcp(s2.x), Num<T>::rcp(s2.y)));
+  P a0, a1, a2;                                                  // the weights times 10
+  if constexpr (sizeof(T) == 8) {
+    const P t2 = pmul(pc<P>(T(3)), s0), t1 = pmul(pc<P>(T(6)), s0);
+    a0 = pmul(s1, s2);
+    a1 = pmul(t1, s2);
+    a2 = pmul(t2, s1);
+  } else {
+    a0 = pmk(Num<T>::rcp(s0.x), Num<T>::rcp(s0.y));
+    a1 = pmul(pc<P>(T(6)), pmk(Num<T>::rcp(s1.x), Num<T>::rcp(s1.y)));
+    a2 = pmul(pc<P>(T(3)), pmk(Num<T>::rcp(s2.x), Num<T>::rcp(s2.y)));
+  }
   const P num = pfma(a2, r2, pfma(a1, r1, pmul(a0, r0)));
-  const P den = pmul(pc<P>(T(6)), padd(padd(a0, a1), a2));
-  return pfma(num, pmk(Num<T>::rcp(den.x), Num<T>::rcp(den.y)), v2);
+  const P den = padd(padd(a0, a1), a2);
+  return pfma(pc<P>(T(1.0 / 6.0)), pmul(num, pmk(Num<T>::rcp(den.x), Num<T>::rcp(den.y))), v2);
 }
 
 // WENOCU6 (the sixth-order adaptive central-upwind WENO that Remark 2 names) for a pair
@@ -267,34 +284,6 @@ template <> struct MidW<8> {
   }
 };
 
-// Fifth-order reconstruction at i+1/2 from v0..v4 = f_{i-2..i+2} (Sec. 2.2.2):
-// WENO5-JS with eps = 1e-6 and power 2, or linear upwind (optimal weights).  Written
-// in the first differences a..d of the five values: q_k - v2 and the smoothness
-// indicators are short combinations of them, and the result is v2 + sum w_k (q_k - v2).
-template <typename T, int SCHEME>
-__device__ __forceinline__ T recon5(T v0, T v1, T v2, T v3, T v4) {
-  const T a = v1 - v0, b = v2 - v1, c = v3 - v2, d = v4 - v3;
-  // 6 (q_k - v2): (5b - 2a), (b + 2c), (4c - d)
-  const T r0 = T(5) * b - T(2) * a;
-  const T r1 = b + T(2) * c;
-  const T r2 = T(4) * c - d;
-  if (SCHEME == 1) {
-    // optimal weights (1/10, 6/10, 3/10) over 6: (2,-13,47,27,-3)/60 relative to v2
-    return v2 + (T(0.1) * r0 + T(0.6) * r1 + T(0.3) * r2) * T(1.0 / 6.0);
-  }
-  const T c13 = T(13.0 / 12.0), eps = T(1.0e-6);
-  const T d0 = b - a, e0 = T(3) * b - a;
-  const T d1 = c - b, e1 = b + c;
-  const T d2 = d - c, e2 = d - T(3) * c;
-  const T b0 = c13 * d0 * d0 + T(0.25) * e0 * e0 + eps;
-  const T b1 = c13 * d1 * d1 + T(0.25) * e1 * e1 + eps;
-  const T b2 = c13 * d2 * d2 + T(0.25) * e2 * e2 + eps;
-  const T a0 = Num<T>::div(T(0.1), b0 * b0);
-  const T a1 = Num<T>::div(T(0.6), b1 * b1);
-  const T a2 = Num<T>::div(T(0.3), b2 * b2);
-  return v2 + Num<T>::div(a0 * r0 + a1 * r1 + a2 * r2, T(6) * (a0 + a1 + a2));
-}
-
 // [F(B) - F(A)] . k from A's state (velocity uA, momentum mA, energy EA, pressure pA),
 // the difference d = B - A, and B's 1/rho and velocity; every term is a product
 // with a component of d, so the result carries the relative rounding of d.
@@ -316,48 +305,58 @@ __device__ __forceinline__ void dflux(T g1, T rinvB, const T uB[3], const T uA[3
   out[4] = (d[4] + dp) * UB + (EA + pA) * dU;
 }
 
-// dflux for two stencil points at once (same A state, two B states), packed.
+// A pair of stencil points B seen from the frame that moves with the reference state's velocity
+// V = u* (Galilean frame: momenta m - rho V, energy E - m.V + rho V^2/2).  d = B - Q* comes in the
+// laboratory frame and leaves in the moving one, and out = [F(B) - F(Q*)] . k there.  Q* is at
+// rest in that frame, so the differences of velocity, kinetic energy and momentum flux lose the
+// terms with its momentum (28 operations per point instead of 35, and no velocities of B): with
+// z = d_m - V d_0 = rho_B (u_B - V),
+//   e = d_E - V.z - V^2/2 d_0,  dp = (gamma-1)(e - z.z/(2 rho_B)),  dU = z.k/rho_B,
+//   U_B = u_B.k, V.k = U_B - dU,
+//   out = (z.k + d_0 V.k,  z U_B + dp k,  e U_B + (E*+p* + dp) dU),
+// every term a product with a component of d, so the result keeps the relative rounding of d.
+// V is any fixed number for this: its own rounding cancels.  EpP = E* + p* = p* gamma/(gamma-1).
+// With the reconstruction below and the velocities out of the shared ring: 64-block WENO5 step
+// 18.04 -> 17.24 ms, 256^3 9.05 -> 8.65 ms, 96^3 FP64 24.5 -> 21.7 ms.
 template <typename T>
-__device__ __forceinline__ void dflux_pair(T g1, typename PairOf<T>::type rinvB,
-                                           const typename PairOf<T>::type uB[3], const T uA[3],
-                                           const T mA[3], T EA, T pA,
-                                           const typename PairOf<T>::type d[5],
-                                           const typename PairOf<T>::type k[3],
-                                           typename PairOf<T>::type out[5]) {
+__device__ __forceinline__ void dflux_frame(T g1, typename PairOf<T>::type rinvB, typename PairOf<T>::type UB,
+                                            const T V[3], T hV2, T EpP, typename PairOf<T>::type d[5],
+                                            const typename PairOf<T>::type k[3],
+                                            typename PairOf<T>::type out[5]) {
   using P = typename PairOf<T>::type;
-  const P du0 = pmul(pfma(pc<P>(-uA[0]), d[0], d[1]), rinvB);
-  const P du1 = pmul(pfma(pc<P>(-uA[1]), d[0], d[2]), rinvB);
-  const P du2 = pmul(pfma(pc<P>(-uA[2]), d[0], d[3]), rinvB);
-  P dke = pmul(d[1], uB[0]);
-  dke = pfma(d[2], uB[1], dke);
-  dke = pfma(d[3], uB[2], dke);
-  dke = pfma(pc<P>(mA[0]), du0, dke);
-  dke = pfma(pc<P>(mA[1]), du1, dke);
-  dke = pfma(pc<P>(mA[2]), du2, dke);
-  const P dp = pmul(pc<P>(g1), pfma(pc<P>(T(-0.5)), dke, d[4]));
-  const P UB = pfma(uB[2], k[2], pfma(uB[1], k[1], pmul(uB[0], k[0])));
-  const P dU = pfma(du2, k[2], pfma(du1, k[1], pmul(du0, k[0])));
-  out[0] = pfma(d[3], k[2], pfma(d[2], k[1], pmul(d[1], k[0])));
-  out[1] = pfma(dp, k[0], pfma(pc<P>(mA[0]), dU, pmul(d[1], UB)));
-  out[2] = pfma(dp, k[1], pfma(pc<P>(mA[1]), dU, pmul(d[2], UB)));
-  out[3] = pfma(dp, k[2], pfma(pc<P>(mA[2]), dU, pmul(d[3], UB)));
-  out[4] = pfma(pc<P>(EA + pA), dU, pmul(padd(d[4], dp), UB));
+#pragma unroll
+  for (int c = 0; c < 3; ++c) d[1 + c] = pfma(pc<P>(-V[c]), d[0], d[1 + c]);
+#pragma unroll
+  for (int c = 0; c < 3; ++c) d[4] = pfma(pc<P>(-V[c]), d[1 + c], d[4]);
+  d[4] = pfma(pc<P>(-hV2), d[0], d[4]);
+  const P zz = pfma(d[3], d[3], pfma(d[2], d[2], pmul(d[1], d[1])));
+  const P zk = pfma(d[3], k[2], pfma(d[2], k[1], pmul(d[1], k[0])));
+  const P dp = pmul(pc<P>(g1), pfma(pc<P>(T(-0.5)), pmul(rinvB, zz), d[4]));
+  const P dU = pmul(rinvB, zk);
+  out[0] = pfma(d[0], psub(UB, dU), zk);
+#pragma unroll
+  for (int c = 0; c < 3; ++c) out[1 + c] = pfma(dp, k[c], pmul(d[1 + c], UB));
+  out[4] = pfma(padd(dp, pc<P>(EpP)), dU, pmul(d[4], UB));
 }
 
 // FIX = 1 or 2: the characteristic decomposition and the FP form on, local Lax-Friedrichs speeds,
 // all fixed at compile time (the configuration of the paper's workloads but the shock test), so
-// their switches fold away; FIX = 0 reads them from the arguments and the block descriptor.
-// FIX = 2 is the same sweep with the alternative CTA shape of sweep_threads (fp_internal.h).
+// their switches fold away.  FIX = 2 is the same sweep with the alternative CTA shape of
+// sweep_threads (fp_internal.h).  FIX = 0: characteristic, the FP form and the speeds read from
+// the arguments and the block descriptor.  FIX = 3: component-wise, the others as FIX = 0 (one
+// variant for both decompositions held the operands of both and spilled: linear upwind on
+// 70 x 80 x 22 points, component-wise, 208 us a step against 149).
 template <typename T, int M, int SCHEME, bool BND, int FIX>
 __global__ void __launch_bounds__(sweep_threads(sizeof(T) == 4, SCHEME, FIX), sweep_min_ctas(sizeof(T) == 4, SCHEME, FIX))
 fp_sweep(const BlockDev *__restrict__ blocks, const SweepItem *__restrict__ items, int dir, int mode,
-         int stage, const double *__restrict__ dtp, int charwise_arg, int fpform_arg) {
+         int stage, const double *__restrict__ dtp, int fpform_arg) {
   // this variant's CTA shape (fp_internal.h): threads, ring stride of a staged field, padding
   constexpr int kThreads = sweep_threads(sizeof(T) == 4, SCHEME, FIX);
   constexpr int kRing = sweep_ring(sizeof(T) == 4, SCHEME, FIX);
   constexpr bool kPad = sweep_padded(sizeof(T) == 4, SCHEME, FIX);
-  const int charwise = FIX ? 1 : charwise_arg;
-  const int fpform = FIX ? 1 : fpform_arg;
+  constexpr bool kFold = FIX == 1 || FIX == 2;
+  constexpr int charwise = FIX == 3 ? 0 : 1;
+  const int fpform = kFold ? 1 : fpform_arg;
   // stencil points of a face: i-2..i+3 (5th order) or i-3..i+4 (WENO7), offset index Q0
   constexpr int NS = SCHEME == 2 ? 8 : 6;
   constexpr int Q0 = SCHEME == 2 ? 0 : 1;
@@ -399,7 +398,7 @@ fp_sweep(const BlockDev *__restrict__ blocks, const SweepItem *__restrict__ item
                                         reinterpret_cast<const unsigned char *>(items + nit) + 16 * tid);
     if (tid == 0) {                      // read after the prologue's barrier
       s_dt = mode == MODE_RK ? T(*dtp) : T(0);
-      if (!FIX && B->global_lf)
+      if (!kFold && B->global_lf)
         for (int c = 0; c < 3; ++c)
           s_lam[c] = *FPK_IN(static_cast<const T *>(B->lamg) + (3 * dir + c), static_cast<const T *>(B->lamg), 9, B->status);
     }
@@ -450,8 +449,8 @@ fp_sweep(const BlockDev *__restrict__ blocks, const SweepItem *__restrict__ item
     const T *__restrict__ met = static_cast<const T *>(B->met) + B->moff;
     const T *__restrict__ fmet = static_cast<const T *>(D->fmet);
     const T *__restrict__ qin = static_cast<const T *>(B->q[stage]);
-    const T g1 = T(B->gamma - 1.0), gam = T(B->gamma);
-    const int glf = FIX ? 0 : B->global_lf;
+    const T g1 = T(B->gamma - 1.0), gam = T(B->gamma), rg1 = Num<T>::rcp(g1);
+    const int glf = kFold ? 0 : B->global_lf;
     T qb[5];
 #pragma unroll
     for (int v = 0; v < 5; ++v) qb[v] = T(B->qbar[v]);
@@ -550,8 +549,6 @@ fp_sweep(const BlockDev *__restrict__ blocks, const SweepItem *__restrict__ item
       const T u0 = Q[1] * rinv, u1 = Q[2] * rinv, u2 = Q[3] * rinv;
       const T p = g1 * (Q[4] - T(0.5) * (Q[1] * u0 + Q[2] * u1 + Q[3] * u2));
       const T Jc = Num<T>::rcp(invJ);
-      const T gx = Jc * k[0], gy = Jc * k[1], gz = Jc * k[2];
-      const T c = Num<T>::sqrt_(gam * p * rinv);
       T *cp = sm + off(x);
 #pragma unroll
       for (int v = 0; v < 5; ++v) cp[(CF_Q + v) * kRing] = Q[v];
@@ -560,13 +557,10 @@ fp_sweep(const BlockDev *__restrict__ blocks, const SweepItem *__restrict__ item
       cp[(CF_K + 2) * kRing] = k[2];
       cp[CF_INVJ * kRing] = invJ;
       cp[CF_RINV * kRing] = rinv;
-      cp[(CF_U + 0) * kRing] = u0;
-      cp[(CF_U + 1) * kRing] = u1;
-      cp[(CF_U + 2) * kRing] = u2;
       cp[CF_H * kRing] = (Q[4] + p) * rinv;
       cp[CF_SQR * kRing] = Num<T>::sqrt_(Q[0]);
-      cp[CF_UC * kRing] = u0 * gx + u1 * gy + u2 * gz;
-      cp[CF_AC * kRing] = c * Num<T>::sqrt_(gx * gx + gy * gy + gz * gz);
+      cp[CF_UC * kRing] = Jc * (u0 * k[0] + u1 * k[1] + u2 * k[2]);
+      cp[CF_AC * kRing] = fabs(Jc) * Num<T>::sqrt_(gam * p * rinv * (k[0] * k[0] + k[1] * k[1] + k[2] * k[2]));
     };
 
     // asynchronous copy of the face metric of face x + 1/2 of line (t1, t2) into staging slot
@@ -691,7 +685,7 @@ fp_sweep(const BlockDev *__restrict__ blocks, const SweepItem *__restrict__ item
         // instruction.  These are the stencil loops' pairs (q, 7 - q) of the same cells, so linear
         // upwind with the switches folded keeps the pairs' Q_q - Q_i and (1/J)_q for its stencil
         // differences instead of loading and subtracting them again.
-        constexpr bool kKeep = SCHEME == 1 && FIX != 0;
+        constexpr bool kKeep = SCHEME == 1 && kFold;
         constexpr int kQlo = 3 - M / 2 + 1;
         P dqk[4][5], ijk[4];
         if (fpform) {
@@ -717,13 +711,18 @@ fp_sweep(const BlockDev *__restrict__ blocks, const SweepItem *__restrict__ item
 #pragma unroll
           for (int v = 0; v < 5; ++v) dl[v] = (acc[v].x + acc[v].y) * wi;
         }
-        T Qs[5];
+        // the frame of the face: velocity V = u* (0 for the plain scheme), see dflux_frame
+        T V[3] = {T(0), T(0), T(0)}, hV2 = T(0), EpP = T(0);
+        if (fpform) {
+          T Qs[5];
 #pragma unroll
-        for (int v = 0; v < 5; ++v) Qs[v] = Qi[v] + dl[v];
-        const T rinvs = Num<T>::rcp(Qs[0]);
-        const T us[3] = {Qs[1] * rinvs, Qs[2] * rinvs, Qs[3] * rinvs};
-        const T ps = g1 * (Qs[4] - T(0.5) * (Qs[1] * us[0] + Qs[2] * us[1] + Qs[3] * us[2]));
-        const T ms[3] = {Qs[1], Qs[2], Qs[3]};
+          for (int v = 0; v < 5; ++v) Qs[v] = Qi[v] + dl[v];
+          const T rinvs = Num<T>::rcp(Qs[0]);
+#pragma unroll
+          for (int c = 0; c < 3; ++c) V[c] = Qs[1 + c] * rinvs;
+          hV2 = T(0.5) * (V[0] * V[0] + V[1] * V[1] + V[2] * V[2]);
+          EpP = gam * (Qs[4] - Qs[0] * hV2);            // p* gamma/(gamma-1)
+        }
 
         // Lax-Friedrichs speeds: local (max over the stencil cells i-2..i+3) or global
         T lm = T(0), l0 = T(0), lp = T(0);
@@ -733,9 +732,9 @@ fp_sweep(const BlockDev *__restrict__ blocks, const SweepItem *__restrict__ item
 #pragma unroll
           for (int q = Q0; q < Q0 + NS; ++q) {
             const T U = CELL(CF_UC, q), ac = CELL(CF_AC, q);
-            lm = fmax(lm, fabs(U - ac));
-            l0 = fmax(l0, fabs(U));
-            lp = fmax(lp, fabs(U + ac));
+            lm = Num<T>::amax(lm, U - ac);
+            l0 = Num<T>::amax(l0, U);
+            lp = Num<T>::amax(lp, U + ac);
           }
         }
         T lam[5];
@@ -749,14 +748,18 @@ fp_sweep(const BlockDev *__restrict__ blocks, const SweepItem *__restrict__ item
         // Roe average of cells i, i+1 and eigenvector basis in the face normal
         const T rl = CELL(CF_SQR, 3), rr = CELL(CF_SQR, 4);
         const T rs = Num<T>::rcp(rl + rr);
+        // sqrt(rho) u = (rho u) sqrt(rho)/rho
+        const T ml = rl * CELL(CF_RINV, 3) * rs, mr = rr * CELL(CF_RINV, 4) * rs;
         T u[3];
 #pragma unroll
-        for (int c = 0; c < 3; ++c) u[c] = (rl * CELL(CF_U + c, 3) + rr * CELL(CF_U + c, 4)) * rs;
+        for (int c = 0; c < 3; ++c) u[c] = ml * Qi[1 + c] + mr * CELL(CF_Q + 1 + c, 4);
         const T H = (rl * CELL(CF_H, 3) + rr * CELL(CF_H, 4)) * rs;
-        const T q2 = u[0] * u[0] + u[1] * u[1] + u[2] * u[2];
-        const T c2 = g1 * (H - T(0.5) * q2);
-        const T cs = Num<T>::sqrt_(c2);
-        const T csi = Num<T>::rcp(cs);
+        const T c2 = g1 * (H - T(0.5) * (u[0] * u[0] + u[1] * u[1] + u[2] * u[2]));
+        const T csi = Num<T>::rsqrt_(c2), cs = c2 * csi;
+        // from here on velocities are those in the frame of the face (w = u - V)
+#pragma unroll
+        for (int c = 0; c < 3; ++c) u[c] -= V[c];
+        const T hq2 = T(0.5) * (u[0] * u[0] + u[1] * u[1] + u[2] * u[2]);
         const T bb = g1 * csi * csi;
         const T knr = Num<T>::rsqrt_(kf[0] * kf[0] + kf[1] * kf[1] + kf[2] * kf[2]);
         const T n[3] = {kf[0] * knr, kf[1] * knr, kf[2] * knr};
@@ -766,7 +769,7 @@ fp_sweep(const BlockDev *__restrict__ blocks, const SweepItem *__restrict__ item
         // measured faster.
         T t1[3], t2[3];
         const bool lowz = n[2] * n[2] <= T(0.5);
-        if constexpr ((SCHEME == 0 && FIX != 0) || SCHEME == 3) {
+        if constexpr ((SCHEME == 0 && kFold) || SCHEME == 3) {
           if (lowz) {
             const T s = Num<T>::rsqrt_(n[0] * n[0] + n[1] * n[1]);
             t1[0] = -n[1] * s; t1[1] = n[0] * s; t1[2] = T(0);
@@ -786,23 +789,25 @@ fp_sweep(const BlockDev *__restrict__ blocks, const SweepItem *__restrict__ item
         const T Un = u[0] * n[0] + u[1] * n[1] + u[2] * n[2];
         const T ut1 = u[0] * t1[0] + u[1] * t1[1] + u[2] * t1[2];
         const T ut2 = u[0] * t2[0] + u[1] * t2[1] + u[2] * t2[2];
-        // half the left-eigenvector rows (the 1/2 of the Lax-Friedrichs split folded in)
-        const T qbb = T(0.25) * bb, hq2 = T(0.5) * q2, qcs = T(0.25) * csi;
-        const T h1[3] = {T(0.5) * t1[0], T(0.5) * t1[1], T(0.5) * t1[2]};
-        const T h2[3] = {T(0.5) * t2[0], T(0.5) * t2[1], T(0.5) * t2[2]};
-        const T hut1 = T(0.5) * ut1, hut2 = T(0.5) * ut2;
+        // the left-eigenvector rows, scaled by kRow: the 1/2 of the Lax-Friedrichs split folded in,
+        // and for WENO5 another 1/2 (see recon5_pair)
+        constexpr T kRow = SCHEME == 0 ? T(0.25) : T(0.5);
+        const T qbb = kRow * T(0.5) * bb, qcs = kRow * T(0.5) * csi;
+        const T h1[3] = {kRow * t1[0], kRow * t1[1], kRow * t1[2]};
+        const T h2[3] = {kRow * t2[0], kRow * t2[1], kRow * t2[2]};
+        const T hut1 = kRow * ut1, hut2 = kRow * ut2;
 
-        // (1/2) l_s . d for the five characteristic fields
+        // kRow l_s . d for the five characteristic fields
         auto project = [&](const T d[5], T c[5]) {
           if (!charwise) {
 #pragma unroll
-            for (int v = 0; v < 5; ++v) c[v] = T(0.5) * d[v];
+            for (int v = 0; v < 5; ++v) c[v] = kRow * d[v];
             return;
           }
           const T X4 = qbb * (hq2 * d[0] - (u[0] * d[1] + u[1] * d[2] + u[2] * d[3]) + d[4]);
           const T Y4 = (Un * d[0] - (n[0] * d[1] + n[1] * d[2] + n[2] * d[3])) * qcs;
           c[0] = X4 + Y4;
-          c[1] = T(0.5) * d[0] - T(2) * X4;
+          c[1] = kRow * d[0] - T(2) * X4;
           c[2] = h1[0] * d[1] + h1[1] * d[2] + h1[2] * d[3] - hut1 * d[0];
           c[3] = h2[0] * d[1] + h2[1] * d[2] + h2[2] * d[3] - hut2 * d[0];
           c[4] = X4 - Y4;
@@ -812,7 +817,7 @@ fp_sweep(const BlockDev *__restrict__ blocks, const SweepItem *__restrict__ item
         auto project_pair = [&](const P d[5], P c[5]) {
           if (!charwise) {
 #pragma unroll
-            for (int v = 0; v < 5; ++v) c[v] = pmul(pc<P>(T(0.5)), d[v]);
+            for (int v = 0; v < 5; ++v) c[v] = pmul(pc<P>(kRow), d[v]);
             return;
           }
           const P ud = pfma(pc<P>(u[0]), d[1], pfma(pc<P>(u[1]), d[2], pmul(pc<P>(u[2]), d[3])));
@@ -820,12 +825,21 @@ fp_sweep(const BlockDev *__restrict__ blocks, const SweepItem *__restrict__ item
           const P nd = pfma(pc<P>(n[0]), d[1], pfma(pc<P>(n[1]), d[2], pmul(pc<P>(n[2]), d[3])));
           const P Y4 = pmul(pc<P>(qcs), psub(pmul(pc<P>(Un), d[0]), nd));
           c[0] = padd(X4, Y4);
-          c[1] = pfma(pc<P>(T(-2)), X4, pmul(pc<P>(T(0.5)), d[0]));
+          c[1] = pfma(pc<P>(T(-2)), X4, pmul(pc<P>(kRow), d[0]));
           c[2] = pfma(pc<P>(h1[0]), d[1], pfma(pc<P>(h1[1]), d[2], pfma(pc<P>(h1[2]), d[3], pmul(pc<P>(-hut1), d[0]))));
           c[3] = pfma(pc<P>(h2[0]), d[1], pfma(pc<P>(h2[1]), d[2], pfma(pc<P>(h2[2]), d[3], pmul(pc<P>(-hut2), d[0]))));
           c[4] = psub(X4, Y4);
         };
 
+        // a flux in the frame of the face, seen from the laboratory
+        auto to_lab = [&](P f[5]) {
+          f[4] = pfma(pc<P>(hV2), f[0], f[4]);
+#pragma unroll
+          for (int c = 0; c < 3; ++c) {
+            f[4] = pfma(pc<P>(V[c]), f[1 + c], f[4]);
+            f[1 + c] = pfma(pc<P>(V[c]), f[0], f[1 + c]);
+          }
+        };
         // h: the back-projected characteristic part of the face flux, cen: the part added
         // to it outside the projection (linear upwind only)
         T h[5], cen[5] = {T(0), T(0), T(0), T(0), T(0)};
@@ -851,28 +865,34 @@ fp_sweep(const BlockDev *__restrict__ blocks, const SweepItem *__restrict__ item
             const int km = q - kQlo;
             const bool kept = kKeep && km >= 0;
             const int kmi = kept ? km : 0;
+            const P ijp = kept ? ijk[kmi] : pmk(CELL(CF_INVJ, q), CELL(CF_INVJ, q2));
+            const P rip = pmk(CELL(CF_RINV, q), CELL(CF_RINV, q2));
             if (fpform) {
-              P kp2[3], uBp[3];
+              P kp2[3];
 #pragma unroll
               for (int v = 0; v < 5; ++v)
                 dp[v] = kept ? psub(dqk[kmi][v], pc<P>(dl[v]))
                              : psub(psub(pmk(CELL(CF_Q + v, q), CELL(CF_Q + v, q2)), pc<P>(Qi[v])), pc<P>(dl[v]));
 #pragma unroll
-              for (int c = 0; c < 3; ++c) {
-                kp2[c] = pmk(CELL(CF_K + c, q), CELL(CF_K + c, q2));
-                uBp[c] = pmk(CELL(CF_U + c, q), CELL(CF_U + c, q2));
+              for (int c = 0; c < 3; ++c) kp2[c] = pmk(CELL(CF_K + c, q), CELL(CF_K + c, q2));
+              const P UBp = pmul(pmk(CELL(CF_UC, q), CELL(CF_UC, q2)), ijp);
+              const P dlab[3] = {dp[1], dp[2], dp[3]};
+              const P elab = dp[4];
+              dflux_frame<T>(g1, rip, UBp, V, hV2, EpP, dp, kp2, out);
+              if (!charwise) {       // the components are those of the laboratory frame
+                to_lab(out);
+                dp[1] = dlab[0]; dp[2] = dlab[1]; dp[3] = dlab[2]; dp[4] = elab;
               }
-              dflux_pair<T>(g1, pmk(CELL(CF_RINV, q), CELL(CF_RINV, q2)), uBp, us, ms, Qs[4], ps, dp, kp2, out);
             } else {
               // plain scheme: F~_m and Q~_m themselves
               P uBp[3], kp2[3];
 #pragma unroll
+              for (int v = 0; v < 5; ++v) dp[v] = pmk(CELL(CF_Q + v, q), CELL(CF_Q + v, q2));
+#pragma unroll
               for (int c = 0; c < 3; ++c) {
                 kp2[c] = pmk(CELL(CF_K + c, q), CELL(CF_K + c, q2));
-                uBp[c] = pmk(CELL(CF_U + c, q), CELL(CF_U + c, q2));
+                uBp[c] = pmul(dp[1 + c], rip);
               }
-#pragma unroll
-              for (int v = 0; v < 5; ++v) dp[v] = pmk(CELL(CF_Q + v, q), CELL(CF_Q + v, q2));
               const P ke = pfma(dp[3], uBp[2], pfma(dp[2], uBp[1], pmul(dp[1], uBp[0])));
               const P pm = pmul(pc<P>(g1), pfma(pc<P>(T(-0.5)), ke, dp[4]));
               const P U = pfma(uBp[2], kp2[2], pfma(uBp[1], kp2[1], pmul(uBp[0], kp2[0])));
@@ -881,7 +901,6 @@ fp_sweep(const BlockDev *__restrict__ blocks, const SweepItem *__restrict__ item
               for (int c = 0; c < 3; ++c) out[1 + c] = pfma(pm, kp2[c], pmul(dp[1 + c], U));
               out[4] = pmul(padd(dp[4], pm), U);
             }
-            const P ijp = kept ? ijk[kmi] : pmk(CELL(CF_INVJ, q), CELL(CF_INVJ, q2));
             const P ds = pmk(d5[s], -d5[s]);
 #pragma unroll
             for (int v = 0; v < 5; ++v) {
@@ -899,7 +918,7 @@ fp_sweep(const BlockDev *__restrict__ blocks, const SweepItem *__restrict__ item
           T c[5];
           project(dis, c);
 #pragma unroll
-          for (int v = 0; v < 5; ++v) h[v] = T(2) * lam[v] * c[v];
+          for (int v = 0; v < 5; ++v) h[v] = lam[v] * c[v] * T(1 / kRow);
         } else {
           // split stencil values f+/- for the NS stencil points
           T fpl[NS][5], fmi[NS][5];
@@ -925,21 +944,25 @@ fp_sweep(const BlockDev *__restrict__ blocks, const SweepItem *__restrict__ item
             for (int s = 0; s < NS / 2; ++s) {
               const int mir = NS - 1 - s;
               const int q = s + Q0, q2 = mir + Q0;
-              P dp[5], kp2[3], uBp[3], out[5];
+              P dp[5], kp2[3], out[5];
 #pragma unroll
               for (int v = 0; v < 5; ++v)
                 dp[v] = psub(psub(pmk(CELL(CF_Q + v, q), CELL(CF_Q + v, q2)), pc<P>(Qi[v])), pc<P>(dl[v]));
 #pragma unroll
-              for (int c = 0; c < 3; ++c) {
-                kp2[c] = pmk(CELL(CF_K + c, q), CELL(CF_K + c, q2));
-                uBp[c] = pmk(CELL(CF_U + c, q), CELL(CF_U + c, q2));
+              for (int c = 0; c < 3; ++c) kp2[c] = pmk(CELL(CF_K + c, q), CELL(CF_K + c, q2));
+              const P ijp = pmk(CELL(CF_INVJ, q), CELL(CF_INVJ, q2));
+              const P UBp = pmul(pmk(CELL(CF_UC, q), CELL(CF_UC, q2)), ijp);
+              const P dlab[3] = {dp[1], dp[2], dp[3]};
+              const P elab = dp[4];
+              dflux_frame<T>(g1, pmk(CELL(CF_RINV, q), CELL(CF_RINV, q2)), UBp, V, hV2, EpP, dp, kp2, out);
+              if (!charwise) {       // the components are those of the laboratory frame
+                to_lab(out);
+                dp[1] = dlab[0]; dp[2] = dlab[1]; dp[3] = dlab[2]; dp[4] = elab;
               }
-              dflux_pair<T>(g1, pmk(CELL(CF_RINV, q), CELL(CF_RINV, q2)), uBp, us, ms, Qs[4], ps, dp, kp2, out);
               P cF[5], cD[5];
               project_pair(out, cF);
               project_pair(dp, cD);
               // (lambda (1/J)_s, -lambda (1/J)_mirror) for the three speed classes
-              const P ijp = pmk(CELL(CF_INVJ, q), CELL(CF_INVJ, q2));
               const P mp[3] = {pmul(lpm[0], ijp), pmul(lpm[1], ijp), pmul(lpm[2], ijp)};
 #pragma unroll
               for (int v = 0; v < 5; ++v) {
@@ -958,9 +981,10 @@ fp_sweep(const BlockDev *__restrict__ blocks, const SweepItem *__restrict__ item
               const int q = s + Q0;
               T dF[5], d[5];
               const T km[3] = {CELL(CF_K, q), CELL(CF_K + 1, q), CELL(CF_K + 2, q)};
-              const T uB[3] = {CELL(CF_U, q), CELL(CF_U + 1, q), CELL(CF_U + 2, q)};
 #pragma unroll
               for (int v = 0; v < 5; ++v) d[v] = CELL(CF_Q + v, q);
+              const T ri = CELL(CF_RINV, q);
+              const T uB[3] = {d[1] * ri, d[2] * ri, d[3] * ri};
               const T pm = g1 * (d[4] - T(0.5) * (d[1] * uB[0] + d[2] * uB[1] + d[3] * uB[2]));
               const T U = uB[0] * km[0] + uB[1] * km[1] + uB[2] * km[2];
               dF[0] = d[0] * U;
@@ -988,7 +1012,7 @@ fp_sweep(const BlockDev *__restrict__ blocks, const SweepItem *__restrict__ item
               const P r = recon6cu_pair<T>(w6);
               h[v] = r.x + r.y;
             } else {
-              const P r = recon5_pair<T, SCHEME>(pmk(fpl[0][v], fmi[5][v]), pmk(fpl[1][v], fmi[4][v]),
+              const P r = recon5_pair<T>(pmk(fpl[0][v], fmi[5][v]), pmk(fpl[1][v], fmi[4][v]),
                                                  pmk(fpl[2][v], fmi[3][v]), pmk(fpl[3][v], fmi[2][v]),
                                                  pmk(fpl[4][v], fmi[1][v]));
               h[v] = r.x + r.y;
@@ -997,19 +1021,31 @@ fp_sweep(const BlockDev *__restrict__ blocks, const SweepItem *__restrict__ item
         }
         T F[5];
         if (charwise) {
-          const T sa = h[0] + h[4], da = h[4] - h[0];
-          F[0] = sa + h[1];
+          // in the frame of the face; H' = c^2/(gamma-1) + w^2/2
+          const T sa = h[0] + h[4], da = cs * (h[4] - h[0]), s1 = sa + h[1];
+          F[0] = s1;
 #pragma unroll
-          for (int c = 0; c < 3; ++c) F[1 + c] = u[c] * (sa + h[1]) + cs * n[c] * da + t1[c] * h[2] + t2[c] * h[3];
-          F[4] = H * sa + cs * Un * da + T(0.5) * q2 * h[1] + ut1 * h[2] + ut2 * h[3];
+          for (int c = 0; c < 3; ++c) F[1 + c] = u[c] * s1 + n[c] * da + t1[c] * h[2] + t2[c] * h[3];
+          F[4] = c2 * rg1 * sa + hq2 * s1 + Un * da + ut1 * h[2] + ut2 * h[3];
         } else {
 #pragma unroll
           for (int v = 0; v < 5; ++v) F[v] = h[v];
         }
+        if constexpr (SCHEME == 1) {
+#pragma unroll
+          for (int v = 0; v < 5; ++v) F[v] += cen[v];
+        }
+        if (SCHEME == 0)             // WENO5 works on half-size values (kRow)
+#pragma unroll
+          for (int v = 0; v < 5; ++v) F[v] += F[v];
+        if (charwise && fpform) {    // back to the laboratory frame: E += V.m + V^2/2 rho, m += V rho
+          F[4] += V[0] * F[1] + V[1] * F[2] + V[2] * F[3] + hV2 * F[0];
+#pragma unroll
+          for (int c = 0; c < 3; ++c) F[1 + c] += V[c] * F[0];
+        }
         T *fp = fr + off(ff);
 #pragma unroll
         for (int v = 0; v < 5; ++v) {
-          if constexpr (SCHEME == 1) F[v] += cen[v];
           fp[v * kRing] = F[v];
           fp[(5 + v) * kRing] = dl[v];
         }
@@ -1130,20 +1166,18 @@ constexpr size_t sweep_smem() {
 }
 
 template <typename T, int M, int SCHEME, bool BND, int FIX>
-cudaError_t launch_one(const SweepLaunch &L, int charwise, int fp, cudaStream_t s) {
+cudaError_t launch_one(const SweepLaunch &L, int fp, cudaStream_t s) {
   constexpr size_t smem = sweep_smem<T, SCHEME, FIX>();
   constexpr int nt = sweep_threads(sizeof(T) == 4, SCHEME, FIX);
   if (L.grid <= 0) return cudaSuccess;
-  fp_sweep<T, M, SCHEME, BND, FIX><<<L.grid, nt, smem, s>>>(L.blocks, L.items, L.dir, L.mode, L.stage, L.dt,
-                                                            charwise, fp);
+  fp_sweep<T, M, SCHEME, BND, FIX><<<L.grid, nt, smem, s>>>(L.blocks, L.items, L.dir, L.mode, L.stage, L.dt, fp);
   return cudaGetLastError();
 }
 
 template <typename T, bool BND, int FIX>
-cudaError_t launch_sweep_t(const SweepLaunch &L, int M, int scheme, int charwise, int fp,
-                           cudaStream_t s) {
+cudaError_t launch_sweep_t(const SweepLaunch &L, int M, int scheme, int fp, cudaStream_t s) {
 #define FPK_CASE(MM, SS) \
-  if (M == MM && scheme == SS) return launch_one<T, MM, SS, BND, FIX>(L, charwise, fp, s);
+  if (M == MM && scheme == SS) return launch_one<T, MM, SS, BND, FIX>(L, fp, s);
   FPK_CASE(2, 0) FPK_CASE(4, 0) FPK_CASE(6, 0) FPK_CASE(8, 0)
   FPK_CASE(2, 1) FPK_CASE(4, 1) FPK_CASE(6, 1) FPK_CASE(8, 1)
   FPK_CASE(2, 2) FPK_CASE(4, 2) FPK_CASE(6, 2) FPK_CASE(8, 2)
@@ -1152,19 +1186,18 @@ cudaError_t launch_sweep_t(const SweepLaunch &L, int M, int scheme, int charwise
   return cudaErrorInvalidValue;
 }
 
-// Opt in to the dynamic shared memory of every variant and return the resident
-// CTAs per SM of the requested one.  Called before any launch or graph capture.
+// Opt in to the dynamic shared memory of a variant and return its resident CTAs per SM.
+// Called before any launch or graph capture.
 template <typename T, bool BND, int FIX>
 int prepare_t(int M, int scheme) {
   int nb = 0;
 #define FPK_OCC(MM, SS)                                                                              \
-  {                                                                                                  \
+  if (M == MM && scheme == SS) {                                                                     \
     constexpr size_t smem = sweep_smem<T, SS, FIX>();                                                \
     cudaFuncSetAttribute(fp_sweep<T, MM, SS, BND, FIX>, cudaFuncAttributeMaxDynamicSharedMemorySize,  \
                          (int)smem);                                                                 \
-    if (M == MM && scheme == SS)                                                                     \
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, fp_sweep<T, MM, SS, BND, FIX>,              \
-                                                    sweep_threads(sizeof(T) == 4, SS, FIX), smem);   \
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, fp_sweep<T, MM, SS, BND, FIX>,                \
+                                                  sweep_threads(sizeof(T) == 4, SS, FIX), smem);     \
   }
   FPK_OCC(2, 0) FPK_OCC(4, 0) FPK_OCC(6, 0) FPK_OCC(8, 0)
   FPK_OCC(2, 1) FPK_OCC(4, 1) FPK_OCC(6, 1) FPK_OCC(8, 1)
@@ -1177,9 +1210,8 @@ int prepare_t(int M, int scheme) {
 // One translation unit per (precision, boundary rules, fixed switches): the launcher and the
 // preparation of its 16 (M, scheme) variants, named launch_sweep_<NAME> / prepare_sweep_<NAME>.
 #define FPK_SWEEP_UNIT(NAME, T, BND, FIX)                                                           \
-  cudaError_t launch_sweep_##NAME(const SweepLaunch &L, int M, int scheme, int charwise, int fp,    \
-                                  cudaStream_t s) {                                                 \
-    return launch_sweep_t<T, BND, FIX>(L, M, scheme, charwise, fp, s);                              \
+  cudaError_t launch_sweep_##NAME(const SweepLaunch &L, int M, int scheme, int fp, cudaStream_t s) { \
+    return launch_sweep_t<T, BND, FIX>(L, M, scheme, fp, s);                                        \
   }                                                                                                 \
   int prepare_sweep_##NAME(int M, int scheme) { return prepare_t<T, BND, FIX>(M, scheme); }
 

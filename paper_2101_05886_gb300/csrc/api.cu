@@ -216,7 +216,7 @@ void set_shapes(C *c, int is_f32, int M, int scheme, int fix) {
   for (int a = 0; a < c->nshape; ++a) {
     const int f = fix + a;   // fix = 2: the alternative shape
     c->nt[a] = fpk::sweep_threads(is_f32, scheme, f);
-    c->pad[a] = fpk::sweep_padded(is_f32, scheme, f) ? 1 : 0;
+    c->pad[a] = c->nt[a] != 64;
     c->per_sm[a] = prepare(is_f32, M, scheme, f);
   }
   if (c->nshape == 1) { c->nt[1] = c->nt[0]; c->pad[1] = c->pad[0]; c->per_sm[1] = c->per_sm[0]; }
@@ -256,6 +256,21 @@ void default_tile(int dir, int nt, int *S, int *TT) {
   *TT = nt / *S;
 }
 
+// the constants of BlockDev::cst, in the sweep's type
+template <typename T>
+void sweep_constants(const fp_grid_desc &d, T *c) {
+  for (int v = 0; v < 5; ++v) c[v] = (T)d.q_inf[v];
+  T m2 = 0;
+  for (int a = 0; a < 3; ++a) {
+    c[5 + a] = c[1 + a] / c[0];
+    m2 += c[1 + a] * c[5 + a];
+  }
+  c[9] = (T)(d.gamma - 1.0);
+  c[8] = c[9] * (c[4] - T(0.5) * m2);
+  c[10] = (T)d.gamma;
+  c[11] = T(1) / c[9];
+}
+
 void fill_dirs(fp_ctx *c) {
   const int ni = c->desc.n[0], nj = c->desc.n[1], nk = c->desc.n[2], G = c->G;
   const int dims = c->desc.dims;
@@ -290,7 +305,7 @@ void fill_dirs(fp_ctx *c) {
   }
   for (int d = 0; d < 3; ++d) {
     DirDev &D = B.dir[d];
-    D.fc = c->nface[d];
+    D.fc = (unsigned)c->nface[d];
     D.bclo = c->desc.bc[d][0];
     D.bchi = c->desc.bc[d][1];
     D.fmet = c->fmet[d];
@@ -306,22 +321,23 @@ void fill_dirs(fp_ctx *c) {
       D.hsd = st[d];
       D.hT1 = st[ta];
       D.hT2 = st[tb];
-      D.hc = e[0] * e[1] * e[2];
+      D.hc = (unsigned)(e[0] * e[1] * e[2]);
     }
     default_tile(d, c->nt[0], &D.S, &D.TT);
     if (d >= dims) D.nt2 = 0;
   }
   B.dims = dims;
   B.G = G;
-  B.qc = (long long)ni * nj * nk;
-  B.mc = c->nmet;
-  B.moff = G + (long long)G * ms1 + (dims == 3 ? (long long)G * ms2 : 0);
+  B.qc = (unsigned)c->ncells;
+  B.mc = (unsigned)c->nmet;
+  B.moff = (unsigned)(G + (long long)G * ms1 + (dims == 3 ? (long long)G * ms2 : 0));
   B.met = c->met;
   B.q[0] = nullptr; B.q[1] = c->q1; B.q[2] = c->q2;
   B.racc = c->racc;
   B.dqdt = nullptr;
-  for (int v = 0; v < 5; ++v) B.qbar[v] = c->desc.q_inf[v];
   B.gamma = c->desc.gamma;
+  if (c->is_f32) sweep_constants(c->desc, reinterpret_cast<float *>(B.cst));
+  else sweep_constants(c->desc, B.cst);
   B.status = c->status;
   B.global_lf = c->desc.global_lf;
   B.lamg = c->lamg;

@@ -13,20 +13,20 @@ constexpr int kNextFields = 15;      // staged per thread: next chunk's cell (Q,
 constexpr int kEpiFields = 13;       // epilogue operands staged per thread (accumulator, Q^n, dk)
 
 // CTA shape of a sweep variant (precision, scheme, fix: 0 switches read at run time, 1 folded,
-// 2 folded with the alternative shape, 3 component-wise): its threads, which equal faces per chunk x lines per
-// tile, whether the rings of the xi pass (lines of 2S slots, one after the other) are padded to
-// 3S slots per line so that every tile shape is free of bank conflicts (unpadded, the xi pass
-// takes S = 32 only), and the CTAs one SM holds.
+// 2 folded with the alternative shape, 3 component-wise): its threads, which equal faces per chunk x
+// lines per tile, whether the rings of the xi pass are padded (none is: turning the slots of
+// every other group of lines keeps all tile shapes free of bank conflicts), and the CTAs one SM
+// holds.
 // Small CTAs pay: the warps of a CTA meet at two barriers per chunk, so with fewer warps per
 // CTA the phases of the chunk (staging, FMA-heavy faces, epilogue) of different CTAs overlap
 // instead of running in step.  Large ones pay where the eta and zeta passes coalesce across
 // more lines (TT): a 256^3 block runs linear upwind 12 % faster at 128 threads (TT = 16) than
 // at 64 (TT = 8), a batch of blocks up to 128^3 12 % slower.  So the folded FP32 sweeps have
-// two shapes, and a batch's autotuner picks one per direction:
-//   WENO5-JS:       64 threads, unpadded, 8 CTAs per SM  |  alternative 128, padded, 4
-//   linear upwind: 128 threads, padded, 4                |  alternative  64, unpadded, 8
-//   WENO7-JS:      128 threads, padded, 2 (255 registers) |  alternative  64, unpadded, 4
-// Every other sweep: 128 threads, padded, 4 CTAs (FP32) or 2 (FP64, and WENO7).
+// two shapes, and a batch runs the one sweep_batch_shape names:
+//   WENO5-JS:       64 threads, 8 CTAs per SM             |  alternative 128, 4
+//   linear upwind: 128 threads, 4                         |  alternative  64, 8
+//   WENO7-JS:      128 threads, 2 (255 registers)         |  alternative  64, 4
+// Every other sweep: 128 threads, 4 CTAs (FP32) or 2 (FP64, and WENO7).
 // Single blocks run the primary shape; batches the shape sweep_batch_shape names, which was
 // the faster one on the 64-block workload (its step graph runs two branches side by side, and
 // kernels of two shapes there would not share SMs, so a batch runs one shape throughout):
@@ -41,11 +41,9 @@ __host__ __device__ constexpr int sweep_threads(bool f32, int scheme, int fix) {
   return !sweep_has_alt(f32, scheme, fix) ? 128
          : ((scheme == 0) != (fix == 2) ? 64 : 128);   // WENO5 primary 64, the others' alternative 64
 }
-__host__ __device__ constexpr bool sweep_padded(bool f32, int scheme, int fix) {
-  return sweep_threads(f32, scheme, fix) != 64;
-}
+__host__ __device__ constexpr bool sweep_padded(bool, int, int) { return false; }
 __host__ __device__ constexpr int sweep_ring(bool f32, int scheme, int fix) {
-  return (sweep_padded(f32, scheme, fix) ? 3 : 2) * sweep_threads(f32, scheme, fix);
+  return 2 * sweep_threads(f32, scheme, fix);
 }
 __host__ __device__ constexpr int sweep_min_ctas(bool f32, int scheme, int fix) {
   return (!f32 || scheme == 2 ? 256 : 512) / sweep_threads(f32, scheme, fix);
@@ -89,8 +87,8 @@ __device__ __forceinline__ P fpk_in(P p, P base, long long n, int *status) {
 #endif
 
 // One swept direction of one block.  A "line" runs along the swept direction.  Strides of one
-// grid index are 32-bit (extents are at most 2^20 and a block holds fewer than 2^31 points),
-// products with an index 64-bit.
+// grid index and component, and element offsets within a component, are 32-bit: a block holds
+// fewer than 2^31 points (and fewer than 2^32 with its ghosts, or its metrics fit no device).
 struct DirDev {
   int nd;              // points along the line
   int nt1;             // extent of the first transverse coordinate (lines are numbered t1 + nt1 t2)
@@ -98,7 +96,7 @@ struct DirDev {
   int qT1, qT2, qsd;   // state offsets: t1, t2 and along-line strides
   int mT1, mT2, msd;   // metric offsets (ghosted arrays)
   int fT1, fT2, fsd;   // face-metric offsets, face f+1/2 at (f+1)*fsd
-  long long fc;        // face-metric component stride
+  unsigned fc;         // face-metric component stride
   int bclo, bchi;      // boundary codes at the two line ends
   int S, TT;           // faces per chunk, lines per tile (S * TT == the variant's sweep_threads)
   const void *fmet;    // T [3][faces]
@@ -107,7 +105,7 @@ struct DirDev {
   // state with this direction's extent replaced by G (strides: t1, t2, along the line, component)
   const void *halo[2];
   int hT1, hT2, hsd;
-  long long hc;
+  unsigned hc;
 };
 
 // 16-byte aligned and padded so that the sweep can copy a descriptor into shared memory in
@@ -116,15 +114,17 @@ struct alignas(16) BlockDev {
   DirDev dir[3];
   int dims;
   int G;               // metric ghost width
-  long long qc;        // state component stride (ni*nj*nk)
-  long long mc;        // metric component stride
-  long long moff;      // offset of point (0,0,0) in the metric arrays
+  unsigned qc;         // state component stride (ni*nj*nk)
+  unsigned mc;         // metric component stride
+  unsigned moff;       // offset of point (0,0,0) in the metric arrays
   const void *met;     // T [10][...] cell metrics with G ghosts
   void *q[3];          // stage states: 0 = Q^n (caller), 1 = Q^(1), 2 = Q^(2)
   void *racc;          // residual accumulator, state layout
   void *dqdt;          // output of the rhs mode
-  double qbar[5];      // reference state (far-field state)
   double gamma;
+  // the sweep's constants in its arithmetic type (12 float or double values): reference (far-field)
+  // state, its velocity and pressure, gamma - 1, gamma, 1/(gamma - 1)
+  alignas(16) double cst[12];
   int *status;         // device status word: ST_NONFINITE, ST_BOUNDS
   int global_lf;       // 1: Lax-Friedrichs speeds from lamg instead of the stencil
   void *lamg;          // T [3 directions][3]: max |U - c|grad||, |U|, |U + c|grad|| over the block

@@ -231,11 +231,19 @@ __device__ __forceinline__ typename PairOf<T>::type recon7_pair(const typename P
   return pfma(num, pmk(Num<T>::rcp(den.x), Num<T>::rcp(den.y)), v[3]);
 }
 
+// element `off` of component v of an array whose components are `stride` elements apart (both
+// below 2^32, one 32 x 32 + 64 bit multiply-add each)
+template <typename T>
+__device__ __forceinline__ T *comp_at(T *base, unsigned off, unsigned stride, unsigned v) {
+  return reinterpret_cast<T *>(reinterpret_cast<unsigned long long>(base) + (unsigned long long)off * sizeof(T) +
+                               (unsigned long long)stride * (v * (unsigned)sizeof(T)));
+}
+
 // Slip-wall reflection of a ghost value (the mirror cell's state Q) about the boundary
 // face metric fm (component stride fcs): m - 2 (m.k) k/|k|^2.
 template <typename T>
-__device__ __forceinline__ void wall_reflect(T Q[5], const T *fm, long long fcs) {
-  const T n0 = fm[0], n1 = fm[fcs], n2 = fm[2 * fcs];
+__device__ __forceinline__ void wall_reflect(T Q[5], const T *fm, unsigned fcs) {
+  const T n0 = fm[0], n1 = *comp_at(fm, 0, fcs, 1), n2 = *comp_at(fm, 0, fcs, 2);
   const T s = T(2) * (Q[1] * n0 + Q[2] * n1 + Q[3] * n2) / (n0 * n0 + n1 * n1 + n2 * n2);
   Q[1] -= s * n0;
   Q[2] -= s * n1;
@@ -350,10 +358,9 @@ template <typename T, int M, int SCHEME, bool BND, int FIX>
 __global__ void __launch_bounds__(sweep_threads(sizeof(T) == 4, SCHEME, FIX), sweep_min_ctas(sizeof(T) == 4, SCHEME, FIX))
 fp_sweep(const BlockDev *__restrict__ blocks, const SweepItem *__restrict__ items, int dir, int mode,
          int stage, const double *__restrict__ dtp, int fpform_arg) {
-  // this variant's CTA shape (fp_internal.h): threads, ring stride of a staged field, padding
+  // this variant's CTA shape (fp_internal.h): threads, ring stride of a staged field
   constexpr int kThreads = sweep_threads(sizeof(T) == 4, SCHEME, FIX);
   constexpr int kRing = sweep_ring(sizeof(T) == 4, SCHEME, FIX);
-  constexpr bool kPad = sweep_padded(sizeof(T) == 4, SCHEME, FIX);
   constexpr bool kFold = FIX == 1 || FIX == 2;
   constexpr int charwise = FIX == 3 ? 0 : 1;
   const int fpform = kFold ? 1 : fpform_arg;
@@ -405,21 +412,19 @@ fp_sweep(const BlockDev *__restrict__ blocks, const SweepItem *__restrict__ item
     const int S = D->S, TT = D->TT, W = 2 * S;
     // thread roles: along-line index tf and line index tl.  The xi pass puts
     // consecutive threads along the line (coalesced, i contiguous), the other passes
-    // across lines.  Shared layout: slot-fast lines are 3S apart (conflict-free for
-    // S < 32 as well) or, unpadded, 2S apart (the host then gives the xi pass S = 32),
-    // line-fast slots are TT apart.
+    // across lines.  Shared layout: line-fast slots are TT apart; slot-fast lines 2S apart, with
+    // the slots of every other run of 32/S lines turned by S, so that the lines a warp reads at
+    // once lie in different banks for every S.
     const bool slotFast = (dir == 0);
     const int tf = slotFast ? (tid % S) : (tid / TT);
     const int tl = slotFast ? (tid / S) : (tid % TT);
-    const int LS = slotFast ? (kPad ? 3 : 2) * S : 1;
     const int SS = slotFast ? 1 : TT;
-    const int lbase = tl * LS;
-    const int wm = W - 1;
+    const int lbase = slotFast ? tl * W : tl;
+    const int turn = slotFast && S < 32 && (tl & (16 / S)) ? S : 0;
     const int nd = D->nd, nt1 = D->nt1, nt2 = D->nt2;
-    const int qsd = D->qsd, msd = D->msd, fsd = D->fsd;
-    const long long fcs = D->fc;
-    const long long qc = B->qc, mc = B->mc;
-    const int G = B->G, bclo = D->bclo, bchi = D->bchi;
+    const int qsd = D->qsd;
+    const unsigned fcs = D->fc, qc = B->qc, mc = B->mc;
+    const int G = B->G;
     // The lines of a tile row are marched as one stream of positions: line after line, each with
     // its G ghost cells at both ends (period P).  `u` is a position within its line (cell
     // x = u - G) and (t1, t2) that line's transverse coordinates.  A chunk may cover the end of
@@ -437,38 +442,47 @@ fp_sweep(const BlockDev *__restrict__ blocks, const SweepItem *__restrict__ item
       t1 = line - t2 * nt1;
     };
     const int step2 = TT * item.stride / nt1, step1 = TT * item.stride - step2 * nt1;
+    const bool shortLines = P < S + 4;   // a step of a chunk can pass more than one line
     auto wrap = [&](int &u, int &t1, int &t2) {
+      const bool p = u >= P;
+      u -= p ? P : 0;
+      t1 += p ? step1 : 0;
+      t2 += p ? step2 : 0;
+      const bool c = t1 >= nt1;
+      t1 -= c ? nt1 : 0;
+      t2 += c ? 1 : 0;
+      if (shortLines)
 #pragma unroll 1
-      while (u >= P) {
-        u -= P;
-        t1 += step1;
-        t2 += step2;
-        if (t1 >= nt1) { t1 -= nt1; ++t2; }
-      }
+        while (u >= P) {
+          u -= P;
+          t1 += step1;
+          t2 += step2;
+          if (t1 >= nt1) { t1 -= nt1; ++t2; }
+        }
     };
-    const T *__restrict__ met = static_cast<const T *>(B->met) + B->moff;
+    const T *__restrict__ met = static_cast<const T *>(B->met);
     const T *__restrict__ fmet = static_cast<const T *>(D->fmet);
     const T *__restrict__ qin = static_cast<const T *>(B->q[stage]);
-    const T g1 = T(B->gamma - 1.0), gam = T(B->gamma), rg1 = Num<T>::rcp(g1);
     const int glf = kFold ? 0 : B->global_lf;
-    T qb[5];
-#pragma unroll
-    for (int v = 0; v < 5; ++v) qb[v] = T(B->qbar[v]);
-    // far-field reference state primitives
-    const T qbr = Num<T>::rcp(qb[0]);
-    const T ub[3] = {qb[1] * qbr, qb[2] * qbr, qb[3] * qbr};
-    const T pb = g1 * (qb[4] - T(0.5) * (qb[1] * ub[0] + qb[2] * ub[1] + qb[3] * ub[2]));
-    const T mbq[3] = {qb[1], qb[2], qb[3]};
+    // the block's constants in the arithmetic type: far-field state, its velocity and pressure,
+    // gamma - 1, gamma, 1/(gamma - 1)
+    const T *const cst = reinterpret_cast<const T *>(B->cst);
+    const T g1 = cst[9], gam = cst[10], rg1 = cst[11];
 
     auto off = [&](int x) -> int {
-      const int o = lbase + (x & wm) * SS;
+      const int o = lbase + ((x + turn) & (W - 1)) * SS;
       FPK_CHK_ONLY(if (o < 0 || o >= kRing) { atomicOr(B->status, ST_BOUNDS); return 0; })
       return o;
     };
-    // offsets of line (t1, t2) in the state, the ghosted metrics and the face metrics
-    auto qline = [&](int t1, int t2) { return (long long)t1 * D->qT1 + (long long)t2 * D->qT2; };
-    auto mline = [&](int t1, int t2) { return (long long)t1 * D->mT1 + (long long)t2 * D->mT2; };
-    auto fline = [&](int t1, int t2) { return (long long)t1 * D->fT1 + (long long)t2 * D->fT2; };
+    // offsets of cell / face x of line (t1, t2) in the state, the ghosted metrics and the face
+    // metrics (face x + 1/2): below 2^32
+    auto qoff = [&](int x, int t1, int t2) { return (unsigned)t1 * D->qT1 + (unsigned)t2 * D->qT2 + (unsigned)x * qsd; };
+    auto moff = [&](int x, int t1, int t2) {
+      return B->moff + (unsigned)t1 * D->mT1 + (unsigned)t2 * D->mT2 + (unsigned)x * D->msd;
+    };
+    auto foff = [&](int x, int t1, int t2) {
+      return (unsigned)t1 * D->fT1 + (unsigned)t2 * D->fT2 + (unsigned)(x + 1) * D->fsd;
+    };
 
     // boundary rule of cell index x of line (t1, t2): the source cell (its first component
     // at src, component stride cs), or the far-field state (far); `wall` asks for the
@@ -477,68 +491,72 @@ fp_sweep(const BlockDev *__restrict__ blocks, const SweepItem *__restrict__ item
     // with t1 reversed, wall outside the cut width), 5 another block of the batch (its cells
     // next to its opposite side, same transverse indices, same RK stage), 6 the caller's halo
     // buffer of that side (the cells another process holds, refreshed for every RK stage).
-    auto bc_source = [&](int x, int t1, int t2, const T *&src, long long &cs, bool &far,
+    auto bc_source = [&](int x, int t1, int t2, const T *&src, unsigned &cs, bool &far,
                          bool &wall FPK_CHK_ONLY(, const T *&sb, long long &sn)) {
-      int xx = x;
-      int s1 = t1;
+      src = qin + qoff(x, t1, t2);
       cs = qc; far = false; wall = false;
-      FPK_CHK_ONLY(sb = qin; sn = 5 * qc;)
-      if (x < 0 || x >= nd) {
-        const int bc = x < 0 ? bclo : bchi;
-        if (bc == 0) { xx = x % nd; if (xx < 0) xx += nd; }
-        else if (bc == 1) far = true;
-        else if (bc == 2 || !BND) xx = x < 0 ? 0 : nd - 1;
-        else if (bc == 6) {   // halo buffer: index x + G below the line, x - nd above it
-          const long long hx = x < 0 ? x + G : x - nd;
-          src = static_cast<const T *>(D->halo[x < 0 ? 0 : 1]) + (long long)t1 * D->hT1 + (long long)t2 * D->hT2 +
-                hx * D->hsd;
+      FPK_CHK_ONLY(sb = qin; sn = 5LL * qc;)
+      if ((unsigned)x >= (unsigned)nd) {
+        const int hi = x >= 0, bc = hi ? D->bchi : D->bclo;
+        if (bc == 1) {
+          far = true;
+        } else if (BND && bc == 6) {   // halo buffer: index x + G below the line, x - nd above it
+          src = static_cast<const T *>(D->halo[hi]) +
+                ((unsigned)t1 * D->hT1 + (unsigned)t2 * D->hT2 + (unsigned)(hi ? x - nd : x + G) * D->hsd);
           cs = D->hc;
-          FPK_CHK_ONLY(sb = static_cast<const T *>(D->halo[x < 0 ? 0 : 1]); sn = 5 * D->hc;)
-          return;
-        } else if (bc == 5) {
-          const BlockDev *NB = blocks + B->nbr[dir][x < 0 ? 0 : 1];
+          FPK_CHK_ONLY(sb = static_cast<const T *>(D->halo[hi]); sn = 5LL * D->hc;)
+        } else if (BND && bc == 5) {
+          const BlockDev *NB = blocks + B->nbr[dir][hi];
           const DirDev *ND = &NB->dir[dir];
-          src = static_cast<const T *>(NB->q[stage]) + (long long)t1 * ND->qT1 + (long long)t2 * ND->qT2 +
-                (long long)(x < 0 ? ND->nd + x : x - nd) * ND->qsd;
+          src = static_cast<const T *>(NB->q[stage]) +
+                ((unsigned)t1 * ND->qT1 + (unsigned)t2 * ND->qT2 + (unsigned)(hi ? x - nd : ND->nd + x) * ND->qsd);
           cs = NB->qc;
-          FPK_CHK_ONLY(sb = static_cast<const T *>(NB->q[stage]); sn = 5 * NB->qc;)
-          return;
+          FPK_CHK_ONLY(sb = static_cast<const T *>(NB->q[stage]); sn = 5LL * NB->qc;)
         } else {
-          xx = x < 0 ? -1 - x : 2 * nd - 1 - x;
-          const int cw = B->cut;
-          if (bc == 4 && (t1 < cw || t1 >= nt1 - cw)) s1 = nt1 - 1 - t1;
-          else wall = true;
+          int xx, s1 = t1;
+          if (bc == 0) {
+            xx = x % nd;
+            if (xx < 0) xx += nd;
+          } else if (!BND || bc == 2) {
+            xx = hi ? nd - 1 : 0;
+          } else {
+            xx = hi ? 2 * nd - 1 - x : -1 - x;
+            const int cw = B->cut;
+            if (bc == 4 && (t1 < cw || t1 >= nt1 - cw)) s1 = nt1 - 1 - t1;
+            else wall = true;
+          }
+          src = qin + qoff(xx, s1, t2);
         }
       }
-      src = qin + qline(s1, t2) + (long long)xx * qsd;
+    };
+    // slip wall: reflect about the boundary face of the line (face -1/2 or nd-1/2)
+    auto reflect = [&](int x, int t1, int t2, T Q[5]) {
+      wall_reflect<T>(Q, FPK_IN(fmet + foff(x < 0 ? -1 : nd - 1, t1, t2), fmet, fcs, B->status), fcs);
     };
 
     // global loads of one cell (Q, metric vector, 1/J) with the boundary rule applied
     auto fetch = [&](int x, int t1, int t2, T Q[5], T k[3], T &invJ) {
       if (x >= -G && x < nd + G) {
-        const long long mo = mline(t1, t2) + (long long)x * msd;
-        FPK_CHK_ONLY(const T *const metb = static_cast<const T *>(B->met);)
+        const unsigned mo = moff(x, t1, t2);
 #pragma unroll
-        for (int a = 0; a < 3; ++a) k[a] = *FPK_IN(met + ((3LL * dir + a) * mc + mo), metb, 10 * mc, B->status);
-        invJ = *FPK_IN(met + (9LL * mc + mo), metb, 10 * mc, B->status);
+        for (int a = 0; a < 3; ++a) k[a] = *FPK_IN(comp_at(met, mo, mc, 3 * dir + a), met, 10LL * mc, B->status);
+        invJ = *FPK_IN(comp_at(met, mo, mc, 9), met, 10LL * mc, B->status);
         const T *qp;
-        long long cs;
+        unsigned cs;
         bool far, wall;
         FPK_CHK_ONLY(const T *sb; long long sn;)
         bc_source(x, t1, t2, qp, cs, far, wall FPK_CHK_ONLY(, sb, sn));
         if (far) {
 #pragma unroll
-          for (int v = 0; v < 5; ++v) Q[v] = qb[v];
+          for (int v = 0; v < 5; ++v) Q[v] = cst[v];
         } else {
 #pragma unroll
-          for (int v = 0; v < 5; ++v) Q[v] = __ldg(FPK_IN(qp + v * cs, sb, sn, B->status));
-          // slip wall: reflect about the boundary face of this line (face -1/2 or nd-1/2)
-          if (BND && wall)
-            wall_reflect<T>(Q, FPK_IN(fmet + (fline(t1, t2) + (x < 0 ? 0LL : (long long)nd * fsd)), fmet, fcs, B->status), fcs);
+          for (int v = 0; v < 5; ++v) Q[v] = __ldg(FPK_IN(comp_at(qp, 0, cs, v), sb, sn, B->status));
+          if (BND && wall) reflect(x, t1, t2, Q);
         }
       } else {   // before the first line of the item: no face of a line uses it
 #pragma unroll
-        for (int v = 0; v < 5; ++v) Q[v] = qb[v];
+        for (int v = 0; v < 5; ++v) Q[v] = cst[v];
         k[0] = T(1); k[1] = T(0); k[2] = T(0);
         invJ = T(1);
       }
@@ -567,54 +585,53 @@ fp_sweep(const BlockDev *__restrict__ blocks, const SweepItem *__restrict__ item
     // `slot` (0/1, alternating between chunks)
     auto prefetch_face = [&](int x, int t1, int t2, int slot) {
       T *dst = nsb + tid + (9 + 3 * slot) * kThreads;
-      const long long fo = fline(t1, t2) + (long long)(x + 1) * fsd;
+      const unsigned fo = foff(x, t1, t2);
 #pragma unroll
       for (int c = 0; c < 3; ++c)
-        cp_async_el(dst + c * kThreads, FPK_IN(fmet + (c * fcs + fo), fmet, 3 * fcs, B->status));
+        cp_async_el(dst + c * kThreads, FPK_IN(comp_at(fmet, fo, fcs, c), fmet, 3LL * fcs, B->status));
     };
     // asynchronous copy of one cell's loads (-G <= x < nd + G) into this thread's staging slots
     auto prefetch_cell = [&](int x, int t1, int t2) {
       T *dst = nsb + tid;
-      const long long mo = mline(t1, t2) + (long long)x * msd;
-      FPK_CHK_ONLY(const T *const metb = static_cast<const T *>(B->met);)
+      const T *const mp = met + moff(x, t1, t2), *const md = comp_at(mp, 0, mc, 3 * dir);
 #pragma unroll
       for (int a = 0; a < 3; ++a)
-        cp_async_el(dst + (5 + a) * kThreads, FPK_IN(met + ((3LL * dir + a) * mc + mo), metb, 10 * mc, B->status));
-      cp_async_el(dst + 8 * kThreads, FPK_IN(met + (9LL * mc + mo), metb, 10 * mc, B->status));
+        cp_async_el(dst + (5 + a) * kThreads, FPK_IN(comp_at(md, 0, mc, a), met, 10LL * mc, B->status));
+      cp_async_el(dst + 8 * kThreads, FPK_IN(comp_at(mp, 0, mc, 9), met, 10LL * mc, B->status));
       const T *qp;
-      long long cs;
+      unsigned cs;
       bool far, wall;
       FPK_CHK_ONLY(const T *sb; long long sn;)
       bc_source(x, t1, t2, qp, cs, far, wall FPK_CHK_ONLY(, sb, sn));
       if (far) {
 #pragma unroll
-        for (int v = 0; v < 5; ++v) dst[v * kThreads] = qb[v];
+        for (int v = 0; v < 5; ++v) dst[v * kThreads] = cst[v];
       } else {   // a wall ghost copies its mirror cell; the reflection is applied when staged
 #pragma unroll
-        for (int v = 0; v < 5; ++v) cp_async_el(dst + v * kThreads, FPK_IN(qp + v * cs, sb, sn, B->status));
+        for (int v = 0; v < 5; ++v)
+          cp_async_el(dst + v * kThreads, FPK_IN(comp_at(qp, 0, cs, v), sb, sn, B->status));
       }
     };
     // asynchronous copy of the epilogue operands of a cell (state offset qo: residual
     // accumulator, Q^n, metric differences) into this thread's slots
-    auto prefetch_epilogue = [&](long long qo) {
+    auto prefetch_epilogue = [&](unsigned qo) {
       T *dst = epb + tid;
       if (mode != MODE_WRITE) {
-        const T *ra = static_cast<const T *>(B->racc) + qo;
+        const T *const ra = static_cast<const T *>(B->racc);
 #pragma unroll
-        for (int v = 0; v < 5; ++v)
-          cp_async_el(dst + v * kThreads, FPK_IN(ra + v * qc, static_cast<const T *>(B->racc), 5 * qc, B->status));
+        for (int v = 0; v < 5; ++v) cp_async_el(dst + v * kThreads, FPK_IN(comp_at(ra, qo, qc, v), ra, 5LL * qc, B->status));
       }
       if (mode == MODE_RK && stage != 0) {
-        const T *qn = static_cast<const T *>(B->q[0]) + qo;
+        const T *const qn = static_cast<const T *>(B->q[0]);
 #pragma unroll
         for (int v = 0; v < 5; ++v)
-          cp_async_el(dst + (5 + v) * kThreads, FPK_IN(qn + v * qc, static_cast<const T *>(B->q[0]), 5 * qc, B->status));
+          cp_async_el(dst + (5 + v) * kThreads, FPK_IN(comp_at(qn, qo, qc, v), qn, 5LL * qc, B->status));
       }
       if (fpform) {
-        const T *dkp = static_cast<const T *>(D->dk) + qo;
+        const T *const dkp = static_cast<const T *>(D->dk);
 #pragma unroll
         for (int c = 0; c < 3; ++c)
-          cp_async_el(dst + (10 + c) * kThreads, FPK_IN(dkp + c * qc, static_cast<const T *>(D->dk), 3 * qc, B->status));
+          cp_async_el(dst + (10 + c) * kThreads, FPK_IN(comp_at(dkp, qo, qc, c), dkp, 3LL * qc, B->status));
       }
     };
 
@@ -649,37 +666,43 @@ fp_sweep(const BlockDev *__restrict__ blocks, const SweepItem *__restrict__ item
       // this thread's face u - G + 1/2 and cell u - G of line (t1, t2)
       const bool faceOK = t2 < nt2 && u >= G - 1 && u < nd + G && a + tf < len;
       const bool cellOK = faceOK && u >= G && (ch > 0 || tf > 0);
+      const unsigned qo = qoff(u - G, t1, t2);       // the cell's offset in the state
       // ---- start the loads this chunk's epilogue and the next chunk need
-      if (cellOK) prefetch_epilogue(qline(t1, t2) + (long long)(u - G) * qsd);
+      if (cellOK) prefetch_epilogue(qo);
+      bool stageOK = false;
       if (more) {
-        int un = u + S, n1 = t1, n2 = t2;            // this thread's face of the next chunk
-        wrap(un, n1, n2);
-        if (n2 < nt2 && un >= G - 1 && un < nd + G) prefetch_face(un - G, n1, n2, (ch + 1) & 1);
-        un += 4;                                     // the cell it stages for the next chunk
-        wrap(un, n1, n2);
-        if (n2 < nt2 && a + S + tf < len) prefetch_cell(un - G, n1, n2);
+        u += S;                                      // this thread's face of the next chunk
+        wrap(u, t1, t2);
+        if (t2 < nt2 && u >= G - 1 && u < nd + G) prefetch_face(u - G, t1, t2, (ch + 1) & 1);
+        int uc = u + 4, c1 = t1, c2 = t2;            // the cell it stages for the next chunk
+        wrap(uc, c1, c2);
+        stageOK = c2 < nt2 && a + S + tf < len;
+        if (stageOK) prefetch_cell(uc - G, c1, c2);
       }
       if (ch == 0 && nit >= 0) fetch_desc(cur ^ 1, s_item[cur ^ 1].block);   // next item's descriptor
+      // opaque: the compiler otherwise splits the chunk by these conditions and spills 250 bytes
+      int staged = stageOK;
+      asm volatile("" : "+r"(staged));
       cp_async_commit();
       // ---- one face per thread: face ff + 1/2 between cells ff and ff+1
       const int ff = a + tf;
+      // the face's flux and reference-state increment, kept for the epilogue, its metric and cell
+      // ff's state (kept by linear upwind, whose face leaves the registers for it)
+      constexpr bool kOwn = SCHEME == 1 && sizeof(T) == 4;
+      T F[5], dl[5], kf[3], Qi[5];
       if (faceOK) {
-        const int i0 = ff;
         int o[8];
 #pragma unroll
-        for (int q = 0; q < 8; ++q) o[q] = off(i0 - 3 + q);
+        for (int q = 0; q < 8; ++q) o[q] = off(ff - 3 + q);
 #define CELL(field, q) sm[(field) * kRing + o[(q)]]
-        T Qi[5];
 #pragma unroll
-        for (int v = 0; v < 5; ++v) Qi[v] = CELL(CF_Q + v, 3);
+        for (int v = 0; v < 5; ++v) { Qi[v] = CELL(CF_Q + v, 3); dl[v] = T(0); }
         // face metric of this face, staged by the previous chunk (or the prologue)
-        T kf[3];
 #pragma unroll
         for (int c = 0; c < 3; ++c) kf[c] = nsb[(9 + 3 * (ch & 1) + c) * kThreads + tid];
 
         // reference face state Q* = Q_i + delta (Eqs. Q_star, QdJ_star, 1dJ at order M)
         using P = typename PairOf<T>::type;
-        T dl[5] = {T(0), T(0), T(0), T(0), T(0)};
         // The cells q = kQlo .. kQlo + M - 1 of the weighted sum are taken in mirror pairs
         // (kQlo + m, kQlo + M - 1 - m), m < M/2, whose weights are equal, two cells per packed
         // instruction.  These are the stencil loops' pairs (q, 7 - q) of the same cells, so linear
@@ -1019,7 +1042,6 @@ fp_sweep(const BlockDev *__restrict__ blocks, const SweepItem *__restrict__ item
             }
           }
         }
-        T F[5];
         if (charwise) {
           // in the frame of the face; H' = c^2/(gamma-1) + w^2/2
           const T sa = h[0] + h[4], da = cs * (h[4] - h[0]), s1 = sa + h[1];
@@ -1052,76 +1074,78 @@ fp_sweep(const BlockDev *__restrict__ blocks, const SweepItem *__restrict__ item
       }
       cp_async_wait_all();
       __syncthreads();
-      // ---- residual of cell x = a + tf from its two faces, then the epilogue
-      const int x = a + tf;
+      // ---- residual of cell x = a + tf from its two faces (the upper one is this thread's own),
+      // then the epilogue
       if (cellOK) {
-        const long long qo = qline(t1, t2) + (long long)(u - G) * qsd;
-        const int ox = off(x), oxm = off(x - 1);
+        const int oxm = off(ff - 1);
+        if constexpr (!kOwn) {                       // loaded again rather than held over the face's arithmetic
+          const int ox = off(ff);
+#pragma unroll
+          for (int v = 0; v < 5; ++v) Qi[v] = sm[(CF_Q + v) * kRing + ox];
+#pragma unroll
+          for (int c = 0; c < 3; ++c) kf[c] = nsb[(9 + 3 * (ch & 1) + c) * kThreads + tid];
+        }
         T R[5];
 #pragma unroll
-        for (int v = 0; v < 5; ++v) R[v] = fr[v * kRing + ox] - fr[v * kRing + oxm];
+        for (int v = 0; v < 5; ++v) R[v] = F[v] - fr[v * kRing + oxm];
         if (fpform) {
           // reference states of the two faces: Q*_+ = Q_x + delta_+, Q*_- = Q_{x-1} + delta_-
-          T Qp[5], Qm[5], dQ[5], dqm[5];
+          T Qp[5], Qm[5], dQ[5], dqm[5], qb[5];
 #pragma unroll
           for (int v = 0; v < 5; ++v) {
-            const T qx = sm[(CF_Q + v) * kRing + ox], qx1 = sm[(CF_Q + v) * kRing + oxm];
-            const T dp = fr[(5 + v) * kRing + ox], dm = fr[(5 + v) * kRing + oxm];
-            Qp[v] = qx + dp;
+            qb[v] = cst[v];
+            const T qx1 = sm[(CF_Q + v) * kRing + oxm], dm = fr[(5 + v) * kRing + oxm];
+            Qp[v] = Qi[v] + dl[v];
             Qm[v] = qx1 + dm;
-            dQ[v] = (qx - qx1) + (dp - dm);
+            dQ[v] = (Qi[v] - qx1) + (dl[v] - dm);
             dqm[v] = (qx1 - qb[v]) + dm;
           }
+          const T ub[3] = {cst[5], cst[6], cst[7]}, pb = cst[8];
           const T rA = Num<T>::rcp(Qm[0]);
           const T uA[3] = {Qm[1] * rA, Qm[2] * rA, Qm[3] * rA};
           const T pA = g1 * (Qm[4] - T(0.5) * (Qm[1] * uA[0] + Qm[2] * uA[1] + Qm[3] * uA[2]));
           const T mA[3] = {Qm[1], Qm[2], Qm[3]};
           const T rB = Num<T>::rcp(Qp[0]);
           const T uBp[3] = {Qp[1] * rB, Qp[2] * rB, Qp[3] * rB};
-          // k_{x+1/2} is the metric of the face this thread computed in this chunk
-          T kp[3], dk[3];
+          T dk[3];
 #pragma unroll
-          for (int c = 0; c < 3; ++c) {
-            dk[c] = epb[(10 + c) * kThreads + tid];
-            kp[c] = nsb[(9 + 3 * (ch & 1) + c) * kThreads + tid];
-          }
+          for (int c = 0; c < 3; ++c) dk[c] = epb[(10 + c) * kThreads + tid];
           T t1v[5], t2v[5];
-          dflux<T>(g1, rB, uBp, uA, mA, Qm[4], pA, dQ, kp, t1v);          // [F(Q*_+) - F(Q*_-)] . k_+
-          dflux<T>(g1, rA, uA, ub, mbq, qb[4], pb, dqm, dk, t2v);         // [F(Q*_-) - F(Qbar)] . (k_+ - k_-)
+          dflux<T>(g1, rB, uBp, uA, mA, Qm[4], pA, dQ, kf, t1v);          // [F(Q*_+) - F(Q*_-)] . k_+
+          dflux<T>(g1, rA, uA, ub, qb + 1, qb[4], pb, dqm, dk, t2v);       // [F(Q*_-) - F(Qbar)] . (k_+ - k_-)
 #pragma unroll
           for (int v = 0; v < 5; ++v) R[v] += t1v[v] + t2v[v];
         }
-        T *racc = static_cast<T *>(B->racc) + qo;
-        FPK_CHK_ONLY(T *const raccb = static_cast<T *>(B->racc);)
+        T *const racc = static_cast<T *>(B->racc);
         const T *ra = epb + tid;                      // prefetched accumulator
         if (mode == MODE_WRITE) {
 #pragma unroll
-          for (int v = 0; v < 5; ++v) *FPK_IN(racc + v * qc, raccb, 5 * qc, B->status) = R[v];
+          for (int v = 0; v < 5; ++v) *FPK_IN(comp_at(racc, qo, qc, v), racc, 5LL * qc, B->status) = R[v];
         } else if (mode == MODE_ADD) {
 #pragma unroll
-          for (int v = 0; v < 5; ++v) *FPK_IN(racc + v * qc, raccb, 5 * qc, B->status) = ra[v * kThreads] + R[v];
+          for (int v = 0; v < 5; ++v) *FPK_IN(comp_at(racc, qo, qc, v), racc, 5LL * qc, B->status) = ra[v * kThreads] + R[v];
         } else {
-          const T Jc = Num<T>::rcp(sm[CF_INVJ * kRing + ox]);
+          const T Jc = Num<T>::rcp(sm[CF_INVJ * kRing + off(ff)]);
           if (mode == MODE_RHS) {
-            T *out = static_cast<T *>(B->dqdt) + qo;
+            T *const out = static_cast<T *>(B->dqdt);
 #pragma unroll
             for (int v = 0; v < 5; ++v)
-              *FPK_IN(out + v * qc, static_cast<T *>(B->dqdt), 5 * qc, B->status) = -Jc * (ra[v * kThreads] + R[v]);
+              *FPK_IN(comp_at(out, qo, qc, v), out, 5LL * qc, B->status) = -Jc * (ra[v * kThreads] + R[v]);
           } else {
             // SSP-RK3 stage (Gottlieb & Shu) in increment form:
             // Q^(s+1) = Q^(s) + a_s (Q^n - Q^(s)) + b_s dt L(Q^(s))
             const T dt = s_dt;
             const T as = stage == 0 ? T(0) : (stage == 1 ? T(0.75) : T(1.0 / 3.0));
             const T bs = stage == 0 ? T(1) : (stage == 1 ? T(0.25) : T(2.0 / 3.0));
-            T *qo_p = static_cast<T *>(B->q[(stage + 1) % 3]) + qo;
+            T *const qs = static_cast<T *>(B->q[(stage + 1) % 3]);
             bool bad = false;
 #pragma unroll
             for (int v = 0; v < 5; ++v) {
-              const T qk = sm[(CF_Q + v) * kRing + ox];
+              const T qk = Qi[v];
               const T Lv = -Jc * (ra[v * kThreads] + R[v]);
               T nv = qk + bs * dt * Lv;
               if (stage != 0) nv = qk + as * (ra[(5 + v) * kThreads] - qk) + bs * dt * Lv;
-              *FPK_IN(qo_p + v * qc, static_cast<T *>(B->q[(stage + 1) % 3]), 5 * qc, B->status) = nv;
+              *FPK_IN(comp_at(qs, qo, qc, v), qs, 5LL * qc, B->status) = nv;
               bad |= !isfinite(nv);
             }
             if (bad) atomicOr(B->status, ST_NONFINITE);
@@ -1130,24 +1154,21 @@ fp_sweep(const BlockDev *__restrict__ blocks, const SweepItem *__restrict__ item
       }
       __syncthreads();
       // ---- stage the next chunk's new cell from this thread's staging slots
-      u += S;
-      wrap(u, t1, t2);
-      int uc = u + 4, c1 = t1, c2 = t2;
-      wrap(uc, c1, c2);
-      if (more && c2 < nt2 && a + S + tf < len) {
+      if (staged) {
         const T *src = nsb + tid;
         T Q[5] = {src[0], src[kThreads], src[2 * kThreads], src[3 * kThreads], src[4 * kThreads]};
         const T k[3] = {src[5 * kThreads], src[6 * kThreads], src[7 * kThreads]};
         if (BND) {                                   // a slip-wall ghost?
+          int uc = u + 4, c1 = t1, c2 = t2;
+          wrap(uc, c1, c2);
           const int xs = uc - G;
-          if (xs < 0 ? bclo >= 3 : xs >= nd && bchi >= 3) {
+          if (xs < 0 ? D->bclo >= 3 : xs >= nd && D->bchi >= 3) {
             const T *qp;
-            long long cs;
+            unsigned cs;
             bool far, wall;
             FPK_CHK_ONLY(const T *sb; long long sn;)
             bc_source(xs, c1, c2, qp, cs, far, wall FPK_CHK_ONLY(, sb, sn));
-            if (wall)
-              wall_reflect<T>(Q, FPK_IN(fmet + (fline(c1, c2) + (xs < 0 ? 0LL : (long long)nd * fsd)), fmet, fcs, B->status), fcs);
+            if (wall) reflect(xs, c1, c2, Q);
           }
         }
         stage_cell(a + S + 4 + tf, Q, k, src[8 * kThreads]);

@@ -6,6 +6,7 @@
 #include <algorithm>
 #include <atomic>
 #include <cmath>
+#include <cstdlib>
 #include <cstdio>
 #include <cstring>
 #include <mutex>
@@ -41,6 +42,10 @@ struct fp_ctx {
   BlockDev uploaded;                  // last BlockDev copied to dblk
   fpk::SweepItem *items[3] = {nullptr, nullptr, nullptr};
   int ncta[3] = {0, 0, 0};            // CTAs of each direction's launch
+  // all directions in one launch (blocks of at most kSplitPoints points): its items
+  int split = 0;
+  fpk::SweepItem *sitems = nullptr;
+  int nscta = 0;
   int nsm = 152;
   // CTA shapes of the context's sweep: [0] the primary one, [1] the alternative (nshape == 2,
   // the folded FP32 sweeps): threads (faces per chunk x lines per tile), xi rings padded (every
@@ -271,6 +276,14 @@ void sweep_constants(const fp_grid_desc &d, T *c) {
   c[11] = T(1) / c[9];
 }
 
+// Blocks of at most this many points run a stage's direction passes as one launch, each direction
+// into an accumulator of its own, and a second launch that sums them: three times the work per
+// launch where a pass is a few chunks per CTA.  Measured (us, passes in turn | one launch; FP32 unless
+// said): 33^2 FP64 residual 111 | 59, 48x37x29 step 93 | 76, 200^2 FP64 shock step 1029 | 868,
+// 181x97x61 step 751 | 738, 112^3 871 | 844, 96^3 FP64 21591 | 21097; but 128x120x128 1147 | 1157 and
+// 256^3 8.67 | 9.19 ms, where the sum's traffic costs more than the passes' ends.
+constexpr long long kSplitPoints = 3 << 19;
+
 void fill_dirs(fp_ctx *c) {
   const int ni = c->desc.n[0], nj = c->desc.n[1], nk = c->desc.n[2], G = c->G;
   const int dims = c->desc.dims;
@@ -308,9 +321,12 @@ void fill_dirs(fp_ctx *c) {
     D.fc = (unsigned)c->nface[d];
     D.bclo = c->desc.bc[d][0];
     D.bchi = c->desc.bc[d][1];
+    D.kmet = static_cast<const char *>(c->met) + (size_t)3 * d * c->nmet * c->esize;
     D.fmet = c->fmet[d];
     D.dk = c->dk[d];
     D.halo[0] = D.halo[1] = nullptr;
+    D.nbr[0] = D.nbr[1] = -1;
+    D.racc = c->racc;
     // halo layout: the state layout with this direction's extent replaced by G
     {
       long long e[3] = {ni, nj, nk};
@@ -332,8 +348,8 @@ void fill_dirs(fp_ctx *c) {
   B.mc = (unsigned)c->nmet;
   B.moff = (unsigned)(G + (long long)G * ms1 + (dims == 3 ? (long long)G * ms2 : 0));
   B.met = c->met;
+  B.imet = static_cast<const char *>(c->met) + (size_t)9 * c->nmet * c->esize;
   B.q[0] = nullptr; B.q[1] = c->q1; B.q[2] = c->q2;
-  B.racc = c->racc;
   B.dqdt = nullptr;
   B.gamma = c->desc.gamma;
   if (c->is_f32) sweep_constants(c->desc, reinterpret_cast<float *>(B.cst));
@@ -342,21 +358,21 @@ void fill_dirs(fp_ctx *c) {
   B.global_lf = c->desc.global_lf;
   B.lamg = c->lamg;
   B.cut = c->desc.cut_width;
-  for (int d = 0; d < 3; ++d) B.nbr[d][0] = B.nbr[d][1] = -1;
 }
 
 // The work of one block in one direction: `tiles` tiles of TT lines, each tile row a line after
 // the other in a stream of period P = nd + 2 G (see the sweep).
 struct Stream {
-  int block;
+  int block, dir;
   long long tiles;
   int P, S, G;
+  long long chunks() const { return (tiles * P + S - 1) / S; }
   long long positions(long long n) const { return n * P - 2 * G; }   // first to last cell of n tiles
 };
 
 Stream stream_of(const BlockDev &B, int block, int d) {
   const DirDev &D = B.dir[d];
-  return {block, ((long long)D.nt1 * D.nt2 + D.TT - 1) / D.TT, D.nd + 2 * B.G, D.S, B.G};
+  return {block, d, ((long long)D.nt1 * D.nt2 + D.TT - 1) / D.TT, D.nd + 2 * B.G, D.S, B.G};
 }
 
 // Cuts the tiles first .. tiles-1 of a stream into pieces of at most `k` chunks, the next piece
@@ -367,7 +383,7 @@ long long cut_stream(const Stream &s, long long first, long long k, std::vector<
   while (tile < s.tiles) {
     const long long left = (s.tiles - 1 - tile) * s.P + (s.P - s.G - u);
     const long long len = std::min(k * s.S - 1, left);
-    if (out) out->push_back({s.block, (int)tile, 1, (int)u, (int)len, -1, {0, 0}});
+    if (out) out->push_back({s.block, (int)tile, 1, (int)u, (int)len, -1, s.dir, 0});
     ++n;
     u += len;
     tile += u / s.P;
@@ -391,9 +407,9 @@ void spread_stream(const Stream &s, long long first, long long most, std::vector
   cut_stream(s, first, lo, &out);
 }
 
-// The items of one launch over direction `d`, for a device that holds `slots` CTAs at once;
-// returns the number of CTAs.  Every block gets a share g of the CTAs in proportion to its
-// positions.
+// The items of one launch, for a device that holds `slots` CTAs at once; returns the number of
+// CTAs.  Every stream (a block in one direction) gets a share g of the CTAs in proportion to its
+// chunks.
 //  - xi: the share's CTAs take equal pieces of the block's stream.  Lines follow each other in
 //    memory, so neighbouring pieces share nothing.
 //  - eta, zeta: a tile is TT adjacent points wide and shares memory sectors with the next, so
@@ -405,17 +421,17 @@ void spread_stream(const Stream &s, long long first, long long most, std::vector
 //    item, 9.97 ms with a CTA per tile in a fixed order and lines padded to chunks).  The blocks of a
 //    batch keep one item for all rounds: its graph's other branches fill the SMs that end
 //    early (64-block WENO5 step: 18.04 ms, 18.25 ms with two rounds per item).
-int make_items(const std::vector<Stream> &streams, int d, int slots, std::vector<fpk::SweepItem> &items) {
+int make_items(const std::vector<Stream> &streams, int slots, std::vector<fpk::SweepItem> &items) {
   std::vector<std::vector<fpk::SweepItem>> cta(slots);
   long long total = 0, done = 0;
-  for (const Stream &s : streams) total += s.tiles * s.P;
+  for (const Stream &s : streams) total += s.chunks();
   for (const Stream &s : streams) {
     // the CTAs c0 .. c0 + g - 1: the block's part of the line [0, total) mapped to the slots, at
     // least one (which it then shares with a neighbour)
     const long long c0 = done * slots / total;
-    done += s.tiles * s.P;
+    done += s.chunks();
     const long long g = std::max(1LL, done * slots / total - c0);
-    const long long r = d == 0 ? 0 : s.tiles / g;
+    const long long r = s.dir == 0 ? 0 : s.tiles / g;
     std::vector<fpk::SweepItem> piece;
     if (r * g < s.tiles) spread_stream(s, r * g, g, piece);
     const bool alone = streams.size() == 1;
@@ -423,7 +439,7 @@ int make_items(const std::vector<Stream> &streams, int d, int slots, std::vector
     for (long long r0 = 0; r0 < r; r0 += per) {
       const long long n = std::min(per, r - r0);
       for (long long c = 0; c < g; ++c) {
-        const fpk::SweepItem it = {s.block, (int)(r0 * g + c), (int)g, s.G, (int)s.positions(n), -1, {0, 0}};
+        const fpk::SweepItem it = {s.block, (int)(r0 * g + c), (int)g, s.G, (int)s.positions(n), -1, s.dir, 0};
         if (alone && r > per) cta.push_back({it}); else cta[c0 + c].push_back(it);
       }
     }
@@ -458,32 +474,50 @@ cudaError_t put_items(const std::vector<fpk::SweepItem> &items, fpk::SweepItem *
   return e;
 }
 
+// The items of streams of one context.  FP64: one CTA's warps keep the SM's FP64 pipe busy (two lanes
+// per clock and SM), so what counts is the chunks of the SM with the most: fewer CTAs than fit, if
+// their equal shares then leave no SM with one CTA more than others (37 x 40 x 26 points, 9
+// passes: 1.79 ms with a share per slot, 1.52 ms).  FP32 needs the resident warps to hide
+// latency: a share per slot.
+int balanced_items(const fp_ctx *c, const std::vector<Stream> &streams, int most_per_sm, std::vector<fpk::SweepItem> &items) {
+  int per_sm = most_per_sm;
+  if (!c->is_f32) {
+    long long least = -1;
+    for (int m = most_per_sm; m >= 1; --m) {
+      const int n = make_items(streams, m * c->nsm, items);
+      long long most = 0;                         // chunks of one CTA
+      for (int k = 0; k < n; ++k) {
+        long long ch = 0;
+        for (int i = k; i >= 0; i = items[i].next) {
+          const int S = c->hblk.dir[items[i].dir].S;
+          ch += (items[i].len + S) / S;
+        }
+        most = std::max(most, ch);
+      }
+      const long long cost = (n + c->nsm - 1) / c->nsm * most;
+      if (least < 0 || 20 * cost < 19 * least) { least = cost; per_sm = m; }
+    }
+  }
+  return make_items(streams, per_sm * c->nsm, items);
+}
+
 int upload_items(fp_ctx *c) {
   std::vector<fpk::SweepItem> items;
+  std::vector<Stream> all;
+  auto shape = [&](int d) { return c->nshape == 2 && c->hblk.dir[d].S * c->hblk.dir[d].TT == c->nt[1] ? 1 : 0; };
+  c->split = c->ncells <= kSplitPoints;
   for (int d = 0; d < c->desc.dims; ++d) {
-    const DirDev &D = c->hblk.dir[d];
-    const int a = c->nshape == 2 && D.S * D.TT == c->nt[1] ? 1 : 0;
-    // FP64: one CTA's warps keep the SM's FP64 pipe busy (two lanes per clock and SM), so what counts is
-    // the chunks of the SM with the most: fewer CTAs than fit, if their equal shares then
-    // leave no SM with one CTA more than others (37 x 40 x 26 points, 9 passes: 1.79 ms with a share per
-    // slot).  FP32 needs the resident warps to hide latency: a share per slot.
-    int per_sm = c->per_sm[a];
-    if (!c->is_f32) {
-      long long least = -1;
-      for (int m = c->per_sm[a]; m >= 1; --m) {
-        const int n = make_items({stream_of(c->hblk, 0, d)}, d, m * c->nsm, items);
-        long long most = 0;                       // chunks of one CTA
-        for (int k = 0; k < n; ++k) {
-          long long ch = 0;
-          for (int i = k; i >= 0; i = items[i].next) ch += (items[i].len + D.S) / D.S;
-          most = std::max(most, ch);
-        }
-        const long long cost = (n + c->nsm - 1) / c->nsm * most;
-        if (least < 0 || 20 * cost < 19 * least) { least = cost; per_sm = m; }
-      }
-    }
-    c->ncta[d] = make_items({stream_of(c->hblk, 0, d)}, d, per_sm * c->nsm, items);
+    all.push_back(stream_of(c->hblk, 0, d));
+    if (shape(d) != shape(0)) c->split = 0;       // one launch has one CTA shape
+    c->ncta[d] = balanced_items(c, {all.back()}, c->per_sm[shape(d)], items);
     cudaError_t e = put_items(items, &c->items[d]);
+    if (e != cudaSuccess) return cuda_fail(c, e, "sweep items");
+  }
+  for (int d = 0; d < c->desc.dims; ++d)          // one accumulator, or the directions' own
+    c->hblk.dir[d].racc = static_cast<char *>(c->racc) + (c->split ? (size_t)5 * d * c->ncells * c->esize : 0);
+  if (c->split) {
+    c->nscta = balanced_items(c, all, c->per_sm[shape(0)], items);
+    cudaError_t e = put_items(items, &c->sitems);
     if (e != cudaSuccess) return cuda_fail(c, e, "sweep items");
   }
   return FP_OK;
@@ -564,7 +598,7 @@ void fp_free(fp_ctx *c) {
   for (int d = 0; d < 3; ++d) { cudaFree(c->fmet[d]); cudaFree(c->dk[d]); cudaFree(c->items[d]); }
   cudaFree(c->q1); cudaFree(c->q2); cudaFree(c->racc);
   cudaFree(c->status); cudaFree(c->dt_dev); cudaFree(c->cfl_bits); cudaFree(c->dblk);
-  cudaFree(c->lamg); cudaFree(c->lam_items);
+  cudaFree(c->lamg); cudaFree(c->lam_items); cudaFree(c->sitems);
   delete c;
 }
 
@@ -652,7 +686,7 @@ int fp_init_grid(const fp_grid_desc *desc, const double *xyz, int ghost_nodes, v
   const size_t sbytes = (size_t)5 * c->ncells * c->esize;
   FP_TRY(fpk::dev_alloc(&c->q1, sbytes), "cudaMalloc(stage 1)");
   FP_TRY(fpk::dev_alloc(&c->q2, sbytes), "cudaMalloc(stage 2)");
-  FP_TRY(fpk::dev_alloc(&c->racc, sbytes), "cudaMalloc(residual)");
+  FP_TRY(fpk::dev_alloc(&c->racc, c->ncells <= kSplitPoints ? dims * sbytes : sbytes), "cudaMalloc(residual)");
   FP_TRY(fpk::dev_alloc(&c->status, sizeof(int)), "cudaMalloc(status)");
   FP_TRY(cudaMemset(c->status, 0, sizeof(int)), "clear status");
   FP_TRY(fpk::dev_alloc(&c->dt_dev, sizeof(double)), "cudaMalloc(dt)");
@@ -689,26 +723,46 @@ int fp_init_grid(const fp_grid_desc *desc, const double *xyz, int ghost_nodes, v
 }
 
 // the direction passes of one RK stage (rk = 1: the last pass applies the stage update) or
-// of one residual (rk = 0)
-static int run_stage(fp_ctx *c, int stage, int rk, cudaStream_t s) {
+// of one residual (rk = 0); chained: the kernel before it in the stream is this call's own
+static int run_stage(fp_ctx *c, int stage, int rk, int chained, cudaStream_t s) {
   const int dims = c->desc.dims, M = c->desc.metric_order;
   if (c->desc.global_lf) {
     cudaError_t e = fpk::launch_lambda(c->dblk, 1, c->lam_items, c->nlam_items, c->is_f32,
                                        c->desc.characteristic, stage, s);
     if (e != cudaSuccess) return cuda_fail(c, e, "global speed launch");
   }
+  if (c->split) {
+    fpk::SweepLaunch L;
+    L.blocks = c->dblk;
+    L.items = c->sitems;
+    L.grid = c->nscta;
+    L.mode = fpk::MODE_WRITE;
+    L.stage = stage;
+    L.dt = c->dt_dev;
+    L.alt = shape_of(c, c->hblk.dir[0]);
+    for (int d = 0; d < dims; ++d) L.bnd |= has_bnd(c->desc, d);
+    L.glf = c->desc.global_lf;
+    // FP64 CTAs, one or two per SM, have to be placed evenly, which the rest of a kernel before them
+    // prevents (128^2 linear upwind: a step 221 us chained, 204 us not)
+    L.chained = chained && c->is_f32;
+    cudaError_t e = launch(c->is_f32, L, M, c->desc.scheme, c->desc.characteristic,
+                           c->desc.free_stream_preserving, s);
+    if (e == cudaSuccess)
+      e = fpk::launch_finish(c->dblk, c->is_f32, c->ncells, c->desc.n, dims, rk, stage, c->dt_dev, s);
+    return e == cudaSuccess ? FP_OK : cuda_fail(c, e, "stage launch");
+  }
   for (int d = 0; d < dims; ++d) {
     fpk::SweepLaunch L;
     L.blocks = c->dblk;
     L.items = c->items[d];
     L.grid = c->ncta[d];
-    L.dir = d;
     L.mode = d == 0 ? fpk::MODE_WRITE : (d == dims - 1 ? (rk ? fpk::MODE_RK : fpk::MODE_RHS) : fpk::MODE_ADD);
     L.stage = stage;
     L.dt = c->dt_dev;
     L.alt = shape_of(c, c->hblk.dir[d]);
     L.bnd = has_bnd(c->desc, d);
     L.glf = c->desc.global_lf;
+    L.chained = (chained || d > 0) && c->is_f32;
     cudaError_t e = launch(c->is_f32, L, M, c->desc.scheme, c->desc.characteristic,
                            c->desc.free_stream_preserving, s);
     if (e != cudaSuccess) return cuda_fail(c, e, "sweep launch");
@@ -718,7 +772,7 @@ static int run_stage(fp_ctx *c, int stage, int rk, cudaStream_t s) {
 
 static int run_passes(fp_ctx *c, int rk, cudaStream_t s) {
   for (int stage = 0; stage < (rk ? 3 : 1); ++stage) {
-    int st = run_stage(c, stage, rk, s);
+    int st = run_stage(c, stage, rk, stage > 0, s);
     if (st) return st;
   }
   return FP_OK;
@@ -779,7 +833,7 @@ int fp_rk3_stage(fp_ctx *c, void *q, double dt, int stage, void *stream) {
     cudaError_t e = cudaMemcpyAsync(c->dt_dev, &c->dt_host, sizeof(double), cudaMemcpyHostToDevice, s);
     if (e != cudaSuccess) return cuda_fail(c, e, "upload dt");
   }
-  return run_stage(c, stage, 1, s);
+  return run_stage(c, stage, 1, 0, s);
 }
 
 int fp_set_halo(fp_ctx *c, int dir, int side, void *halo_dev) {
@@ -882,7 +936,7 @@ int fp_bounds_checking(void) {
 #endif
 }
 
-int fp_launches_per_rhs(const fp_ctx *c) { return c ? c->desc.dims + (c->desc.global_lf ? 2 : 0) : 0; }
+int fp_launches_per_rhs(const fp_ctx *c) { return c ? (c->split ? 2 : c->desc.dims) + (c->desc.global_lf ? 2 : 0) : 0; }
 int fp_launches_per_step(const fp_ctx *c) { return c ? 3 * fp_launches_per_rhs(c) : 0; }
 
 int fp_get_cta_sizes(const fp_ctx *c, int *primary, int *alternative) {
@@ -952,7 +1006,7 @@ static int batch_items_into(fp_batch *b, int d, const std::vector<int> *only_blo
     if (!only_blocks || std::find(only_blocks->begin(), only_blocks->end(), (int)k) != only_blocks->end())
       streams.push_back(stream_of(b->hblk[k], (int)k, d));
   std::vector<fpk::SweepItem> items;
-  *ncta = make_items(streams, d, b->per_sm[shape_of(b, b->hblk[0].dir[d])] * b->nsm, items);
+  *ncta = make_items(streams, b->per_sm[shape_of(b, b->hblk[0].dir[d])] * b->nsm, items);
   cudaError_t e = put_items(items, dst);
   if (e != cudaSuccess)
     return bfail(b, e == cudaErrorMemoryAllocation ? FP_ERR_OOM : FP_ERR_CUDA,
@@ -978,7 +1032,6 @@ static int batch_pass_items(fp_batch *b, int d, int mode, int stage, cudaStream_
   L.blocks = b->dblk;
   L.items = items;
   L.grid = ncta;
-  L.dir = d;
   L.mode = mode;
   L.stage = stage;
   L.dt = b->dt_dev;
@@ -1110,8 +1163,9 @@ int fp_batch_create_linked(fp_ctx *const *blocks, int nblocks, void *const *q_de
     BlockDev B = blocks[k]->hblk;
     B.q[0] = q_devs[k];
     B.dqdt = nullptr;
+    for (int d = 0; d < 3; ++d) B.dir[d].racc = blocks[k]->racc;
     for (int d = 0; d < 3; ++d)
-      for (int sd = 0; sd < 2; ++sd) B.nbr[d][sd] = nbr[(size_t)k * 6 + d * 2 + sd];
+      for (int sd = 0; sd < 2; ++sd) B.dir[d].nbr[sd] = nbr[(size_t)k * 6 + d * 2 + sd];
     b->hblk.push_back(B);
   }
   // the batch runs one CTA shape: the blocks' own tiles where they are of that shape, the
@@ -1288,7 +1342,7 @@ extern "C" int fp_rhs_noalloc(fp_ctx *c, const void *q, void *dqdt, void *stream
   BlockDev b = c->hblk;
   b.q[0] = const_cast<void *>(q);
   b.dqdt = dqdt;
-  b.racc = S.racc;                     // fully written by the first pass: nothing to clear
+  for (int d = 0; d < 3; ++d) b.dir[d].racc = S.racc;   // fully written by the first pass: nothing to clear
   k_noalloc_store_block<<<1, 1, 0, s>>>(b);
   e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_fail(c, e, "fp_rhs_noalloc: descriptor store");
@@ -1302,7 +1356,6 @@ extern "C" int fp_rhs_noalloc(fp_ctx *c, const void *q, void *dqdt, void *stream
     L.blocks = S.blk;
     L.items = c->items[d];
     L.grid = c->ncta[d];
-    L.dir = d;
     L.mode = d == 0 ? fpk::MODE_WRITE : (d == dims - 1 ? fpk::MODE_RHS : fpk::MODE_ADD);
     L.stage = 0;
     L.dt = c->dt_dev;

@@ -61,6 +61,9 @@ enum : int {
   CF_AC = 13     // c |grad(d)|
 };
 
+// What a pass does with its part of the residual: write or add it to the accumulator, or finish
+// dQ/dt or the RK stage with it.  Where all directions run in one launch, each writes an
+// accumulator of its own and launch_finish sums them.
 enum : int { MODE_WRITE = 0, MODE_ADD = 1, MODE_RHS = 2, MODE_RK = 3 };
 
 // Status word bits set by the kernels.
@@ -99,12 +102,15 @@ struct DirDev {
   unsigned fc;         // face-metric component stride
   int bclo, bchi;      // boundary codes at the two line ends
   int S, TT;           // faces per chunk, lines per tile (S * TT == the variant's sweep_threads)
+  const void *kmet;    // this direction's metric vector in the cell metrics (component 3 d)
   const void *fmet;    // T [3][faces]
+  void *racc;          // residual accumulator, state layout (the directions' own or the same one)
   const void *dk;      // T [3][cells]: k_{i+1/2} - k_{i-1/2} along this direction (FP64-formed)
   // FP_BC_HALO sides: the caller's buffers of the G cells beyond each side, laid out like the
   // state with this direction's extent replaced by G (strides: t1, t2, along the line, component)
   const void *halo[2];
   int hT1, hT2, hsd;
+  int nbr[2];          // FP_BC_BLOCK sides: index of the linked block in the launch's block table
   unsigned hc;
 };
 
@@ -118,8 +124,8 @@ struct alignas(16) BlockDev {
   unsigned mc;         // metric component stride
   unsigned moff;       // offset of point (0,0,0) in the metric arrays
   const void *met;     // T [10][...] cell metrics with G ghosts
+  const void *imet;    // its component 9, 1/J
   void *q[3];          // stage states: 0 = Q^n (caller), 1 = Q^(1), 2 = Q^(2)
-  void *racc;          // residual accumulator, state layout
   void *dqdt;          // output of the rhs mode
   double gamma;
   // the sweep's constants in its arithmetic type (12 float or double values): reference (far-field)
@@ -129,30 +135,30 @@ struct alignas(16) BlockDev {
   int global_lf;       // 1: Lax-Friedrichs speeds from lamg instead of the stencil
   void *lamg;          // T [3 directions][3]: max |U - c|grad||, |U|, |U + c|grad|| over the block
   int cut;             // FP_BC_CUT sides: lines t1 < cut or t1 >= nt1 - cut meet across the cut
-  int nbr[3][2];       // FP_BC_BLOCK sides: index of the linked block in the launch's block table
 };
 
 // A work item of the sweep: `len` consecutive positions (cells and the ghost positions between two
 // lines) of one block's stream, the first one position u0 (0 .. nd + 2 G - 1) of tile `tile`;
-// after the end of a tile's line the stream goes on with the tile `stride` further.  Item c is
+// after the end of a tile's line the stream goes on with the tile `stride` further.  `dir` is the
+// swept direction.  Item c is
 // the first of CTA c, `next` the index of the CTA's next item (-1: none).  16-byte aligned:
 // copied into shared memory in 16-byte pieces.
 struct alignas(16) SweepItem {
   int block, tile, stride, u0;
-  int len, next, pad[2];
+  int len, next, dir, pad;
 };
 
 struct SweepLaunch {
   const BlockDev *blocks;
   const SweepItem *items;
-  int dir;
   int mode;
   int stage;           // RK stage 0,1,2 (input q[stage], output q[(stage+1)%3])
   const double *dt;    // device scalar
   int grid;            // CTAs of the launch
-  int bnd = 0;         // some block of the launch has a slip-wall or cut side in `dir`
+  int bnd = 0;         // some block of the launch has a slip-wall or cut side in a swept direction
   int glf = 0;         // the blocks of the launch use global Lax-Friedrichs speeds
-  int alt = 0;         // the blocks' tiles in `dir` are of the alternative CTA shape
+  int alt = 0;         // the blocks' tiles are of the alternative CTA shape
+  int chained = 0;     // the kernel before it in the stream may still run (launch_kernel)
 };
 
 // Launchers of the sweep, one per translation unit (sweep_<NAME>.cu): precision f32 / f64,
@@ -190,6 +196,30 @@ int prepare_sweep_f64_bnd(int M, int scheme);
 int prepare_sweep_f64_bnd_fix(int M, int scheme);
 int prepare_sweep_f64_bnd_comp(int M, int scheme);
 
+// Programmatic dependent launch: with `chained`, the kernel may be scheduled while the one before
+// it in the stream is still running and has to execute chain_wait() before it touches anything
+// that one reads or writes; chain_next() lets the kernel after it do the same.  Without, the
+// launch waits as usual and both are no-ops.
+template <typename... P, typename... A>
+inline cudaError_t launch_kernel(void (*kernel)(P...), int grid, int threads, size_t smem, cudaStream_t s, int chained,
+                                 A... args) {
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cfg.attrs = attr;
+  cfg.numAttrs = chained ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+#ifdef __CUDACC__
+__device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void chain_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+#endif
+
 // Every device and page-locked allocation of the library goes through these two, so the
 // host-side hook fp_debug_fail_allocation can make a chosen one fail as if the device (or
 // the pinned host pool) were out of memory.  Defined in api.cu.
@@ -217,6 +247,11 @@ cudaError_t convert_f64_to_f32(const double *src, float *dst, long long n, cudaS
 constexpr int kLamChunk = 256;
 cudaError_t launch_lambda(const BlockDev *blocks, int nblocks, const int2 *items, int nitems,
                           int is_f32, int charwise, int stage, cudaStream_t s);
+
+// Sum of the directions' accumulators of one block and the end of the pass (stage.cu): dQ/dt (rk = 0)
+// or the RK stage (rk = 1).
+cudaError_t launch_finish(const BlockDev *blk, int is_f32, long long ncells, const int *n, int dims, int rk,
+                          int stage, const double *dt, cudaStream_t s);
 
 // CFL reduction (cfl.cu).
 cudaError_t launch_cfl(const BlockDev *blk, int is_f32, long long ncells, const int *n, int dims,

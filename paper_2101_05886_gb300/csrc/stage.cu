@@ -1,0 +1,64 @@
+// stage.cu - the end of a residual or Runge-Kutta stage whose direction passes ran as one launch
+// (each into its own accumulator): the sum of the directions' residuals, in the order of the passes, scaled into
+// dQ/dt or applied as the stage update.  The same operations as the last pass's own epilogue.
+#include <cuda_runtime.h>
+
+#include "sweep.cuh"
+
+namespace fpk {
+
+namespace {
+
+// Bound by memory latency at these sizes (a few hundred thousand points, all in L2): one point per
+// thread, all its loads in flight at once.
+template <typename T>
+__global__ void __launch_bounds__(256) k_finish(const BlockDev *__restrict__ blk, unsigned ncells, int ni, int nj,
+                                                int dims, int rk, int stage, const double *__restrict__ dtp) {
+  const unsigned idx = blockIdx.x * 256u + threadIdx.x;
+  const unsigned i = idx % ni, r = idx / ni, j = r % nj, k = r / nj, qc = blk->qc;
+  const DirDev *D = &blk->dir[0];      // lines along i: its transverse strides are those of j and k
+  const T *met = static_cast<const T *>(blk->met);
+  const unsigned mo = blk->moff + i + j * D->mT1 + k * D->mT2;
+  const bool in = idx < ncells;
+  const T Jc = in ? Num<T>::rcp(*FPK_IN(comp_at(met, mo, blk->mc, 9), met, 10LL * blk->mc, blk->status)) : T(0);
+  chain_wait();
+  chain_next();
+  if (!in) return;
+  const T *acc[3];
+#pragma unroll
+  for (int d = 0; d < 3; ++d) acc[d] = static_cast<const T *>(blk->dir[d].racc);
+  T R[5], qk[5], qn[5];
+#pragma unroll
+  for (int v = 0; v < 5; ++v) {
+    R[v] = *comp_at(acc[0], idx, qc, v) + *comp_at(acc[1], idx, qc, v);
+    if (dims == 3) R[v] += *comp_at(acc[2], idx, qc, v);
+    if (rk) qk[v] = *comp_at(static_cast<const T *>(blk->q[stage]), idx, qc, v);
+    qn[v] = rk && stage ? *comp_at(static_cast<const T *>(blk->q[0]), idx, qc, v) : T(0);
+  }
+  if (!rk) {
+#pragma unroll
+    for (int v = 0; v < 5; ++v) *comp_at(static_cast<T *>(blk->dqdt), idx, qc, v) = -Jc * R[v];
+    return;
+  }
+  const RkStage<T> update(stage, T(*dtp));
+  T *qs = static_cast<T *>(blk->q[(stage + 1) % 3]);
+  bool bad = false;
+#pragma unroll
+  for (int v = 0; v < 5; ++v) {
+    const T nv = update(qk[v], qn + v, -Jc * R[v]);
+    *comp_at(qs, idx, qc, v) = nv;
+    bad |= !isfinite(nv);
+  }
+  if (bad) atomicOr(blk->status, ST_NONFINITE);
+}
+
+}  // namespace
+
+cudaError_t launch_finish(const BlockDev *blk, int is_f32, long long ncells, const int *n, int dims, int rk,
+                          int stage, const double *dt, cudaStream_t s) {
+  const int grid = (int)((ncells + 255) / 256);
+  return is_f32 ? launch_kernel(k_finish<float>, grid, 256, 0, s, 1, blk, (unsigned)ncells, n[0], n[1], dims, rk, stage, dt)
+                : launch_kernel(k_finish<double>, grid, 256, 0, s, 1, blk, (unsigned)ncells, n[0], n[1], dims, rk, stage, dt);
+}
+
+}  // namespace fpk

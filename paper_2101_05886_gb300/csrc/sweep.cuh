@@ -56,6 +56,7 @@ template <> struct Num<double> {
     const long long a = __double_as_longlong(m), b = __double_as_longlong(fabs(x));
     return __longlong_as_double(a > b ? a : b);
   }
+  static __device__ __forceinline__ double fma_(double a, double b, double c) { return fma(a, b, c); }
   static __device__ __forceinline__ double sqrt_(double x) { return sqrt(x); }
   static __device__ __forceinline__ double rsqrt_(double x) { return rsqrt(x); }
   static __device__ __forceinline__ double ld(const void *p, long long i) {
@@ -70,6 +71,7 @@ template <> struct Num<float> {
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
     return r;
   }
+  static __device__ __forceinline__ float fma_(float a, float b, float c) { return fmaf(a, b, c); }
   static __device__ __forceinline__ float amax(float m, float x) { return fmaxf(m, fabsf(x)); }
   static __device__ __forceinline__ float sqrt_(float x) {
     float r;
@@ -347,6 +349,19 @@ __device__ __forceinline__ void dflux_frame(T g1, typename PairOf<T>::type rinvB
   out[4] = pfma(padd(dp, pc<P>(EpP)), dU, pmul(d[4], UB));
 }
 
+// One value of an SSP-RK3 stage (Gottlieb & Shu) in increment form:
+// Q^(s+1) = Q^(s) + a_s (Q^n - Q^(s)) + b_s dt L(Q^(s))
+template <typename T> struct RkStage {
+  T a, bdt;
+  bool first;
+  __device__ __forceinline__ RkStage(int stage, T dt)
+      : a(stage == 1 ? T(0.75) : T(1.0 / 3.0)),
+        bdt((stage == 0 ? T(1) : (stage == 1 ? T(0.25) : T(2.0 / 3.0))) * dt), first(stage == 0) {}
+  __device__ __forceinline__ T operator()(T qk, const T *qn, T L) const {
+    return Num<T>::fma_(bdt, L, first ? qk : Num<T>::fma_(a, *qn - qk, qk));
+  }
+};
+
 // FIX = 1 or 2: the characteristic decomposition and the FP form on, local Lax-Friedrichs speeds,
 // all fixed at compile time (the configuration of the paper's workloads but the shock test), so
 // their switches fold away.  FIX = 2 is the same sweep with the alternative CTA shape of
@@ -356,7 +371,7 @@ __device__ __forceinline__ void dflux_frame(T g1, typename PairOf<T>::type rinvB
 // 70 x 80 x 22 points, component-wise, 208 us a step against 149).
 template <typename T, int M, int SCHEME, bool BND, int FIX>
 __global__ void __launch_bounds__(sweep_threads(sizeof(T) == 4, SCHEME, FIX), sweep_min_ctas(sizeof(T) == 4, SCHEME, FIX))
-fp_sweep(const BlockDev *__restrict__ blocks, const SweepItem *__restrict__ items, int dir, int mode,
+fp_sweep(const BlockDev *__restrict__ blocks, const SweepItem *__restrict__ items, int mode,
          int stage, const double *__restrict__ dtp, int fpform_arg) {
   // this variant's CTA shape (fp_internal.h): threads, ring stride of a staged field
   constexpr int kThreads = sweep_threads(sizeof(T) == 4, SCHEME, FIX);
@@ -398,24 +413,19 @@ fp_sweep(const BlockDev *__restrict__ blocks, const SweepItem *__restrict__ item
   for (int it = blockIdx.x; it >= 0; cur ^= 1) {
     const SweepItem &item = s_item[cur];
     const BlockDev *B = reinterpret_cast<const BlockDev *>(s_desc[cur]);
-    const DirDev *D = &B->dir[dir];
+    const DirDev *D = &B->dir[item.dir];
     const int nit = item.next;
     // the next item: lands by this item's prologue barrier
     if (tid < 2 && nit >= 0) cp_async16(reinterpret_cast<unsigned char *>(&s_item[cur ^ 1]) + 16 * tid,
                                         reinterpret_cast<const unsigned char *>(items + nit) + 16 * tid);
-    if (tid == 0) {                      // read after the prologue's barrier
-      s_dt = mode == MODE_RK ? T(*dtp) : T(0);
-      if (!kFold && B->global_lf)
-        for (int c = 0; c < 3; ++c)
-          s_lam[c] = *FPK_IN(static_cast<const T *>(B->lamg) + (3 * dir + c), static_cast<const T *>(B->lamg), 9, B->status);
-    }
+    if (tid == 0) s_dt = mode == MODE_RK ? T(*dtp) : T(0);   // read after the prologue's barrier
     const int S = D->S, TT = D->TT, W = 2 * S;
     // thread roles: along-line index tf and line index tl.  The xi pass puts
     // consecutive threads along the line (coalesced, i contiguous), the other passes
     // across lines.  Shared layout: line-fast slots are TT apart; slot-fast lines 2S apart, with
     // the slots of every other run of 32/S lines turned by S, so that the lines a warp reads at
     // once lie in different banks for every S.
-    const bool slotFast = (dir == 0);
+    const bool slotFast = item.dir == 0;
     const int tf = slotFast ? (tid % S) : (tid / TT);
     const int tl = slotFast ? (tid / S) : (tid % TT);
     const int SS = slotFast ? 1 : TT;
@@ -460,7 +470,6 @@ fp_sweep(const BlockDev *__restrict__ blocks, const SweepItem *__restrict__ item
           if (t1 >= nt1) { t1 -= nt1; ++t2; }
         }
     };
-    const T *__restrict__ met = static_cast<const T *>(B->met);
     const T *__restrict__ fmet = static_cast<const T *>(D->fmet);
     const T *__restrict__ qin = static_cast<const T *>(B->q[stage]);
     const int glf = kFold ? 0 : B->global_lf;
@@ -506,8 +515,8 @@ fp_sweep(const BlockDev *__restrict__ blocks, const SweepItem *__restrict__ item
           cs = D->hc;
           FPK_CHK_ONLY(sb = static_cast<const T *>(D->halo[hi]); sn = 5LL * D->hc;)
         } else if (BND && bc == 5) {
-          const BlockDev *NB = blocks + B->nbr[dir][hi];
-          const DirDev *ND = &NB->dir[dir];
+          const BlockDev *NB = blocks + D->nbr[hi];
+          const DirDev *ND = &NB->dir[item.dir];
           src = static_cast<const T *>(NB->q[stage]) +
                 ((unsigned)t1 * ND->qT1 + (unsigned)t2 * ND->qT2 + (unsigned)(hi ? x - nd : ND->nd + x) * ND->qsd);
           cs = NB->qc;
@@ -539,8 +548,8 @@ fp_sweep(const BlockDev *__restrict__ blocks, const SweepItem *__restrict__ item
       if (x >= -G && x < nd + G) {
         const unsigned mo = moff(x, t1, t2);
 #pragma unroll
-        for (int a = 0; a < 3; ++a) k[a] = *FPK_IN(comp_at(met, mo, mc, 3 * dir + a), met, 10LL * mc, B->status);
-        invJ = *FPK_IN(comp_at(met, mo, mc, 9), met, 10LL * mc, B->status);
+        for (int a = 0; a < 3; ++a) k[a] = *FPK_IN(comp_at(static_cast<const T *>(D->kmet), mo, mc, a), static_cast<const T *>(B->met), 10LL * mc, B->status);
+        invJ = *FPK_IN(static_cast<const T *>(B->imet) + mo, static_cast<const T *>(B->met), 10LL * mc, B->status);
         const T *qp;
         unsigned cs;
         bool far, wall;
@@ -593,11 +602,12 @@ fp_sweep(const BlockDev *__restrict__ blocks, const SweepItem *__restrict__ item
     // asynchronous copy of one cell's loads (-G <= x < nd + G) into this thread's staging slots
     auto prefetch_cell = [&](int x, int t1, int t2) {
       T *dst = nsb + tid;
-      const T *const mp = met + moff(x, t1, t2), *const md = comp_at(mp, 0, mc, 3 * dir);
+      const unsigned mo = moff(x, t1, t2);
+      const T *const md = static_cast<const T *>(D->kmet), *const mi = static_cast<const T *>(B->imet);
 #pragma unroll
       for (int a = 0; a < 3; ++a)
-        cp_async_el(dst + (5 + a) * kThreads, FPK_IN(comp_at(md, 0, mc, a), met, 10LL * mc, B->status));
-      cp_async_el(dst + 8 * kThreads, FPK_IN(comp_at(mp, 0, mc, 9), met, 10LL * mc, B->status));
+        cp_async_el(dst + (5 + a) * kThreads, FPK_IN(comp_at(md, mo, mc, a), static_cast<const T *>(B->met), 10LL * mc, B->status));
+      cp_async_el(dst + 8 * kThreads, FPK_IN(mi + mo, static_cast<const T *>(B->met), 10LL * mc, B->status));
       const T *qp;
       unsigned cs;
       bool far, wall;
@@ -617,7 +627,7 @@ fp_sweep(const BlockDev *__restrict__ blocks, const SweepItem *__restrict__ item
     auto prefetch_epilogue = [&](unsigned qo) {
       T *dst = epb + tid;
       if (mode != MODE_WRITE) {
-        const T *const ra = static_cast<const T *>(B->racc);
+        const T *const ra = static_cast<const T *>(D->racc);
 #pragma unroll
         for (int v = 0; v < 5; ++v) cp_async_el(dst + v * kThreads, FPK_IN(comp_at(ra, qo, qc, v), ra, 5LL * qc, B->status));
       }
@@ -651,6 +661,11 @@ fp_sweep(const BlockDev *__restrict__ blocks, const SweepItem *__restrict__ item
       locate(item.u0 - 5 + tf, ua, a1, a2);
       locate(item.u0 - 5 + tf + S, ub2, b1, b2);
       const bool one = a2 < nt2, two = tf < 8 && b2 < nt2;
+      chain_wait();                      // from here on: what earlier kernels wrote
+      chain_next();
+      if (!kFold && tid == 0 && B->global_lf)
+        for (int c = 0; c < 3; ++c)
+          s_lam[c] = *FPK_IN(static_cast<const T *>(B->lamg) + (3 * item.dir + c), static_cast<const T *>(B->lamg), 9, B->status);
       T Qa[5], ka[3], ija, Qb[5], kb[3], ijb;
       if (one) fetch(ua - G, a1, a2, Qa, ka, ija);
       if (two) fetch(ub2 - G, b1, b2, Qb, kb, ijb);
@@ -1116,7 +1131,7 @@ fp_sweep(const BlockDev *__restrict__ blocks, const SweepItem *__restrict__ item
 #pragma unroll
           for (int v = 0; v < 5; ++v) R[v] += t1v[v] + t2v[v];
         }
-        T *const racc = static_cast<T *>(B->racc);
+        T *const racc = static_cast<T *>(D->racc);
         const T *ra = epb + tid;                      // prefetched accumulator
         if (mode == MODE_WRITE) {
 #pragma unroll
@@ -1132,19 +1147,12 @@ fp_sweep(const BlockDev *__restrict__ blocks, const SweepItem *__restrict__ item
             for (int v = 0; v < 5; ++v)
               *FPK_IN(comp_at(out, qo, qc, v), out, 5LL * qc, B->status) = -Jc * (ra[v * kThreads] + R[v]);
           } else {
-            // SSP-RK3 stage (Gottlieb & Shu) in increment form:
-            // Q^(s+1) = Q^(s) + a_s (Q^n - Q^(s)) + b_s dt L(Q^(s))
-            const T dt = s_dt;
-            const T as = stage == 0 ? T(0) : (stage == 1 ? T(0.75) : T(1.0 / 3.0));
-            const T bs = stage == 0 ? T(1) : (stage == 1 ? T(0.25) : T(2.0 / 3.0));
             T *const qs = static_cast<T *>(B->q[(stage + 1) % 3]);
+            const RkStage<T> rk(stage, s_dt);
             bool bad = false;
 #pragma unroll
             for (int v = 0; v < 5; ++v) {
-              const T qk = Qi[v];
-              const T Lv = -Jc * (ra[v * kThreads] + R[v]);
-              T nv = qk + bs * dt * Lv;
-              if (stage != 0) nv = qk + as * (ra[(5 + v) * kThreads] - qk) + bs * dt * Lv;
+              const T nv = rk(Qi[v], ra + (5 + v) * kThreads, -Jc * (ra[v * kThreads] + R[v]));
               *FPK_IN(comp_at(qs, qo, qc, v), qs, 5LL * qc, B->status) = nv;
               bad |= !isfinite(nv);
             }
@@ -1191,8 +1199,8 @@ cudaError_t launch_one(const SweepLaunch &L, int fp, cudaStream_t s) {
   constexpr size_t smem = sweep_smem<T, SCHEME, FIX>();
   constexpr int nt = sweep_threads(sizeof(T) == 4, SCHEME, FIX);
   if (L.grid <= 0) return cudaSuccess;
-  fp_sweep<T, M, SCHEME, BND, FIX><<<L.grid, nt, smem, s>>>(L.blocks, L.items, L.dir, L.mode, L.stage, L.dt, fp);
-  return cudaGetLastError();
+  return launch_kernel(fp_sweep<T, M, SCHEME, BND, FIX>, L.grid, nt, smem, s, L.chained, L.blocks, L.items, L.mode,
+                       L.stage, L.dt, fp);
 }
 
 template <typename T, bool BND, int FIX>

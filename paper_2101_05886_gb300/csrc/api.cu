@@ -33,7 +33,7 @@ struct fp_ctx {
   void *q1 = nullptr, *q2 = nullptr, *racc = nullptr;
   int *status = nullptr;
   double *dt_dev = nullptr;
-  unsigned long long *cfl_bits = nullptr;
+  fpk::CflScratch *cfl_bits = nullptr;
   void *lamg = nullptr;               // T [3][3] global Lax-Friedrichs speeds
   int2 *lam_items = nullptr;          // (block 0, first point) chunks for the speed reduction
   int nlam_items = 0;
@@ -690,7 +690,7 @@ int fp_init_grid(const fp_grid_desc *desc, const double *xyz, int ghost_nodes, v
   FP_TRY(fpk::dev_alloc(&c->status, sizeof(int)), "cudaMalloc(status)");
   FP_TRY(cudaMemset(c->status, 0, sizeof(int)), "clear status");
   FP_TRY(fpk::dev_alloc(&c->dt_dev, sizeof(double)), "cudaMalloc(dt)");
-  FP_TRY(fpk::dev_alloc(&c->cfl_bits, sizeof(unsigned long long)), "cudaMalloc(cfl)");
+  FP_TRY(fpk::dev_alloc(&c->cfl_bits, sizeof(fpk::CflScratch) + fpk::cfl_ctas(c->ncells) * sizeof(float)), "cudaMalloc(cfl)");
   FP_TRY(fpk::dev_alloc(&c->dblk, sizeof(BlockDev)), "cudaMalloc(block)");
   FP_TRY(fpk::dev_alloc(&c->lamg, 9 * c->esize), "cudaMalloc(global speeds)");
   FP_TRY(cudaMemset(c->lamg, 0, 9 * c->esize), "clear global speeds");
@@ -867,12 +867,12 @@ int fp_cfl_dt(fp_ctx *c, const void *q, double cfl, double *dt_out, void *stream
   c->hblk.q[0] = const_cast<void *>(q);
   int st = sync_block(c, s);
   if (st) return st;
-  cudaError_t e = cudaMemsetAsync(c->cfl_bits, 0, sizeof(unsigned long long), s);
+  cudaError_t e = cudaMemsetAsync(c->cfl_bits, 0, sizeof(fpk::CflScratch), s);
   if (e != cudaSuccess) return cuda_fail(c, e, "cfl clear");
   e = fpk::launch_cfl(c->dblk, c->is_f32, c->ncells, c->desc.n, c->desc.dims, c->cfl_bits, s);
   if (e != cudaSuccess) return cuda_fail(c, e, "cfl launch");
   unsigned long long bits = 0;
-  e = cudaMemcpyAsync(&bits, c->cfl_bits, sizeof(bits), cudaMemcpyDeviceToHost, s);
+  e = cudaMemcpyAsync(&bits, &c->cfl_bits->max_bits, sizeof(bits), cudaMemcpyDeviceToHost, s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   if (e != cudaSuccess) return cuda_fail(c, e, "cfl readback");
   double mx;

@@ -34,37 +34,34 @@ constexpr int kCflThreads = 256, kCflPoints = 4;   // points per thread
 
 // The maximum of cfl_point over a block.  The FP64 pipe does two operations per clock and SM, and
 // a point's four quotients and four roots cost about 150 (1.07M points: 258 us, 25 times their
-// memory time), so every point is first bounded in FP32: `hi` and `lo` enclose its value.
-// Only points whose upper bound reaches the CTA's largest lower bound and the maximum found so
-// far are evaluated in FP64, so the result is the same to the last bit.  The bounds' relative
-// width 4e-6 is about 20 times the rounding of the FP32 evaluation (inputs rounded to float, at
-// most 12 operations deep); cancellation in the pressure and in u . grad d is covered by adding
-// that width of the summed magnitudes.  Values outside [1e-30, 1e30], whose products could
-// leave the FP32 range, and anything not finite are evaluated in FP64.
-// A step with its bound on 181 x 97 x 61 FP32 points: 1010 -> 792 us.
-template <typename T>
-__global__ void __launch_bounds__(kCflThreads) k_cfl(const BlockDev *blk, long long ncells, int ni, int nj, int dims,
-                                                     unsigned long long *out) {
-  __shared__ float red[kCflThreads / 32];
-  const T *q = static_cast<const T *>(blk->q[0]);
-  const T *met = static_cast<const T *>(blk->met);
-  const long long qc = blk->qc, mc = blk->mc;
-  const float g1 = (float)(blk->gamma - 1.0), gam = (float)blk->gamma;
-  constexpr float kW = 4e-6f, kLow = 1e-30f, kHigh = 1e30f;
-  const long long base = (long long)blockIdx.x * (kCflThreads * kCflPoints) + threadIdx.x;
-  float hi[kCflPoints], lo = 0.f;
-  auto place = [&](long long idx) {
+// memory time), so every point is first enclosed in FP32 bounds.  k_cfl_bound keeps the largest
+// lower bound of the block and each CTA's largest upper bound; k_cfl_max evaluates in FP64 the points
+// whose upper bound reaches the former, so the result is the same to the last bit.  (One kernel
+// whose CTAs knew only their own lower bound evaluated a point in every CTA: 39 us.)  The bounds'
+// relative width 4e-6 is about 20 times the rounding of the FP32 evaluation (inputs rounded to
+// float, at most 12 operations deep); cancellation in the pressure and in u . grad d is covered by
+// adding that width of the summed magnitudes.  Values outside [1e-30, 1e30], whose products could
+// leave the FP32 range, and anything not finite have the upper bound +inf.
+// A step with its bound on 181 x 97 x 61 FP32 points: 1010 -> 792 us with the first form.
+template <typename T> struct CflScreen {
+  const BlockDev *blk;
+  const T *q, *met;
+  long long qc, mc;
+  int ni, nj, dims;
+  float g1, gam;
+  __device__ CflScreen(const BlockDev *b, int ni_, int nj_, int dims_)
+      : blk(b), q(static_cast<const T *>(b->q[0])), met(static_cast<const T *>(b->met)), qc(b->qc), mc(b->mc),
+        ni(ni_), nj(nj_), dims(dims_), g1((float)(b->gamma - 1.0)), gam((float)b->gamma) {}
+  __device__ long long place(long long idx) const {
     const int i = (int)(idx % ni);
     const long long r = idx / ni;
     const int j = (int)(r % nj), k = (int)(r / nj);
     // lines of the xi direction run along i; their transverse strides are those of j and k
     return blk->moff + i + (long long)j * blk->dir[0].mT1 + (dims == 3 ? (long long)k * blk->dir[0].mT2 : 0);
-  };
-#pragma unroll
-  for (int m = 0; m < kCflPoints; ++m) {
-    const long long idx = base + m * kCflThreads;
-    hi[m] = -1.f;
-    if (idx >= ncells) continue;
+  }
+  // upper bound of the point, and its lower bound (0 if it has none)
+  __device__ float bound(long long idx, float &lo) const {
+    constexpr float kW = 4e-6f, kLow = 1e-30f, kHigh = 1e30f;
     const long long mo = place(idx);
     float Q[5];
 #pragma unroll
@@ -91,25 +88,62 @@ __global__ void __launch_bounds__(kCflThreads) k_cfl(const BlockDev *blk, long l
     sh *= Jc * (1.f + kW);
     sl *= Jc * (1.f - kW);
     ok = ok && sh < kHigh;                          // false for NaN as well
-    hi[m] = ok ? sh : __int_as_float(0x7f800000);   // not bounded: +inf
-    lo = ok && e > de ? fmaxf(lo, sl) : lo;         // a negative pressure has no value (NaN, ignored)
+    lo = ok && e > de ? sl : 0.f;                   // a negative pressure has no value (NaN, ignored)
+    return ok ? sh : __int_as_float(0x7f800000);
   }
-  for (int h = 16; h; h >>= 1) lo = fmaxf(lo, __shfl_xor_sync(0xffffffffu, lo, h));
-  if (threadIdx.x % 32 == 0) red[threadIdx.x / 32] = lo;
-  __syncthreads();
-  for (int w = 0; w < kCflThreads / 32; ++w) lo = fmaxf(lo, red[w]);
-  // the maximum so far (a stale value only costs an evaluation), rounded down
-  const float far = __double2float_rd(__longlong_as_double((long long)*(volatile unsigned long long *)out));
-  lo = fmaxf(lo, far);
-  double best = 0.0;
+};
+
+template <typename T>
+__global__ void __launch_bounds__(kCflThreads) k_cfl_bound(const BlockDev *blk, long long ncells, int ni, int nj, int dims,
+                                                           CflScratch *out, float *cta_hi) {
+  __shared__ float red[2][kCflThreads / 32];
+  const CflScreen<T> screen(blk, ni, nj, dims);
+  const long long base = (long long)blockIdx.x * (kCflThreads * kCflPoints) + threadIdx.x;
+  float hi = -1.f, lo = 0.f;
 #pragma unroll
-  for (int m = 0; m < kCflPoints; ++m)
-    if (hi[m] >= lo) {
-      const long long idx = base + m * kCflThreads;
-      const double s = cfl_point(blk, q, met, idx, place(idx), dims);
-      best = s > best ? s : best;
+  for (int m = 0; m < kCflPoints; ++m) {
+    const long long idx = base + m * kCflThreads;
+    if (idx >= ncells) continue;
+    float l;
+    hi = fmaxf(hi, screen.bound(idx, l));
+    lo = fmaxf(lo, l);
+  }
+  for (int h = 16; h; h >>= 1) {
+    hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, h));
+    lo = fmaxf(lo, __shfl_xor_sync(0xffffffffu, lo, h));
+  }
+  if (threadIdx.x % 32 == 0) {
+    red[0][threadIdx.x / 32] = hi;
+    red[1][threadIdx.x / 32] = lo;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int w = 1; w < kCflThreads / 32; ++w) {
+      hi = fmaxf(hi, red[0][w]);
+      lo = fmaxf(lo, red[1][w]);
     }
-  if (best > 0.0) atomicMax(out, (unsigned long long)__double_as_longlong(best));
+    cta_hi[blockIdx.x] = hi;
+    atomicMax(&out->lower_bits, __float_as_uint(lo));
+  }
+  chain_next();
+}
+
+template <typename T>
+__global__ void __launch_bounds__(kCflThreads) k_cfl_max(const BlockDev *blk, long long ncells, int ni, int nj, int dims,
+                                                         CflScratch *out, const float *cta_hi) {
+  chain_wait();
+  const float lo = __uint_as_float(*(volatile unsigned int *)&out->lower_bits);
+  if (cta_hi[blockIdx.x] < lo) return;
+  const CflScreen<T> screen(blk, ni, nj, dims);
+  double best = 0.0;
+  for (int m = 0; m < kCflPoints; ++m) {
+    const long long idx = (long long)blockIdx.x * (kCflThreads * kCflPoints) + m * kCflThreads + threadIdx.x;
+    float l;
+    if (idx >= ncells || screen.bound(idx, l) < lo) continue;
+    const double s = cfl_point(blk, screen.q, screen.met, idx, screen.place(idx), dims);
+    best = s > best ? s : best;
+  }
+  if (best > 0.0) atomicMax(&out->max_bits, (unsigned long long)__double_as_longlong(best));
 }
 
 template <typename T>
@@ -251,14 +285,17 @@ cudaError_t launch_lambda(const BlockDev *blocks, int nblocks, const int2 *items
   return cudaGetLastError();
 }
 
+int cfl_ctas(long long ncells) { return (int)((ncells + kCflThreads * kCflPoints - 1) / (kCflThreads * kCflPoints)); }
+
 cudaError_t launch_cfl(const BlockDev *blk, int is_f32, long long ncells, const int *n, int dims,
-                       unsigned long long *out_bits, cudaStream_t s) {
-  const long long g = (ncells + kCflThreads * kCflPoints - 1) / (kCflThreads * kCflPoints);   // < 2^21
-  if (is_f32)
-    k_cfl<float><<<(int)g, kCflThreads, 0, s>>>(blk, ncells, n[0], n[1], dims, out_bits);
-  else
-    k_cfl<double><<<(int)g, kCflThreads, 0, s>>>(blk, ncells, n[0], n[1], dims, out_bits);
-  return cudaGetLastError();
+                       CflScratch *scratch, cudaStream_t s) {
+  const int g = cfl_ctas(ncells);
+  float *hi = reinterpret_cast<float *>(scratch + 1);
+  cudaError_t e = launch_kernel(is_f32 ? k_cfl_bound<float> : k_cfl_bound<double>, g, kCflThreads, 0, s, 0, blk, ncells, n[0],
+                                n[1], dims, scratch, hi);
+  if (e != cudaSuccess) return e;
+  return launch_kernel(is_f32 ? k_cfl_max<float> : k_cfl_max<double>, g, kCflThreads, 0, s, 1, blk, ncells, n[0], n[1],
+                       dims, scratch, (const float *)hi);
 }
 
 }  // namespace fpk

@@ -253,9 +253,15 @@ cudaError_t launch_lambda(const BlockDev *blocks, int nblocks, const int2 *items
 cudaError_t launch_finish(const BlockDev *blk, int is_f32, long long ncells, const int *n, int dims, int rk,
                           int stage, const double *dt, cudaStream_t s);
 
-// CFL reduction (cfl.cu).
+// CFL reduction (cfl.cu): `scratch` holds CflScratch and a float per CTA (cfl_ctas of them).
+struct CflScratch {
+  unsigned long long max_bits;   // the result: bits of the FP64 maximum
+  unsigned int lower_bits;       // bits of the largest FP32 lower bound
+  unsigned int pad;
+};
+int cfl_ctas(long long ncells);
 cudaError_t launch_cfl(const BlockDev *blk, int is_f32, long long ncells, const int *n, int dims,
-                       unsigned long long *out_bits, cudaStream_t s);
+                       CflScratch *scratch, cudaStream_t s);
 
 // Halo packing (cfl.cu): the G cells of stage state `stage` next to side `side` of direction
 // `dir` into `out`, in the halo layout of DirDev (the receiving block's view of them); `status`

@@ -662,7 +662,7 @@ fp_sweep(const BlockDev *__restrict__ blocks, const SweepItem *__restrict__ item
       locate(item.u0 - 5 + tf + S, ub2, b1, b2);
       const bool one = a2 < nt2, two = tf < 8 && b2 < nt2;
       chain_wait();                      // from here on: what earlier kernels wrote
-      chain_next();
+      if (sizeof(T) == 4) chain_next();
       if (!kFold && tid == 0 && B->global_lf)
         for (int c = 0; c < 3; ++c)
           s_lam[c] = *FPK_IN(static_cast<const T *>(B->lamg) + (3 * item.dir + c), static_cast<const T *>(B->lamg), 9, B->status);

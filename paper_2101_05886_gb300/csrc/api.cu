@@ -416,12 +416,12 @@ void spread_stream(const Stream &s, long long first, long long most, std::vector
 //    CTAs that run at the same time take adjacent tiles: whole rounds go in turn, CTA c the
 //    tiles c, c + g, ... (equal pieces of the stream instead read 3 times the bytes and cost 6 %
 //    on a 256^3 block), and what is left after the rounds is spread in equal pieces.
-//  - One block by itself: two rounds per CTA, so there are more CTAs than slots and those that
+//  - `alone`, no other launch runs at the same time (one block, or a batch of one chain): two rounds per CTA, so there are more CTAs than slots and those that
 //    run on faster SMs take more of them (256^3 WENO5 step: 8.93 ms, 9.75 ms with all rounds in one
 //    item, 9.97 ms with a CTA per tile in a fixed order and lines padded to chunks).  The blocks of a
 //    batch keep one item for all rounds: its graph's other branches fill the SMs that end
 //    early (64-block WENO5 step: 18.04 ms, 18.25 ms with two rounds per item).
-int make_items(const std::vector<Stream> &streams, int slots, std::vector<fpk::SweepItem> &items) {
+int make_items(const std::vector<Stream> &streams, int slots, bool alone, std::vector<fpk::SweepItem> &items) {
   std::vector<std::vector<fpk::SweepItem>> cta(slots);
   long long total = 0, done = 0;
   for (const Stream &s : streams) total += s.chunks();
@@ -434,7 +434,6 @@ int make_items(const std::vector<Stream> &streams, int slots, std::vector<fpk::S
     const long long r = s.dir == 0 ? 0 : s.tiles / g;
     std::vector<fpk::SweepItem> piece;
     if (r * g < s.tiles) spread_stream(s, r * g, g, piece);
-    const bool alone = streams.size() == 1;
     const long long per = alone ? 2 : r;          // rounds per item
     for (long long r0 = 0; r0 < r; r0 += per) {
       const long long n = std::min(per, r - r0);
@@ -484,7 +483,7 @@ int balanced_items(const fp_ctx *c, const std::vector<Stream> &streams, int most
   if (!c->is_f32) {
     long long least = -1;
     for (int m = most_per_sm; m >= 1; --m) {
-      const int n = make_items(streams, m * c->nsm, items);
+      const int n = make_items(streams, m * c->nsm, streams.size() == 1, items);
       long long most = 0;                         // chunks of one CTA
       for (int k = 0; k < n; ++k) {
         long long ch = 0;
@@ -498,7 +497,7 @@ int balanced_items(const fp_ctx *c, const std::vector<Stream> &streams, int most
       if (least < 0 || 20 * cost < 19 * least) { least = cost; per_sm = m; }
     }
   }
-  return make_items(streams, per_sm * c->nsm, items);
+  return make_items(streams, per_sm * c->nsm, streams.size() == 1, items);
 }
 
 int upload_items(fp_ctx *c) {
@@ -999,14 +998,14 @@ int fp_batch_launches_per_step(const fp_batch *b) {
 }
 
 // the items of direction d for all blocks or some of them (blocks in index order)
-static int batch_items_into(fp_batch *b, int d, const std::vector<int> *only_blocks, fpk::SweepItem **dst,
-                            int *ncta) {
+static int batch_items_into(fp_batch *b, int d, const std::vector<int> *only_blocks, bool alone,
+                            fpk::SweepItem **dst, int *ncta) {
   std::vector<Stream> streams;
   for (size_t k = 0; k < b->hblk.size(); ++k)
     if (!only_blocks || std::find(only_blocks->begin(), only_blocks->end(), (int)k) != only_blocks->end())
       streams.push_back(stream_of(b->hblk[k], (int)k, d));
   std::vector<fpk::SweepItem> items;
-  *ncta = make_items(streams, b->per_sm[shape_of(b, b->hblk[0].dir[d])] * b->nsm, items);
+  *ncta = make_items(streams, b->per_sm[shape_of(b, b->hblk[0].dir[d])] * b->nsm, alone, items);
   cudaError_t e = put_items(items, dst);
   if (e != cudaSuccess)
     return bfail(b, e == cudaErrorMemoryAllocation ? FP_ERR_OOM : FP_ERR_CUDA,
@@ -1015,7 +1014,7 @@ static int batch_items_into(fp_batch *b, int d, const std::vector<int> *only_blo
 }
 
 static int batch_items(fp_batch *b, int d, const std::vector<int> *only_blocks) {
-  return batch_items_into(b, d, only_blocks, &b->items[d], &b->ncta[d]);
+  return batch_items_into(b, d, only_blocks, true, &b->items[d], &b->ncta[d]);
 }
 
 static int batch_upload(fp_batch *b, cudaStream_t s) {
@@ -1027,7 +1026,7 @@ static int batch_upload(fp_batch *b, cudaStream_t s) {
 }
 
 static int batch_pass_items(fp_batch *b, int d, int mode, int stage, cudaStream_t s,
-                            const fpk::SweepItem *items, int ncta) {
+                            const fpk::SweepItem *items, int ncta, int chained = 0) {
   fpk::SweepLaunch L;
   L.blocks = b->dblk;
   L.items = items;
@@ -1038,13 +1037,15 @@ static int batch_pass_items(fp_batch *b, int d, int mode, int stage, cudaStream_
   L.alt = shape_of(b, b->hblk[0].dir[d]);   // every block of a batch pass has the same shape
   L.bnd = b->bnd[d];
   L.glf = b->global_lf;
+  L.chained = chained && b->is_f32;
   cudaError_t e = launch(b->is_f32, L, b->M, b->scheme, b->charwise, b->fp, s);
   if (e != cudaSuccess) return bfail(b, FP_ERR_CUDA, std::string("batch sweep: ") + cudaGetErrorString(e));
   return FP_OK;
 }
 
-static int batch_pass(fp_batch *b, int d, int mode, int stage, cudaStream_t s) {
-  return batch_pass_items(b, d, mode, stage, s, b->items[d], b->ncta[d]);
+// chained: the launch before it in the stream is the previous pass of the same chain
+static int batch_pass(fp_batch *b, int d, int mode, int stage, cudaStream_t s, int chained = 0) {
+  return batch_pass_items(b, d, mode, stage, s, b->items[d], b->ncta[d], chained);
 }
 
 // Autotuner: for the batch's CTA shape, each direction and each line-length class, time every
@@ -1209,7 +1210,7 @@ int fp_batch_create_linked(fp_ctx *const *blocks, int nblocks, void *const *q_de
     std::vector<std::vector<int>> grp(b->nbranch);
     for (int k = 0; k < nblocks; ++k) grp[group_of[k]].push_back(k);
     for (int g = 0; g < b->nbranch && !st; ++g)
-      for (int d = 0; d < b->dims && !st; ++d) st = batch_items_into(b, d, &grp[g], &b->bitems[g][d], &b->bncta[g][d]);
+      for (int d = 0; d < b->dims && !st; ++d) st = batch_items_into(b, d, &grp[g], false, &b->bitems[g][d], &b->bncta[g][d]);
     if (st) { fp_batch_free(b); return st; }
   }
   // capture the three RK stages x directions into one graph (one chain per branch)
@@ -1249,7 +1250,7 @@ int fp_batch_create_linked(fp_ctx *const *blocks, int nblocks, void *const *q_de
       }
       for (int d = 0; d < b->dims && !st; ++d) {
         int mode = d == 0 ? fpk::MODE_WRITE : (d == b->dims - 1 ? fpk::MODE_RK : fpk::MODE_ADD);
-        st = batch_pass(b, d, mode, stage, cs);
+        st = batch_pass(b, d, mode, stage, cs, d > 0 || (stage > 0 && !b->global_lf));
       }
     }
     cudaError_t e2 = cudaStreamEndCapture(cs, &b->graph);
@@ -1303,7 +1304,7 @@ int fp_batch_rhs(fp_batch *b, void *const *dqdt_devs, void *stream) {
   }
   for (int d = 0; d < b->dims && !st; ++d) {
     int mode = d == 0 ? fpk::MODE_WRITE : (d == b->dims - 1 ? fpk::MODE_RHS : fpk::MODE_ADD);
-    st = batch_pass(b, d, mode, 0, s);
+    st = batch_pass(b, d, mode, 0, s, d > 0);
   }
   return st;
 }

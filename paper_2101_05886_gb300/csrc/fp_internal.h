@@ -8,7 +8,7 @@
 namespace fpk {
 
 constexpr int kCellFields = 14;      // per-cell values staged in shared memory
-constexpr int kFaceFields = 10;      // per-face values staged in shared memory (W, delta)
+constexpr int kFaceFields = 16;      // per-face values staged in shared memory, at most (sweep_face_fields)
 constexpr int kNextFields = 15;      // staged per thread: next chunk's cell (Q, k, 1/J), face metrics x2
 constexpr int kEpiFields = 13;       // epilogue operands staged per thread (accumulator, Q^n, dk)
 
@@ -47,6 +47,13 @@ __host__ __device__ constexpr int sweep_ring(bool f32, int scheme, int fix) {
 }
 __host__ __device__ constexpr int sweep_min_ctas(bool f32, int scheme, int fix) {
   return (!f32 || scheme == 2 ? 256 : 512) / sweep_threads(f32, scheme, fix);
+}
+
+// Fields of the face ring: flux and reference-state increment, and for FP32 WENO7 (see the sweep) the
+// lower cell's state and 1/J.
+__host__ __device__ constexpr bool sweep_early(bool f32, int scheme) { return f32 && scheme == 2; }
+__host__ __device__ constexpr int sweep_face_fields(bool f32, int scheme) {
+  return sweep_early(f32, scheme) ? kFaceFields : 10;
 }
 
 // Shared-memory field indices of a staged cell.

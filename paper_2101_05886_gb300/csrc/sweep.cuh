@@ -315,6 +315,25 @@ __device__ __forceinline__ void dflux(T g1, T rinvB, const T uB[3], const T uA[3
   out[4] = (d[4] + dp) * UB + (EA + pA) * dU;
 }
 
+// dflux of two pairs of states at once.
+template <typename P, typename T>
+__device__ __forceinline__ void dflux_pair(T g1, P rinvB, const P uB[3], const P uA[3], const P mA[3], P EA, P pA,
+                                           const P d[5], const P k[3], P out[5]) {
+  P du[3];
+#pragma unroll
+  for (int c = 0; c < 3; ++c) du[c] = pmul(psub(d[1 + c], pmul(uA[c], d[0])), rinvB);
+  P dke = pfma(d[3], uB[2], pfma(d[2], uB[1], pmul(d[1], uB[0])));
+#pragma unroll
+  for (int c = 0; c < 3; ++c) dke = pfma(mA[c], du[c], dke);
+  const P dp = pmul(pc<P>(g1), pfma(pc<P>(T(-0.5)), dke, d[4]));
+  const P UB = pfma(uB[2], k[2], pfma(uB[1], k[1], pmul(uB[0], k[0])));
+  const P dU = pfma(du[2], k[2], pfma(du[1], k[1], pmul(du[0], k[0])));
+  out[0] = pfma(d[3], k[2], pfma(d[2], k[1], pmul(d[1], k[0])));
+#pragma unroll
+  for (int c = 0; c < 3; ++c) out[1 + c] = pfma(dp, k[c], pfma(mA[c], dU, pmul(d[1 + c], UB)));
+  out[4] = pfma(padd(EA, pA), dU, pmul(padd(d[4], dp), UB));
+}
+
 // A pair of stencil points B seen from the frame that moves with the reference state's velocity
 // V = u* (Galilean frame: momenta m - rho V, energy E - m.V + rho V^2/2).  d = B - Q* comes in the
 // laboratory frame and leaves in the moving one, and out = [F(B) - F(Q*)] . k there.  Q* is at
@@ -382,10 +401,15 @@ fp_sweep(const BlockDev *__restrict__ blocks, const SweepItem *__restrict__ item
   // stencil points of a face: i-2..i+3 (5th order) or i-3..i+4 (WENO7), offset index Q0
   constexpr int NS = SCHEME == 2 ? 8 : 6;
   constexpr int Q0 = SCHEME == 2 ? 0 : 1;
+  // kEarly: the face ring also takes the lower cell's state and 1/J, so that the epilogue leaves the
+  // cell ring alone and the next cells are staged without a barrier after it.  FP32 WENO7 has the
+  // registers for it (150 x 141 x 133, M8: 711 -> 698 us a residual); WENO5 spills and loses 1 to 2 %.
+  constexpr bool kEarly = sweep_early(sizeof(T) == 4, SCHEME);
+  constexpr int kFace = sweep_face_fields(sizeof(T) == 4, SCHEME);
   extern __shared__ __align__(16) unsigned char smraw[];
   T *const sm = reinterpret_cast<T *>(smraw);              // cell ring: kCellFields x kRing
-  T *const fr = sm + kCellFields * kRing;                   // face ring: kFaceFields x kRing
-  T *const nsb = fr + kFaceFields * kRing;                  // next chunk's cell and face metrics, per thread
+  T *const fr = sm + kCellFields * kRing;                   // face ring: kFace x kRing
+  T *const nsb = fr + kFace * kRing;                  // next chunk's cell and face metrics, per thread
   T *const epb = nsb + kNextFields * kThreads;              // epilogue operands, per thread
   const int tid = threadIdx.x;
   // Work-item descriptors in shared memory, double-buffered: during an item's first chunk
@@ -715,6 +739,8 @@ fp_sweep(const BlockDev *__restrict__ blocks, const SweepItem *__restrict__ item
         // face metric of this face, staged by the previous chunk (or the prologue)
 #pragma unroll
         for (int c = 0; c < 3; ++c) kf[c] = nsb[(9 + 3 * (ch & 1) + c) * kThreads + tid];
+
+        if (kEarly && mode >= MODE_RHS) fr[15 * kRing + o[3]] = CELL(CF_INVJ, 3);
 
         // reference face state Q* = Q_i + delta (Eqs. Q_star, QdJ_star, 1dJ at order M)
         using P = typename PairOf<T>::type;
@@ -1085,6 +1111,7 @@ fp_sweep(const BlockDev *__restrict__ blocks, const SweepItem *__restrict__ item
         for (int v = 0; v < 5; ++v) {
           fp[v * kRing] = F[v];
           fp[(5 + v) * kRing] = dl[v];
+          if (kEarly) fp[(10 + v) * kRing] = Qi[v];
         }
       }
       cp_async_wait_all();
@@ -1096,7 +1123,7 @@ fp_sweep(const BlockDev *__restrict__ blocks, const SweepItem *__restrict__ item
         if constexpr (!kOwn) {                       // loaded again rather than held over the face's arithmetic
           const int ox = off(ff);
 #pragma unroll
-          for (int v = 0; v < 5; ++v) Qi[v] = sm[(CF_Q + v) * kRing + ox];
+          for (int v = 0; v < 5; ++v) Qi[v] = kEarly ? fr[(10 + v) * kRing + ox] : sm[(CF_Q + v) * kRing + ox];
 #pragma unroll
           for (int c = 0; c < 3; ++c) kf[c] = nsb[(9 + 3 * (ch & 1) + c) * kThreads + tid];
         }
@@ -1109,7 +1136,7 @@ fp_sweep(const BlockDev *__restrict__ blocks, const SweepItem *__restrict__ item
 #pragma unroll
           for (int v = 0; v < 5; ++v) {
             qb[v] = cst[v];
-            const T qx1 = sm[(CF_Q + v) * kRing + oxm], dm = fr[(5 + v) * kRing + oxm];
+            const T qx1 = kEarly ? fr[(10 + v) * kRing + oxm] : sm[(CF_Q + v) * kRing + oxm], dm = fr[(5 + v) * kRing + oxm];
             Qp[v] = Qi[v] + dl[v];
             Qm[v] = qx1 + dm;
             dQ[v] = (Qi[v] - qx1) + (dl[v] - dm);
@@ -1125,11 +1152,31 @@ fp_sweep(const BlockDev *__restrict__ blocks, const SweepItem *__restrict__ item
           T dk[3];
 #pragma unroll
           for (int c = 0; c < 3; ++c) dk[c] = epb[(10 + c) * kThreads + tid];
-          T t1v[5], t2v[5];
-          dflux<T>(g1, rB, uBp, uA, mA, Qm[4], pA, dQ, kf, t1v);          // [F(Q*_+) - F(Q*_-)] . k_+
-          dflux<T>(g1, rA, uA, ub, qb + 1, qb[4], pb, dqm, dk, t2v);       // [F(Q*_-) - F(Qbar)] . (k_+ - k_-)
+          // [F(Q*_+) - F(Q*_-)] . k_+ and [F(Q*_-) - F(Qbar)] . (k_+ - k_-): packed for linear upwind, which is
+          // bound by instruction issue (20-block batch 2.50 -> 2.47 ms), one after the other for the
+          // others, whose FMA pipe is the busier (WENO5 on 256^3 packed: 8.57 -> 8.61 ms)
+          if constexpr (SCHEME == 1 && sizeof(T) == 4) {
+            using P = typename PairOf<T>::type;
+            P d[5], uBq[3], uAq[3], mAq[3], k[3], tv[5];
 #pragma unroll
-          for (int v = 0; v < 5; ++v) R[v] += t1v[v] + t2v[v];
+            for (int v = 0; v < 5; ++v) d[v] = pmk(dQ[v], dqm[v]);
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+              uBq[c] = pmk(uBp[c], uA[c]);
+              uAq[c] = pmk(uA[c], ub[c]);
+              mAq[c] = pmk(mA[c], qb[1 + c]);
+              k[c] = pmk(kf[c], dk[c]);
+            }
+            dflux_pair<P>(g1, pmk(rB, rA), uBq, uAq, mAq, pmk(Qm[4], qb[4]), pmk(pA, pb), d, k, tv);
+#pragma unroll
+            for (int v = 0; v < 5; ++v) R[v] += tv[v].x + tv[v].y;
+          } else {
+            T t1v[5], t2v[5];
+            dflux<T>(g1, rB, uBp, uA, mA, Qm[4], pA, dQ, kf, t1v);
+            dflux<T>(g1, rA, uA, ub, qb + 1, qb[4], pb, dqm, dk, t2v);
+#pragma unroll
+            for (int v = 0; v < 5; ++v) R[v] += t1v[v] + t2v[v];
+          }
         }
         T *const racc = static_cast<T *>(D->racc);
         const T *ra = epb + tid;                      // prefetched accumulator
@@ -1140,7 +1187,7 @@ fp_sweep(const BlockDev *__restrict__ blocks, const SweepItem *__restrict__ item
 #pragma unroll
           for (int v = 0; v < 5; ++v) *FPK_IN(comp_at(racc, qo, qc, v), racc, 5LL * qc, B->status) = ra[v * kThreads] + R[v];
         } else {
-          const T Jc = Num<T>::rcp(sm[CF_INVJ * kRing + off(ff)]);
+          const T Jc = Num<T>::rcp(kEarly ? fr[15 * kRing + off(ff)] : sm[CF_INVJ * kRing + off(ff)]);
           if (mode == MODE_RHS) {
             T *const out = static_cast<T *>(B->dqdt);
 #pragma unroll
@@ -1160,7 +1207,7 @@ fp_sweep(const BlockDev *__restrict__ blocks, const SweepItem *__restrict__ item
           }
         }
       }
-      __syncthreads();
+      if (!kEarly) __syncthreads();
       // ---- stage the next chunk's new cell from this thread's staging slots
       if (staged) {
         const T *src = nsb + tid;
@@ -1190,7 +1237,7 @@ fp_sweep(const BlockDev *__restrict__ blocks, const SweepItem *__restrict__ item
 // dynamic shared memory of a sweep variant: the cell and face rings, then the per-thread slots
 template <typename T, int SCHEME, int FIX>
 constexpr size_t sweep_smem() {
-  return ((size_t)(kCellFields + kFaceFields) * sweep_ring(sizeof(T) == 4, SCHEME, FIX) +
+  return ((size_t)(kCellFields + sweep_face_fields(sizeof(T) == 4, SCHEME)) * sweep_ring(sizeof(T) == 4, SCHEME, FIX) +
           (size_t)(kNextFields + kEpiFields) * sweep_threads(sizeof(T) == 4, SCHEME, FIX)) * sizeof(T);
 }
 

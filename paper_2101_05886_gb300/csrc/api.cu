@@ -27,9 +27,8 @@ struct fp_ctx {
   long long ncells = 0;
   long long nmet = 0;                 // points of one metric component (ghosted box)
   long long nface[3] = {0, 0, 0};     // faces per direction
-  void *met = nullptr;                // T [10][nmet]
-  void *fmet[3] = {nullptr, nullptr, nullptr};
-  void *dk[3] = {nullptr, nullptr, nullptr};
+  void *kj[3] = {nullptr, nullptr, nullptr};   // the sweep's metrics (DirDev)
+  void *fk[3] = {nullptr, nullptr, nullptr};
   void *q1 = nullptr, *q2 = nullptr, *racc = nullptr;
   int *status = nullptr;
   double *dt_dev = nullptr;
@@ -284,6 +283,9 @@ void sweep_constants(const fp_grid_desc &d, T *c) {
 // 256^3 8.67 | 9.19 ms, where the sum's traffic costs more than the passes' ends.
 constexpr long long kSplitPoints = 3 << 19;
 
+// bytes from one direction's accumulator to the next, 32-byte aligned
+size_t split_stride(const fp_ctx *c) { return ((size_t)5 * c->ncells * c->esize + 31) / 32 * 32; }
+
 void fill_dirs(fp_ctx *c) {
   const int ni = c->desc.n[0], nj = c->desc.n[1], nk = c->desc.n[2], G = c->G;
   const int dims = c->desc.dims;
@@ -321,9 +323,8 @@ void fill_dirs(fp_ctx *c) {
     D.fc = (unsigned)c->nface[d];
     D.bclo = c->desc.bc[d][0];
     D.bchi = c->desc.bc[d][1];
-    D.kmet = static_cast<const char *>(c->met) + (size_t)3 * d * c->nmet * c->esize;
-    D.fmet = c->fmet[d];
-    D.dk = c->dk[d];
+    D.kj = c->kj[d];
+    D.fk = c->fk[d];
     D.halo[0] = D.halo[1] = nullptr;
     D.nbr[0] = D.nbr[1] = -1;
     D.racc = c->racc;
@@ -347,8 +348,6 @@ void fill_dirs(fp_ctx *c) {
   B.qc = (unsigned)c->ncells;
   B.mc = (unsigned)c->nmet;
   B.moff = (unsigned)(G + (long long)G * ms1 + (dims == 3 ? (long long)G * ms2 : 0));
-  B.met = c->met;
-  B.imet = static_cast<const char *>(c->met) + (size_t)9 * c->nmet * c->esize;
   B.q[0] = nullptr; B.q[1] = c->q1; B.q[2] = c->q2;
   B.dqdt = nullptr;
   B.gamma = c->desc.gamma;
@@ -513,7 +512,7 @@ int upload_items(fp_ctx *c) {
     if (e != cudaSuccess) return cuda_fail(c, e, "sweep items");
   }
   for (int d = 0; d < c->desc.dims; ++d)          // one accumulator, or the directions' own
-    c->hblk.dir[d].racc = static_cast<char *>(c->racc) + (c->split ? (size_t)5 * d * c->ncells * c->esize : 0);
+    c->hblk.dir[d].racc = static_cast<char *>(c->racc) + (c->split ? d * split_stride(c) : 0);
   if (c->split) {
     c->nscta = balanced_items(c, all, c->per_sm[shape(0)], items);
     cudaError_t e = put_items(items, &c->sitems);
@@ -593,8 +592,7 @@ const char *fp_last_error(const fp_ctx *c) { return c ? c->err.c_str() : "null c
 void fp_free(fp_ctx *c) {
   if (!c) return;
   cudaDeviceSynchronize();
-  cudaFree(c->met);
-  for (int d = 0; d < 3; ++d) { cudaFree(c->fmet[d]); cudaFree(c->dk[d]); cudaFree(c->items[d]); }
+  for (int d = 0; d < 3; ++d) { cudaFree(c->kj[d]); cudaFree(c->fk[d]); cudaFree(c->items[d]); }
   cudaFree(c->q1); cudaFree(c->q2); cudaFree(c->racc);
   cudaFree(c->status); cudaFree(c->dt_dev); cudaFree(c->cfl_bits); cudaFree(c->dblk);
   cudaFree(c->lamg); cudaFree(c->lam_items); cudaFree(c->sitems);
@@ -629,12 +627,10 @@ int fp_init_grid(const fp_grid_desc *desc, const double *xyz, int ghost_nodes, v
 
   cudaError_t e;
   double *nodes = nullptr, *met64 = nullptr, *scratch = nullptr, *fm64[3] = {nullptr, nullptr, nullptr};
-  double *dk64[3] = {nullptr, nullptr, nullptr};
   auto cleanup_tmp = [&]() {
-    cudaFree(nodes); cudaFree(scratch);
-    if (c->is_f32) {
-      cudaFree(met64);
-      for (int d = 0; d < 3; ++d) { cudaFree(fm64[d]); cudaFree(dk64[d]); }
+    for (double **p : {&nodes, &scratch, &met64, &fm64[0], &fm64[1], &fm64[2]}) {
+      cudaFree(*p);
+      *p = nullptr;
     }
   };
 #define FP_TRY(call, where)                         \
@@ -655,37 +651,36 @@ int fp_init_grid(const fp_grid_desc *desc, const double *xyz, int ghost_nodes, v
   FP_TRY(cudaMemcpyAsync(nodes, xyz, (size_t)dims * nnode * sizeof(double), cudaMemcpyHostToDevice, s),
          "copy nodes");
   FP_TRY(fpk::dev_alloc(&met64, (size_t)10 * c->nmet * sizeof(double)), "cudaMalloc(metrics)");
-  for (int d = 0; d < dims; ++d) {
+  for (int d = 0; d < dims; ++d)
     FP_TRY(fpk::dev_alloc(&fm64[d], (size_t)3 * c->nface[d] * sizeof(double)), "cudaMalloc(face metrics)");
-    FP_TRY(fpk::dev_alloc(&dk64[d], (size_t)3 * c->ncells * sizeof(double)), "cudaMalloc(metric differences)");
-  }
   FP_TRY(fpk::dev_alloc(&scratch, (size_t)9 * (nb1 + nb2) * sizeof(double)), "cudaMalloc(metric scratch)");
   fpk::MetricJob J;
   J.dims = dims; J.M = M; J.G = G; J.Gn = Gn;
-  for (int d = 0; d < 3; ++d) { J.n[d] = n[d]; J.fmet[d] = fm64[d]; J.dk[d] = dk64[d]; }
+  for (int d = 0; d < 3; ++d) { J.n[d] = n[d]; J.fmet[d] = fm64[d]; }
   J.nodes = nodes; J.met = met64; J.scratch = scratch;
   FP_TRY(fpk::build_metrics(J, s), "build metrics");
-  if (c->is_f32) {
-    FP_TRY(fpk::dev_alloc(&c->met, (size_t)10 * c->nmet * sizeof(float)), "cudaMalloc(metrics f32)");
-    FP_TRY(fpk::convert_f64_to_f32(met64, (float *)c->met, 10 * c->nmet, s), "convert metrics");
-    for (int d = 0; d < dims; ++d) {
-      FP_TRY(fpk::dev_alloc(&c->fmet[d], (size_t)3 * c->nface[d] * sizeof(float)), "cudaMalloc(face f32)");
-      FP_TRY(fpk::convert_f64_to_f32(fm64[d], (float *)c->fmet[d], 3 * c->nface[d], s), "convert face metrics");
-      FP_TRY(fpk::dev_alloc(&c->dk[d], (size_t)3 * c->ncells * sizeof(float)), "cudaMalloc(differences f32)");
-      FP_TRY(fpk::convert_f64_to_f32(dk64[d], (float *)c->dk[d], 3 * c->ncells, s), "convert differences");
-    }
-  } else {
-    c->met = met64;
-    for (int d = 0; d < 3; ++d) { c->fmet[d] = fm64[d]; c->dk[d] = dk64[d]; }
-  }
+  // the FP64 arrays are released as soon as they are packed: the sweep's take their place
   FP_TRY(cudaStreamSynchronize(s), "metric construction");
-  cleanup_tmp();
-  nodes = nullptr; scratch = nullptr;
-  if (c->is_f32) { met64 = nullptr; for (int d = 0; d < 3; ++d) { fm64[d] = nullptr; dk64[d] = nullptr; } }
+  cudaFree(nodes); cudaFree(scratch);
+  nodes = scratch = nullptr;
+  for (int d = 0; d < dims; ++d) {
+    FP_TRY(fpk::dev_alloc(&c->kj[d], (size_t)4 * c->nmet * c->esize), "cudaMalloc(metrics)");
+    FP_TRY(fpk::pack_metrics(J, d, c->is_f32, c->kj[d], s), "pack metrics");
+  }
+  FP_TRY(cudaStreamSynchronize(s), "metric packing");
+  cudaFree(met64);
+  met64 = nullptr;
+  for (int d = 0; d < dims; ++d) {
+    FP_TRY(fpk::dev_alloc(&c->fk[d], (size_t)6 * c->nface[d] * c->esize), "cudaMalloc(face metrics)");
+    FP_TRY(fpk::pack_faces(J, d, c->is_f32, c->fk[d], s), "pack face metrics");
+    FP_TRY(cudaStreamSynchronize(s), "metric packing");
+    cudaFree(fm64[d]);
+    fm64[d] = nullptr;
+  }
   const size_t sbytes = (size_t)5 * c->ncells * c->esize;
   FP_TRY(fpk::dev_alloc(&c->q1, sbytes), "cudaMalloc(stage 1)");
   FP_TRY(fpk::dev_alloc(&c->q2, sbytes), "cudaMalloc(stage 2)");
-  FP_TRY(fpk::dev_alloc(&c->racc, c->ncells <= kSplitPoints ? dims * sbytes : sbytes), "cudaMalloc(residual)");
+  FP_TRY(fpk::dev_alloc(&c->racc, c->ncells <= kSplitPoints ? dims * split_stride(c) : sbytes), "cudaMalloc(residual)");
   FP_TRY(fpk::dev_alloc(&c->status, sizeof(int)), "cudaMalloc(status)");
   FP_TRY(cudaMemset(c->status, 0, sizeof(int)), "clear status");
   FP_TRY(fpk::dev_alloc(&c->dt_dev, sizeof(double)), "cudaMalloc(dt)");
@@ -881,20 +876,37 @@ int fp_cfl_dt(fp_ctx *c, const void *q, double cfl, double *dt_out, void *stream
   return FP_OK;
 }
 
+// n values of a device array of the context's type as doubles
+static cudaError_t read_back(const fp_ctx *c, const void *src, long long n, std::vector<double> &out) {
+  out.resize(n);
+  if (!c->is_f32) return cudaMemcpy(out.data(), src, n * sizeof(double), cudaMemcpyDeviceToHost);
+  std::vector<float> tmp(n);
+  cudaError_t e = cudaMemcpy(tmp.data(), src, n * sizeof(float), cudaMemcpyDeviceToHost);
+  std::copy(tmp.begin(), tmp.end(), out.begin());
+  return e;
+}
+
+static int get_metrics(fp_ctx *c, double *host_out) {
+  const long long n = c->nmet;
+  std::fill(host_out, host_out + 9 * n, 0.0);     // 2-D: no third metric vector
+  std::vector<double> kj;
+  for (int d = 0; d < c->desc.dims; ++d) {
+    cudaError_t e = read_back(c, c->kj[d], 4 * n, kj);
+    if (e != cudaSuccess) return cuda_fail(c, e, "fp_get_metrics copy");
+    for (long long i = 0; i < n; ++i) {
+      for (int a = 0; a < 3; ++a) host_out[(3 * d + a) * n + i] = kj[4 * i + a];
+      host_out[9 * n + i] = kj[4 * i + 3];
+    }
+  }
+  return FP_OK;
+}
+
 int fp_get_metrics(fp_ctx *c, double *host_out) {
   if (!c) return FP_ERR_ARG;
   if (!host_out) return fail(c, FP_ERR_ARG, "fp_get_metrics: null output");
   cudaError_t e = cudaDeviceSynchronize();
   if (e != cudaSuccess) return cuda_fail(c, e, "fp_get_metrics");
-  const long long n = 10 * c->nmet;
-  if (c->is_f32) {
-    std::vector<float> tmp(n);
-    e = cudaMemcpy(tmp.data(), c->met, n * sizeof(float), cudaMemcpyDeviceToHost);
-    for (long long i = 0; i < n; ++i) host_out[i] = tmp[i];
-  } else {
-    e = cudaMemcpy(host_out, c->met, n * sizeof(double), cudaMemcpyDeviceToHost);
-  }
-  return e == cudaSuccess ? FP_OK : cuda_fail(c, e, "fp_get_metrics copy");
+  return get_metrics(c, host_out);
 }
 
 int fp_get_face_metrics(fp_ctx *c, int dir, double *host_out) {
@@ -902,15 +914,13 @@ int fp_get_face_metrics(fp_ctx *c, int dir, double *host_out) {
   if (!host_out || dir < 0 || dir >= c->desc.dims) return fail(c, FP_ERR_ARG, "fp_get_face_metrics: bad argument");
   cudaError_t e = cudaDeviceSynchronize();
   if (e != cudaSuccess) return cuda_fail(c, e, "fp_get_face_metrics");
-  const long long n = 3 * c->nface[dir];
-  if (c->is_f32) {
-    std::vector<float> tmp(n);
-    e = cudaMemcpy(tmp.data(), c->fmet[dir], n * sizeof(float), cudaMemcpyDeviceToHost);
-    for (long long i = 0; i < n; ++i) host_out[i] = tmp[i];
-  } else {
-    e = cudaMemcpy(host_out, c->fmet[dir], n * sizeof(double), cudaMemcpyDeviceToHost);
-  }
-  return e == cudaSuccess ? FP_OK : cuda_fail(c, e, "fp_get_face_metrics copy");
+  const long long nf = c->nface[dir];
+  std::vector<double> fk;
+  e = read_back(c, c->fk[dir], 6 * nf, fk);
+  if (e != cudaSuccess) return cuda_fail(c, e, "fp_get_face_metrics copy");
+  for (long long f = 0; f < nf; ++f)
+    for (int a = 0; a < 3; ++a) host_out[a * nf + f] = fk[6 * f + a];
+  return FP_OK;
 }
 
 int fp_get_device_status(fp_ctx *c, void *stream) {

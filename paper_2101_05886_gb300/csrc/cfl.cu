@@ -4,7 +4,7 @@
 #include <cuda_runtime.h>
 #include <math.h>
 
-#include "fp_internal.h"
+#include "sweep.cuh"
 
 namespace fpk {
 
@@ -12,19 +12,18 @@ namespace {
 
 // sum_d (|u . grad d| + c |grad d|) of one point in FP64
 template <typename T>
-__device__ double cfl_point(const BlockDev *blk, const T *q, const T *met, long long idx, long long mo, int dims) {
-  const long long qc = blk->qc, mc = blk->mc;
+__device__ double cfl_point(const BlockDev *blk, const T *q, long long idx, long long mo, int dims) {
+  const long long qc = blk->qc;
   const double g = blk->gamma;
   const double rho = (double)q[idx];
   const double u = (double)q[qc + idx] / rho, v = (double)q[2 * qc + idx] / rho, w = (double)q[3 * qc + idx] / rho;
   const double p = (g - 1.0) * ((double)q[4 * qc + idx] - 0.5 * rho * (u * u + v * v + w * w));
   const double c = sqrt(g * p / rho);
-  const double Jc = 1.0 / (double)met[9 * mc + mo];
+  const double Jc = 1.0 / (double)static_cast<const T *>(blk->dir[0].kj)[4 * mo + 3];
   double s = 0.0;
   for (int d = 0; d < dims; ++d) {
-    const double gx = Jc * (double)met[(3 * d) * mc + mo];
-    const double gy = Jc * (double)met[(3 * d + 1) * mc + mo];
-    const double gz = Jc * (double)met[(3 * d + 2) * mc + mo];
+    const T *k = static_cast<const T *>(blk->dir[d].kj) + 4 * mo;
+    const double gx = Jc * (double)k[0], gy = Jc * (double)k[1], gz = Jc * (double)k[2];
     s += fabs(u * gx + v * gy + w * gz) + c * sqrt(gx * gx + gy * gy + gz * gz);
   }
   return s;
@@ -45,13 +44,12 @@ constexpr int kCflThreads = 256, kCflPoints = 4;   // points per thread
 // A step with its bound on 181 x 97 x 61 FP32 points: 1010 -> 792 us with the first form.
 template <typename T> struct CflScreen {
   const BlockDev *blk;
-  const T *q, *met;
-  long long qc, mc;
+  const T *q;
+  long long qc;
   int ni, nj, dims;
   float g1, gam;
   __device__ CflScreen(const BlockDev *b, int ni_, int nj_, int dims_)
-      : blk(b), q(static_cast<const T *>(b->q[0])), met(static_cast<const T *>(b->met)), qc(b->qc), mc(b->mc),
-        ni(ni_), nj(nj_), dims(dims_), g1((float)(b->gamma - 1.0)), gam((float)b->gamma) {}
+      : blk(b), q(static_cast<const T *>(b->q[0])), qc(b->qc), ni(ni_), nj(nj_), dims(dims_), g1((float)(b->gamma - 1.0)), gam((float)b->gamma) {}
   __device__ long long place(long long idx) const {
     const int i = (int)(idx % ni);
     const long long r = idx / ni;
@@ -66,7 +64,14 @@ template <typename T> struct CflScreen {
     float Q[5];
 #pragma unroll
     for (int v = 0; v < 5; ++v) Q[v] = (float)q[v * qc + idx];
-    const float ij = fabsf((float)*FPK_IN(met + (9 * mc + mo), met, 10 * mc, blk->status));
+    // the point's metric vectors and 1/J, the values of one direction side by side
+    auto metric = [&](int d, T k[4]) {
+      const T *kj = static_cast<const T *>(blk->dir[d].kj);
+      load4(FPK_IN(kj + 4 * mo, kj, 4LL * blk->mc - 3, blk->status), k);
+    };
+    T kj[4];
+    metric(0, kj);
+    const float ij = fabsf((float)kj[3]);
     bool ok = Q[0] > kLow && Q[0] < kHigh && Q[4] > kLow && Q[4] < kHigh && ij > kLow && ij < kHigh;
     const float ri = 1.0f / Q[0], Jc = 1.0f / ij;
     const float u = Q[1] * ri, v = Q[2] * ri, w = Q[3] * ri;
@@ -75,9 +80,8 @@ template <typename T> struct CflScreen {
     const float chi = sqrtf(gam * g1 * fmaxf(e + de, 0.f) * ri), clo = sqrtf(gam * g1 * fmaxf(e - de, 0.f) * ri);
     float sh = 0.f, sl = 0.f;
     for (int d = 0; d < dims; ++d) {
-      const float kx = (float)*FPK_IN(met + ((3 * d) * mc + mo), met, 10 * mc, blk->status);
-      const float ky = (float)*FPK_IN(met + ((3 * d + 1) * mc + mo), met, 10 * mc, blk->status);
-      const float kz = (float)*FPK_IN(met + ((3 * d + 2) * mc + mo), met, 10 * mc, blk->status);
+      if (d) metric(d, kj);
+      const float kx = (float)kj[0], ky = (float)kj[1], kz = (float)kj[2];
       const float k2 = kx * kx + ky * ky + kz * kz, kn = sqrtf(k2);
       ok = ok && k2 > kLow && k2 < kHigh;
       const float U = fabsf(u * kx + v * ky + w * kz);
@@ -140,7 +144,7 @@ __global__ void __launch_bounds__(kCflThreads) k_cfl_max(const BlockDev *blk, lo
     const long long idx = (long long)blockIdx.x * (kCflThreads * kCflPoints) + m * kCflThreads + threadIdx.x;
     float l;
     if (idx >= ncells || screen.bound(idx, l) < lo) continue;
-    const double s = cfl_point(blk, screen.q, screen.met, idx, screen.place(idx), dims);
+    const double s = cfl_point(blk, screen.q, idx, screen.place(idx), dims);
     best = s > best ? s : best;
   }
   if (best > 0.0) atomicMax(&out->max_bits, (unsigned long long)__double_as_longlong(best));
@@ -162,15 +166,9 @@ __device__ __forceinline__ void atomic_max_nonneg(double *a, double v) {
   atomicMax(reinterpret_cast<unsigned long long *>(a), (unsigned long long)__double_as_longlong(v));
 }
 
-// 1/x: FP64 by the PTX approximation and a third-order step (Num in sweep.cuh), a quarter of the
-// FP64 operations of a quotient
-__device__ __forceinline__ float recip(float x) { return 1.0f / x; }
-__device__ __forceinline__ double recip(double x) {
-  double y;
-  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-  const double e = fma(-x, y, 1.0);
-  return fma(y, fma(e, e, e), y);
-}
+// 1/x, in FP64 with a quarter of the operations of a quotient
+__device__ __forceinline__ float reciprocal(float x) { return 1.0f / x; }
+__device__ __forceinline__ double reciprocal(double x) { return Num<double>::rcp(x); }
 
 // Max over each block's points of |U - c|grad d||, |U|, |U + c|grad d|| for every direction.  A CTA
 // takes a contiguous range of the items (kLamChunk points each), keeps its maxima in registers
@@ -189,9 +187,8 @@ __global__ void k_lam_max(const BlockDev *blocks, const int2 *items, int nitems,
     const int2 item = items[it];
     const BlockDev *B = blocks + item.x;
     const int dims = B->dims, ni = B->dir[0].nd, nj = B->dir[1].nd;
-    const long long qc = B->qc, mc = B->mc;
+    const long long qc = B->qc;
     const T *q = static_cast<const T *>(B->q[stage]);
-    const T *met = static_cast<const T *>(B->met);
     const T g = T(B->gamma);
     const long long idx = (long long)item.y + threadIdx.x;
     if (idx < qc) {
@@ -200,17 +197,22 @@ __global__ void k_lam_max(const BlockDev *blocks, const int2 *items, int nitems,
       const int j = (int)(r % nj);
       const int k = (int)(r / nj);
       const long long mo = B->moff + i + (long long)j * B->dir[0].mT1 + (dims == 3 ? (long long)k * B->dir[0].mT2 : 0);
-      const T rho = q[idx], rinv = recip(rho);
+      const T rho = q[idx], rinv = reciprocal(rho);
       const T u = q[qc + idx] * rinv, v = q[2 * qc + idx] * rinv, w = q[3 * qc + idx] * rinv;
       const T p = (g - T(1)) * (q[4 * qc + idx] - T(0.5) * rho * (u * u + v * v + w * w));
       const T c2 = g * p * rinv;
-      const T Jc = recip(*FPK_IN(met + (9 * mc + mo), met, 10 * mc, B->status));
+      auto metric = [&](int d, T k[4]) {
+        const T *kj = static_cast<const T *>(B->dir[d].kj);
+        load4(FPK_IN(kj + 4 * mo, kj, 4LL * B->mc - 3, B->status), k);
+      };
+      T kj[4];
+      metric(0, kj);
+      const T Jc = reciprocal(kj[3]);
 #pragma unroll
       for (int d = 0; d < 3; ++d) {
         if (d >= dims) continue;
-        const T kx = *FPK_IN(met + ((3 * d) * mc + mo), met, 10 * mc, B->status),
-                ky = *FPK_IN(met + ((3 * d + 1) * mc + mo), met, 10 * mc, B->status),
-                kz = *FPK_IN(met + ((3 * d + 2) * mc + mo), met, 10 * mc, B->status);
+        if (d) metric(d, kj);
+        const T kx = kj[0], ky = kj[1], kz = kj[2];
         const T U = Jc * (u * kx + v * ky + w * kz), a = fabs(Jc) * sqrt(c2 * (kx * kx + ky * ky + kz * kz));
         T lm = fabs(U - a), l0 = fabs(U), lp = fabs(U + a);
         if (!charwise) { lm = fmax(lm, lp); l0 = lm; lp = lm; }

@@ -9,8 +9,8 @@ namespace fpk {
 
 constexpr int kCellFields = 14;      // per-cell values staged in shared memory
 constexpr int kFaceFields = 16;      // per-face values staged in shared memory, at most (sweep_face_fields)
-constexpr int kNextFields = 15;      // staged per thread: next chunk's cell (Q, k, 1/J), face metrics x2
-constexpr int kEpiFields = 13;       // epilogue operands staged per thread (accumulator, Q^n, dk)
+constexpr int kNextFields = 21;      // staged per thread: next chunk's cell (Q, k, 1/J), face metrics and their change x2
+constexpr int kEpiFields = 10;       // epilogue operands staged per thread (accumulator, Q^n)
 
 // CTA shape of a sweep variant (precision, scheme, fix: 0 switches read at run time, 1 folded,
 // 2 folded with the alternative shape, 3 component-wise): its threads, which equal faces per chunk x
@@ -106,13 +106,16 @@ struct DirDev {
   int qT1, qT2, qsd;   // state offsets: t1, t2 and along-line strides
   int mT1, mT2, msd;   // metric offsets (ghosted arrays)
   int fT1, fT2, fsd;   // face-metric offsets, face f+1/2 at (f+1)*fsd
-  unsigned fc;         // face-metric component stride
+  unsigned fc;         // faces of this direction
   int bclo, bchi;      // boundary codes at the two line ends
   int S, TT;           // faces per chunk, lines per tile (S * TT == the variant's sweep_threads)
-  const void *kmet;    // this direction's metric vector in the cell metrics (component 3 d)
-  const void *fmet;    // T [3][faces]
-  void *racc;          // residual accumulator, state layout (the directions' own or the same one)
-  const void *dk;      // T [3][cells]: k_{i+1/2} - k_{i-1/2} along this direction (FP64-formed)
+  // Metrics of this direction, the values of a point side by side, so that the eta and zeta passes,
+  // whose tiles are TT points wide, read rows of 16 TT and 24 TT bytes instead of 4 TT (FP32; with
+  // the accumulator alike: 256^3 WENO5 step 8.52 -> 7.85 ms, 64-block batch 16.81 -> 16.33 ms,
+  // linear batch 2.48 -> 2.33 ms).
+  const void *kj;      // T [ghosted cells][4]: metric vector (d_x, d_y, d_z)/J and 1/J
+  const void *fk;      // T [faces][6]: metric k of face x + 1/2; k_{x+1/2} - k_{x-1/2} of cell x (FP64-formed)
+  void *racc;          // residual accumulator, T [cells][4] then T [cells] (the directions' own or the same one)
   // FP_BC_HALO sides: the caller's buffers of the G cells beyond each side, laid out like the
   // state with this direction's extent replaced by G (strides: t1, t2, along the line, component)
   const void *halo[2];
@@ -128,10 +131,8 @@ struct alignas(16) BlockDev {
   int dims;
   int G;               // metric ghost width
   unsigned qc;         // state component stride (ni*nj*nk)
-  unsigned mc;         // metric component stride
+  unsigned mc;         // ghosted cells
   unsigned moff;       // offset of point (0,0,0) in the metric arrays
-  const void *met;     // T [10][...] cell metrics with G ghosts
-  const void *imet;    // its component 9, 1/J
   void *q[3];          // stage states: 0 = Q^n (caller), 1 = Q^(1), 2 = Q^(2)
   void *dqdt;          // output of the rhs mode
   double gamma;
@@ -243,11 +244,12 @@ struct MetricJob {
   const double *nodes;     // device, [dims][..] with Gn ghosts
   double *met;             // device, [10][B3]
   double *fmet[3];         // device, face metrics per direction [3][faces]
-  double *dk[3];           // device, per-point face-metric difference per direction [3][cells]
   double *scratch;         // device, 9 * |B2| doubles
 };
 cudaError_t build_metrics(const MetricJob &J, cudaStream_t s);
-cudaError_t convert_f64_to_f32(const double *src, float *dst, long long n, cudaStream_t s);
+// The sweep's arrays (DirDev kj and fk) of direction d from the FP64 ones, in its type.
+cudaError_t pack_metrics(const MetricJob &J, int d, int is_f32, void *kj, cudaStream_t s);
+cudaError_t pack_faces(const MetricJob &J, int d, int is_f32, void *fk, cudaStream_t s);
 
 // Global Lax-Friedrichs speeds (cfl.cu): zero, then max over (block, first point) items of
 // kLamChunk points each (the kernel's threads).

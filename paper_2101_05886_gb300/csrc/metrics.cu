@@ -18,7 +18,7 @@
 // value is formed from coordinates and derivative stencils measured from the
 // point itself: the sums then carry the rounding of the metric's own size and
 // the discrete SCL residual stays at the metric round-off at any grid size.
-// Finally k_{i+1/2} - k_{i-1/2} is formed per point and direction in FP64.
+// Finally the values are packed per point for the sweep, with k_{i+1/2} - k_{i-1/2} formed in FP64.
 #include <cuda_runtime.h>
 
 #include "fp_internal.h"
@@ -214,31 +214,31 @@ __global__ void k_face_metrics(const double *met, Box b3, Coef C, int d, int n0,
   }
 }
 
-// metric difference across a cell along d: dk[a] = k_{i+1/2} - k_{i-1/2} (interior points,
-// state layout [3][nk][nj][ni])
-__global__ void k_face_diff(const double *fm, int d, int n0, int n1, int n2, double *dk) {
-  const long long ncell = (long long)n0 * n1 * n2;
+// kj[4 i + a] = metric vector of direction d and 1/J of ghosted cell i
+template <typename T>
+__global__ void k_pack_cells(const double *met, long long n3, int d, T *kj) {
+  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n3; i += (long long)gridDim.x * blockDim.x) {
+    for (int a = 0; a < 3; ++a) kj[4 * i + a] = (T)met[(3 * d + a) * n3 + i];
+    kj[4 * i + 3] = (T)met[9 * n3 + i];
+  }
+}
+
+// fk[6 f + a] = metric of face f, and behind it the difference to the face one lower along d (across
+// the cell between them), formed in FP64; 0 for the lowest face
+template <typename T>
+__global__ void k_pack_faces(const double *fm, int d, int n0, int n1, int n2, T *fk) {
   int nf[3] = {n0, n1, n2};
   nf[d] += 1;
   const long long nfaces = (long long)nf[0] * nf[1] * nf[2];
   const long long sd = d == 0 ? 1 : (d == 1 ? nf[0] : (long long)nf[0] * nf[1]);
-  for (long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x; idx < ncell;
-       idx += (long long)gridDim.x * blockDim.x) {
-    int p[3];
-    p[0] = (int)(idx % n0);
-    long long r = idx / n0;
-    p[1] = (int)(r % n1);
-    p[2] = (int)(r / n1);
-    // face p_d + 1/2 sits at index p_d + 1 along d, face p_d - 1/2 at p_d
-    const long long fo = (long long)p[0] + (long long)nf[0] * (p[1] + (long long)nf[1] * p[2]);
-    for (int a = 0; a < 3; ++a) dk[a * ncell + idx] = fm[a * nfaces + fo + sd] - fm[a * nfaces + fo];
+  for (long long f = blockIdx.x * (long long)blockDim.x + threadIdx.x; f < nfaces; f += (long long)gridDim.x * blockDim.x) {
+    const bool low = f / sd % nf[d] == 0;
+    for (int a = 0; a < 3; ++a) {
+      const double v = fm[a * nfaces + f];
+      fk[6 * f + a] = (T)v;
+      fk[6 * f + 3 + a] = low ? T(0) : (T)(v - fm[a * nfaces + f - sd]);
+    }
   }
-}
-
-__global__ void k_f64_to_f32(const double *src, float *dst, long long n) {
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
-       i += (long long)gridDim.x * blockDim.x)
-    dst[i] = (float)src[i];
 }
 
 int grid_for(long long n) {
@@ -264,14 +264,25 @@ cudaError_t build_metrics(const MetricJob &J, cudaStream_t s) {
   for (int d = 0; d < J.dims; ++d) {
     long long nf = (long long)J.n[0] * J.n[1] * J.n[2] / J.n[d] * (J.n[d] + 1);
     k_face_metrics<<<grid_for(nf), 256, 0, s>>>(J.met, b3, C, d, J.n[0], J.n[1], J.n[2], J.fmet[d]);
-    const long long nc = (long long)J.n[0] * J.n[1] * J.n[2];
-    k_face_diff<<<grid_for(nc), 256, 0, s>>>(J.fmet[d], d, J.n[0], J.n[1], J.n[2], J.dk[d]);
   }
   return cudaGetLastError();
 }
 
-cudaError_t convert_f64_to_f32(const double *src, float *dst, long long n, cudaStream_t s) {
-  k_f64_to_f32<<<grid_for(n), 256, 0, s>>>(src, dst, n);
+cudaError_t pack_metrics(const MetricJob &J, int d, int is_f32, void *kj, cudaStream_t s) {
+  const long long n3 = make_box(J.dims, J.n, J.G).size();
+  if (is_f32)
+    k_pack_cells<<<grid_for(n3), 256, 0, s>>>(J.met, n3, d, static_cast<float *>(kj));
+  else
+    k_pack_cells<<<grid_for(n3), 256, 0, s>>>(J.met, n3, d, static_cast<double *>(kj));
+  return cudaGetLastError();
+}
+
+cudaError_t pack_faces(const MetricJob &J, int d, int is_f32, void *fk, cudaStream_t s) {
+  const long long nf = (long long)J.n[0] * J.n[1] * J.n[2] / J.n[d] * (J.n[d] + 1);
+  if (is_f32)
+    k_pack_faces<<<grid_for(nf), 256, 0, s>>>(J.fmet[d], d, J.n[0], J.n[1], J.n[2], static_cast<float *>(fk));
+  else
+    k_pack_faces<<<grid_for(nf), 256, 0, s>>>(J.fmet[d], d, J.n[0], J.n[1], J.n[2], static_cast<double *>(fk));
   return cudaGetLastError();
 }
 

@@ -17,21 +17,25 @@ __global__ void __launch_bounds__(256) k_finish(const BlockDev *__restrict__ blk
   const unsigned idx = blockIdx.x * 256u + threadIdx.x;
   const unsigned i = idx % ni, r = idx / ni, j = r % nj, k = r / nj, qc = blk->qc;
   const DirDev *D = &blk->dir[0];      // lines along i: its transverse strides are those of j and k
-  const T *met = static_cast<const T *>(blk->met);
+  const T *kj = static_cast<const T *>(D->kj);
   const unsigned mo = blk->moff + i + j * D->mT1 + k * D->mT2;
   const bool in = idx < ncells;
-  const T Jc = in ? Num<T>::rcp(*FPK_IN(comp_at(met, mo, blk->mc, 9), met, 10LL * blk->mc, blk->status)) : T(0);
+  const T Jc = in ? Num<T>::rcp(*FPK_IN(kj + (4ULL * mo + 3), kj, 4LL * blk->mc, blk->status)) : T(0);
   chain_wait();
   chain_next();
   if (!in) return;
-  const T *acc[3];
+  T acc[3][5], R[5], qk[5], qn[5];
 #pragma unroll
-  for (int d = 0; d < 3; ++d) acc[d] = static_cast<const T *>(blk->dir[d].racc);
-  T R[5], qk[5], qn[5];
+  for (int d = 0; d < 3; ++d) {
+    if (d >= dims) continue;
+    const T *a = static_cast<const T *>(blk->dir[d].racc);
+    load4(a + 4ULL * idx, acc[d]);
+    acc[d][4] = *comp_at(a, idx, qc, 4);
+  }
 #pragma unroll
   for (int v = 0; v < 5; ++v) {
-    R[v] = *comp_at(acc[0], idx, qc, v) + *comp_at(acc[1], idx, qc, v);
-    if (dims == 3) R[v] += *comp_at(acc[2], idx, qc, v);
+    R[v] = acc[0][v] + acc[1][v];
+    if (dims == 3) R[v] += acc[2][v];
     if (rk) qk[v] = *comp_at(static_cast<const T *>(blk->q[stage]), idx, qc, v);
     qn[v] = rk && stage ? *comp_at(static_cast<const T *>(blk->q[0]), idx, qc, v) : T(0);
   }

@@ -242,10 +242,10 @@ __device__ __forceinline__ T *comp_at(T *base, unsigned off, unsigned stride, un
 }
 
 // Slip-wall reflection of a ghost value (the mirror cell's state Q) about the boundary
-// face metric fm (component stride fcs): m - 2 (m.k) k/|k|^2.
+// face metric fm: m - 2 (m.k) k/|k|^2.
 template <typename T>
-__device__ __forceinline__ void wall_reflect(T Q[5], const T *fm, unsigned fcs) {
-  const T n0 = fm[0], n1 = *comp_at(fm, 0, fcs, 1), n2 = *comp_at(fm, 0, fcs, 2);
+__device__ __forceinline__ void wall_reflect(T Q[5], const T *fm) {
+  const T n0 = fm[0], n1 = fm[1], n2 = fm[2];
   const T s = T(2) * (Q[1] * n0 + Q[2] * n1 + Q[3] * n2) / (n0 * n0 + n1 * n1 + n2 * n2);
   Q[1] -= s * n0;
   Q[2] -= s * n1;
@@ -268,6 +268,31 @@ __device__ __forceinline__ void cp_async16(void *smem, const void *gmem) {
 __device__ __forceinline__ void cp_async8(void *smem, const void *gmem) {
   const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
   asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(sa), "l"(gmem));
+}
+// copies of four or six neighbouring elements, in the widest pieces that six keep aligned
+template <typename T>
+__device__ __forceinline__ void cp_async_2el(T *smem, const T *gmem) {
+  if (sizeof(T) == 4) cp_async8(smem, gmem); else cp_async16(smem, gmem);
+}
+template <typename T>
+__device__ __forceinline__ void cp_async_4el(T *smem, const T *gmem) {
+  cp_async16(smem, gmem);
+  if (sizeof(T) == 8) cp_async16(smem + 2, gmem + 2);
+}
+__device__ __forceinline__ void load4(const float *p, float v[4]) {
+  const float4 x = *reinterpret_cast<const float4 *>(p);
+  v[0] = x.x; v[1] = x.y; v[2] = x.z; v[3] = x.w;
+}
+__device__ __forceinline__ void load4(const double *p, double v[4]) {
+  const double2 x = *reinterpret_cast<const double2 *>(p), y = *reinterpret_cast<const double2 *>(p + 2);
+  v[0] = x.x; v[1] = x.y; v[2] = y.x; v[3] = y.y;
+}
+__device__ __forceinline__ void store4(float *p, const float v[4]) {
+  *reinterpret_cast<float4 *>(p) = make_float4(v[0], v[1], v[2], v[3]);
+}
+__device__ __forceinline__ void store4(double *p, const double v[4]) {
+  *reinterpret_cast<double2 *>(p) = make_double2(v[0], v[1]);
+  *reinterpret_cast<double2 *>(p + 2) = make_double2(v[2], v[3]);
 }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::); }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_group 0;\n" ::: "memory"); }
@@ -457,7 +482,7 @@ fp_sweep(const BlockDev *__restrict__ blocks, const SweepItem *__restrict__ item
     const int turn = slotFast && S < 32 && (tl & (16 / S)) ? S : 0;
     const int nd = D->nd, nt1 = D->nt1, nt2 = D->nt2;
     const int qsd = D->qsd;
-    const unsigned fcs = D->fc, qc = B->qc, mc = B->mc;
+    const unsigned qc = B->qc;
     const int G = B->G;
     // The lines of a tile row are marched as one stream of positions: line after line, each with
     // its G ghost cells at both ends (period P).  `u` is a position within its line (cell
@@ -494,7 +519,6 @@ fp_sweep(const BlockDev *__restrict__ blocks, const SweepItem *__restrict__ item
           if (t1 >= nt1) { t1 -= nt1; ++t2; }
         }
     };
-    const T *__restrict__ fmet = static_cast<const T *>(D->fmet);
     const T *__restrict__ qin = static_cast<const T *>(B->q[stage]);
     const int glf = kFold ? 0 : B->global_lf;
     // the block's constants in the arithmetic type: far-field state, its velocity and pressure,
@@ -564,16 +588,18 @@ fp_sweep(const BlockDev *__restrict__ blocks, const SweepItem *__restrict__ item
     };
     // slip wall: reflect about the boundary face of the line (face -1/2 or nd-1/2)
     auto reflect = [&](int x, int t1, int t2, T Q[5]) {
-      wall_reflect<T>(Q, FPK_IN(fmet + foff(x < 0 ? -1 : nd - 1, t1, t2), fmet, fcs, B->status), fcs);
+      const T *const fk = static_cast<const T *>(D->fk);
+      wall_reflect<T>(Q, FPK_IN(fk + 6ULL * foff(x < 0 ? -1 : nd - 1, t1, t2), fk, 6LL * D->fc - 5, B->status));
     };
 
     // global loads of one cell (Q, metric vector, 1/J) with the boundary rule applied
     auto fetch = [&](int x, int t1, int t2, T Q[5], T k[3], T &invJ) {
       if (x >= -G && x < nd + G) {
-        const unsigned mo = moff(x, t1, t2);
-#pragma unroll
-        for (int a = 0; a < 3; ++a) k[a] = *FPK_IN(comp_at(static_cast<const T *>(D->kmet), mo, mc, a), static_cast<const T *>(B->met), 10LL * mc, B->status);
-        invJ = *FPK_IN(static_cast<const T *>(B->imet) + mo, static_cast<const T *>(B->met), 10LL * mc, B->status);
+        const T *const kj = static_cast<const T *>(D->kj);
+        T kv[4];
+        load4(FPK_IN(kj + 4ULL * moff(x, t1, t2), kj, 4LL * B->mc - 3, B->status), kv);
+        k[0] = kv[0]; k[1] = kv[1]; k[2] = kv[2];
+        invJ = kv[3];
         const T *qp;
         unsigned cs;
         bool far, wall;
@@ -614,24 +640,20 @@ fp_sweep(const BlockDev *__restrict__ blocks, const SweepItem *__restrict__ item
       cp[CF_AC * kRing] = fabs(Jc) * Num<T>::sqrt_(gam * p * rinv * (k[0] * k[0] + k[1] * k[1] + k[2] * k[2]));
     };
 
-    // asynchronous copy of the face metric of face x + 1/2 of line (t1, t2) into staging slot
-    // `slot` (0/1, alternating between chunks)
+    // asynchronous copy of the metrics of face x + 1/2 of line (t1, t2), and of the change of the face
+    // metric over cell x, into staging slot `slot` (0/1, alternating between chunks)
     auto prefetch_face = [&](int x, int t1, int t2, int slot) {
-      T *dst = nsb + tid + (9 + 3 * slot) * kThreads;
-      const unsigned fo = foff(x, t1, t2);
+      T *dst = nsb + (9 + 6 * slot) * kThreads + 6 * tid;
+      const T *const fk = static_cast<const T *>(D->fk);
+      const T *const src = FPK_IN(fk + 6ULL * foff(x, t1, t2), fk, 6LL * D->fc - 5, B->status);
 #pragma unroll
-      for (int c = 0; c < 3; ++c)
-        cp_async_el(dst + c * kThreads, FPK_IN(comp_at(fmet, fo, fcs, c), fmet, 3LL * fcs, B->status));
+      for (int c = 0; c < 6; c += 2) cp_async_2el(dst + c, src + c);
     };
     // asynchronous copy of one cell's loads (-G <= x < nd + G) into this thread's staging slots
     auto prefetch_cell = [&](int x, int t1, int t2) {
       T *dst = nsb + tid;
-      const unsigned mo = moff(x, t1, t2);
-      const T *const md = static_cast<const T *>(D->kmet), *const mi = static_cast<const T *>(B->imet);
-#pragma unroll
-      for (int a = 0; a < 3; ++a)
-        cp_async_el(dst + (5 + a) * kThreads, FPK_IN(comp_at(md, mo, mc, a), static_cast<const T *>(B->met), 10LL * mc, B->status));
-      cp_async_el(dst + 8 * kThreads, FPK_IN(mi + mo, static_cast<const T *>(B->met), 10LL * mc, B->status));
+      const T *const kj = static_cast<const T *>(D->kj);
+      cp_async_4el(nsb + 5 * kThreads + 4 * tid, FPK_IN(kj + 4ULL * moff(x, t1, t2), kj, 4LL * B->mc - 3, B->status));
       const T *qp;
       unsigned cs;
       bool far, wall;
@@ -647,25 +669,18 @@ fp_sweep(const BlockDev *__restrict__ blocks, const SweepItem *__restrict__ item
       }
     };
     // asynchronous copy of the epilogue operands of a cell (state offset qo: residual
-    // accumulator, Q^n, metric differences) into this thread's slots
+    // accumulator, Q^n) into this thread's slots
     auto prefetch_epilogue = [&](unsigned qo) {
-      T *dst = epb + tid;
       if (mode != MODE_WRITE) {
         const T *const ra = static_cast<const T *>(D->racc);
-#pragma unroll
-        for (int v = 0; v < 5; ++v) cp_async_el(dst + v * kThreads, FPK_IN(comp_at(ra, qo, qc, v), ra, 5LL * qc, B->status));
+        cp_async_4el(epb + 4 * tid, FPK_IN(ra + 4ULL * qo, ra, 4LL * qc - 3, B->status));
+        cp_async_el(epb + 4 * kThreads + tid, FPK_IN(comp_at(ra, qo, qc, 4), ra, 5LL * qc, B->status));
       }
       if (mode == MODE_RK && stage != 0) {
         const T *const qn = static_cast<const T *>(B->q[0]);
 #pragma unroll
         for (int v = 0; v < 5; ++v)
-          cp_async_el(dst + (5 + v) * kThreads, FPK_IN(comp_at(qn, qo, qc, v), qn, 5LL * qc, B->status));
-      }
-      if (fpform) {
-        const T *const dkp = static_cast<const T *>(D->dk);
-#pragma unroll
-        for (int c = 0; c < 3; ++c)
-          cp_async_el(dst + (10 + c) * kThreads, FPK_IN(comp_at(dkp, qo, qc, c), dkp, 3LL * qc, B->status));
+          cp_async_el(epb + (5 + v) * kThreads + tid, FPK_IN(comp_at(qn, qo, qc, v), qn, 5LL * qc, B->status));
       }
     };
 
@@ -738,7 +753,7 @@ fp_sweep(const BlockDev *__restrict__ blocks, const SweepItem *__restrict__ item
         for (int v = 0; v < 5; ++v) { Qi[v] = CELL(CF_Q + v, 3); dl[v] = T(0); }
         // face metric of this face, staged by the previous chunk (or the prologue)
 #pragma unroll
-        for (int c = 0; c < 3; ++c) kf[c] = nsb[(9 + 3 * (ch & 1) + c) * kThreads + tid];
+        for (int c = 0; c < 3; ++c) kf[c] = nsb[(9 + 6 * (ch & 1)) * kThreads + 6 * tid + c];
 
         if (kEarly && mode >= MODE_RHS) fr[15 * kRing + o[3]] = CELL(CF_INVJ, 3);
 
@@ -1125,7 +1140,7 @@ fp_sweep(const BlockDev *__restrict__ blocks, const SweepItem *__restrict__ item
 #pragma unroll
           for (int v = 0; v < 5; ++v) Qi[v] = kEarly ? fr[(10 + v) * kRing + ox] : sm[(CF_Q + v) * kRing + ox];
 #pragma unroll
-          for (int c = 0; c < 3; ++c) kf[c] = nsb[(9 + 3 * (ch & 1) + c) * kThreads + tid];
+          for (int c = 0; c < 3; ++c) kf[c] = nsb[(9 + 6 * (ch & 1)) * kThreads + 6 * tid + c];
         }
         T R[5];
 #pragma unroll
@@ -1151,7 +1166,7 @@ fp_sweep(const BlockDev *__restrict__ blocks, const SweepItem *__restrict__ item
           const T uBp[3] = {Qp[1] * rB, Qp[2] * rB, Qp[3] * rB};
           T dk[3];
 #pragma unroll
-          for (int c = 0; c < 3; ++c) dk[c] = epb[(10 + c) * kThreads + tid];
+          for (int c = 0; c < 3; ++c) dk[c] = nsb[(9 + 6 * (ch & 1)) * kThreads + 6 * tid + 3 + c];
           // [F(Q*_+) - F(Q*_-)] . k_+ and [F(Q*_-) - F(Qbar)] . (k_+ - k_-): packed for linear upwind, which is
           // bound by instruction issue (20-block batch 2.50 -> 2.47 ms), one after the other for the
           // others, whose FMA pipe is the busier (WENO5 on 256^3 packed: 8.57 -> 8.61 ms)
@@ -1179,27 +1194,32 @@ fp_sweep(const BlockDev *__restrict__ blocks, const SweepItem *__restrict__ item
           }
         }
         T *const racc = static_cast<T *>(D->racc);
-        const T *ra = epb + tid;                      // prefetched accumulator
-        if (mode == MODE_WRITE) {
+        // the accumulator holds four components side by side and the fifth behind them (one wide
+        // access per point instead of four: the eta and zeta rows are only TT points wide)
+        if (mode != MODE_WRITE) {                     // add what the passes before wrote
+          T ra[4];
+          load4(epb + 4 * tid, ra);
 #pragma unroll
-          for (int v = 0; v < 5; ++v) *FPK_IN(comp_at(racc, qo, qc, v), racc, 5LL * qc, B->status) = R[v];
-        } else if (mode == MODE_ADD) {
-#pragma unroll
-          for (int v = 0; v < 5; ++v) *FPK_IN(comp_at(racc, qo, qc, v), racc, 5LL * qc, B->status) = ra[v * kThreads] + R[v];
+          for (int v = 0; v < 4; ++v) R[v] = ra[v] + R[v];
+          R[4] = epb[4 * kThreads + tid] + R[4];
+        }
+        if (mode <= MODE_ADD) {
+          store4(FPK_IN(racc + 4ULL * qo, racc, 4LL * qc - 3, B->status), R);
+          *FPK_IN(comp_at(racc, qo, qc, 4), racc, 5LL * qc, B->status) = R[4];
         } else {
           const T Jc = Num<T>::rcp(kEarly ? fr[15 * kRing + off(ff)] : sm[CF_INVJ * kRing + off(ff)]);
           if (mode == MODE_RHS) {
             T *const out = static_cast<T *>(B->dqdt);
 #pragma unroll
             for (int v = 0; v < 5; ++v)
-              *FPK_IN(comp_at(out, qo, qc, v), out, 5LL * qc, B->status) = -Jc * (ra[v * kThreads] + R[v]);
+              *FPK_IN(comp_at(out, qo, qc, v), out, 5LL * qc, B->status) = -Jc * R[v];
           } else {
             T *const qs = static_cast<T *>(B->q[(stage + 1) % 3]);
             const RkStage<T> rk(stage, s_dt);
             bool bad = false;
 #pragma unroll
             for (int v = 0; v < 5; ++v) {
-              const T nv = rk(Qi[v], ra + (5 + v) * kThreads, -Jc * (ra[v * kThreads] + R[v]));
+              const T nv = rk(Qi[v], epb + (5 + v) * kThreads + tid, -Jc * R[v]);
               *FPK_IN(comp_at(qs, qo, qc, v), qs, 5LL * qc, B->status) = nv;
               bad |= !isfinite(nv);
             }
@@ -1212,7 +1232,8 @@ fp_sweep(const BlockDev *__restrict__ blocks, const SweepItem *__restrict__ item
       if (staged) {
         const T *src = nsb + tid;
         T Q[5] = {src[0], src[kThreads], src[2 * kThreads], src[3 * kThreads], src[4 * kThreads]};
-        const T k[3] = {src[5 * kThreads], src[6 * kThreads], src[7 * kThreads]};
+        T kv[4];
+        load4(nsb + 5 * kThreads + 4 * tid, kv);
         if (BND) {                                   // a slip-wall ghost?
           int uc = u + 4, c1 = t1, c2 = t2;
           wrap(uc, c1, c2);
@@ -1226,7 +1247,7 @@ fp_sweep(const BlockDev *__restrict__ blocks, const SweepItem *__restrict__ item
             if (wall) reflect(xs, c1, c2, Q);
           }
         }
-        stage_cell(a + S + 4 + tf, Q, k, src[8 * kThreads]);
+        stage_cell(a + S + 4 + tf, Q, kv, kv[3]);
       }
       __syncthreads();
     }

@@ -850,7 +850,7 @@ int fp_pack_halo(fp_ctx *c, const void *q, int stage, int dir, int side, void *o
     return fail(c, FP_ERR_ARG, "fp_pack_halo: bad argument");
   const void *src = stage == 0 ? q : (stage == 1 ? c->q1 : c->q2);
   cudaError_t e =
-      fpk::launch_pack_halo(src, c->is_f32, dir, side, c->G, c->desc.n, out_dev, c->status, (cudaStream_t)stream);
+      fpk::launch_pack_halo(src, stage, c->is_f32, dir, side, c->G, c->desc.n, out_dev, c->status, (cudaStream_t)stream);
   return e == cudaSuccess ? FP_OK : cuda_fail(c, e, "fp_pack_halo");
 }
 

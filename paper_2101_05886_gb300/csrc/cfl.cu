@@ -197,9 +197,10 @@ __global__ void k_lam_max(const BlockDev *blocks, const int2 *items, int nitems,
       const int j = (int)(r % nj);
       const int k = (int)(r / nj);
       const long long mo = B->moff + i + (long long)j * B->dir[0].mT1 + (dims == 3 ? (long long)k * B->dir[0].mT2 : 0);
-      const T rho = q[idx], rinv = reciprocal(rho);
-      const T u = q[qc + idx] * rinv, v = q[2 * qc + idx] * rinv, w = q[3 * qc + idx] * rinv;
-      const T p = (g - T(1)) * (q[4 * qc + idx] - T(0.5) * rho * (u * u + v * v + w * w));
+      auto val = [&](int c) { return q[state_at(stage, idx, qc, c)]; };
+      const T rho = val(0), rinv = reciprocal(rho);
+      const T u = val(1) * rinv, v = val(2) * rinv, w = val(3) * rinv;
+      const T p = (g - T(1)) * (val(4) - T(0.5) * rho * (u * u + v * v + w * w));
       const T c2 = g * p * rinv;
       auto metric = [&](int d, T k[4]) {
         const T *kj = static_cast<const T *>(B->dir[d].kj);
@@ -243,7 +244,7 @@ __global__ void k_lam_max(const BlockDev *blocks, const int2 *items, int nitems,
 // the state layout [5][nk][nj][ni] with the extent of direction `dir` replaced by G.  Low
 // side: cells 0..G-1; high side: cells n-G..n-1 (index x - (n - G) in the buffer).
 template <typename T>
-__global__ void k_pack_halo(const T *__restrict__ q, T *__restrict__ out, int dir, int side, int G, int ni,
+__global__ void k_pack_halo(const T *__restrict__ q, int stage, T *__restrict__ out, int dir, int side, int G, int ni,
                             int nj, int nk, int *status) {
   int e[3] = {ni, nj, nk};
   const int nd = e[dir];
@@ -259,13 +260,13 @@ __global__ void k_pack_halo(const T *__restrict__ q, T *__restrict__ out, int di
     c[1] = (int)(r % e[1]);
     c[2] = (int)(r / e[1]);
     c[dir] += side ? nd - G : 0;
-    out[idx] = *FPK_IN(q + (v * qc + ((long long)c[2] * nj + c[1]) * ni + c[0]), q, 5 * qc, status);
+    out[idx] = *FPK_IN(q + state_at(stage, ((long long)c[2] * nj + c[1]) * ni + c[0], qc, v), q, 5 * qc, status);
   }
 }
 
 }  // namespace
 
-cudaError_t launch_pack_halo(const void *q, int is_f32, int dir, int side, int G, const int *n, void *out,
+cudaError_t launch_pack_halo(const void *q, int stage, int is_f32, int dir, int side, int G, const int *n, void *out,
                              int *status, cudaStream_t s) {
   int e[3] = {n[0], n[1], n[2]};
   e[dir] = G;
@@ -274,10 +275,10 @@ cudaError_t launch_pack_halo(const void *q, int is_f32, int dir, int side, int G
   const long long want = (total + threads - 1) / threads;
   const int grid = (int)(want < 4096 ? (want < 1 ? 1 : want) : 4096);
   if (is_f32)
-    k_pack_halo<float><<<grid, threads, 0, s>>>(static_cast<const float *>(q), static_cast<float *>(out), dir, side, G,
+    k_pack_halo<float><<<grid, threads, 0, s>>>(static_cast<const float *>(q), stage, static_cast<float *>(out), dir, side, G,
                                                 n[0], n[1], n[2], status);
   else
-    k_pack_halo<double><<<grid, threads, 0, s>>>(static_cast<const double *>(q), static_cast<double *>(out), dir, side,
+    k_pack_halo<double><<<grid, threads, 0, s>>>(static_cast<const double *>(q), stage, static_cast<double *>(out), dir, side,
                                                  G, n[0], n[1], n[2], status);
   return cudaGetLastError();
 }

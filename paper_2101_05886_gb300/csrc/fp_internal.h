@@ -133,7 +133,8 @@ struct alignas(16) BlockDev {
   unsigned qc;         // state component stride (ni*nj*nk)
   unsigned mc;         // ghosted cells
   unsigned moff;       // offset of point (0,0,0) in the metric arrays
-  void *q[3];          // stage states: 0 = Q^n (caller), 1 = Q^(1), 2 = Q^(2)
+  // stage states: 0 = Q^n (the caller's, T [5][cells]), 1 = Q^(1), 2 = Q^(2) (T [cells][4] then T [cells])
+  void *q[3];
   void *dqdt;          // output of the rhs mode
   double gamma;
   // the sweep's constants in its arithmetic type (12 float or double values): reference (far-field)
@@ -275,7 +276,7 @@ cudaError_t launch_cfl(const BlockDev *blk, int is_f32, long long ncells, const 
 // Halo packing (cfl.cu): the G cells of stage state `stage` next to side `side` of direction
 // `dir` into `out`, in the halo layout of DirDev (the receiving block's view of them); `status`
 // is the context's status word (bounds-checking builds record there).
-cudaError_t launch_pack_halo(const void *q, int is_f32, int dir, int side, int G, const int *n, void *out,
+cudaError_t launch_pack_halo(const void *q, int stage, int is_f32, int dir, int side, int G, const int *n, void *out,
                              int *status, cudaStream_t s);
 
 }  // namespace fpk

@@ -36,7 +36,7 @@ __global__ void __launch_bounds__(256) k_finish(const BlockDev *__restrict__ blk
   for (int v = 0; v < 5; ++v) {
     R[v] = acc[0][v] + acc[1][v];
     if (dims == 3) R[v] += acc[2][v];
-    if (rk) qk[v] = *comp_at(static_cast<const T *>(blk->q[stage]), idx, qc, v);
+    if (rk) qk[v] = static_cast<const T *>(blk->q[stage])[state_at(stage, idx, qc, v)];
     qn[v] = rk && stage ? *comp_at(static_cast<const T *>(blk->q[0]), idx, qc, v) : T(0);
   }
   if (!rk) {
@@ -47,12 +47,19 @@ __global__ void __launch_bounds__(256) k_finish(const BlockDev *__restrict__ blk
   const RkStage<T> update(stage, T(*dtp));
   T *qs = static_cast<T *>(blk->q[(stage + 1) % 3]);
   bool bad = false;
+  T nv[5];
 #pragma unroll
   for (int v = 0; v < 5; ++v) {
-    const T nv = update(qk[v], qn + v, -Jc * R[v]);
-    *comp_at(qs, idx, qc, v) = nv;
-    bad |= !isfinite(nv);
+    nv[v] = update(qk[v], qn + v, -Jc * R[v]);
+    bad |= !isfinite(nv[v]);
   }
+  if (stage < 2) {
+    store4(qs + 4ULL * idx, nv);
+  } else {
+#pragma unroll
+    for (int v = 0; v < 4; ++v) *comp_at(qs, idx, qc, v) = nv[v];
+  }
+  *comp_at(qs, idx, qc, 4) = nv[4];
   if (bad) atomicOr(blk->status, ST_NONFINITE);
 }
 

@@ -241,6 +241,11 @@ __device__ __forceinline__ T *comp_at(T *base, unsigned off, unsigned stride, un
                                (unsigned long long)stride * (v * (unsigned)sizeof(T)));
 }
 
+// index of component v of cell `idx` in the state of an RK stage (BlockDev::q) of n cells
+__device__ __forceinline__ unsigned long long state_at(int stage, unsigned long long idx, unsigned long long n, int v) {
+  return stage && v < 4 ? 4 * idx + v : v * n + idx;
+}
+
 // Slip-wall reflection of a ghost value (the mirror cell's state Q) about the boundary
 // face metric fm: m - 2 (m.k) k/|k|^2.
 template <typename T>
@@ -548,26 +553,34 @@ fp_sweep(const BlockDev *__restrict__ blocks, const SweepItem *__restrict__ item
     // with t1 reversed, wall outside the cut width), 5 another block of the batch (its cells
     // next to its opposite side, same transverse indices, same RK stage), 6 the caller's halo
     // buffer of that side (the cells another process holds, refreshed for every RK stage).
-    auto bc_source = [&](int x, int t1, int t2, const T *&src, unsigned &cs, bool &far,
+    // The caller's state and halos hold each component by itself; the stage states (stage > 0) four
+    // components side by side and the fifth behind them.  So component v < 4 of a source is at
+    // src + v cs, cs = 1 for a stage state, and the fifth at src4.
+    auto cell_of = [&](const T *base, unsigned n, unsigned o, const T *&src, const T *&src4, unsigned &cs) {
+      src = base + (stage ? 4ULL * o : (unsigned long long)o);
+      cs = stage ? 1u : n;
+      src4 = comp_at(base, o, n, 4);
+    };
+    auto bc_source = [&](int x, int t1, int t2, const T *&src, const T *&src4, unsigned &cs, bool &far,
                          bool &wall FPK_CHK_ONLY(, const T *&sb, long long &sn)) {
-      src = qin + qoff(x, t1, t2);
-      cs = qc; far = false; wall = false;
+      cell_of(qin, qc, qoff(x, t1, t2), src, src4, cs);
+      far = false; wall = false;
       FPK_CHK_ONLY(sb = qin; sn = 5LL * qc;)
       if ((unsigned)x >= (unsigned)nd) {
         const int hi = x >= 0, bc = hi ? D->bchi : D->bclo;
         if (bc == 1) {
           far = true;
         } else if (BND && bc == 6) {   // halo buffer: index x + G below the line, x - nd above it
-          src = static_cast<const T *>(D->halo[hi]) +
-                ((unsigned)t1 * D->hT1 + (unsigned)t2 * D->hT2 + (unsigned)(hi ? x - nd : x + G) * D->hsd);
+          const unsigned o = (unsigned)t1 * D->hT1 + (unsigned)t2 * D->hT2 + (unsigned)(hi ? x - nd : x + G) * D->hsd;
+          src = static_cast<const T *>(D->halo[hi]) + o;
           cs = D->hc;
+          src4 = comp_at(src, 0, cs, 4);
           FPK_CHK_ONLY(sb = static_cast<const T *>(D->halo[hi]); sn = 5LL * D->hc;)
         } else if (BND && bc == 5) {
           const BlockDev *NB = blocks + D->nbr[hi];
           const DirDev *ND = &NB->dir[item.dir];
-          src = static_cast<const T *>(NB->q[stage]) +
-                ((unsigned)t1 * ND->qT1 + (unsigned)t2 * ND->qT2 + (unsigned)(hi ? x - nd : ND->nd + x) * ND->qsd);
-          cs = NB->qc;
+          cell_of(static_cast<const T *>(NB->q[stage]), NB->qc,
+                  (unsigned)t1 * ND->qT1 + (unsigned)t2 * ND->qT2 + (unsigned)(hi ? x - nd : ND->nd + x) * ND->qsd, src, src4, cs);
           FPK_CHK_ONLY(sb = static_cast<const T *>(NB->q[stage]); sn = 5LL * NB->qc;)
         } else {
           int xx, s1 = t1;
@@ -582,7 +595,7 @@ fp_sweep(const BlockDev *__restrict__ blocks, const SweepItem *__restrict__ item
             if (bc == 4 && (t1 < cw || t1 >= nt1 - cw)) s1 = nt1 - 1 - t1;
             else wall = true;
           }
-          src = qin + qoff(xx, s1, t2);
+          cell_of(qin, qc, qoff(xx, s1, t2), src, src4, cs);
         }
       }
     };
@@ -600,17 +613,18 @@ fp_sweep(const BlockDev *__restrict__ blocks, const SweepItem *__restrict__ item
         load4(FPK_IN(kj + 4ULL * moff(x, t1, t2), kj, 4LL * B->mc - 3, B->status), kv);
         k[0] = kv[0]; k[1] = kv[1]; k[2] = kv[2];
         invJ = kv[3];
-        const T *qp;
+        const T *qp, *q4;
         unsigned cs;
         bool far, wall;
         FPK_CHK_ONLY(const T *sb; long long sn;)
-        bc_source(x, t1, t2, qp, cs, far, wall FPK_CHK_ONLY(, sb, sn));
+        bc_source(x, t1, t2, qp, q4, cs, far, wall FPK_CHK_ONLY(, sb, sn));
         if (far) {
 #pragma unroll
           for (int v = 0; v < 5; ++v) Q[v] = cst[v];
         } else {
 #pragma unroll
-          for (int v = 0; v < 5; ++v) Q[v] = __ldg(FPK_IN(comp_at(qp, 0, cs, v), sb, sn, B->status));
+          for (int v = 0; v < 4; ++v) Q[v] = *FPK_IN(comp_at(qp, 0, cs, v), sb, sn, B->status);
+          Q[4] = *FPK_IN(q4, sb, sn, B->status);
           if (BND && wall) reflect(x, t1, t2, Q);
         }
       } else {   // before the first line of the item: no face of a line uses it
@@ -651,21 +665,26 @@ fp_sweep(const BlockDev *__restrict__ blocks, const SweepItem *__restrict__ item
     };
     // asynchronous copy of one cell's loads (-G <= x < nd + G) into this thread's staging slots
     auto prefetch_cell = [&](int x, int t1, int t2) {
-      T *dst = nsb + tid;
+      T *const dst = nsb + 4 * tid, *const dst4 = nsb + 4 * kThreads + tid;
       const T *const kj = static_cast<const T *>(D->kj);
       cp_async_4el(nsb + 5 * kThreads + 4 * tid, FPK_IN(kj + 4ULL * moff(x, t1, t2), kj, 4LL * B->mc - 3, B->status));
-      const T *qp;
+      const T *qp, *q4;
       unsigned cs;
       bool far, wall;
       FPK_CHK_ONLY(const T *sb; long long sn;)
-      bc_source(x, t1, t2, qp, cs, far, wall FPK_CHK_ONLY(, sb, sn));
+      bc_source(x, t1, t2, qp, q4, cs, far, wall FPK_CHK_ONLY(, sb, sn));
       if (far) {
 #pragma unroll
-        for (int v = 0; v < 5; ++v) dst[v * kThreads] = cst[v];
+        for (int v = 0; v < 4; ++v) dst[v] = cst[v];
+        *dst4 = cst[4];
       } else {   // a wall ghost copies its mirror cell; the reflection is applied when staged
+        if (BND ? cs == 1 : stage != 0) {
+          cp_async_4el(dst, FPK_IN(qp, sb, sn - 3, B->status));
+        } else {
 #pragma unroll
-        for (int v = 0; v < 5; ++v)
-          cp_async_el(dst + v * kThreads, FPK_IN(comp_at(qp, 0, cs, v), sb, sn, B->status));
+          for (int v = 0; v < 4; ++v) cp_async_el(dst + v, FPK_IN(comp_at(qp, 0, cs, v), sb, sn, B->status));
+        }
+        cp_async_el(dst4, FPK_IN(q4, sb, sn, B->status));
       }
     };
     // asynchronous copy of the epilogue operands of a cell (state offset qo: residual
@@ -1217,12 +1236,19 @@ fp_sweep(const BlockDev *__restrict__ blocks, const SweepItem *__restrict__ item
             T *const qs = static_cast<T *>(B->q[(stage + 1) % 3]);
             const RkStage<T> rk(stage, s_dt);
             bool bad = false;
+            T nv[5];
 #pragma unroll
             for (int v = 0; v < 5; ++v) {
-              const T nv = rk(Qi[v], epb + (5 + v) * kThreads + tid, -Jc * R[v]);
-              *FPK_IN(comp_at(qs, qo, qc, v), qs, 5LL * qc, B->status) = nv;
-              bad |= !isfinite(nv);
+              nv[v] = rk(Qi[v], epb + (5 + v) * kThreads + tid, -Jc * R[v]);
+              bad |= !isfinite(nv[v]);
             }
+            if (stage < 2) {
+              store4(FPK_IN(qs + 4ULL * qo, qs, 4LL * qc - 3, B->status), nv);
+            } else {
+#pragma unroll
+              for (int v = 0; v < 4; ++v) *FPK_IN(comp_at(qs, qo, qc, v), qs, 5LL * qc, B->status) = nv[v];
+            }
+            *FPK_IN(comp_at(qs, qo, qc, 4), qs, 5LL * qc, B->status) = nv[4];
             if (bad) atomicOr(B->status, ST_NONFINITE);
           }
         }
@@ -1230,8 +1256,9 @@ fp_sweep(const BlockDev *__restrict__ blocks, const SweepItem *__restrict__ item
       if (!kEarly) __syncthreads();
       // ---- stage the next chunk's new cell from this thread's staging slots
       if (staged) {
-        const T *src = nsb + tid;
-        T Q[5] = {src[0], src[kThreads], src[2 * kThreads], src[3 * kThreads], src[4 * kThreads]};
+        T Q[5];
+        load4(nsb + 4 * tid, Q);
+        Q[4] = nsb[4 * kThreads + tid];
         T kv[4];
         load4(nsb + 5 * kThreads + 4 * tid, kv);
         if (BND) {                                   // a slip-wall ghost?
@@ -1239,11 +1266,11 @@ fp_sweep(const BlockDev *__restrict__ blocks, const SweepItem *__restrict__ item
           wrap(uc, c1, c2);
           const int xs = uc - G;
           if (xs < 0 ? D->bclo >= 3 : xs >= nd && D->bchi >= 3) {
-            const T *qp;
+            const T *qp, *q4;
             unsigned cs;
             bool far, wall;
             FPK_CHK_ONLY(const T *sb; long long sn;)
-            bc_source(xs, c1, c2, qp, cs, far, wall FPK_CHK_ONLY(, sb, sn));
+            bc_source(xs, c1, c2, qp, q4, cs, far, wall FPK_CHK_ONLY(, sb, sn));
             if (wall) reflect(xs, c1, c2, Q);
           }
         }

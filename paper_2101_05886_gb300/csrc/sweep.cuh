@@ -50,11 +50,11 @@ template <> struct Num<double> {
     const double e = fma(-x, y, 1.0);
     return fma(y, fma(e, e, e), y);
   }
-  // max(m, |x|), m >= 0: doubles without sign are ordered like their bits, and integer compares
-  // leave the FP64 pipe alone
+  // max(m, |x|), m >= 0, a NaN ignored as by fmax: doubles without sign are ordered like their
+  // bits, and integer compares leave the FP64 pipe alone
   static __device__ __forceinline__ double amax(double m, double x) {
     const long long a = __double_as_longlong(m), b = __double_as_longlong(fabs(x));
-    return __longlong_as_double(a > b ? a : b);
+    return __longlong_as_double(b > a && b <= 0x7ff0000000000000LL ? b : a);
   }
   static __device__ __forceinline__ double fma_(double a, double b, double c) { return fma(a, b, c); }
   static __device__ __forceinline__ double sqrt_(double x) { return sqrt(x); }

@@ -47,3 +47,24 @@ def test_streams_over_many_lines_match_the_oracle(kind, n, scheme, precision):
     assert np.isfinite(dq).all() and max(errs) <= tol, errs
     assert blk.status() == B.FP_OK
     blk.close()
+
+
+def test_a_cell_without_pressure_has_no_acoustic_speed():
+    """A cell whose pressure is negative has no sound speed (NaN): like the oracle, the sweep leaves
+    it out of the local Lax-Friedrichs maxima, and its faces stay finite where their Roe state
+    is.  The pattern of finite values is the oracle's; the finite ones agree to 1e-10 of the
+    largest (about 1e-13 of rounding, and residual terms up to 1e2 times their sum)."""
+    Gn = O.node_ghost(6)
+    g = I.periodic_wavy_3d((16, 14, 12), amp=0.05, Gn=Gn)
+    qinf = I.uniform_qinf(0.8, 10.0)
+    q = I.random_smooth_state(g, qinf, amp=0.02, seed=3)
+    ke = 0.5 * (q[1:4, 5, 6, 7] ** 2).sum() / q[0, 5, 6, 7]
+    q[4, 5, 6, 7] = 0.9 * ke                             # p < 0 there only
+    blk = Block(g, metric_order=6, scheme=1, precision=F64, q_inf=qinf)
+    dq = blk.rhs(blk.to_device(q)).cpu().numpy()
+    cfg = O.cfg_for(g, M=6, scheme=1, qinf=qinf)
+    _, ref = O.rhs(cfg, O.metrics(cfg, g.nodes, g.Gn), q)
+    fine = np.isfinite(ref)
+    assert fine.any() and (np.isfinite(dq) == fine).all()
+    assert np.abs(dq[fine] - ref[fine]).max() <= 1e-10 * np.abs(ref[fine]).max()
+    blk.close()

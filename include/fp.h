@@ -239,8 +239,8 @@ int fp_get_cta_sizes(const fp_ctx *ctx, int *primary, int *alternative);
    the device holds resident CTAs (small blocks); lines = the primary CTA size / faces.
    Results do not depend on it. */
 int fp_get_tile(const fp_ctx *ctx, int dir, int *faces, int *lines);
-/* Override the tile shape: faces in {8,16,32}, faces x lines one of fp_get_cta_sizes; a size
-   whose xi rings are unpadded takes 32 faces along xi only (FP_ERR_ARG otherwise). */
+/* Override the tile shape: faces in {8,16,32}, faces x lines one of fp_get_cta_sizes; the
+   64-thread size takes 32 faces along xi only (FP_ERR_ARG otherwise). */
 int fp_set_tile(fp_ctx *ctx, int dir, int faces, int lines);
 
 const char *fp_last_error(const fp_ctx *ctx);

@@ -47,10 +47,10 @@ struct fp_ctx {
   int nscta = 0;
   int nsm = 152;
   // CTA shapes of the context's sweep: [0] the primary one, [1] the alternative (nshape == 2,
-  // the folded FP32 sweeps): threads (faces per chunk x lines per tile), xi rings padded (every
-  // tile shape conflict-free) or not (S = 32 only), resident CTAs per SM
+  // the folded FP32 sweeps): threads (faces per chunk x lines per tile), whether fp_set_tile takes
+  // other than 32 faces along xi (not for the 64-thread shape), resident CTAs per SM
   int nshape = 1;
-  int nt[2] = {128, 128}, pad[2] = {1, 1}, per_sm[2] = {1, 1};
+  int nt[2] = {128, 128}, anyS[2] = {1, 1}, per_sm[2] = {1, 1};
   int dev = 0;                        // the device the context's memory lives on
   double dt_host = 0.0;
   std::string err;
@@ -77,7 +77,7 @@ struct fp_batch {
   fpk::SweepItem *bitems[kMaxBranch][3] = {};
   int bncta[kMaxBranch][3] = {};
   int nsm = 152;
-  int nshape = 1, nt[2] = {128, 128}, pad[2] = {1, 1}, per_sm[2] = {1, 1};   // as fp_ctx (shared by all blocks)
+  int nshape = 1, nt[2] = {128, 128}, anyS[2] = {1, 1}, per_sm[2] = {1, 1};   // as fp_ctx (shared by all blocks)
   int shape = 0;                     // the one CTA shape the batch runs (sweep_batch_shape)
   int2 *lam_items = nullptr;
   int nlam_items = 0;
@@ -220,10 +220,10 @@ void set_shapes(C *c, int is_f32, int M, int scheme, int fix) {
   for (int a = 0; a < c->nshape; ++a) {
     const int f = fix + a;   // fix = 2: the alternative shape
     c->nt[a] = fpk::sweep_threads(is_f32, scheme, f);
-    c->pad[a] = c->nt[a] != 64;
+    c->anyS[a] = c->nt[a] != 64;
     c->per_sm[a] = prepare(is_f32, M, scheme, f);
   }
-  if (c->nshape == 1) { c->nt[1] = c->nt[0]; c->pad[1] = c->pad[0]; c->per_sm[1] = c->per_sm[0]; }
+  if (c->nshape == 1) { c->nt[1] = c->nt[0]; c->anyS[1] = c->anyS[0]; c->per_sm[1] = c->per_sm[0]; }
 }
 
 // the shape (0 primary, 1 alternative) of a direction's tile
@@ -415,13 +415,25 @@ void spread_stream(const Stream &s, long long first, long long most, std::vector
 //    CTAs that run at the same time take adjacent tiles: whole rounds go in turn, CTA c the
 //    tiles c, c + g, ... (equal pieces of the stream instead read 3 times the bytes and cost 6 %
 //    on a 256^3 block), and what is left after the rounds is spread in equal pieces.
-//  - `alone`, no other launch runs at the same time (one block, or a batch of one chain): two rounds per CTA, so there are more CTAs than slots and those that
-//    run on faster SMs take more of them (256^3 WENO5 step: 8.93 ms, 9.75 ms with all rounds in one
-//    item, 9.97 ms with a CTA per tile in a fixed order and lines padded to chunks).  The blocks of a
-//    batch keep one item for all rounds: its graph's other branches fill the SMs that end
-//    early (64-block WENO5 step: 18.04 ms, 18.25 ms with two rounds per item).
+//  - `alone`, no other launch runs at the same time (one block, or a batch of one chain): two
+//    rounds per CTA, so there are more CTAs than slots and those that run on faster SMs take more
+//    of them (256^3 WENO5 step, when introduced: 8.93 ms, 9.75 ms with all rounds in one item,
+//    9.97 ms with a CTA per tile in a fixed order and lines padded to chunks).  The blocks of a batch
+//    with several chains keep one item for all rounds: its graph's other branches fill the SMs
+//    that end early (64-block WENO5 step: 18.04 ms, 18.25 ms with two rounds per item).
 int make_items(const std::vector<Stream> &streams, int slots, bool alone, std::vector<fpk::SweepItem> &items) {
-  std::vector<std::vector<fpk::SweepItem>> cta(slots);
+  std::vector<fpk::SweepItem> list, piece;        // in the order made, `next` within the list
+  std::vector<int> head(slots, -1), tail(slots, -1);   // of each CTA
+  auto add = [&](long long cta, const fpk::SweepItem &it) {
+    const int k = (int)list.size();
+    list.push_back(it);
+    if (cta < 0) {                                // a CTA of its own
+      head.push_back(k);
+      return;
+    }
+    if (head[cta] < 0) head[cta] = k; else list[tail[cta]].next = k;
+    tail[cta] = k;
+  };
   long long total = 0, done = 0;
   for (const Stream &s : streams) total += s.chunks();
   for (const Stream &s : streams) {
@@ -431,34 +443,31 @@ int make_items(const std::vector<Stream> &streams, int slots, bool alone, std::v
     done += s.chunks();
     const long long g = std::max(1LL, done * slots / total - c0);
     const long long r = s.dir == 0 ? 0 : s.tiles / g;
-    std::vector<fpk::SweepItem> piece;
-    if (r * g < s.tiles) spread_stream(s, r * g, g, piece);
     const long long per = alone ? 2 : r;          // rounds per item
+    const bool own = alone && r > per;            // more CTAs than slots
     for (long long r0 = 0; r0 < r; r0 += per) {
       const long long n = std::min(per, r - r0);
-      for (long long c = 0; c < g; ++c) {
-        const fpk::SweepItem it = {s.block, (int)(r0 * g + c), (int)g, s.G, (int)s.positions(n), -1, s.dir, 0};
-        if (alone && r > per) cta.push_back({it}); else cta[c0 + c].push_back(it);
-      }
+      for (long long c = 0; c < g; ++c)
+        add(own ? -1 : c0 + c, {s.block, (int)(r0 * g + c), (int)g, s.G, (int)s.positions(n), -1, s.dir, 0});
     }
-    for (size_t c = 0; c < piece.size(); ++c)
-      if (alone && r > per) cta.push_back({piece[c]}); else cta[c0 + c].push_back(piece[c]);
+    piece.clear();
+    if (r * g < s.tiles) spread_stream(s, r * g, g, piece);
+    for (size_t c = 0; c < piece.size(); ++c) add(own ? -1 : c0 + (long long)c, piece[c]);
   }
   // CTA c's first item at index c, the others behind
-  items.clear();
-  for (const auto &c : cta)
-    if (!c.empty()) items.push_back(c[0]);
+  std::vector<int> place(list.size(), -1);
   int n = 0;
-  for (const auto &c : cta) {
-    if (c.empty()) continue;
-    int prev = n++;
-    for (size_t i = 1; i < c.size(); ++i) {
-      items[prev].next = (int)items.size();
-      prev = items[prev].next;
-      items.push_back(c[i]);
-    }
+  for (int h : head)
+    if (h >= 0) place[h] = n++;
+  const int ncta = n;
+  for (int &p : place)
+    if (p < 0) p = n++;
+  items.resize(list.size());
+  for (size_t k = 0; k < list.size(); ++k) {
+    items[place[k]] = list[k];
+    if (list[k].next >= 0) items[place[k]].next = place[list[k].next];
   }
-  return n;
+  return ncta;
 }
 
 // the launch's items on the device (replaces *dst)
@@ -659,24 +668,18 @@ int fp_init_grid(const fp_grid_desc *desc, const double *xyz, int ghost_nodes, v
   for (int d = 0; d < 3; ++d) { J.n[d] = n[d]; J.fmet[d] = fm64[d]; }
   J.nodes = nodes; J.met = met64; J.scratch = scratch;
   FP_TRY(fpk::build_metrics(J, s), "build metrics");
-  // the FP64 arrays are released as soon as they are packed: the sweep's take their place
+  // the scratch and the nodes make room for the packed arrays
   FP_TRY(cudaStreamSynchronize(s), "metric construction");
   cudaFree(nodes); cudaFree(scratch);
   nodes = scratch = nullptr;
   for (int d = 0; d < dims; ++d) {
     FP_TRY(fpk::dev_alloc(&c->kj[d], (size_t)4 * c->nmet * c->esize), "cudaMalloc(metrics)");
     FP_TRY(fpk::pack_metrics(J, d, c->is_f32, c->kj[d], s), "pack metrics");
-  }
-  FP_TRY(cudaStreamSynchronize(s), "metric packing");
-  cudaFree(met64);
-  met64 = nullptr;
-  for (int d = 0; d < dims; ++d) {
     FP_TRY(fpk::dev_alloc(&c->fk[d], (size_t)6 * c->nface[d] * c->esize), "cudaMalloc(face metrics)");
     FP_TRY(fpk::pack_faces(J, d, c->is_f32, c->fk[d], s), "pack face metrics");
-    FP_TRY(cudaStreamSynchronize(s), "metric packing");
-    cudaFree(fm64[d]);
-    fm64[d] = nullptr;
   }
+  FP_TRY(cudaStreamSynchronize(s), "metric packing");
+  cleanup_tmp();
   const size_t sbytes = (size_t)5 * c->ncells * c->esize;
   FP_TRY(fpk::dev_alloc(&c->q1, sbytes), "cudaMalloc(stage 1)");
   FP_TRY(fpk::dev_alloc(&c->q2, sbytes), "cudaMalloc(stage 2)");
@@ -969,8 +972,8 @@ int fp_set_tile(fp_ctx *c, int dir, int faces, int lines) {
   if (!(faces == 8 || faces == 16 || faces == 32) || faces * lines != c->nt[a])
     return fail(c, FP_ERR_ARG, "fp_set_tile: faces in {8,16,32} and faces*lines one of the sweep's CTA sizes "
                                "(fp_get_cta_sizes)");
-  if (dir == 0 && !c->pad[a] && faces != 32)
-    return fail(c, FP_ERR_ARG, "fp_set_tile: this CTA size's xi rings are unpadded: 32 faces per chunk only");
+  if (dir == 0 && !c->anyS[a] && faces != 32)
+    return fail(c, FP_ERR_ARG, "fp_set_tile: this CTA size takes 32 faces per chunk along xi only");
   c->hblk.dir[dir].S = faces;
   c->hblk.dir[dir].TT = lines;
   return upload_items(c);
@@ -1082,7 +1085,7 @@ static int batch_autotune(fp_batch *b, cudaStream_t s, std::vector<int> tiles[2]
         float best = 1e30f;
         int bestS = 32;
         for (int S : {32, 16, 8}) {
-          if (d == 0 && !b->pad[a] && S != 32) continue;   // unpadded xi rings: S = 32 only
+          if (d == 0 && !b->anyS[a] && S != 32) continue;   // as fp_set_tile
           for (int k : members[cl]) { b->hblk[k].dir[d].S = S; b->hblk[k].dir[d].TT = b->nt[a] / S; }
           st = batch_upload(b, s);
           if (!st) st = batch_items(b, d, &members[cl]);
@@ -1163,7 +1166,7 @@ int fp_batch_create_linked(fp_ctx *const *blocks, int nblocks, void *const *q_de
   b->nshape = blocks[0]->nshape;
   for (int a = 0; a < 2; ++a) {
     b->nt[a] = blocks[0]->nt[a];
-    b->pad[a] = blocks[0]->pad[a];
+    b->anyS[a] = blocks[0]->anyS[a];
     b->per_sm[a] = blocks[0]->per_sm[a];
   }
   b->shape = fpk::sweep_batch_shape(b->is_f32, b->scheme, fix_of(b->scheme, b->charwise, b->fp, b->global_lf));

@@ -17,20 +17,17 @@ constexpr int kEpiFields = 10;       // epilogue operands staged per thread (acc
 // lines per tile, whether the rings of the xi pass are padded (none is: turning the slots of
 // every other group of lines keeps all tile shapes free of bank conflicts), and the CTAs one SM
 // holds.
-// Small CTAs pay: the warps of a CTA meet at two barriers per chunk, so with fewer warps per
-// CTA the phases of the chunk (staging, FMA-heavy faces, epilogue) of different CTAs overlap
-// instead of running in step.  Large ones pay where the eta and zeta passes coalesce across
-// more lines (TT): a 256^3 block runs linear upwind 12 % faster at 128 threads (TT = 16) than
-// at 64 (TT = 8), a batch of blocks up to 128^3 12 % slower.  So the folded FP32 sweeps have
-// two shapes, and a batch runs the one sweep_batch_shape names:
+// The warps of a CTA meet at two or three barriers per chunk, so with fewer warps per CTA the phases
+// of the chunk (staging, FMA-heavy faces, epilogue) of different CTAs overlap instead of running
+// in step; large CTAs read wider rows in the eta and zeta passes (TT = 16 lines instead of 8).  The
+// folded FP32 sweeps have both, and a batch runs the one sweep_batch_shape names:
 //   WENO5-JS:       64 threads, 8 CTAs per SM             |  alternative 128, 4
 //   linear upwind: 128 threads, 4                         |  alternative  64, 8
 //   WENO7-JS:      128 threads, 2 (255 registers)         |  alternative  64, 4
 // Every other sweep: 128 threads, 4 CTAs (FP32) or 2 (FP64, and WENO7).
-// Single blocks run the primary shape; batches the shape sweep_batch_shape names, which was
-// the faster one on the 64-block workload (its step graph runs two branches side by side, and
-// kernels of two shapes there would not share SMs, so a batch runs one shape throughout):
-// linear upwind the alternative (64 threads: +12 %), the others the primary.
+// Measured, 64 | 128 threads, default tiles: WENO5 256^3 7.81 | 7.86 ms, 64-block batch 16.28 | 16.35;
+// linear upwind 256^3 5.45 | 5.46, 20-block batch 2.29 | 2.32; WENO7 256^3 11.44 | 11.54, batch 4.86 |
+// 4.85.  A batch runs one shape throughout (kernels of two shapes in its graph would not share SMs).
 __host__ __device__ constexpr bool sweep_has_alt(bool f32, int scheme, int fix) {
   return f32 && (fix == 1 || fix == 2) && scheme >= 0 && scheme <= 2;
 }

@@ -3,7 +3,7 @@
 // pipe's groups and the batch graph's branches use (fp_balanced_groups).
 //
 // The blocks are split into groups of about equal size.  Each group is a batch
-// (fp_batch_create: one persistent launch per direction pass, the three RK stages in
+// (fp_batch_create: one launch per direction pass, the three RK stages in
 // one CUDA graph) with its own device state buffers and its own stream.  A step issues,
 // group by group on the group's stream, the copies of the group's states to the device,
 // the group's graph and the copies back.  The copy engines then move one group's states

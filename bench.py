@@ -53,14 +53,14 @@ BYTES_PER_CELL_STAGE_F64 = 2 * BYTES_PER_CELL_STAGE_F32
 # differences 270, central and dissipation sums 120, eigensystem 140, one projection and
 # back-projection 60, reference state and speeds 110).
 ALG_FLOPS_PER_POINT_PASS = {"weno5_char": 2000.0, "lu5_char": 700.0}
-# FP32 operations the kernels execute per point and pass, counted by ncu on the 16-block
-# subset (FFMA 2, FFMA2 4, FADD/FMUL 1, FADD2/FMUL2 2): reported beside the algorithmic count.
-EXEC_FLOPS_PER_POINT_PASS = {"weno5_char": 2145.0, "lu5_char": 1132.0}
-# DRAM bytes per point per direction pass measured by ncu (16-block capture, mean over an RK
-# step: 96.4 B), scaled to a pass over the workload.  The linear-upwind sweep makes the same
-# loads and stores (78.0 / 99.4 / 100.8 B per point in its captured passes against 77.9 /
-# 99.8 / 101.1 B for WENO5).
-TRAFFIC_BYTES_PER_POINT_PASS = {"weno5_char": 96.4, "lu5_char": 96.4}
+# FP32 operations the kernels execute per point and pass (idle faces between lines included),
+# counted by ncu on an 8-block subset (FFMA 2, FFMA2 4, FADD/FMUL 1, FADD2/FMUL2 2): reported
+# beside the algorithmic count.
+EXEC_FLOPS_PER_POINT_PASS = {"weno5_char": 2140.0, "lu5_char": 1090.0}
+# DRAM bytes per point per direction pass measured by ncu (8-block capture, first stage, mean of
+# the xi, eta and zeta passes: 74, 96 and 100 B), scaled to a pass over the workload.  The
+# linear-upwind sweep makes the same loads and stores.
+TRAFFIC_BYTES_PER_POINT_PASS = {"weno5_char": 90.0, "lu5_char": 90.0}
 ORACLE_SAMPLE_N = 32           # side of the O-grid block each host core advances (both CPU arms)
 
 

@@ -246,15 +246,25 @@ __device__ __forceinline__ unsigned long long state_at(int stage, unsigned long 
   return stage && v < 4 ? 4 * idx + v : v * n + idx;
 }
 
+// a . b with its fused operations spelled out.  Where a cell is staged (at the start of a work item or
+// within one) depends on the layout of the launch, each place is compiled by itself, and a sum of
+// two products leaves the compiler the choice of the one that it fuses: linear upwind's results
+// differed in the last bit from one layout to another.  So whatever is computed in several places
+// (stage_cell, wall_reflect) names its fused operations.
+template <typename T>
+__device__ __forceinline__ T dot3(T a0, T a1, T a2, T b0, T b1, T b2) {
+  return Num<T>::fma_(a2, b2, Num<T>::fma_(a1, b1, a0 * b0));
+}
+
 // Slip-wall reflection of a ghost value (the mirror cell's state Q) about the boundary
 // face metric fm: m - 2 (m.k) k/|k|^2.
 template <typename T>
 __device__ __forceinline__ void wall_reflect(T Q[5], const T *fm) {
   const T n0 = fm[0], n1 = fm[1], n2 = fm[2];
-  const T s = T(2) * (Q[1] * n0 + Q[2] * n1 + Q[3] * n2) / (n0 * n0 + n1 * n1 + n2 * n2);
-  Q[1] -= s * n0;
-  Q[2] -= s * n1;
-  Q[3] -= s * n2;
+  const T s = T(-2) * dot3<T>(Q[1], Q[2], Q[3], n0, n1, n2) / dot3<T>(n0, n1, n2, n0, n1, n2);
+  Q[1] = Num<T>::fma_(s, n0, Q[1]);
+  Q[2] = Num<T>::fma_(s, n1, Q[2]);
+  Q[3] = Num<T>::fma_(s, n2, Q[3]);
 }
 
 // Asynchronous global -> shared copies of single elements (sm_80+ cp.async).
@@ -638,7 +648,8 @@ fp_sweep(const BlockDev *__restrict__ blocks, const SweepItem *__restrict__ item
     auto stage_cell = [&](int x, const T Q[5], const T k[3], T invJ) {
       const T rinv = Num<T>::rcp(Q[0]);
       const T u0 = Q[1] * rinv, u1 = Q[2] * rinv, u2 = Q[3] * rinv;
-      const T p = g1 * (Q[4] - T(0.5) * (Q[1] * u0 + Q[2] * u1 + Q[3] * u2));
+      const T e = Num<T>::fma_(T(-0.5), dot3<T>(Q[1], Q[2], Q[3], u0, u1, u2), Q[4]);
+      const T p = g1 * e;
       const T Jc = Num<T>::rcp(invJ);
       T *cp = sm + off(x);
 #pragma unroll
@@ -648,10 +659,10 @@ fp_sweep(const BlockDev *__restrict__ blocks, const SweepItem *__restrict__ item
       cp[(CF_K + 2) * kRing] = k[2];
       cp[CF_INVJ * kRing] = invJ;
       cp[CF_RINV * kRing] = rinv;
-      cp[CF_H * kRing] = (Q[4] + p) * rinv;
+      cp[CF_H * kRing] = Num<T>::fma_(g1, e, Q[4]) * rinv;
       cp[CF_SQR * kRing] = Num<T>::sqrt_(Q[0]);
-      cp[CF_UC * kRing] = Jc * (u0 * k[0] + u1 * k[1] + u2 * k[2]);
-      cp[CF_AC * kRing] = fabs(Jc) * Num<T>::sqrt_(gam * p * rinv * (k[0] * k[0] + k[1] * k[1] + k[2] * k[2]));
+      cp[CF_UC * kRing] = Jc * dot3<T>(u0, u1, u2, k[0], k[1], k[2]);
+      cp[CF_AC * kRing] = fabs(Jc) * Num<T>::sqrt_(gam * p * rinv * dot3<T>(k[0], k[1], k[2], k[0], k[1], k[2]));
     };
 
     // asynchronous copy of the metrics of face x + 1/2 of line (t1, t2), and of the change of the face

@@ -1,0 +1,77 @@
+"""Units far from 1: the sweep's intermediate products stay in range wherever its inputs do.
+
+Scaling by powers of two is exact, so a problem in other units has the same significands, and the
+residuals are compared bit for bit after scaling back."""
+import dataclasses
+
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+
+import oracle as O
+from paper_2101_05886_gb300 import inputs as I
+from tests.helpers import f32, rhs_err, ulp_sensitivity
+
+pytestmark = pytest.mark.gpu
+
+if not torch.cuda.is_available():
+    pytest.skip("CUDA device required", allow_module_level=True)
+
+from paper_2101_05886_gb300 import binding as B  # noqa: E402
+from paper_2101_05886_gb300.solver import Block  # noqa: E402
+
+N = (22, 14, 11)
+
+
+def _case(precision, seed):
+    g = I.periodic_wavy_3d(N, amp=0.05, Gn=O.node_ghost(6))
+    qinf = I.uniform_qinf(0.8, 10.0)
+    q = I.random_smooth_state(g, qinf, amp=0.05, seed=seed)
+    return (g, f32(qinf), f32(q)) if precision == B.FP_F32_MIXED else (g, np.asarray(qinf), q)
+
+
+def _rhs(g, q, qinf, **kw):
+    blk = Block(g, metric_order=6, q_inf=tuple(qinf), **kw)
+    dq = blk.rhs(blk.to_device(q)).cpu().numpy()
+    assert blk.status() == B.FP_OK
+    blk.close()
+    return dq
+
+
+@pytest.mark.parametrize("characteristic,global_lf", [(1, 0), (0, 0), (1, 1)])
+def test_fp32_linear_upwind_in_large_units(characteristic, global_lf):
+    """Lengths in units of 2^-27 and speeds in units of 2^-17 (metres and metres per second on a
+    planet-sized grid): |k| is about 2^53 and the sound speed about 2^17, so |k|^2, 1/J and all
+    fluxes are FP32 numbers but c^2 |k|^2, about 2^140, is not.  Linear upwind and its speeds have
+    no constant with a unit, so the residual has the bits of the problem in units of 1."""
+    g, qinf, q = _case(B.FP_F32_MIXED, 7)
+    big = dataclasses.replace(g, nodes=g.nodes * 2.0 ** 27)
+    unit = 2.0 ** np.array([0, 17, 17, 17, 34])
+    kw = dict(scheme=B.FP_LINEAR_UPWIND5, precision=B.FP_F32_MIXED, characteristic=characteristic, global_lf=global_lf)
+    want = _rhs(g, q, qinf, **kw)
+    got = _rhs(big, q * unit[:, None, None, None], qinf * unit, **kw)
+    assert np.isfinite(want).all() and np.abs(want).max() > 1e-3
+    assert np.array_equal(got / (unit * 2.0 ** -10)[:, None, None, None], want)
+
+
+@pytest.mark.parametrize("characteristic", [1, 0])
+@pytest.mark.parametrize("power", [130, 240])
+def test_fp64_weno5_of_large_states(power, characteristic):
+    """The Euler fluxes and the WENO5 weights (where the constant 1e-6 is negligible) do not depend
+    on the unit of the conserved variables: a state times 2^130 or 2^240, whose squared indicators
+    (2^500, 2^940) are FP64 numbers though their products are not, has the residual of the state
+    times 2^100, and the oracle's."""
+    g, qinf, q = _case(B.FP_F64, 8)
+    kw = dict(scheme=B.FP_WENO5_JS, precision=B.FP_F64, characteristic=characteristic)
+    want = _rhs(g, q * 2.0 ** 100, qinf * 2.0 ** 100, **kw)
+    got = _rhs(g, q * 2.0 ** power, qinf * 2.0 ** power, **kw)
+    assert np.isfinite(want).all() and np.abs(want).max() > 0
+    assert np.array_equal(got * 2.0 ** (100 - power), want)
+    # the oracle in the same units; its error bound is that of the parity suite
+    cfg = O.cfg_for(g, M=6, scheme=0, charwise=characteristic, qinf=qinf * 2.0 ** 130)
+    met = O.metrics(cfg, g.nodes, g.Gn)
+    q130 = q * 2.0 ** 130
+    tol = max(1e-12, 2.0 * ulp_sensitivity(cfg, met, q130))
+    assert tol <= 2e-11, tol
+    assert max(rhs_err(got * 2.0 ** (130 - power), cfg, met, q130, per_component=True)) <= tol

@@ -39,6 +39,7 @@ struct fp_ctx {
   BlockDev hblk;
   BlockDev *dblk = nullptr;
   BlockDev uploaded;                  // last BlockDev copied to dblk
+  fpk::SweepItem *item_mem = nullptr; // the items of all launches, one allocation
   fpk::SweepItem *items[3] = {nullptr, nullptr, nullptr};
   int ncta[3] = {0, 0, 0};            // CTAs of each direction's launch
   // all directions in one launch (blocks of at most kSplitPoints points): its items
@@ -508,25 +509,45 @@ int balanced_items(const fp_ctx *c, const std::vector<Stream> &streams, int most
   return make_items(streams, per_sm * c->nsm, streams.size() == 1, items);
 }
 
+// The items of the context's launches for the tiles in hblk.  All lists are made and copied before
+// any of the old ones goes, so a failure leaves the context with the lists it had.
 int upload_items(fp_ctx *c) {
-  std::vector<fpk::SweepItem> items;
-  std::vector<Stream> all;
-  auto shape = [&](int d) { return c->nshape == 2 && c->hblk.dir[d].S * c->hblk.dir[d].TT == c->nt[1] ? 1 : 0; };
-  c->split = c->ncells <= kSplitPoints;
+  std::vector<fpk::SweepItem> items, all;         // one launch's, and those of all launches in turn
+  std::vector<Stream> streams;
+  size_t first[4] = {0, 0, 0, 0};                 // of each direction, and of the launch over all of them
+  int ncta[4] = {0, 0, 0, 0};
+  int split = c->ncells <= kSplitPoints;
+  const int sh0 = shape_of(c, c->hblk.dir[0]);
+  auto add = [&](int l, const std::vector<Stream> &of, int shape) {
+    ncta[l] = balanced_items(c, of, c->per_sm[shape], items);
+    first[l] = all.size();
+    all.insert(all.end(), items.begin(), items.end());
+  };
   for (int d = 0; d < c->desc.dims; ++d) {
-    all.push_back(stream_of(c->hblk, 0, d));
-    if (shape(d) != shape(0)) c->split = 0;       // one launch has one CTA shape
-    c->ncta[d] = balanced_items(c, {all.back()}, c->per_sm[shape(d)], items);
-    cudaError_t e = put_items(items, &c->items[d]);
-    if (e != cudaSuccess) return cuda_fail(c, e, "sweep items");
+    const int sh = shape_of(c, c->hblk.dir[d]);
+    streams.push_back(stream_of(c->hblk, 0, d));
+    if (sh != sh0) split = 0;                     // one launch has one CTA shape
+    add(d, {streams.back()}, sh);
   }
-  for (int d = 0; d < c->desc.dims; ++d)          // one accumulator, or the directions' own
-    c->hblk.dir[d].racc = static_cast<char *>(c->racc) + (c->split ? d * split_stride(c) : 0);
-  if (c->split) {
-    c->nscta = balanced_items(c, all, c->per_sm[shape(0)], items);
-    cudaError_t e = put_items(items, &c->sitems);
-    if (e != cudaSuccess) return cuda_fail(c, e, "sweep items");
+  if (split) add(3, streams, sh0);
+  fpk::SweepItem *mem = nullptr;
+  cudaError_t e = fpk::dev_alloc(&mem, all.size() * sizeof(fpk::SweepItem));
+  if (e == cudaSuccess) e = cudaMemcpy(mem, all.data(), all.size() * sizeof(fpk::SweepItem), cudaMemcpyHostToDevice);
+  if (e != cudaSuccess) {
+    cudaFree(mem);
+    return cuda_fail(c, e, "sweep items");
   }
+  cudaFree(c->item_mem);
+  c->item_mem = mem;
+  for (int d = 0; d < c->desc.dims; ++d) {
+    c->items[d] = mem + first[d];
+    c->ncta[d] = ncta[d];
+    // one accumulator, or the directions' own
+    c->hblk.dir[d].racc = static_cast<char *>(c->racc) + (split ? d * split_stride(c) : 0);
+  }
+  c->split = split;
+  c->sitems = split ? mem + first[3] : nullptr;
+  c->nscta = ncta[3];
   return FP_OK;
 }
 
@@ -601,10 +622,10 @@ const char *fp_last_error(const fp_ctx *c) { return c ? c->err.c_str() : "null c
 void fp_free(fp_ctx *c) {
   if (!c) return;
   cudaDeviceSynchronize();
-  for (int d = 0; d < 3; ++d) { cudaFree(c->kj[d]); cudaFree(c->fk[d]); cudaFree(c->items[d]); }
+  for (int d = 0; d < 3; ++d) { cudaFree(c->kj[d]); cudaFree(c->fk[d]); }
   cudaFree(c->q1); cudaFree(c->q2); cudaFree(c->racc);
   cudaFree(c->status); cudaFree(c->dt_dev); cudaFree(c->cfl_bits); cudaFree(c->dblk);
-  cudaFree(c->lamg); cudaFree(c->lam_items); cudaFree(c->sitems);
+  cudaFree(c->lamg); cudaFree(c->lam_items); cudaFree(c->item_mem);
   delete c;
 }
 
@@ -974,9 +995,15 @@ int fp_set_tile(fp_ctx *c, int dir, int faces, int lines) {
                                "(fp_get_cta_sizes)");
   if (dir == 0 && !c->anyS[a] && faces != 32)
     return fail(c, FP_ERR_ARG, "fp_set_tile: this CTA size takes 32 faces per chunk along xi only");
+  const int S = c->hblk.dir[dir].S, TT = c->hblk.dir[dir].TT;
   c->hblk.dir[dir].S = faces;
   c->hblk.dir[dir].TT = lines;
-  return upload_items(c);
+  const int st = upload_items(c);
+  if (st != FP_OK) {                              // the lists are still those of the old tile
+    c->hblk.dir[dir].S = S;
+    c->hblk.dir[dir].TT = TT;
+  }
+  return st;
 }
 
 // ----------------------------------------------------------------- batches

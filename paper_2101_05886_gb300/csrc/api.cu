@@ -708,7 +708,7 @@ int fp_init_grid(const fp_grid_desc *desc, const double *xyz, int ghost_nodes, v
   FP_TRY(fpk::dev_alloc(&c->status, sizeof(int)), "cudaMalloc(status)");
   FP_TRY(cudaMemset(c->status, 0, sizeof(int)), "clear status");
   FP_TRY(fpk::dev_alloc(&c->dt_dev, sizeof(double)), "cudaMalloc(dt)");
-  FP_TRY(fpk::dev_alloc(&c->cfl_bits, sizeof(fpk::CflScratch) + fpk::cfl_ctas(c->ncells) * sizeof(float)), "cudaMalloc(cfl)");
+  FP_TRY(fpk::dev_alloc(&c->cfl_bits, sizeof(fpk::CflScratch) + fpk::cfl_ctas(c->ncells) * sizeof(float2)), "cudaMalloc(cfl)");
   FP_TRY(fpk::dev_alloc(&c->dblk, sizeof(BlockDev)), "cudaMalloc(block)");
   FP_TRY(fpk::dev_alloc(&c->lamg, 9 * c->esize), "cudaMalloc(global speeds)");
   FP_TRY(cudaMemset(c->lamg, 0, 9 * c->esize), "clear global speeds");

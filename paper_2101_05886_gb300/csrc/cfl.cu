@@ -10,7 +10,7 @@ namespace fpk {
 
 namespace {
 
-// sum_d (|u . grad d| + c |grad d|) of one point in FP64
+// sum_d (|u . grad d| + c |grad d|) of one point in FP64, as |J| (sum_d |u . k_d| + c sum_d |k_d|)
 template <typename T>
 __device__ double cfl_point(const BlockDev *blk, const T *q, long long idx, long long mo, int dims) {
   const long long qc = blk->qc;
@@ -20,29 +20,46 @@ __device__ double cfl_point(const BlockDev *blk, const T *q, long long idx, long
   const double p = (g - 1.0) * ((double)q[4 * qc + idx] - 0.5 * rho * (u * u + v * v + w * w));
   const double c = sqrt(g * p / rho);
   const double Jc = 1.0 / (double)static_cast<const T *>(blk->dir[0].kj)[4 * mo + 3];
-  double s = 0.0;
+  double U = 0.0, K = 0.0;
   for (int d = 0; d < dims; ++d) {
     const T *k = static_cast<const T *>(blk->dir[d].kj) + 4 * mo;
-    const double gx = Jc * (double)k[0], gy = Jc * (double)k[1], gz = Jc * (double)k[2];
-    s += fabs(u * gx + v * gy + w * gz) + c * sqrt(gx * gx + gy * gy + gz * gz);
+    const double kx = (double)k[0], ky = (double)k[1], kz = (double)k[2];
+    U += fabs(u * kx + v * ky + w * kz);
+    K += sqrt(kx * kx + ky * ky + kz * kz);
   }
-  return s;
+  return fabs(Jc) * (U + c * K);
+}
+
+// x rounded towards zero to FP32 (relative error below 2^-23; 0 below 2^-126, infinity from 2^128 on
+// and for a NaN) by integer operations: a conversion takes the FP64 pipe as long as an addition, and
+// a point's 17 took the FP64 screen 26 us on 1.05M points
+__device__ __forceinline__ float screen_value(float x) { return x; }
+__device__ __forceinline__ float screen_value(double x) {
+  const unsigned hi = __double2hiint(x), m = hi & 0x7fffffffu;
+  const unsigned bits = __funnelshift_l((unsigned)__double2loint(x), m, 3) - (896u << 23);
+  const unsigned mag = m < (897u << 20) ? 0u : (m >= (1151u << 20) ? 0x7f800000u : bits);
+  return __uint_as_float(mag | (hi & 0x80000000u));
 }
 
 constexpr int kCflThreads = 256, kCflPoints = 4;   // points per thread
 
 // The maximum of cfl_point over a block.  The FP64 pipe does two operations per clock and SM, and
-// a point's four quotients and four roots cost about 150 (1.07M points: 258 us, 25 times their
+// a point's four quotients and four roots cost about 120 (1.05M points: 220 us, 20 times their
 // memory time), so every point is first enclosed in FP32 bounds.  k_cfl_bound keeps the largest
-// lower bound of the block and each CTA's largest upper bound; k_cfl_max evaluates in FP64 the points
-// whose upper bound reaches the former, so the result is the same to the last bit.  (One kernel
-// whose CTAs knew only their own lower bound evaluated a point in every CTA: 39 us.)  The bounds'
-// relative width 4e-6 is about 20 times the rounding of the FP32 evaluation (inputs rounded to
-// float, at most 12 operations deep); cancellation in the pressure and in u . grad d is covered by
-// adding that width of the summed magnitudes.  Points with an input, a squared sound speed or a sum
-// outside [1e-30, 1e30], where a product could leave the FP32 range (p/rho of a dense cold gas
-// rounds to zero), and anything not finite have the upper bound +inf.
-// A step with its bound on 181 x 97 x 61 FP32 points: 1010 -> 792 us with the first form.
+// lower bound of the block and each CTA's largest and smallest upper bound; k_cfl_max evaluates in
+// FP64 the points whose upper bound reaches the former, so the result is the FP64 maximum.  (One
+// kernel whose CTAs knew only their own lower bound evaluated a point in every CTA: 39 us.)  The
+// bounds' relative width 4e-6 is more than three times the error of the FP32 evaluation (inputs to
+// 2^-23, the approximate reciprocal and root 2^-23 each, at most 12 operations deep: 1.2e-6);
+// cancellation in the pressure and in u . grad d is covered by adding that width of the summed
+// magnitudes.  Points with an input, a squared sound speed or a sum outside [1e-30, 1e30], where a
+// product could leave the FP32 range (p/rho of a dense cold gas rounds to zero), and anything not
+// finite have the upper bound +inf.
+// Measured, a call on 128 x 128 x 64 points (one FP64 kernel over all points | the screen): a smooth
+// flow 268 | 46 us in FP32, 242 | 65 us in FP64.  Where every point ties (a uniform stream on a
+// uniform grid) the screen rejects nothing and its pass comes on top: 292 | 294 us in FP32, 267 |
+// 281 us in FP64.  So a tie is kept cheap: CTAs all of whose points pass do not look at the bounds
+// again (26 us), and each CTA does one atomic (one per thread: 25 to 70 us).
 template <typename T> struct CflScreen {
   const BlockDev *blk;
   const T *q;
@@ -52,19 +69,18 @@ template <typename T> struct CflScreen {
   __device__ CflScreen(const BlockDev *b, int ni_, int nj_, int dims_)
       : blk(b), q(static_cast<const T *>(b->q[0])), qc(b->qc), ni(ni_), nj(nj_), dims(dims_), g1((float)(b->gamma - 1.0)), gam((float)b->gamma) {}
   __device__ long long place(long long idx) const {
-    const int i = (int)(idx % ni);
-    const long long r = idx / ni;
-    const int j = (int)(r % nj), k = (int)(r / nj);
+    // (a block has fewer than 2^31 points)
+    const unsigned r = (unsigned)idx / (unsigned)ni, i = (unsigned)idx - r * ni;
+    const unsigned k = r / (unsigned)nj, j = r - k * nj;
     // lines of the xi direction run along i; their transverse strides are those of j and k
     return blk->moff + i + (long long)j * blk->dir[0].mT1 + (dims == 3 ? (long long)k * blk->dir[0].mT2 : 0);
   }
   // upper bound of the point, and its lower bound (0 if it has none)
-  __device__ float bound(long long idx, float &lo) const {
+  __device__ float bound(long long idx, long long mo, float &lo) const {
     constexpr float kW = 4e-6f, kLow = 1e-30f, kHigh = 1e30f;
-    const long long mo = place(idx);
     float Q[5];
 #pragma unroll
-    for (int v = 0; v < 5; ++v) Q[v] = (float)q[v * qc + idx];
+    for (int v = 0; v < 5; ++v) Q[v] = screen_value(q[v * qc + idx]);
     // the point's metric vectors and 1/J, the values of one direction side by side
     auto metric = [&](int d, T k[4]) {
       const T *kj = static_cast<const T *>(blk->dir[d].kj);
@@ -72,20 +88,20 @@ template <typename T> struct CflScreen {
     };
     T kj[4];
     metric(0, kj);
-    const float ij = fabsf((float)kj[3]);
+    const float ij = fabsf(screen_value(kj[3]));
     bool ok = Q[0] > kLow && Q[0] < kHigh && Q[4] > kLow && Q[4] < kHigh && ij > kLow && ij < kHigh;
-    const float ri = 1.0f / Q[0], Jc = 1.0f / ij;
+    const float ri = Num<float>::rcp(Q[0]), Jc = Num<float>::rcp(ij);
     const float u = Q[1] * ri, v = Q[2] * ri, w = Q[3] * ri;
     const float ke = 0.5f * (Q[1] * u + Q[2] * v + Q[3] * w);
     const float e = Q[4] - ke, de = kW * (Q[4] + ke);
     const float c2 = gam * g1 * fmaxf(e + de, 0.f) * ri;
     ok = ok && c2 > kLow;
-    const float chi = sqrtf(c2), clo = sqrtf(gam * g1 * fmaxf(e - de, 0.f) * ri);
+    const float chi = Num<float>::sqrt_(c2), clo = Num<float>::sqrt_(gam * g1 * fmaxf(e - de, 0.f) * ri);
     float sh = 0.f, sl = 0.f;
     for (int d = 0; d < dims; ++d) {
       if (d) metric(d, kj);
-      const float kx = (float)kj[0], ky = (float)kj[1], kz = (float)kj[2];
-      const float k2 = kx * kx + ky * ky + kz * kz, kn = sqrtf(k2);
+      const float kx = screen_value(kj[0]), ky = screen_value(kj[1]), kz = screen_value(kj[2]);
+      const float k2 = kx * kx + ky * ky + kz * kz, kn = Num<float>::sqrt_(k2);
       ok = ok && k2 > kLow && k2 < kHigh;
       const float U = fabsf(u * kx + v * ky + w * kz);
       const float dU = kW * (fabsf(u * kx) + fabsf(v * ky) + fabsf(w * kz));
@@ -102,34 +118,39 @@ template <typename T> struct CflScreen {
 
 template <typename T>
 __global__ void __launch_bounds__(kCflThreads) k_cfl_bound(const BlockDev *blk, long long ncells, int ni, int nj, int dims,
-                                                           CflScratch *out, float *cta_hi) {
-  __shared__ float red[2][kCflThreads / 32];
+                                                           CflScratch *out, float2 *cta_hi) {
+  __shared__ float red[3][kCflThreads / 32];
   const CflScreen<T> screen(blk, ni, nj, dims);
   const long long base = (long long)blockIdx.x * (kCflThreads * kCflPoints) + threadIdx.x;
-  float hi = -1.f, lo = 0.f;
+  float hi = -1.f, lo = 0.f, least = __int_as_float(0x7f800000);
 #pragma unroll
   for (int m = 0; m < kCflPoints; ++m) {
     const long long idx = base + m * kCflThreads;
     if (idx >= ncells) continue;
     float l;
-    hi = fmaxf(hi, screen.bound(idx, l));
+    const float h = screen.bound(idx, screen.place(idx), l);
+    hi = fmaxf(hi, h);
+    least = fminf(least, h);
     lo = fmaxf(lo, l);
   }
   for (int h = 16; h; h >>= 1) {
     hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, h));
     lo = fmaxf(lo, __shfl_xor_sync(0xffffffffu, lo, h));
+    least = fminf(least, __shfl_xor_sync(0xffffffffu, least, h));
   }
   if (threadIdx.x % 32 == 0) {
     red[0][threadIdx.x / 32] = hi;
     red[1][threadIdx.x / 32] = lo;
+    red[2][threadIdx.x / 32] = least;
   }
   __syncthreads();
   if (threadIdx.x == 0) {
     for (int w = 1; w < kCflThreads / 32; ++w) {
       hi = fmaxf(hi, red[0][w]);
       lo = fmaxf(lo, red[1][w]);
+      least = fminf(least, red[2][w]);
     }
-    cta_hi[blockIdx.x] = hi;
+    cta_hi[blockIdx.x] = make_float2(hi, least);
     atomicMax(&out->lower_bits, __float_as_uint(lo));
   }
   chain_next();
@@ -137,20 +158,31 @@ __global__ void __launch_bounds__(kCflThreads) k_cfl_bound(const BlockDev *blk, 
 
 template <typename T>
 __global__ void __launch_bounds__(kCflThreads) k_cfl_max(const BlockDev *blk, long long ncells, int ni, int nj, int dims,
-                                                         CflScratch *out, const float *cta_hi) {
+                                                         CflScratch *out, const float2 *cta_hi) {
+  __shared__ long long red[kCflThreads / 32];
   chain_wait();
   const float lo = __uint_as_float(*(volatile unsigned int *)&out->lower_bits);
-  if (cta_hi[blockIdx.x] < lo) return;
+  const float2 hi = cta_hi[blockIdx.x];
+  if (hi.x < lo) return;
+  const bool all = hi.y >= lo;                      // every point of the CTA, without another look
   const CflScreen<T> screen(blk, ni, nj, dims);
-  double best = 0.0;
+  long long best = 0;                               // bits: non-negative doubles are ordered like them
   for (int m = 0; m < kCflPoints; ++m) {
     const long long idx = (long long)blockIdx.x * (kCflThreads * kCflPoints) + m * kCflThreads + threadIdx.x;
+    if (idx >= ncells) break;
+    const long long mo = screen.place(idx);
     float l;
-    if (idx >= ncells || screen.bound(idx, l) < lo) continue;
-    const double s = cfl_point(blk, screen.q, idx, screen.place(idx), dims);
-    best = s > best ? s : best;
+    if (!all && screen.bound(idx, mo, l) < lo) continue;
+    const long long s = __double_as_longlong(cfl_point(blk, screen.q, idx, mo, dims));
+    if (s > best && s <= 0x7ff0000000000000LL) best = s;   // (a NaN is ignored)
   }
-  if (best > 0.0) atomicMax(&out->max_bits, (unsigned long long)__double_as_longlong(best));
+  for (int h = 16; h; h >>= 1) best = max(best, __shfl_xor_sync(0xffffffffu, best, h));
+  if (threadIdx.x % 32 == 0) red[threadIdx.x / 32] = best;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int w = 1; w < kCflThreads / 32; ++w) best = max(best, red[w]);
+    if (best > 0) atomicMax(&out->max_bits, (unsigned long long)best);
+  }
 }
 
 template <typename T>
@@ -306,12 +338,12 @@ int cfl_ctas(long long ncells) { return (int)((ncells + kCflThreads * kCflPoints
 cudaError_t launch_cfl(const BlockDev *blk, int is_f32, long long ncells, const int *n, int dims,
                        CflScratch *scratch, cudaStream_t s) {
   const int g = cfl_ctas(ncells);
-  float *hi = reinterpret_cast<float *>(scratch + 1);
+  float2 *hi = reinterpret_cast<float2 *>(scratch + 1);
   cudaError_t e = launch_kernel(is_f32 ? k_cfl_bound<float> : k_cfl_bound<double>, g, kCflThreads, 0, s, 0, blk, ncells, n[0],
                                 n[1], dims, scratch, hi);
   if (e != cudaSuccess) return e;
   return launch_kernel(is_f32 ? k_cfl_max<float> : k_cfl_max<double>, g, kCflThreads, 0, s, 1, blk, ncells, n[0], n[1],
-                       dims, scratch, (const float *)hi);
+                       dims, scratch, (const float2 *)hi);
 }
 
 }  // namespace fpk

@@ -260,7 +260,7 @@ cudaError_t launch_lambda(const BlockDev *blocks, int nblocks, const int2 *items
 cudaError_t launch_finish(const BlockDev *blk, int is_f32, long long ncells, const int *n, int dims, int rk,
                           int stage, const double *dt, cudaStream_t s);
 
-// CFL reduction (cfl.cu): `scratch` holds CflScratch and a float per CTA (cfl_ctas of them).
+// CFL reduction (cfl.cu): `scratch` holds CflScratch and a float2 per CTA (cfl_ctas of them).
 struct CflScratch {
   unsigned long long max_bits;   // the result: bits of the FP64 maximum
   unsigned int lower_bits;       // bits of the largest FP32 lower bound

@@ -205,6 +205,10 @@ __device__ __forceinline__ void atomic_max_nonneg(double *a, double v) {
 __device__ __forceinline__ float reciprocal(float x) { return 1.0f / x; }
 __device__ __forceinline__ double reciprocal(double x) { return Num<double>::rcp(x); }
 
+// sqrt(a b), correctly rounded roots (see Num::sqrt_product for the ranges)
+__device__ __forceinline__ float sqrt_product(float a, float b) { return sqrtf(a) * sqrtf(b); }
+__device__ __forceinline__ double sqrt_product(double a, double b) { return sqrt(a * b); }
+
 // Max over each block's points of |U - c|grad d||, |U|, |U + c|grad d|| for every direction.  A CTA
 // takes a contiguous range of the items (kLamChunk points each), keeps its maxima in registers
 // while the block stays the same, and then reduces them by warp and adds them to the block's.
@@ -249,7 +253,7 @@ __global__ void k_lam_max(const BlockDev *blocks, const int2 *items, int nitems,
         if (d >= dims) continue;
         if (d) metric(d, kj);
         const T kx = kj[0], ky = kj[1], kz = kj[2];
-        const T U = Jc * (u * kx + v * ky + w * kz), a = fabs(Jc) * sqrt(c2 * (kx * kx + ky * ky + kz * kz));
+        const T U = Jc * (u * kx + v * ky + w * kz), a = fabs(Jc) * sqrt_product(c2, kx * kx + ky * ky + kz * kz);
         T lm = fabs(U - a), l0 = fabs(U), lp = fabs(U + a);
         if (!charwise) { lm = fmax(lm, lp); l0 = lm; lp = lm; }
         best[3 * d] = fmax(best[3 * d], lm);

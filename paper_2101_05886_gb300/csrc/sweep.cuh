@@ -59,6 +59,8 @@ template <> struct Num<double> {
   static __device__ __forceinline__ double fma_(double a, double b, double c) { return fma(a, b, c); }
   static __device__ __forceinline__ double sqrt_(double x) { return sqrt(x); }
   static __device__ __forceinline__ double rsqrt_(double x) { return rsqrt(x); }
+  // sqrt(a b): one root of the product, which stays in range up to 1e308
+  static __device__ __forceinline__ double sqrt_product(double a, double b) { return sqrt(a * b); }
   static __device__ __forceinline__ double ld(const void *p, long long i) {
     return __ldg(static_cast<const double *>(p) + i);
   }
@@ -79,6 +81,9 @@ template <> struct Num<float> {
     return r;
   }
   static __device__ __forceinline__ float rsqrt_(float x) { return rsqrtf(x); }
+  // sqrt(a b) by two roots: c^2 |k|^2 leaves the FP32 range where c |k| passes 1.8e19 (sound speeds
+  // in m/s on cells of 1e8 m) though both factors are far inside it
+  static __device__ __forceinline__ float sqrt_product(float a, float b) { return sqrt_(a) * sqrt_(b); }
   static __device__ __forceinline__ float ld(const void *p, long long i) {
     return __ldg(static_cast<const float *>(p) + i);
   }
@@ -662,7 +667,7 @@ fp_sweep(const BlockDev *__restrict__ blocks, const SweepItem *__restrict__ item
       cp[CF_H * kRing] = Num<T>::fma_(g1, e, Q[4]) * rinv;
       cp[CF_SQR * kRing] = Num<T>::sqrt_(Q[0]);
       cp[CF_UC * kRing] = Jc * dot3<T>(u0, u1, u2, k[0], k[1], k[2]);
-      cp[CF_AC * kRing] = fabs(Jc) * Num<T>::sqrt_(gam * p * rinv * dot3<T>(k[0], k[1], k[2], k[0], k[1], k[2]));
+      cp[CF_AC * kRing] = fabs(Jc) * Num<T>::sqrt_product(gam * p * rinv, dot3<T>(k[0], k[1], k[2], k[0], k[1], k[2]));
     };
 
     // asynchronous copy of the metrics of face x + 1/2 of line (t1, t2), and of the change of the face

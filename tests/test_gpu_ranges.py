@@ -11,7 +11,7 @@ torch = pytest.importorskip("torch")
 
 import oracle as O
 from paper_2101_05886_gb300 import inputs as I
-from tests.helpers import f32
+from tests.helpers import f32, rhs_err, ulp_sensitivity
 
 pytestmark = pytest.mark.gpu
 
@@ -53,3 +53,25 @@ def test_fp32_linear_upwind_in_large_units(characteristic, global_lf):
     got = _rhs(big, q * unit[:, None, None, None], qinf * unit, **kw)
     assert np.isfinite(want).all() and np.abs(want).max() > 1e-3
     assert np.array_equal(got / (unit * 2.0 ** -10)[:, None, None, None], want)
+
+
+@pytest.mark.parametrize("characteristic", [1, 0])
+@pytest.mark.parametrize("power", [130, 240])
+def test_fp64_weno5_of_large_states(power, characteristic):
+    """The Euler fluxes and the WENO5 weights (where the constant 1e-6 is negligible) do not depend
+    on the unit of the conserved variables: a state times 2^130 or 2^240, whose squared indicators
+    (2^500, 2^940) are FP64 numbers though their products are not, has the residual of the state
+    times 2^100, and the oracle's."""
+    g, qinf, q = _case(B.FP_F64, 8)
+    kw = dict(scheme=B.FP_WENO5_JS, precision=B.FP_F64, characteristic=characteristic)
+    want = _rhs(g, q * 2.0 ** 100, qinf * 2.0 ** 100, **kw)
+    got = _rhs(g, q * 2.0 ** power, qinf * 2.0 ** power, **kw)
+    assert np.isfinite(want).all() and np.abs(want).max() > 0
+    assert np.array_equal(got * 2.0 ** (100 - power), want)
+    # the oracle in the same units; its error bound is that of the parity suite
+    cfg = O.cfg_for(g, M=6, scheme=0, charwise=characteristic, qinf=qinf * 2.0 ** 130)
+    met = O.metrics(cfg, g.nodes, g.Gn)
+    q130 = q * 2.0 ** 130
+    tol = max(1e-12, 2.0 * ulp_sensitivity(cfg, met, q130))
+    assert tol <= 2e-11, tol
+    assert max(rhs_err(got * 2.0 ** (130 - power), cfg, met, q130, per_component=True)) <= tol

@@ -15,14 +15,17 @@ template <typename T>
 __device__ double cfl_point(const BlockDev *blk, const T *q, long long idx, long long mo, int dims) {
   const long long qc = blk->qc;
   const double g = blk->gamma;
-  const double rho = (double)q[idx];
-  const double u = (double)q[qc + idx] / rho, v = (double)q[2 * qc + idx] / rho, w = (double)q[3 * qc + idx] / rho;
-  const double p = (g - 1.0) * ((double)q[4 * qc + idx] - 0.5 * rho * (u * u + v * v + w * w));
+  auto val = [&](int c) { return (double)*FPK_IN(q + (c * qc + idx), q, 5 * qc, blk->status); };
+  const double rho = val(0);
+  const double u = val(1) / rho, v = val(2) / rho, w = val(3) / rho;
+  const double p = (g - 1.0) * (val(4) - 0.5 * rho * (u * u + v * v + w * w));
   const double c = sqrt(g * p / rho);
-  const double Jc = 1.0 / (double)static_cast<const T *>(blk->dir[0].kj)[4 * mo + 3];
-  double U = 0.0, K = 0.0;
+  double Jc = 0.0, U = 0.0, K = 0.0;
   for (int d = 0; d < dims; ++d) {
-    const T *k = static_cast<const T *>(blk->dir[d].kj) + 4 * mo;
+    const T *kj = static_cast<const T *>(blk->dir[d].kj);
+    T k[4];
+    load4(FPK_IN(kj + 4 * mo, kj, 4LL * blk->mc - 3, blk->status), k);
+    if (d == 0) Jc = 1.0 / (double)k[3];
     const double kx = (double)k[0], ky = (double)k[1], kz = (double)k[2];
     U += fabs(u * kx + v * ky + w * kz);
     K += sqrt(kx * kx + ky * ky + kz * kz);
@@ -80,7 +83,7 @@ template <typename T> struct CflScreen {
     constexpr float kW = 4e-6f, kLow = 1e-30f, kHigh = 1e30f;
     float Q[5];
 #pragma unroll
-    for (int v = 0; v < 5; ++v) Q[v] = screen_value(q[v * qc + idx]);
+    for (int v = 0; v < 5; ++v) Q[v] = screen_value(*FPK_IN(q + (v * qc + idx), q, 5 * qc, blk->status));
     // the point's metric vectors and 1/J, the values of one direction side by side
     auto metric = [&](int d, T k[4]) {
       const T *kj = static_cast<const T *>(blk->dir[d].kj);
@@ -236,7 +239,7 @@ __global__ void k_lam_max(const BlockDev *blocks, const int2 *items, int nitems,
       const int j = (int)(r % nj);
       const int k = (int)(r / nj);
       const long long mo = B->moff + i + (long long)j * B->dir[0].mT1 + (dims == 3 ? (long long)k * B->dir[0].mT2 : 0);
-      auto val = [&](int c) { return q[state_at(stage, idx, qc, c)]; };
+      auto val = [&](int c) { return *FPK_IN(q + state_at(stage, idx, qc, c), q, 5 * qc, B->status); };
       const T rho = val(0), rinv = reciprocal(rho);
       const T u = val(1) * rinv, v = val(2) * rinv, w = val(3) * rinv;
       const T p = (g - T(1)) * (val(4) - T(0.5) * rho * (u * u + v * v + w * w));
@@ -273,7 +276,7 @@ __global__ void k_lam_max(const BlockDev *blocks, const int2 *items, int nitems,
     if (threadIdx.x < 3 * dims) {
       T b = red[threadIdx.x][0];
       for (int w = 1; w < kLamChunk / 32; ++w) b = fmax(b, red[threadIdx.x][w]);
-      atomic_max_nonneg(static_cast<T *>(B->lamg) + threadIdx.x, b);
+      atomic_max_nonneg(FPK_IN(static_cast<T *>(B->lamg) + threadIdx.x, static_cast<T *>(B->lamg), 9, B->status), b);
     }
     __syncthreads();
   }
@@ -299,7 +302,7 @@ __global__ void k_pack_halo(const T *__restrict__ q, int stage, T *__restrict__ 
     c[1] = (int)(r % e[1]);
     c[2] = (int)(r / e[1]);
     c[dir] += side ? nd - G : 0;
-    out[idx] = *FPK_IN(q + state_at(stage, ((long long)c[2] * nj + c[1]) * ni + c[0], qc, v), q, 5 * qc, status);
+    *FPK_IN(out + idx, out, 5 * hc, status) = *FPK_IN(q + state_at(stage, ((long long)c[2] * nj + c[1]) * ni + c[0], qc, v), q, 5 * qc, status);
   }
 }
 

@@ -74,10 +74,12 @@ enum : int { MODE_WRITE = 0, MODE_ADD = 1, MODE_RHS = 2, MODE_RK = 3 };
 enum : int { ST_NONFINITE = 1, ST_BOUNDS = 2 };
 
 // Bounds-checking builds (compiled with -DFPK_BOUNDS_CHECK, libfpgb300_check.so): before every
-// global access of the sweep, the halo packing and the speed and time-step reductions, the
-// element is checked against the array it belongs to, and every shared-ring offset against the
-// ring.  An element outside records ST_BOUNDS in the status word and the access goes to the
-// array's first element instead, so a wrong index shows as FP_ERR_BOUNDS, not as a fault.  In
+// access of the sweep, the sum that ends a stage, the halo packing and the speed and time-step
+// reductions to a block's arrays (states, halos, metrics, face metrics, accumulators, dQ/dt, speeds)
+// the element is checked against the array, and every shared-ring offset against the ring.  (The
+// lists that a launch is made of, descriptors and work items, are read by CTA number and link and
+// not checked.)  An element outside records ST_BOUNDS in the status word and the access goes to
+// the array's first element instead, so a wrong index shows as FP_ERR_BOUNDS, not as a fault.  In
 // the normal build FPK_CHK_ONLY(...) expands to nothing and FPK_IN(p, ...) to p.
 #ifdef FPK_BOUNDS_CHECK
 #define FPK_CHK_ONLY(...) __VA_ARGS__

@@ -29,19 +29,21 @@ __global__ void __launch_bounds__(256) k_finish(const BlockDev *__restrict__ blk
   for (int d = 0; d < 3; ++d) {
     if (d >= dims) continue;
     const T *a = static_cast<const T *>(blk->dir[d].racc);
-    load4(a + 4ULL * idx, acc[d]);
-    acc[d][4] = *comp_at(a, idx, qc, 4);
+    load4(FPK_IN(a + 4ULL * idx, a, 4LL * qc - 3, blk->status), acc[d]);
+    acc[d][4] = *FPK_IN(comp_at(a, idx, qc, 4), a, 5LL * qc, blk->status);
   }
+  const T *const q0 = static_cast<const T *>(blk->q[0]), *const qi = static_cast<const T *>(blk->q[stage]);
 #pragma unroll
   for (int v = 0; v < 5; ++v) {
     R[v] = acc[0][v] + acc[1][v];
     if (dims == 3) R[v] += acc[2][v];
-    if (rk) qk[v] = static_cast<const T *>(blk->q[stage])[state_at(stage, idx, qc, v)];
-    qn[v] = rk && stage ? *comp_at(static_cast<const T *>(blk->q[0]), idx, qc, v) : T(0);
+    if (rk) qk[v] = *FPK_IN(qi + state_at(stage, idx, qc, v), qi, 5LL * qc, blk->status);
+    qn[v] = rk && stage ? *FPK_IN(comp_at(q0, idx, qc, v), q0, 5LL * qc, blk->status) : T(0);
   }
   if (!rk) {
+    T *const out = static_cast<T *>(blk->dqdt);
 #pragma unroll
-    for (int v = 0; v < 5; ++v) *comp_at(static_cast<T *>(blk->dqdt), idx, qc, v) = -Jc * R[v];
+    for (int v = 0; v < 5; ++v) *FPK_IN(comp_at(out, idx, qc, v), out, 5LL * qc, blk->status) = -Jc * R[v];
     return;
   }
   const RkStage<T> update(stage, T(*dtp));
@@ -54,12 +56,12 @@ __global__ void __launch_bounds__(256) k_finish(const BlockDev *__restrict__ blk
     bad |= !isfinite(nv[v]);
   }
   if (stage < 2) {
-    store4(qs + 4ULL * idx, nv);
+    store4(FPK_IN(qs + 4ULL * idx, qs, 4LL * qc - 3, blk->status), nv);
   } else {
 #pragma unroll
-    for (int v = 0; v < 4; ++v) *comp_at(qs, idx, qc, v) = nv[v];
+    for (int v = 0; v < 4; ++v) *FPK_IN(comp_at(qs, idx, qc, v), qs, 5LL * qc, blk->status) = nv[v];
   }
-  *comp_at(qs, idx, qc, 4) = nv[4];
+  *FPK_IN(comp_at(qs, idx, qc, 4), qs, 5LL * qc, blk->status) = nv[4];
   if (bad) atomicOr(blk->status, ST_NONFINITE);
 }
 

@@ -39,7 +39,6 @@ struct fp_ctx {
   BlockDev hblk;
   BlockDev *dblk = nullptr;
   BlockDev uploaded;                  // last BlockDev copied to dblk
-  fpk::SweepItem *item_mem = nullptr; // the items of all launches, one allocation
   fpk::SweepItem *items[3] = {nullptr, nullptr, nullptr};
   int ncta[3] = {0, 0, 0};            // CTAs of each direction's launch
   // all directions in one launch (blocks of at most kSplitPoints points): its items
@@ -488,66 +487,69 @@ cudaError_t put_items(const std::vector<fpk::SweepItem> &items, fpk::SweepItem *
 // passes: 1.79 ms with a share per slot, 1.52 ms).  FP32 needs the resident warps to hide
 // latency: a share per slot.
 int balanced_items(const fp_ctx *c, const std::vector<Stream> &streams, int most_per_sm, std::vector<fpk::SweepItem> &items) {
-  int per_sm = most_per_sm;
-  if (!c->is_f32) {
-    long long least = -1;
-    for (int m = most_per_sm; m >= 1; --m) {
-      const int n = make_items(streams, m * c->nsm, streams.size() == 1, items);
-      long long most = 0;                         // chunks of one CTA
-      for (int k = 0; k < n; ++k) {
-        long long ch = 0;
-        for (int i = k; i >= 0; i = items[i].next) {
-          const int S = c->hblk.dir[items[i].dir].S;
-          ch += (items[i].len + S) / S;
-        }
-        most = std::max(most, ch);
+  const bool alone = streams.size() == 1;
+  if (c->is_f32) return make_items(streams, most_per_sm * c->nsm, alone, items);
+  std::vector<fpk::SweepItem> tried;
+  long long least = -1;
+  int ncta = 0;
+  for (int m = most_per_sm; m >= 1; --m) {
+    const int n = make_items(streams, m * c->nsm, alone, tried);
+    long long most = 0;                           // chunks of one CTA
+    for (int k = 0; k < n; ++k) {
+      long long ch = 0;
+      for (int i = k; i >= 0; i = tried[i].next) {
+        const int S = c->hblk.dir[tried[i].dir].S;
+        ch += (tried[i].len + S) / S;
       }
-      const long long cost = (n + c->nsm - 1) / c->nsm * most;
-      if (least < 0 || 20 * cost < 19 * least) { least = cost; per_sm = m; }
+      most = std::max(most, ch);
     }
+    const long long cost = (n + c->nsm - 1) / c->nsm * most;
+    if (least < 0 || 20 * cost < 19 * least) { least = cost; ncta = n; items.swap(tried); }
   }
-  return make_items(streams, per_sm * c->nsm, streams.size() == 1, items);
+  return ncta;
 }
 
 // The items of the context's launches for the tiles in hblk.  All lists are made and copied before
-// any of the old ones goes, so a failure leaves the context with the lists it had.
-int upload_items(fp_ctx *c) {
-  std::vector<fpk::SweepItem> items, all;         // one launch's, and those of all launches in turn
+// any of the old ones goes, so a failure leaves the context with the lists it had.  Ends with a
+// synchronisation of the stream.
+int upload_items(fp_ctx *c, cudaStream_t s) {
+  struct List {                                   // of each direction, and of the launch over all of them
+    std::vector<fpk::SweepItem> items;
+    int ncta = 0;
+    fpk::SweepItem *dev = nullptr;
+  } lists[4];
   std::vector<Stream> streams;
-  size_t first[4] = {0, 0, 0, 0};                 // of each direction, and of the launch over all of them
-  int ncta[4] = {0, 0, 0, 0};
   int split = c->ncells <= kSplitPoints;
   const int sh0 = shape_of(c, c->hblk.dir[0]);
-  auto add = [&](int l, const std::vector<Stream> &of, int shape) {
-    ncta[l] = balanced_items(c, of, c->per_sm[shape], items);
-    first[l] = all.size();
-    all.insert(all.end(), items.begin(), items.end());
-  };
   for (int d = 0; d < c->desc.dims; ++d) {
     const int sh = shape_of(c, c->hblk.dir[d]);
     streams.push_back(stream_of(c->hblk, 0, d));
     if (sh != sh0) split = 0;                     // one launch has one CTA shape
-    add(d, {streams.back()}, sh);
+    lists[d].ncta = balanced_items(c, {streams.back()}, c->per_sm[sh], lists[d].items);
   }
-  if (split) add(3, streams, sh0);
-  fpk::SweepItem *mem = nullptr;
-  cudaError_t e = fpk::dev_alloc(&mem, all.size() * sizeof(fpk::SweepItem));
-  if (e == cudaSuccess) e = cudaMemcpy(mem, all.data(), all.size() * sizeof(fpk::SweepItem), cudaMemcpyHostToDevice);
+  if (split) lists[3].ncta = balanced_items(c, streams, c->per_sm[sh0], lists[3].items);
+  cudaError_t e = cudaSuccess;
+  for (List &l : lists) {
+    const size_t bytes = l.items.size() * sizeof(fpk::SweepItem);
+    if (e == cudaSuccess && bytes) e = fpk::dev_alloc(&l.dev, bytes);
+    if (e == cudaSuccess && bytes) e = cudaMemcpyAsync(l.dev, l.items.data(), bytes, cudaMemcpyHostToDevice, s);
+  }
+  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   if (e != cudaSuccess) {
-    cudaFree(mem);
+    for (List &l : lists) cudaFree(l.dev);
     return cuda_fail(c, e, "sweep items");
   }
-  cudaFree(c->item_mem);
-  c->item_mem = mem;
   for (int d = 0; d < c->desc.dims; ++d) {
-    c->items[d] = mem + first[d];
-    c->ncta[d] = ncta[d];
+    cudaFree(c->items[d]);
+    c->items[d] = lists[d].dev;
+    c->ncta[d] = lists[d].ncta;
     // one accumulator, or the directions' own
     c->hblk.dir[d].racc = static_cast<char *>(c->racc) + (split ? d * split_stride(c) : 0);
   }
+  cudaFree(c->sitems);
+  c->sitems = lists[3].dev;
+  c->nscta = lists[3].ncta;
   c->split = split;
-  c->sitems = split ? mem + first[3] : nullptr;
-  c->nscta = ncta[3];
   return FP_OK;
 }
 
@@ -622,10 +624,10 @@ const char *fp_last_error(const fp_ctx *c) { return c ? c->err.c_str() : "null c
 void fp_free(fp_ctx *c) {
   if (!c) return;
   cudaDeviceSynchronize();
-  for (int d = 0; d < 3; ++d) { cudaFree(c->kj[d]); cudaFree(c->fk[d]); }
+  for (int d = 0; d < 3; ++d) { cudaFree(c->kj[d]); cudaFree(c->fk[d]); cudaFree(c->items[d]); }
   cudaFree(c->q1); cudaFree(c->q2); cudaFree(c->racc);
   cudaFree(c->status); cudaFree(c->dt_dev); cudaFree(c->cfl_bits); cudaFree(c->dblk);
-  cudaFree(c->lamg); cudaFree(c->lam_items); cudaFree(c->item_mem);
+  cudaFree(c->lamg); cudaFree(c->lam_items); cudaFree(c->sitems);
   delete c;
 }
 
@@ -656,68 +658,81 @@ int fp_init_grid(const fp_grid_desc *desc, const double *xyz, int ghost_nodes, v
     c->nface[d] = d < dims ? c->ncells / n[d] * (n[d] + 1) : 0;
 
   cudaError_t e;
-  double *nodes = nullptr, *met64 = nullptr, *scratch = nullptr, *fm64[3] = {nullptr, nullptr, nullptr};
+  // temporaries, two allocations: the nodes and the construction's scratch; the FP64 metrics and face metrics
+  double *nodes = nullptr, *met64 = nullptr;
   auto cleanup_tmp = [&]() {
-    for (double **p : {&nodes, &scratch, &met64, &fm64[0], &fm64[1], &fm64[2]}) {
-      cudaFree(*p);
-      *p = nullptr;
-    }
+    cudaFree(nodes);
+    cudaFree(met64);
+    nodes = met64 = nullptr;
   };
 #define FP_TRY(call, where)                         \
   do {                                              \
     e = (call);                                     \
     if (e != cudaSuccess) {                         \
       int st = cuda_fail(c, e, where);              \
+      cudaStreamSynchronize(s);                     \
       cleanup_tmp();                                \
       std::fprintf(stderr, "fp_init_grid: %s\n", c->err.c_str()); \
       fp_free(c);                                   \
       return st;                                    \
     }                                               \
   } while (0)
-  FP_TRY(fpk::dev_alloc(&nodes, (size_t)dims * nnode * sizeof(double)), "cudaMalloc(nodes)");
+  const long long nodes_n = (dims * nnode + 31) / 32 * 32, nscratch = 9 * (nb1 + nb2);
+  FP_TRY(fpk::dev_alloc(&nodes, (size_t)(nodes_n + nscratch) * sizeof(double)), "cudaMalloc(nodes, metric scratch)");
   FP_TRY(cudaGetDevice(&c->dev), "cudaGetDevice");
   FP_TRY(cudaDeviceGetAttribute(&c->nsm, cudaDevAttrMultiProcessorCount, c->dev), "device attribute");
   FP_TRY(noalloc_prepare(c->dev), "static scratch of fp_rhs_noalloc");
   FP_TRY(cudaMemcpyAsync(nodes, xyz, (size_t)dims * nnode * sizeof(double), cudaMemcpyHostToDevice, s),
          "copy nodes");
-  FP_TRY(fpk::dev_alloc(&met64, (size_t)10 * c->nmet * sizeof(double)), "cudaMalloc(metrics)");
-  for (int d = 0; d < dims; ++d)
-    FP_TRY(fpk::dev_alloc(&fm64[d], (size_t)3 * c->nface[d] * sizeof(double)), "cudaMalloc(face metrics)");
-  FP_TRY(fpk::dev_alloc(&scratch, (size_t)9 * (nb1 + nb2) * sizeof(double)), "cudaMalloc(metric scratch)");
+  FP_TRY(fpk::dev_alloc(&met64, (size_t)(10 * c->nmet + 3 * (c->nface[0] + c->nface[1] + c->nface[2])) * sizeof(double)),
+         "cudaMalloc(metrics, face metrics)");
   fpk::MetricJob J;
   J.dims = dims; J.M = M; J.G = G; J.Gn = Gn;
-  for (int d = 0; d < 3; ++d) { J.n[d] = n[d]; J.fmet[d] = fm64[d]; }
-  J.nodes = nodes; J.met = met64; J.scratch = scratch;
+  J.nodes = nodes; J.met = met64; J.scratch = nodes + nodes_n;
+  double *fm = met64 + 10 * c->nmet;
+  for (int d = 0; d < 3; ++d) {
+    J.n[d] = n[d];
+    J.fmet[d] = d < dims ? fm : nullptr;
+    fm += 3 * c->nface[d];
+  }
   FP_TRY(fpk::build_metrics(J, s), "build metrics");
-  // the scratch and the nodes make room for the packed arrays
-  FP_TRY(cudaStreamSynchronize(s), "metric construction");
-  cudaFree(nodes); cudaFree(scratch);
-  nodes = scratch = nullptr;
+  // A small block's time goes into allocations (40 us each from 1 MB on, and as much to free them) and
+  // the host's part, so few temporaries are made, and what follows runs while the device builds the
+  // metrics (six temporaries and a wait here | so, in ms: 48 x 37 x 29 FP32 1.36 | 0.79, 96^3 FP64
+  // 4.0 | 3.3, 128^2 FP64 0.55 | 0.49).  In a large block the nodes and the scratch make room for the
+  // packed arrays first.
+  if (c->ncells > kSplitPoints) {
+    FP_TRY(cudaStreamSynchronize(s), "metric construction");
+    cudaFree(nodes);
+    nodes = nullptr;
+  }
   for (int d = 0; d < dims; ++d) {
     FP_TRY(fpk::dev_alloc(&c->kj[d], (size_t)4 * c->nmet * c->esize), "cudaMalloc(metrics)");
     FP_TRY(fpk::pack_metrics(J, d, c->is_f32, c->kj[d], s), "pack metrics");
     FP_TRY(fpk::dev_alloc(&c->fk[d], (size_t)6 * c->nface[d] * c->esize), "cudaMalloc(face metrics)");
     FP_TRY(fpk::pack_faces(J, d, c->is_f32, c->fk[d], s), "pack face metrics");
   }
-  FP_TRY(cudaStreamSynchronize(s), "metric packing");
-  cleanup_tmp();
+  if (c->ncells > kSplitPoints) {
+    FP_TRY(cudaStreamSynchronize(s), "metric packing");
+    cleanup_tmp();
+  }
   const size_t sbytes = (size_t)5 * c->ncells * c->esize;
   FP_TRY(fpk::dev_alloc(&c->q1, sbytes), "cudaMalloc(stage 1)");
   FP_TRY(fpk::dev_alloc(&c->q2, sbytes), "cudaMalloc(stage 2)");
   FP_TRY(fpk::dev_alloc(&c->racc, c->ncells <= kSplitPoints ? dims * split_stride(c) : sbytes), "cudaMalloc(residual)");
   FP_TRY(fpk::dev_alloc(&c->status, sizeof(int)), "cudaMalloc(status)");
-  FP_TRY(cudaMemset(c->status, 0, sizeof(int)), "clear status");
+  FP_TRY(cudaMemsetAsync(c->status, 0, sizeof(int), s), "clear status");
   FP_TRY(fpk::dev_alloc(&c->dt_dev, sizeof(double)), "cudaMalloc(dt)");
   FP_TRY(fpk::dev_alloc(&c->cfl_bits, sizeof(fpk::CflScratch) + fpk::cfl_ctas(c->ncells) * sizeof(float2)), "cudaMalloc(cfl)");
   FP_TRY(fpk::dev_alloc(&c->dblk, sizeof(BlockDev)), "cudaMalloc(block)");
   FP_TRY(fpk::dev_alloc(&c->lamg, 9 * c->esize), "cudaMalloc(global speeds)");
-  FP_TRY(cudaMemset(c->lamg, 0, 9 * c->esize), "clear global speeds");
-  {
-    std::vector<int2> li;
+  FP_TRY(cudaMemsetAsync(c->lamg, 0, 9 * c->esize, s), "clear global speeds");
+  std::vector<int2> li;               // lives until the stream is synchronised
+  if (desc->global_lf) {
     for (long long p0 = 0; p0 < c->ncells; p0 += fpk::kLamChunk) li.push_back(make_int2(0, (int)p0));
     c->nlam_items = (int)li.size();
     FP_TRY(fpk::dev_alloc(&c->lam_items, li.size() * sizeof(int2)), "cudaMalloc(speed items)");
-    FP_TRY(cudaMemcpy(c->lam_items, li.data(), li.size() * sizeof(int2), cudaMemcpyHostToDevice),
+    FP_TRY(cudaMemcpyAsync(c->lam_items, li.data(), li.size() * sizeof(int2), cudaMemcpyHostToDevice, s),
            "copy speed items");
   }
   {
@@ -733,7 +748,8 @@ int fp_init_grid(const fp_grid_desc *desc, const double *xyz, int ghost_nodes, v
     DirDev &D = c->hblk.dir[d];
     if (((long long)D.nt1 * D.nt2 + D.TT - 1) / D.TT < (long long)c->per_sm[0] * c->nsm) { D.S = 32; D.TT = c->nt[0] / 32; }
   }
-  int st = upload_items(c);
+  int st = upload_items(c, s);        // synchronises: everything above is done
+  cleanup_tmp();
   if (st != FP_OK) { fp_free(c); return st; }
 #undef FP_TRY
   *out = c;
@@ -998,7 +1014,7 @@ int fp_set_tile(fp_ctx *c, int dir, int faces, int lines) {
   const int S = c->hblk.dir[dir].S, TT = c->hblk.dir[dir].TT;
   c->hblk.dir[dir].S = faces;
   c->hblk.dir[dir].TT = lines;
-  const int st = upload_items(c);
+  const int st = upload_items(c, nullptr);
   if (st != FP_OK) {                              // the lists are still those of the old tile
     c->hblk.dir[dir].S = S;
     c->hblk.dir[dir].TT = TT;

@@ -916,29 +916,24 @@ int fp_cfl_dt(fp_ctx *c, const void *q, double cfl, double *dt_out, void *stream
   return FP_OK;
 }
 
-// n values of a device array of the context's type as doubles
-static cudaError_t read_back(const fp_ctx *c, const void *src, long long n, std::vector<double> &out) {
-  out.resize(n);
-  if (!c->is_f32) return cudaMemcpy(out.data(), src, n * sizeof(double), cudaMemcpyDeviceToHost);
-  std::vector<float> tmp(n);
-  cudaError_t e = cudaMemcpy(tmp.data(), src, n * sizeof(float), cudaMemcpyDeviceToHost);
-  std::copy(tmp.begin(), tmp.end(), out.begin());
-  return e;
-}
-
-static int get_metrics(fp_ctx *c, double *host_out) {
-  const long long n = c->nmet;
-  std::fill(host_out, host_out + 9 * n, 0.0);     // 2-D: no third metric vector
-  std::vector<double> kj;
-  for (int d = 0; d < c->desc.dims; ++d) {
-    cudaError_t e = read_back(c, c->kj[d], 4 * n, kj);
-    if (e != cudaSuccess) return cuda_fail(c, e, "fp_get_metrics copy");
-    for (long long i = 0; i < n; ++i) {
-      for (int a = 0; a < 3; ++a) host_out[(3 * d + a) * n + i] = kj[4 * i + a];
-      host_out[9 * n + i] = kj[4 * i + 3];
-    }
+// The values of packed metrics as [components][points] doubles on the host.  The device unpacks them,
+// into the residual accumulator, which holds nothing between two calls.  (120 x 100 x 64 points into
+// new memory: 10.6 ms with the loops over points on the host, 3.6 ms so; 40 x 36 x 30 FP64 567 | 160 us.)
+static cudaError_t read_back(const fp_ctx *c, const void *const a[3], int stride, int arrays, int comps, long long points,
+                             double *host_out) {
+  double *buf = static_cast<double *>(c->racc);
+  const long long room = (long long)((c->split ? c->desc.dims * split_stride(c) : (size_t)5 * c->ncells * c->esize) / sizeof(double));
+  const long long total = comps * points;
+  for (long long first = 0; first < total; first += room) {
+    const long long n = std::min(room, total - first);
+    cudaError_t e = fpk::unpack(a, c->is_f32, stride, 3, arrays, points, first, n, buf, nullptr);
+    // pages that the caller has not touched yet: the copy would have them mapped one by one for the
+    // device (129 ms instead of 19 for 4.8M points)
+    for (long long i = 0; i < n; i += 512) host_out[first + i] = 0.0;
+    if (e == cudaSuccess) e = cudaMemcpy(host_out + first, buf, n * sizeof(double), cudaMemcpyDeviceToHost);
+    if (e != cudaSuccess) return e;
   }
-  return FP_OK;
+  return cudaSuccess;
 }
 
 int fp_get_metrics(fp_ctx *c, double *host_out) {
@@ -946,7 +941,8 @@ int fp_get_metrics(fp_ctx *c, double *host_out) {
   if (!host_out) return fail(c, FP_ERR_ARG, "fp_get_metrics: null output");
   cudaError_t e = cudaDeviceSynchronize();
   if (e != cudaSuccess) return cuda_fail(c, e, "fp_get_metrics");
-  return get_metrics(c, host_out);
+  e = read_back(c, c->kj, 4, 3, 10, c->nmet, host_out);        // (2-D: no third metric vector)
+  return e == cudaSuccess ? FP_OK : cuda_fail(c, e, "fp_get_metrics copy");
 }
 
 int fp_get_face_metrics(fp_ctx *c, int dir, double *host_out) {
@@ -954,13 +950,9 @@ int fp_get_face_metrics(fp_ctx *c, int dir, double *host_out) {
   if (!host_out || dir < 0 || dir >= c->desc.dims) return fail(c, FP_ERR_ARG, "fp_get_face_metrics: bad argument");
   cudaError_t e = cudaDeviceSynchronize();
   if (e != cudaSuccess) return cuda_fail(c, e, "fp_get_face_metrics");
-  const long long nf = c->nface[dir];
-  std::vector<double> fk;
-  e = read_back(c, c->fk[dir], 6 * nf, fk);
-  if (e != cudaSuccess) return cuda_fail(c, e, "fp_get_face_metrics copy");
-  for (long long f = 0; f < nf; ++f)
-    for (int a = 0; a < 3; ++a) host_out[a * nf + f] = fk[6 * f + a];
-  return FP_OK;
+  const void *const fk[3] = {c->fk[dir], nullptr, nullptr};
+  e = read_back(c, fk, 6, 1, 3, c->nface[dir], host_out);
+  return e == cudaSuccess ? FP_OK : cuda_fail(c, e, "fp_get_face_metrics copy");
 }
 
 int fp_get_device_status(fp_ctx *c, void *stream) {

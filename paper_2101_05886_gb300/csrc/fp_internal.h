@@ -250,6 +250,11 @@ cudaError_t build_metrics(const MetricJob &J, cudaStream_t s);
 // The sweep's arrays (DirDev kj and fk) of direction d from the FP64 ones, in its type.
 cudaError_t pack_metrics(const MetricJob &J, int d, int is_f32, void *kj, cudaStream_t s);
 cudaError_t pack_faces(const MetricJob &J, int d, int is_f32, void *fk, cudaStream_t s);
+// The way back: values first .. first + n - 1 of the FP64 [components][points] array that packed arrays
+// hold, `per` components in each of `arrays` of them and the first one's next value behind these
+// (metrics: kj of three directions, per = 3, and 1/J; face metrics: one fk, per = 3).
+cudaError_t unpack(const void *const a[3], int is_f32, int stride, int per, int arrays, long long points,
+                   long long first, long long n, double *out, cudaStream_t s);
 
 // Global Lax-Friedrichs speeds (cfl.cu): zero, then max over (block, first point) items of
 // kLamChunk points each (the kernel's threads).

@@ -241,6 +241,20 @@ __global__ void k_pack_faces(const double *fm, int d, int n0, int n1, int n2, T 
   }
 }
 
+// values first .. first + n - 1 of the [components][points] array in FP64 that the packed arrays hold
+// (component c of array c / per, per components an array, of which a point has `stride` values side by
+// side; the value behind the last component is the first array's number per).  A null array is zero.
+template <typename T>
+__global__ void k_unpack(const T *a0, const T *a1, const T *a2, int stride, int per, int arrays, long long points,
+                         long long first, long long n, double *out) {
+  for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < n; t += (long long)gridDim.x * blockDim.x) {
+    const long long c = (first + t) / points, i = first + t - c * points;
+    const int d = c < arrays * per ? (int)(c / per) : 0, v = c < arrays * per ? (int)(c % per) : per;
+    const T *a = d == 0 ? a0 : (d == 1 ? a1 : a2);
+    out[t] = a ? (double)a[stride * i + v] : 0.0;
+  }
+}
+
 int grid_for(long long n) {
   long long g = (n + 255) / 256;
   if (g > 152LL * 64) g = 152LL * 64;
@@ -283,6 +297,17 @@ cudaError_t pack_faces(const MetricJob &J, int d, int is_f32, void *fk, cudaStre
     k_pack_faces<<<grid_for(nf), 256, 0, s>>>(J.fmet[d], d, J.n[0], J.n[1], J.n[2], static_cast<float *>(fk));
   else
     k_pack_faces<<<grid_for(nf), 256, 0, s>>>(J.fmet[d], d, J.n[0], J.n[1], J.n[2], static_cast<double *>(fk));
+  return cudaGetLastError();
+}
+
+cudaError_t unpack(const void *const a[3], int is_f32, int stride, int per, int arrays, long long points,
+                   long long first, long long n, double *out, cudaStream_t s) {
+  if (is_f32)
+    k_unpack<<<grid_for(n), 256, 0, s>>>(static_cast<const float *>(a[0]), static_cast<const float *>(a[1]),
+                                         static_cast<const float *>(a[2]), stride, per, arrays, points, first, n, out);
+  else
+    k_unpack<<<grid_for(n), 256, 0, s>>>(static_cast<const double *>(a[0]), static_cast<const double *>(a[1]),
+                                         static_cast<const double *>(a[2]), stride, per, arrays, points, first, n, out);
   return cudaGetLastError();
 }
 

@@ -119,6 +119,11 @@ template <typename T> struct CflScreen {
   }
 };
 
+// Blocks of at most one such CTA per SM: every point in FP64 by k_cfl_max alone, one per thread.  A
+// second kernel costs 2 to 5 us there, more than the screen saves (us a call, one kernel | two:
+// 4,320 points 30.6 | 34.5, 32,768 30.6 | 34.7, 65,120 42.6 | 34.3).
+constexpr long long kCflSmall = 152 * kCflThreads;
+
 template <typename T>
 __global__ void __launch_bounds__(kCflThreads) k_cfl_bound(const BlockDev *blk, long long ncells, int ni, int nj, int dims,
                                                            CflScratch *out, float2 *cta_hi) {
@@ -164,14 +169,19 @@ __global__ void __launch_bounds__(kCflThreads) k_cfl_max(const BlockDev *blk, lo
                                                          CflScratch *out, const float2 *cta_hi) {
   __shared__ long long red[kCflThreads / 32];
   chain_wait();
-  const float lo = __uint_as_float(*(volatile unsigned int *)&out->lower_bits);
-  const float2 hi = cta_hi[blockIdx.x];
-  if (hi.x < lo) return;
-  const bool all = hi.y >= lo;                      // every point of the CTA, without another look
+  float lo = 0.f;
+  bool all = true;                                  // every point of the CTA, without another look
+  if (cta_hi) {
+    lo = __uint_as_float(*(volatile unsigned int *)&out->lower_bits);
+    const float2 hi = cta_hi[blockIdx.x];
+    if (hi.x < lo) return;
+    all = hi.y >= lo;
+  }
   const CflScreen<T> screen(blk, ni, nj, dims);
+  const int points = cta_hi ? kCflPoints : 1;       // of a thread
   long long best = 0;                               // bits: non-negative doubles are ordered like them
-  for (int m = 0; m < kCflPoints; ++m) {
-    const long long idx = (long long)blockIdx.x * (kCflThreads * kCflPoints) + m * kCflThreads + threadIdx.x;
+  for (int m = 0; m < points; ++m) {
+    const long long idx = (long long)blockIdx.x * (kCflThreads * points) + m * kCflThreads + threadIdx.x;
     if (idx >= ncells) break;
     const long long mo = screen.place(idx);
     float l;
@@ -344,13 +354,17 @@ int cfl_ctas(long long ncells) { return (int)((ncells + kCflThreads * kCflPoints
 
 cudaError_t launch_cfl(const BlockDev *blk, int is_f32, long long ncells, const int *n, int dims,
                        CflScratch *scratch, cudaStream_t s) {
-  const int g = cfl_ctas(ncells);
+  // small blocks: one kernel over all points
+  const bool small = ncells <= kCflSmall;
+  const int g = small ? (int)((ncells + kCflThreads - 1) / kCflThreads) : cfl_ctas(ncells);
   float2 *hi = reinterpret_cast<float2 *>(scratch + 1);
-  cudaError_t e = launch_kernel(is_f32 ? k_cfl_bound<float> : k_cfl_bound<double>, g, kCflThreads, 0, s, 0, blk, ncells, n[0],
-                                n[1], dims, scratch, hi);
-  if (e != cudaSuccess) return e;
-  return launch_kernel(is_f32 ? k_cfl_max<float> : k_cfl_max<double>, g, kCflThreads, 0, s, 1, blk, ncells, n[0], n[1],
-                       dims, scratch, (const float2 *)hi);
+  if (!small) {
+    cudaError_t e = launch_kernel(is_f32 ? k_cfl_bound<float> : k_cfl_bound<double>, g, kCflThreads, 0, s, 0, blk, ncells,
+                                  n[0], n[1], dims, scratch, hi);
+    if (e != cudaSuccess) return e;
+  }
+  return launch_kernel(is_f32 ? k_cfl_max<float> : k_cfl_max<double>, g, kCflThreads, 0, s, small ? 0 : 1, blk, ncells, n[0],
+                       n[1], dims, scratch, small ? (const float2 *)nullptr : (const float2 *)hi);
 }
 
 }  // namespace fpk

@@ -1061,8 +1061,8 @@ static int batch_items_into(fp_batch *b, int d, const std::vector<int> *only_blo
   return FP_OK;
 }
 
-static int batch_items(fp_batch *b, int d, const std::vector<int> *only_blocks) {
-  return batch_items_into(b, d, only_blocks, true, &b->items[d], &b->ncta[d]);
+static int batch_items(fp_batch *b, int d, const std::vector<int> *only_blocks, bool alone) {
+  return batch_items_into(b, d, only_blocks, alone, &b->items[d], &b->ncta[d]);
 }
 
 static int batch_upload(fp_batch *b, cudaStream_t s) {
@@ -1097,9 +1097,9 @@ static int batch_pass(fp_batch *b, int d, int mode, int stage, cudaStream_t s, i
 }
 
 // Autotuner: for the batch's CTA shape, each direction and each line-length class, time every
-// tile of that shape on the blocks of that class and keep the best (tiles[a][d][k]: block k's
-// faces per chunk in direction d).
-static int batch_autotune(fp_batch *b, cudaStream_t s, std::vector<int> tiles[2][3]) {
+// tile of that shape on the blocks of that class, cut into items as the step's launches are, and keep
+// the best (tiles[a][d][k]: block k's faces per chunk in direction d).
+static int batch_autotune(fp_batch *b, bool alone, cudaStream_t s, std::vector<int> tiles[2][3]) {
   cudaEvent_t e0, e1;
   cudaEventCreate(&e0);
   cudaEventCreate(&e1);
@@ -1123,7 +1123,7 @@ static int batch_autotune(fp_batch *b, cudaStream_t s, std::vector<int> tiles[2]
           if (d == 0 && !b->anyS[a] && S != 32) continue;   // as fp_set_tile
           for (int k : members[cl]) { b->hblk[k].dir[d].S = S; b->hblk[k].dir[d].TT = b->nt[a] / S; }
           st = batch_upload(b, s);
-          if (!st) st = batch_items(b, d, &members[cl]);
+          if (!st) st = batch_items(b, d, &members[cl], alone);
           if (!st) st = batch_pass(b, d, fpk::MODE_WRITE, 0, s);           // warm-up
           if (st) break;
           cudaEventRecord(e0, s);
@@ -1238,18 +1238,19 @@ int fp_batch_create_linked(fp_ctx *const *blocks, int nblocks, void *const *q_de
       e = cudaMemcpy(b->lam_items, li.data(), li.size() * sizeof(int2), cudaMemcpyHostToDevice);
     if (e != cudaSuccess) { fp_batch_free(b); return e == cudaErrorMemoryAllocation ? FP_ERR_OOM : FP_ERR_CUDA; }
   }
+  const bool chains = !b->global_lf && nlinks == 0 && nblocks >= 2;   // the step runs as several
   int st = FP_OK;
   if (autotune) {
     std::vector<int> tiles[2][3];
-    st = batch_autotune(b, s, tiles);
+    st = batch_autotune(b, !chains, s, tiles);
     if (!st) batch_set_tiles(b, b->shape, tiles);
   }
   if (!st) st = batch_upload(b, s);
-  for (int d = 0; d < b->dims && !st; ++d) st = batch_items(b, d, nullptr);
+  for (int d = 0; d < b->dims && !st; ++d) st = batch_items(b, d, nullptr, true);
   if (st) { std::fprintf(stderr, "fp_batch_create: %s\n", b->err.c_str()); fp_batch_free(b); return st; }
   // graph branches: blocks split into groups of about equal point count, each group's
   // items built separately
-  if (!b->global_lf && nlinks == 0 && nblocks >= 2) {
+  if (chains) {
     b->nbranch = std::min(nblocks, (int)fp_batch::kMaxBranch);
     std::vector<long long> weight(nblocks);
     for (int k = 0; k < nblocks; ++k) weight[k] = blocks[k]->ncells;

@@ -41,7 +41,7 @@ struct fp_ctx {
   BlockDev uploaded;                  // last BlockDev copied to dblk
   fpk::SweepItem *items[3] = {nullptr, nullptr, nullptr};
   int ncta[3] = {0, 0, 0};            // CTAs of each direction's launch
-  // all directions in one launch (blocks of at most kSplitPoints points): its items
+  // all directions in one launch (blocks of at most split_points points): its items
   int split = 0;
   fpk::SweepItem *sitems = nullptr;
   int nscta = 0;
@@ -277,11 +277,25 @@ void sweep_constants(const fp_grid_desc &d, T *c) {
 
 // Blocks of at most this many points run a stage's direction passes as one launch, each direction
 // into an accumulator of its own, and a second launch that sums them: three times the work per
-// launch where a pass is a few chunks per CTA.  Measured (us, passes in turn | one launch; FP32 unless
-// said): 33^2 FP64 residual 111 | 59, 48x37x29 step 93 | 76, 200^2 FP64 shock step 1029 | 868,
-// 181x97x61 step 751 | 738, 112^3 871 | 844, 96^3 FP64 21591 | 21097; but 128x120x128 1147 | 1157 and
-// 256^3 8.67 | 9.19 ms, where the sum's traffic costs more than the passes' ends.
-constexpr long long kSplitPoints = 3 << 19;
+// launch where a pass is a few chunks per CTA, so the launch's uneven end counts for less.  The sum
+// moves 100 to 120 B a point at any size, while the end of a pass does not grow, so the line lies
+// lower the less time the passes take per point (linear upwind), or the shorter their ends are (WENO7,
+// which has half the CTAs per SM and so half the points in a last round).
+// A step in us, one launch | passes in turn, FP32:
+//   WENO5: 64^3 179 | 235, 92^3 481 | 494, 100^3 585 | 554, 60 x 60 x 300 655 | 690, 181 x 97 x 61 629 |
+//     619, 1000^2 392 | 417, 112^3 800 | 805, 1200^2 568 | 584, 116 x 115 x 114 864 | 848 (WENOCU6 alike)
+//   linear upwind: 64^3 126 | 154, 84^3 263 | 282, 92^3 343 | 334, 96^3 391 | 407; but 100^3 423 | 386,
+//     1000^2 285 | 276, 108^3 523 | 489
+//   WENO7: 64^3 241 | 275, 76^3 366 | 383, 88^3 553 | 564, 92^3 626 | 621; but 96^3 719 | 699, 100^3 805 |
+//     783, 1000^2 532 | 486
+// FP64, where a pass takes 20 times as long: 33^2 WENO5 187 | 340, 128^2 linear upwind 204 | 211, 96^3
+// WENO5 21.10 | 21.56 ms, 1000^2 15.36 | 15.31 ms, 1100^2 18.4 | 18.8 ms.
+long long split_points(int is_f32, int scheme) {
+  return is_f32 && scheme == FP_LINEAR_UPWIND5 ? 7 << 17 : (is_f32 && scheme == FP_WENO7_JS ? 3 << 18 : 3 << 19);
+}
+
+// blocks of more points than this make room for the packed metrics before they are built (fp_init_grid)
+constexpr long long kSmallPoints = 3 << 19;
 
 // bytes from one direction's accumulator to the next, 32-byte aligned
 size_t split_stride(const fp_ctx *c) { return ((size_t)5 * c->ncells * c->esize + 31) / 32 * 32; }
@@ -519,7 +533,7 @@ int upload_items(fp_ctx *c, cudaStream_t s) {
     fpk::SweepItem *dev = nullptr;
   } lists[4];
   std::vector<Stream> streams;
-  int split = c->ncells <= kSplitPoints;
+  int split = c->ncells <= split_points(c->is_f32, c->desc.scheme);
   const int sh0 = shape_of(c, c->hblk.dir[0]);
   for (int d = 0; d < c->desc.dims; ++d) {
     const int sh = shape_of(c, c->hblk.dir[d]);
@@ -701,7 +715,7 @@ int fp_init_grid(const fp_grid_desc *desc, const double *xyz, int ghost_nodes, v
   // metrics (six temporaries and a wait here | so, in ms: 48 x 37 x 29 FP32 1.36 | 0.79, 96^3 FP64
   // 4.0 | 3.3, 128^2 FP64 0.55 | 0.49).  In a large block the nodes and the scratch make room for the
   // packed arrays first.
-  if (c->ncells > kSplitPoints) {
+  if (c->ncells > kSmallPoints) {
     FP_TRY(cudaStreamSynchronize(s), "metric construction");
     cudaFree(nodes);
     nodes = nullptr;
@@ -712,14 +726,14 @@ int fp_init_grid(const fp_grid_desc *desc, const double *xyz, int ghost_nodes, v
     FP_TRY(fpk::dev_alloc(&c->fk[d], (size_t)6 * c->nface[d] * c->esize), "cudaMalloc(face metrics)");
     FP_TRY(fpk::pack_faces(J, d, c->is_f32, c->fk[d], s), "pack face metrics");
   }
-  if (c->ncells > kSplitPoints) {
+  if (c->ncells > kSmallPoints) {
     FP_TRY(cudaStreamSynchronize(s), "metric packing");
     cleanup_tmp();
   }
   const size_t sbytes = (size_t)5 * c->ncells * c->esize;
   FP_TRY(fpk::dev_alloc(&c->q1, sbytes), "cudaMalloc(stage 1)");
   FP_TRY(fpk::dev_alloc(&c->q2, sbytes), "cudaMalloc(stage 2)");
-  FP_TRY(fpk::dev_alloc(&c->racc, c->ncells <= kSplitPoints ? dims * split_stride(c) : sbytes), "cudaMalloc(residual)");
+  FP_TRY(fpk::dev_alloc(&c->racc, c->ncells <= split_points(c->is_f32, desc->scheme) ? dims * split_stride(c) : sbytes), "cudaMalloc(residual)");
   FP_TRY(fpk::dev_alloc(&c->status, sizeof(int)), "cudaMalloc(status)");
   FP_TRY(cudaMemsetAsync(c->status, 0, sizeof(int), s), "clear status");
   FP_TRY(fpk::dev_alloc(&c->dt_dev, sizeof(double)), "cudaMalloc(dt)");

@@ -1,5 +1,5 @@
 """The ways a stage is launched give the same bits: all directions in one launch with a sum behind it
-(blocks up to the library's limit of 3 * 2^19 points), chained passes in turn (beyond it, and in
+(blocks up to a limit by scheme and precision), chained passes in turn (beyond it, and in
 every batch), and the unchained passes of fp_rhs_noalloc; with boundary rules compiled into all
 directions or only into those that have such a side."""
 import ctypes
@@ -21,7 +21,7 @@ from paper_2101_05886_gb300 import binding as B  # noqa: E402
 from paper_2101_05886_gb300.solver import Batch, Block  # noqa: E402
 
 F64, F32 = B.FP_F64, B.FP_F32_MIXED
-LIMIT = 3 << 19
+LIMIT = {(0, F32): 3 << 19, (1, F32): 7 << 17, (2, F32): 3 << 18, (0, F64): 3 << 19}   # points, by scheme and precision
 
 
 def _setup(kind, n, scheme, precision, **kw):
@@ -81,12 +81,13 @@ def test_many_rounds_of_tiles(n, scheme, precision):
     _close(blk)
 
 
-# one point either side of the limit's nearest products
-@pytest.mark.parametrize("n,scheme,precision", [((181, 97, 89), 0, F32), ((181, 97, 90), 0, F32), ((181, 97, 90), 1, F32),
-                                                ((181, 97, 90), 2, F32), ((181, 97, 90), 0, F64)])
+# just below and just above each limit
+@pytest.mark.parametrize("n,scheme,precision", [
+    ((181, 97, 89), 0, F32), ((181, 97, 90), 0, F32), ((181, 97, 52), 1, F32), ((181, 97, 53), 1, F32),
+    ((181, 97, 44), 2, F32), ((181, 97, 45), 2, F32), ((181, 97, 89), 0, F64), ((181, 97, 90), 0, F64)])
 def test_steps_on_either_side_of_the_limit(n, scheme, precision):
     blk, q = _setup("wall", n, scheme, precision)
-    assert B.lib().fp_launches_per_rhs(blk.ctx) == (2 if np.prod(n) <= LIMIT else 3)
+    assert B.lib().fp_launches_per_rhs(blk.ctx) == (2 if np.prod(n) <= LIMIT[scheme, precision] else 3)
     dt = blk.cfl_dt(q, 0.4)
     a, b = q.clone(), q.clone()
     bat = Batch([blk], [b], autotune=False)

@@ -43,7 +43,8 @@ template <typename T> struct Num;
 template <> struct Num<double> {
   // reciprocal of a finite nonzero x: the PTX approximation (relative error about 2^-20) and one
   // step of Householder's third-order iteration, y <- y + y (e + e^2) with e = 1 - x y, which
-  // cubes the error (three operations; two Newton-Raphson steps take four)
+  // cubes the error (three operations; two Newton-Raphson steps take four): within 2^-53 (1 + 2^-4)
+  // of 1/x, as tested
   static __device__ __forceinline__ double rcp(double x) {
     double y;
     asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
@@ -61,9 +62,6 @@ template <> struct Num<double> {
   static __device__ __forceinline__ double rsqrt_(double x) { return rsqrt(x); }
   // sqrt(a b): one root of the product, which stays in range up to 1e308
   static __device__ __forceinline__ double sqrt_product(double a, double b) { return sqrt(a * b); }
-  static __device__ __forceinline__ double ld(const void *p, long long i) {
-    return __ldg(static_cast<const double *>(p) + i);
-  }
 };
 template <> struct Num<float> {
   // the PTX approximate reciprocal (one MUFU operation, max relative error 2^-23);
@@ -84,9 +82,6 @@ template <> struct Num<float> {
   // sqrt(a b) by two roots: c^2 |k|^2 leaves the FP32 range where c |k| passes 1.8e19 (sound speeds
   // in m/s on cells of 1e8 m) though both factors are far inside it
   static __device__ __forceinline__ float sqrt_product(float a, float b) { return sqrt_(a) * sqrt_(b); }
-  static __device__ __forceinline__ float ld(const void *p, long long i) {
-    return __ldg(static_cast<const float *>(p) + i);
-  }
 };
 
 // Pairs of values processed by one instruction: packed FP32x2 arithmetic (sm_100+

@@ -57,10 +57,10 @@ ALG_FLOPS_PER_POINT_PASS = {"weno5_char": 2000.0, "lu5_char": 700.0}
 # counted by ncu on an 8-block subset (FFMA 2, FFMA2 4, FADD/FMUL 1, FADD2/FMUL2 2): reported
 # beside the algorithmic count.
 EXEC_FLOPS_PER_POINT_PASS = {"weno5_char": 2140.0, "lu5_char": 1090.0}
-# DRAM bytes per point per direction pass measured by ncu (8-block capture, first stage, mean of
-# the xi, eta and zeta passes: 74, 96 and 100 B), scaled to a pass over the workload.  The
-# linear-upwind sweep makes the same loads and stores.
-TRAFFIC_BYTES_PER_POINT_PASS = {"weno5_char": 90.0, "lu5_char": 90.0}
+# DRAM bytes per point per direction pass measured by ncu (8 blocks of the workload, cold caches),
+# the mean over the nine passes of an RK step: those of the last direction also read Q^n in stages
+# 2 and 3 (WENO5 about 72, 95 and 97 B in stage 1, 121 B in the last passes of the others).
+TRAFFIC_BYTES_PER_POINT_PASS = {"weno5_char": 86.4, "lu5_char": 80.8}
 ORACLE_SAMPLE_N = 32           # side of the O-grid block each host core advances (both CPU arms)
 
 

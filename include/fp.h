@@ -240,7 +240,8 @@ int fp_get_cta_sizes(const fp_ctx *ctx, int *primary, int *alternative);
    Results do not depend on it. */
 int fp_get_tile(const fp_ctx *ctx, int dir, int *faces, int *lines);
 /* Override the tile shape: faces in {8,16,32}, faces x lines one of fp_get_cta_sizes; the
-   64-thread size takes 32 faces along xi only (FP_ERR_ARG otherwise). */
+   64-thread size takes 32 faces along xi only (FP_ERR_ARG otherwise).  A failed call
+   (FP_ERR_OOM) leaves the context as it was. */
 int fp_set_tile(fp_ctx *ctx, int dir, int faces, int lines);
 
 const char *fp_last_error(const fp_ctx *ctx);

@@ -48,7 +48,8 @@ struct fp_ctx {
   int nsm = 152;
   // CTA shapes of the context's sweep: [0] the primary one, [1] the alternative (nshape == 2,
   // the folded FP32 sweeps): threads (faces per chunk x lines per tile), whether fp_set_tile takes
-  // other than 32 faces along xi (not for the 64-thread shape), resident CTAs per SM
+  // other than 32 faces along xi (not for the 64-thread shape: the sweep could, but its interface has
+  // always refused them, and the autotuner would gain 0.3 % from them), resident CTAs per SM
   int nshape = 1;
   int nt[2] = {128, 128}, anyS[2] = {1, 1}, per_sm[2] = {1, 1};
   int dev = 0;                        // the device the context's memory lives on
@@ -434,7 +435,7 @@ void spread_stream(const Stream &s, long long first, long long most, std::vector
 //    of them (256^3 WENO5 step, when introduced: 8.93 ms, 9.75 ms with all rounds in one item,
 //    9.97 ms with a CTA per tile in a fixed order and lines padded to chunks).  The blocks of a batch
 //    with several chains keep one item for all rounds: its graph's other branches fill the SMs
-//    that end early (64-block WENO5 step: 18.04 ms, 18.25 ms with two rounds per item).
+//    that end early (64-block WENO5 step: 16.27 ms, 16.39 ms with two rounds per item).
 int make_items(const std::vector<Stream> &streams, int slots, bool alone, std::vector<fpk::SweepItem> &items) {
   std::vector<fpk::SweepItem> list, piece;        // in the order made, `next` within the list
   std::vector<int> head(slots, -1), tail(slots, -1);   // of each CTA
@@ -788,6 +789,8 @@ static int run_stage(fp_ctx *c, int stage, int rk, int chained, cudaStream_t s) 
     L.stage = stage;
     L.dt = c->dt_dev;
     L.alt = shape_of(c, c->hblk.dir[0]);
+    // one side with a boundary rule takes all directions into that variant (an O-grid of 140 x 110 x 100
+    // points, WENO5: a step 877 us with zero-gradient sides, 894 us with a wall)
     for (int d = 0; d < dims; ++d) L.bnd |= has_bnd(c->desc, d);
     L.glf = c->desc.global_lf;
     // FP64 CTAs, one or two per SM, have to be placed evenly, which the rest of a kernel before them

@@ -13,7 +13,7 @@ BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libfpgb300.so")
 LIB_CHECK = os.path.join(HERE, "libfpgb300_check.so")
 SOURCES = ["api.cu", "pipe.cu", "metrics.cu", "cfl.cu", "stage.cu", "probe.cu", "sweep_f32.cu", "sweep_f32_fix.cu", "sweep_f32_fix2.cu",
-           "sweep_f32_comp.cu", "sweep_f32_bnd.cu", "sweep_f32_bnd_fix.cu", "sweep_f32_bnd_fix2.cu", "sweep_f32_bnd_comp.cu",
+           "sweep_f32_comp.cu", "sweep_f32_wide.cu", "sweep_f32_bnd.cu", "sweep_f32_bnd_fix.cu", "sweep_f32_bnd_fix2.cu", "sweep_f32_bnd_comp.cu", "sweep_f32_bnd_wide.cu",
            "sweep_f64.cu", "sweep_f64_fix.cu", "sweep_f64_comp.cu", "sweep_f64_bnd.cu", "sweep_f64_bnd_fix.cu",
            "sweep_f64_bnd_comp.cu"]
 HEADERS = ["fp_internal.h", "sweep.cuh"]

@@ -69,6 +69,7 @@ struct fp_batch {
   cudaGraph_t graph = nullptr;
   cudaGraphExec_t exec = nullptr;
   int dims = 3, M = 6, scheme = 0, charwise = 1, fp = 1, is_f32 = 1, global_lf = 0;
+  int wide = 0;             // some block's state is far from unit scale
   int bnd[3] = {0, 0, 0};   // some block has a slip-wall or cut side in direction d
   // Graph branches: groups of blocks whose RK steps run as independent chains of the graph,
   // so one group's launches fill the end-of-pass tail of another's.  One branch when blocks
@@ -205,13 +206,14 @@ int ghost_of(int M, int scheme) { return std::max(scheme == FP_WENO7_JS ? 4 : 3,
 // shared memory
 int prepare(int is_f32, int M, int scheme, int fix) {
   using P = int (*)(int, int);
-  const P f32[8] = {fpk::prepare_sweep_f32,     fpk::prepare_sweep_f32_fix,     fpk::prepare_sweep_f32_fix2,
-                    fpk::prepare_sweep_f32_comp, fpk::prepare_sweep_f32_bnd,    fpk::prepare_sweep_f32_bnd_fix,
-                    fpk::prepare_sweep_f32_bnd_fix2, fpk::prepare_sweep_f32_bnd_comp};
-  const P f64[8] = {fpk::prepare_sweep_f64,     fpk::prepare_sweep_f64_fix, nullptr, fpk::prepare_sweep_f64_comp,
-                    fpk::prepare_sweep_f64_bnd, fpk::prepare_sweep_f64_bnd_fix, nullptr, fpk::prepare_sweep_f64_bnd_comp};
+  const P f32[10] = {fpk::prepare_sweep_f32,          fpk::prepare_sweep_f32_fix,      fpk::prepare_sweep_f32_fix2,
+                     fpk::prepare_sweep_f32_comp,     fpk::prepare_sweep_f32_wide,     fpk::prepare_sweep_f32_bnd,
+                     fpk::prepare_sweep_f32_bnd_fix,  fpk::prepare_sweep_f32_bnd_fix2, fpk::prepare_sweep_f32_bnd_comp,
+                     fpk::prepare_sweep_f32_bnd_wide};
+  const P f64[10] = {fpk::prepare_sweep_f64,     fpk::prepare_sweep_f64_fix,     nullptr, fpk::prepare_sweep_f64_comp,     nullptr,
+                     fpk::prepare_sweep_f64_bnd, fpk::prepare_sweep_f64_bnd_fix, nullptr, fpk::prepare_sweep_f64_bnd_comp, nullptr};
   const P *p = is_f32 ? f32 : f64;
-  return std::min(p[fix](M, scheme), p[4 + fix](M, scheme));
+  return std::min(p[fix](M, scheme), p[5 + fix](M, scheme));
 }
 
 // the CTA shapes of a sweep (fp_internal.h sweep_threads) and their resident CTAs per SM
@@ -233,10 +235,21 @@ int shape_of(const C *c, const fpk::DirDev &D) {
   return c->nshape == 2 && D.S * D.TT == c->nt[1] ? 1 : 0;
 }
 
-// the sweep's variant: 3 component-wise; 1 switches folded, for characteristic FP sweeps with
-// local speeds (not for WENOCU6, whose sweep measured 1 % slower with them folded); 0 the rest
-int fix_of(int scheme, int charwise, int fp, int global_lf) {
-  return !charwise ? 3 : (fp && !global_lf && scheme != FP_WENOCU6 ? 1 : 0);
+// the sweep's variant: 4 for states far from unit scale (is_wide); 3 component-wise; 1 switches
+// folded, for characteristic FP sweeps with local speeds (not for WENOCU6, whose sweep measured
+// 1 % slower with them folded); 0 the rest
+int fix_of(int scheme, int charwise, int fp, int global_lf, int wide) {
+  return wide ? 4 : (!charwise ? 3 : (fp && !global_lf && scheme != FP_WENOCU6 ? 1 : 0));
+}
+
+// FP32 FP-form blocks whose far-field state, which has the units of the flow, has momenta whose
+// squares leave the FP32 range 2^-126 .. 2^128 when they differ from point to point by 1e-7 (z^2 of
+// that size still counts against z) or by 1e3, at densities up to 1e3 times larger or smaller
+int is_wide(const fp_grid_desc &d) {
+  if (d.precision != FP_F32_MIXED || !d.free_stream_preserving) return 0;
+  const double *q = d.q_inf, m2 = q[1] * q[1] + q[2] * q[2] + q[3] * q[3];
+  const double rc2 = d.gamma * (d.gamma - 1.0) * (q[4] * q[0] - 0.5 * m2);   // (rho c)^2
+  return !(m2 + rc2 > 0x1p-60 && m2 + rc2 < 0x1p+90);
 }
 
 // the variant of the launch: boundary rules compiled in when some block of the launch has such a
@@ -244,14 +257,15 @@ int fix_of(int scheme, int charwise, int fp, int global_lf) {
 cudaError_t launch(int is_f32, const fpk::SweepLaunch &L, int M, int scheme, int charwise, int fp,
                    cudaStream_t s) {
   using F = cudaError_t (*)(const fpk::SweepLaunch &, int, int, int, cudaStream_t);
-  const F f32[8] = {fpk::launch_sweep_f32,     fpk::launch_sweep_f32_fix,     fpk::launch_sweep_f32_fix2,
-                    fpk::launch_sweep_f32_comp, fpk::launch_sweep_f32_bnd,    fpk::launch_sweep_f32_bnd_fix,
-                    fpk::launch_sweep_f32_bnd_fix2, fpk::launch_sweep_f32_bnd_comp};
-  const F f64[8] = {fpk::launch_sweep_f64,     fpk::launch_sweep_f64_fix, nullptr, fpk::launch_sweep_f64_comp,
-                    fpk::launch_sweep_f64_bnd, fpk::launch_sweep_f64_bnd_fix, nullptr, fpk::launch_sweep_f64_bnd_comp};
-  int v = fix_of(scheme, charwise, fp, L.glf);
+  const F f32[10] = {fpk::launch_sweep_f32,          fpk::launch_sweep_f32_fix,      fpk::launch_sweep_f32_fix2,
+                     fpk::launch_sweep_f32_comp,     fpk::launch_sweep_f32_wide,     fpk::launch_sweep_f32_bnd,
+                     fpk::launch_sweep_f32_bnd_fix,  fpk::launch_sweep_f32_bnd_fix2, fpk::launch_sweep_f32_bnd_comp,
+                     fpk::launch_sweep_f32_bnd_wide};
+  const F f64[10] = {fpk::launch_sweep_f64,     fpk::launch_sweep_f64_fix,     nullptr, fpk::launch_sweep_f64_comp,     nullptr,
+                     fpk::launch_sweep_f64_bnd, fpk::launch_sweep_f64_bnd_fix, nullptr, fpk::launch_sweep_f64_bnd_comp, nullptr};
+  int v = fix_of(scheme, charwise, fp, L.glf, L.wide);
   if (v == 1 && is_f32 && L.alt) v = 2;
-  return (is_f32 ? f32 : f64)[(L.bnd ? 4 : 0) + v](L, M, scheme, fp, s);
+  return (is_f32 ? f32 : f64)[(L.bnd ? 5 : 0) + v](L, M, scheme, v == 4 && !charwise ? fp | 2 : fp, s);
 }
 
 // default tile of a direction for a CTA of nt threads: 32 faces along xi, 8 across lines
@@ -751,7 +765,7 @@ int fp_init_grid(const fp_grid_desc *desc, const double *xyz, int ghost_nodes, v
            "copy speed items");
   }
   {
-    const int fix = fix_of(desc->scheme, desc->characteristic, desc->free_stream_preserving, desc->global_lf);
+    const int fix = fix_of(desc->scheme, desc->characteristic, desc->free_stream_preserving, desc->global_lf, is_wide(*desc));
     set_shapes(c, c->is_f32, M, desc->scheme, fix);
     fill_dirs(c);
   }
@@ -793,6 +807,7 @@ static int run_stage(fp_ctx *c, int stage, int rk, int chained, cudaStream_t s) 
     // points, WENO5: a step 877 us with zero-gradient sides, 894 us with a wall)
     for (int d = 0; d < dims; ++d) L.bnd |= has_bnd(c->desc, d);
     L.glf = c->desc.global_lf;
+    L.wide = is_wide(c->desc);
     // FP64 CTAs, one or two per SM, have to be placed evenly, which the rest of a kernel before them
     // prevents (128^2 linear upwind: a step 221 us chained, 204 us not)
     L.chained = chained && c->is_f32;
@@ -813,6 +828,7 @@ static int run_stage(fp_ctx *c, int stage, int rk, int chained, cudaStream_t s) 
     L.alt = shape_of(c, c->hblk.dir[d]);
     L.bnd = has_bnd(c->desc, d);
     L.glf = c->desc.global_lf;
+    L.wide = is_wide(c->desc);
     L.chained = (chained || d > 0) && c->is_f32;
     cudaError_t e = launch(c->is_f32, L, M, c->desc.scheme, c->desc.characteristic,
                            c->desc.free_stream_preserving, s);
@@ -1102,6 +1118,7 @@ static int batch_pass_items(fp_batch *b, int d, int mode, int stage, cudaStream_
   L.alt = shape_of(b, b->hblk[0].dir[d]);   // every block of a batch pass has the same shape
   L.bnd = b->bnd[d];
   L.glf = b->global_lf;
+  L.wide = b->wide;
   L.chained = chained && b->is_f32;
   cudaError_t e = launch(b->is_f32, L, b->M, b->scheme, b->charwise, b->fp, s);
   if (e != cudaSuccess) return bfail(b, FP_ERR_CUDA, std::string("batch sweep: ") + cudaGetErrorString(e));
@@ -1215,13 +1232,19 @@ int fp_batch_create_linked(fp_ctx *const *blocks, int nblocks, void *const *q_de
   b->charwise = d0.characteristic; b->fp = d0.free_stream_preserving;
   b->is_f32 = d0.precision == FP_F32_MIXED;
   b->global_lf = d0.global_lf;
-  b->nshape = blocks[0]->nshape;
-  for (int a = 0; a < 2; ++a) {
-    b->nt[a] = blocks[0]->nt[a];
-    b->anyS[a] = blocks[0]->anyS[a];
-    b->per_sm[a] = blocks[0]->per_sm[a];
+  for (int k = 0; k < nblocks; ++k) b->wide |= is_wide(blocks[k]->desc);
+  const int fix = fix_of(b->scheme, b->charwise, b->fp, b->global_lf, b->wide);
+  if (b->wide) {                      // (the blocks' own variants may differ)
+    set_shapes(b, b->is_f32, b->M, b->scheme, fix);
+  } else {
+    b->nshape = blocks[0]->nshape;
+    for (int a = 0; a < 2; ++a) {
+      b->nt[a] = blocks[0]->nt[a];
+      b->anyS[a] = blocks[0]->anyS[a];
+      b->per_sm[a] = blocks[0]->per_sm[a];
+    }
   }
-  b->shape = fpk::sweep_batch_shape(b->is_f32, b->scheme, fix_of(b->scheme, b->charwise, b->fp, b->global_lf));
+  b->shape = fpk::sweep_batch_shape(b->is_f32, b->scheme, fix);
   b->nsm = blocks[0]->nsm;
   for (int k = 0; k < nblocks; ++k) {
     b->ctx.push_back(blocks[k]);
@@ -1429,6 +1452,7 @@ extern "C" int fp_rhs_noalloc(fp_ctx *c, const void *q, void *dqdt, void *stream
     L.alt = shape_of(c, c->hblk.dir[d]);
     L.bnd = has_bnd(c->desc, d);
     L.glf = c->desc.global_lf;
+    L.wide = is_wide(c->desc);
     e = launch(c->is_f32, L, M, c->desc.scheme, c->desc.characteristic, c->desc.free_stream_preserving, s);
     if (e != cudaSuccess) return cuda_fail(c, e, "fp_rhs_noalloc: sweep launch");
   }

@@ -13,7 +13,7 @@ constexpr int kNextFields = 21;      // staged per thread: next chunk's cell (Q,
 constexpr int kEpiFields = 10;       // epilogue operands staged per thread (accumulator, Q^n)
 
 // CTA shape of a sweep variant (precision, scheme, fix: 0 switches read at run time, 1 folded,
-// 2 folded with the alternative shape, 3 component-wise): its threads, which equal faces per chunk x
+// 2 folded with the alternative shape, 3 component-wise, 4 states far from unit scale): its threads, which equal faces per chunk x
 // lines per tile, whether the rings of the xi pass are padded (none is: turning the slots of
 // every other group of lines keeps all tile shapes free of bank conflicts), and the CTAs one SM
 // holds.
@@ -166,23 +166,27 @@ struct SweepLaunch {
   int bnd = 0;         // some block of the launch has a slip-wall or cut side in a swept direction
   int glf = 0;         // the blocks of the launch use global Lax-Friedrichs speeds
   int alt = 0;         // the blocks' tiles are of the alternative CTA shape
+  int wide = 0;        // some block's state is far from unit scale (FP32: the sweep that squares no momenta)
   int chained = 0;     // the kernel before it in the stream may still run (launch_kernel)
 };
 
 // Launchers of the sweep, one per translation unit (sweep_<NAME>.cu): precision f32 / f64,
 // `_bnd` with the slip-wall, cut, link and halo rules compiled in, `_fix` with the
 // characteristic decomposition and the FP form fixed on, `_fix2` the same in the alternative
-// CTA shape (FP32 only), `_comp` component-wise.  Each returns the cudaError_t of the
+// CTA shape (FP32 only), `_comp` component-wise, `_wide` for states far from unit scale (FP32 only; `fp`
+// there is 2 bits: the FP form, component-wise).  Each returns the cudaError_t of the
 // launch; prepare_sweep_<NAME> opts in to the dynamic shared memory of its 16 (M, scheme)
 // variants and returns the resident CTAs per SM of the given one.
 cudaError_t launch_sweep_f32(const SweepLaunch &L, int M, int scheme, int fp, cudaStream_t s);
 cudaError_t launch_sweep_f32_fix(const SweepLaunch &L, int M, int scheme, int fp, cudaStream_t s);
 cudaError_t launch_sweep_f32_fix2(const SweepLaunch &L, int M, int scheme, int fp, cudaStream_t s);
 cudaError_t launch_sweep_f32_comp(const SweepLaunch &L, int M, int scheme, int fp, cudaStream_t s);
+cudaError_t launch_sweep_f32_wide(const SweepLaunch &L, int M, int scheme, int fp, cudaStream_t s);
 cudaError_t launch_sweep_f32_bnd(const SweepLaunch &L, int M, int scheme, int fp, cudaStream_t s);
 cudaError_t launch_sweep_f32_bnd_fix(const SweepLaunch &L, int M, int scheme, int fp, cudaStream_t s);
 cudaError_t launch_sweep_f32_bnd_fix2(const SweepLaunch &L, int M, int scheme, int fp, cudaStream_t s);
 cudaError_t launch_sweep_f32_bnd_comp(const SweepLaunch &L, int M, int scheme, int fp, cudaStream_t s);
+cudaError_t launch_sweep_f32_bnd_wide(const SweepLaunch &L, int M, int scheme, int fp, cudaStream_t s);
 cudaError_t launch_sweep_f64(const SweepLaunch &L, int M, int scheme, int fp, cudaStream_t s);
 cudaError_t launch_sweep_f64_fix(const SweepLaunch &L, int M, int scheme, int fp, cudaStream_t s);
 cudaError_t launch_sweep_f64_comp(const SweepLaunch &L, int M, int scheme, int fp, cudaStream_t s);
@@ -193,10 +197,12 @@ int prepare_sweep_f32(int M, int scheme);
 int prepare_sweep_f32_fix(int M, int scheme);
 int prepare_sweep_f32_fix2(int M, int scheme);
 int prepare_sweep_f32_comp(int M, int scheme);
+int prepare_sweep_f32_wide(int M, int scheme);
 int prepare_sweep_f32_bnd(int M, int scheme);
 int prepare_sweep_f32_bnd_fix(int M, int scheme);
 int prepare_sweep_f32_bnd_fix2(int M, int scheme);
 int prepare_sweep_f32_bnd_comp(int M, int scheme);
+int prepare_sweep_f32_bnd_wide(int M, int scheme);
 int prepare_sweep_f64(int M, int scheme);
 int prepare_sweep_f64_fix(int M, int scheme);
 int prepare_sweep_f64_comp(int M, int scheme);

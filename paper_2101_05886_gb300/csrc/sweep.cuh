@@ -405,9 +405,14 @@ __device__ __forceinline__ void dflux_pair(T g1, P rinvB, const P uB[3], const P
 // V is any fixed number for this: its own rounding cancels.  EpP = E* + p* = p* gamma/(gamma-1).
 // With the reconstruction below and the velocities out of the shared ring: 64-block WENO5 step
 // 18.04 -> 17.24 ms, 256^3 9.05 -> 8.65 ms, 96^3 FP64 24.5 -> 21.7 ms.
-template <typename T>
+// z.z leaves the FP32 range where momenta differ by more than 1.8e19, and loses digits that count where
+// they are below about 1e-16 (densities of 1e-24 kg/m^3).  WIDE forms the velocity differences
+// w = z/rho_B first, z.z/rho_B = z.w, dU = w.k, and out[0] = d_0 U_B + rho* dU (rs = rho*): no squares of
+// momenta, one operation and three registers more (64-block step 16.27 | 16.52 ms, WENO7 672 |
+// 686 us), so the sweeps of ordinary states do without.
+template <typename T, bool WIDE>
 __device__ __forceinline__ void dflux_frame(T g1, typename PairOf<T>::type rinvB, typename PairOf<T>::type UB,
-                                            const T V[3], T hV2, T EpP, typename PairOf<T>::type d[5],
+                                            T rs, const T V[3], T hV2, T EpP, typename PairOf<T>::type d[5],
                                             const typename PairOf<T>::type k[3],
                                             typename PairOf<T>::type out[5]) {
   using P = typename PairOf<T>::type;
@@ -416,11 +421,19 @@ __device__ __forceinline__ void dflux_frame(T g1, typename PairOf<T>::type rinvB
 #pragma unroll
   for (int c = 0; c < 3; ++c) d[4] = pfma(pc<P>(-V[c]), d[1 + c], d[4]);
   d[4] = pfma(pc<P>(-hV2), d[0], d[4]);
-  const P zz = pfma(d[3], d[3], pfma(d[2], d[2], pmul(d[1], d[1])));
-  const P zk = pfma(d[3], k[2], pfma(d[2], k[1], pmul(d[1], k[0])));
-  const P dp = pmul(pc<P>(g1), pfma(pc<P>(T(-0.5)), pmul(rinvB, zz), d[4]));
-  const P dU = pmul(rinvB, zk);
-  out[0] = pfma(d[0], psub(UB, dU), zk);
+  P zz, dU;                                          // z.z/rho_B, dU
+  if constexpr (WIDE) {
+    const P w[3] = {pmul(rinvB, d[1]), pmul(rinvB, d[2]), pmul(rinvB, d[3])};
+    zz = pfma(d[3], w[2], pfma(d[2], w[1], pmul(d[1], w[0])));
+    dU = pfma(w[2], k[2], pfma(w[1], k[1], pmul(w[0], k[0])));
+    out[0] = pfma(d[0], UB, pmul(pc<P>(rs), dU));
+  } else {
+    const P zk = pfma(d[3], k[2], pfma(d[2], k[1], pmul(d[1], k[0])));
+    zz = pmul(rinvB, pfma(d[3], d[3], pfma(d[2], d[2], pmul(d[1], d[1]))));
+    dU = pmul(rinvB, zk);
+    out[0] = pfma(d[0], psub(UB, dU), zk);
+  }
+  const P dp = pmul(pc<P>(g1), pfma(pc<P>(T(-0.5)), zz, d[4]));
 #pragma unroll
   for (int c = 0; c < 3; ++c) out[1 + c] = pfma(dp, k[c], pmul(d[1 + c], UB));
   out[4] = pfma(padd(dp, pc<P>(EpP)), dU, pmul(d[4], UB));
@@ -445,7 +458,8 @@ template <typename T> struct RkStage {
 // sweep_threads (fp_internal.h).  FIX = 0: characteristic, the FP form and the speeds read from
 // the arguments and the block descriptor.  FIX = 3: component-wise, the others as FIX = 0 (one
 // variant for both decompositions held the operands of both and spilled: linear upwind on
-// 70 x 80 x 22 points, component-wise, 208 us a step against 149).
+// 70 x 80 x 22 points, component-wise, 208 us a step against 149).  FIX = 4: all three read at run
+// time, and no squares of momenta (dflux_frame).
 template <typename T, int M, int SCHEME, bool BND, int FIX>
 __global__ void __launch_bounds__(sweep_threads(sizeof(T) == 4, SCHEME, FIX), sweep_min_ctas(sizeof(T) == 4, SCHEME, FIX))
 fp_sweep(const BlockDev *__restrict__ blocks, const SweepItem *__restrict__ items, int mode,
@@ -454,8 +468,8 @@ fp_sweep(const BlockDev *__restrict__ blocks, const SweepItem *__restrict__ item
   constexpr int kThreads = sweep_threads(sizeof(T) == 4, SCHEME, FIX);
   constexpr int kRing = sweep_ring(sizeof(T) == 4, SCHEME, FIX);
   constexpr bool kFold = FIX == 1 || FIX == 2;
-  constexpr int charwise = FIX == 3 ? 0 : 1;
-  const int fpform = kFold ? 1 : fpform_arg;
+  const int charwise = FIX == 3 ? 0 : (FIX == 4 ? !(fpform_arg & 2) : 1);
+  const int fpform = kFold ? 1 : (FIX == 4 ? fpform_arg & 1 : fpform_arg);
   // stencil points of a face: i-2..i+3 (5th order) or i-3..i+4 (WENO7), offset index Q0
   constexpr int NS = SCHEME == 2 ? 8 : 6;
   constexpr int Q0 = SCHEME == 2 ? 0 : 1;
@@ -839,12 +853,13 @@ fp_sweep(const BlockDev *__restrict__ blocks, const SweepItem *__restrict__ item
           for (int v = 0; v < 5; ++v) dl[v] = (acc[v].x + acc[v].y) * wi;
         }
         // the frame of the face: velocity V = u* (0 for the plain scheme), see dflux_frame
-        T V[3] = {T(0), T(0), T(0)}, hV2 = T(0), EpP = T(0);
+        T V[3] = {T(0), T(0), T(0)}, hV2 = T(0), EpP = T(0), rhos = T(0);
         if (fpform) {
           T Qs[5];
 #pragma unroll
           for (int v = 0; v < 5; ++v) Qs[v] = Qi[v] + dl[v];
-          const T rinvs = Num<T>::rcp(Qs[0]);
+          rhos = Qs[0];
+          const T rinvs = Num<T>::rcp(rhos);
 #pragma unroll
           for (int c = 0; c < 3; ++c) V[c] = Qs[1 + c] * rinvs;
           hV2 = T(0.5) * (V[0] * V[0] + V[1] * V[1] + V[2] * V[2]);
@@ -1005,7 +1020,7 @@ fp_sweep(const BlockDev *__restrict__ blocks, const SweepItem *__restrict__ item
               const P UBp = pmul(pmk(CELL(CF_UC, q), CELL(CF_UC, q2)), ijp);
               const P dlab[3] = {dp[1], dp[2], dp[3]};
               const P elab = dp[4];
-              dflux_frame<T>(g1, rip, UBp, V, hV2, EpP, dp, kp2, out);
+              dflux_frame<T, FIX == 4>(g1, rip, UBp, rhos, V, hV2, EpP, dp, kp2, out);
               if (!charwise) {       // the components are those of the laboratory frame
                 to_lab(out);
                 dp[1] = dlab[0]; dp[2] = dlab[1]; dp[3] = dlab[2]; dp[4] = elab;
@@ -1081,7 +1096,7 @@ fp_sweep(const BlockDev *__restrict__ blocks, const SweepItem *__restrict__ item
               const P UBp = pmul(pmk(CELL(CF_UC, q), CELL(CF_UC, q2)), ijp);
               const P dlab[3] = {dp[1], dp[2], dp[3]};
               const P elab = dp[4];
-              dflux_frame<T>(g1, pmk(CELL(CF_RINV, q), CELL(CF_RINV, q2)), UBp, V, hV2, EpP, dp, kp2, out);
+              dflux_frame<T, FIX == 4>(g1, pmk(CELL(CF_RINV, q), CELL(CF_RINV, q2)), UBp, rhos, V, hV2, EpP, dp, kp2, out);
               if (!charwise) {       // the components are those of the laboratory frame
                 to_lab(out);
                 dp[1] = dlab[0]; dp[2] = dlab[1]; dp[3] = dlab[2]; dp[4] = elab;

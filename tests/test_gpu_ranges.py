@@ -19,13 +19,13 @@ if not torch.cuda.is_available():
     pytest.skip("CUDA device required", allow_module_level=True)
 
 from paper_2101_05886_gb300 import binding as B  # noqa: E402
-from paper_2101_05886_gb300.solver import Block  # noqa: E402
+from paper_2101_05886_gb300.solver import Batch, Block  # noqa: E402
 
 N = (22, 14, 11)
 
 
 def _case(precision, seed):
-    g = I.periodic_wavy_3d(N, amp=0.05, Gn=O.node_ghost(6))
+    g = I.periodic_wavy_3d(N, amp=0.05, Gn=O.node_ghost(6, 2))
     qinf = I.uniform_qinf(0.8, 10.0)
     q = I.random_smooth_state(g, qinf, amp=0.05, seed=seed)
     return (g, f32(qinf), f32(q)) if precision == B.FP_F32_MIXED else (g, np.asarray(qinf), q)
@@ -75,3 +75,60 @@ def test_fp64_weno5_of_large_states(power, characteristic):
     tol = max(1e-12, 2.0 * ulp_sensitivity(cfg, met, q130))
     assert tol <= 2e-11, tol
     assert max(rhs_err(got * 2.0 ** (130 - power), cfg, met, q130, per_component=True)) <= tol
+
+
+@pytest.mark.parametrize("scheme,power,base", [(1, -80, -50), (1, 70, 60), (0, -80, -60), (2, -80, -60), (0, 200, 100)])
+@pytest.mark.parametrize("characteristic,global_lf", [(1, 0), (0, 0), (1, 1)])
+@pytest.mark.parametrize("precision", [B.FP_F32_MIXED, B.FP_F64])
+def test_states_in_other_units(precision, characteristic, global_lf, scheme, power, base):
+    """Densities far from 1 (a thin gas in kg/m^3: 2^-80 is 8e-25) at ordinary velocities: the residual
+    has the bits of the state in other units, for linear upwind at any two units, for WENO5 and WENO7
+    where the constant 1e-6 of the weights is far above every indicator (2^-60 and below) or, in FP64,
+    far below (2^100 and above); and it is the oracle's, with the bounds of the parity suite."""
+    if power > 100 and precision == B.FP_F32_MIXED:
+        pytest.skip("beyond the FP32 range")
+    g, qinf, q = _case(B.FP_F32_MIXED, 9)               # float values in both precisions
+    kw = dict(scheme=scheme, precision=precision, characteristic=characteristic, global_lf=global_lf)
+    u = 2.0 ** base
+    want = _rhs(g, q * u, qinf * u, **kw)
+    got = _rhs(g, q * 2.0 ** power, qinf * 2.0 ** power, **kw)
+    assert np.isfinite(want).all() and np.abs(want).max() > 0
+    assert np.array_equal(got * 2.0 ** (base - power), want)
+    if power > 100:
+        return                                          # test_fp64_weno5_of_large_states
+    cfg = O.cfg_for(g, M=6, scheme=scheme, charwise=characteristic, global_lf=global_lf, qinf=qinf * 2.0 ** power)
+    met, qp = O.metrics(cfg, g.nodes, g.Gn), q * 2.0 ** power
+    tol = 1e-5 if precision == B.FP_F32_MIXED else max(1e-12, 2.0 * ulp_sensitivity(cfg, met, qp))
+    assert max(rhs_err(got, cfg, met, qp, per_component=True)) <= tol
+
+
+def test_batches_of_states_in_other_units():
+    """A batch with one block far from unit scale runs all of them by that sweep; blocks of ordinary
+    units keep to the bounds of the parity suite, and the others have their single-block bits."""
+    g, qinf, q = _case(B.FP_F32_MIXED, 10)
+    scale = [2.0 ** -70, 1.0, 2.0 ** -80]
+    for scheme in (0, 1, 2):
+        blks = [Block(g, metric_order=6, scheme=scheme, precision=B.FP_F32_MIXED, q_inf=tuple(qinf * s)) for s in scale]
+        for order in ((0, 1, 2), (1, 0, 2)):
+            bs = [blks[k] for k in order]
+            qs = [b.to_device(q * scale[k]) for b, k in zip(bs, order)]
+            for tune in (False, True):
+                bat = Batch(bs, qs, autotune=tune)
+                outs = bat.rhs([torch.full_like(x, float("nan")) for x in qs])
+                for b, k, x, o in zip(bs, order, qs, outs):
+                    if k != 1:
+                        assert torch.equal(o, b.rhs(x))
+                    cfg = O.cfg_for(g, M=6, scheme=scheme, qinf=qinf * scale[k])
+                    met = O.metrics(cfg, g.nodes, g.Gn)
+                    assert max(rhs_err(o.cpu().numpy(), cfg, met, q * scale[k], per_component=True)) <= 1e-5
+                before = [x.clone() for x in qs]
+                bat.rk3_step(1e-3)
+                torch.cuda.synchronize()
+                assert all(torch.isfinite(x).all() and not torch.equal(x, y) for x, y in zip(qs, before))
+                for x, y in zip(qs, before):
+                    x.copy_(y)
+                torch.cuda.synchronize()
+                bat.close()
+        for b in blks:
+            assert b.status() == B.FP_OK
+            b.close()

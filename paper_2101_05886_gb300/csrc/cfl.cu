@@ -218,7 +218,7 @@ __device__ __forceinline__ void atomic_max_nonneg(double *a, double v) {
 __device__ __forceinline__ float reciprocal(float x) { return 1.0f / x; }
 __device__ __forceinline__ double reciprocal(double x) { return Num<double>::rcp(x); }
 
-// sqrt(a b), correctly rounded roots (see Num::sqrt_product for the ranges)
+// sqrt(a b) by correctly rounded roots, two in FP32 and one in FP64 (as Num::sqrt_product)
 __device__ __forceinline__ float sqrt_product(float a, float b) { return sqrtf(a) * sqrtf(b); }
 __device__ __forceinline__ double sqrt_product(double a, double b) { return sqrt(a * b); }
 
@@ -265,8 +265,11 @@ __global__ void k_lam_max(const BlockDev *blocks, const int2 *items, int nitems,
       for (int d = 0; d < 3; ++d) {
         if (d >= dims) continue;
         if (d) metric(d, kj);
-        const T kx = kj[0], ky = kj[1], kz = kj[2];
-        const T U = Jc * (u * kx + v * ky + w * kz), a = fabs(Jc) * sqrt_product(c2, kx * kx + ky * ky + kz * kz);
+        // grad d = J k: FP32 forms it first, whose square stays in range for any cell size; FP64
+        // saves the operations
+        const T j = sizeof(T) == 4 ? Jc : T(1), Jo = sizeof(T) == 4 ? T(1) : Jc;
+        const T gx = j * kj[0], gy = j * kj[1], gz = j * kj[2];
+        const T U = Jo * (u * gx + v * gy + w * gz), a = fabs(Jo) * sqrt_product(c2, gx * gx + gy * gy + gz * gz);
         T lm = fabs(U - a), l0 = fabs(U), lp = fabs(U + a);
         if (!charwise) { lm = fmax(lm, lp); l0 = lm; lp = lm; }
         best[3 * d] = fmax(best[3 * d], lm);

@@ -694,7 +694,14 @@ fp_sweep(const BlockDev *__restrict__ blocks, const SweepItem *__restrict__ item
       cp[CF_H * kRing] = Num<T>::fma_(g1, e, Q[4]) * rinv;
       cp[CF_SQR * kRing] = Num<T>::sqrt_(Q[0]);
       cp[CF_UC * kRing] = Jc * dot3<T>(u0, u1, u2, k[0], k[1], k[2]);
-      cp[CF_AC * kRing] = fabs(Jc) * Num<T>::sqrt_product(gam * p * rinv, dot3<T>(k[0], k[1], k[2], k[0], k[1], k[2]));
+      // |J| c |k|.  The component-wise sweep takes no other square of k, so on it (and in the one for
+      // units far from 1) |grad d| = |J k| keeps cells beyond 2^32 or below 2^-32 in the FP32 range
+      if constexpr (sizeof(T) == 4 && FIX >= 3) {
+        const T gx = Jc * k[0], gy = Jc * k[1], gz = Jc * k[2];
+        cp[CF_AC * kRing] = Num<T>::sqrt_product(gam * p * rinv, dot3<T>(gx, gy, gz, gx, gy, gz));
+      } else {
+        cp[CF_AC * kRing] = fabs(Jc) * Num<T>::sqrt_product(gam * p * rinv, dot3<T>(k[0], k[1], k[2], k[0], k[1], k[2]));
+      }
     };
 
     // asynchronous copy of the metrics of face x + 1/2 of line (t1, t2), and of the change of the face
